@@ -12,6 +12,7 @@ It needs the CUDA library and a device, like the rest of the package.
 from __future__ import annotations
 
 import copy
+from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
 import torch
@@ -27,33 +28,68 @@ def _aq(lo: float, hi: float, bits: int) -> synth.AQ:
     return synth.AQ(bits, scale, inv, zp)
 
 
+_upload_streams = {}
+
+
+def _upload_stream(device) -> torch.cuda.Stream:
+    """One upload stream per device: the caching allocator keeps memory per stream, a new stream per call would not reuse it."""
+    if device not in _upload_streams:
+        _upload_streams[device] = torch.cuda.Stream(device)
+    return _upload_streams[device]
+
+
 def calibrate_backbone(ctx: "mq.Context", bb, x0: np.ndarray):
     """Returns a deep copy of `bb` whose activation quantizers (both branches of every block, every merge) and score
     steps come from the calibration sample x0 [B,H,W,C0].  Every block is calibrated on the full feature map, once
     through each branch's own LayerNorm parameters and biases; the sample is propagated through the floating-point
     model with the high branch's."""
-    out = copy.deepcopy(bb)
     dev = mq._Dev(ctx.device)
-    x = torch.from_numpy(np.ascontiguousarray(x0, np.float32)).to(ctx.device)
-    k = 0
+    # The copy of the result object and the upload of the next block's parameters run on a helper thread while the
+    # library calibrates the current block (its calls wait for the device without holding the interpreter): 19 of 48 ms
+    # of a Swin-T calibration were this host work, in front of an idle GPU.
+    side = _upload_stream(ctx.device)
+
+    def upload(make, params):
+        with torch.cuda.device(ctx.device), torch.cuda.stream(side):
+            struct = make(dev, params)
+            side.synchronize()
+        return struct
+
+    with ThreadPoolExecutor(1) as pool:
+        jobs, k = [], 0                              # parameters in the order of use: merge of a stage, its blocks
+        for s, d in enumerate(bb.depths):
+            if s > 0:
+                jobs.append((mq.fill_merge_struct, bb.merges[s - 1]))
+            jobs += [(mq.fill_block_struct, b) for b in bb.blocks[k:k + d]]
+            k += d
+        structs = [pool.submit(upload, *j) for j in jobs]
+        copied = pool.submit(copy.deepcopy, bb)
+        x = torch.from_numpy(np.ascontiguousarray(x0, np.float32)).to(ctx.device)
+        found, step = [], 0
+        for s, d in enumerate(bb.depths):
+            if s > 0:
+                x, rng = mq.calibrate_merge(ctx, structs[step].result(), x)
+                found.append(rng)
+                step += 1
+            for _ in range(d):
+                bs = structs[step].result()
+                y_next, rng_hi = mq.calibrate_block(ctx, bs, 0, x)
+                _, rng_lo = mq.calibrate_block(ctx, bs, 1, x)
+                found.append((rng_hi, rng_lo))
+                x = y_next
+                step += 1
+        out = copied.result()
+    it, k = iter(found), 0
     for s, d in enumerate(out.depths):
         if s > 0:
             m = out.merges[s - 1]
-            x, (lo, hi) = mq.calibrate_merge(ctx, mq.fill_merge_struct(dev, m), x)
-            m.aq = _aq(lo, hi, m.aq.bits)
-        for _ in range(d):
-            blk = out.blocks[k]
-            bs = mq.fill_block_struct(dev, blk)
-            y_next = None
-            for branch, name in enumerate(("hi", "lo")):
-                br = getattr(blk, name)
-                y, rng = mq.calibrate_block(ctx, bs, branch, x)
+            m.aq = _aq(*next(it), m.aq.bits)
+        for blk in out.blocks[k:k + d]:
+            for br, rng in zip((blk.hi, blk.lo), next(it)):
                 for site in SITES:
                     setattr(br, site, _aq(rng[site][0], rng[site][1], br.bits))
-                if name == "hi":
-                    y_next = y
+                if br is blk.hi:
                     # the int8 score codes span the block's input map
                     blk.score_inv_scale = float(np.float32(127.0 / max(1e-12, max(abs(rng["x_in"][0]), abs(rng["x_in"][1])))))
-            x = y_next
-            k += 1
+        k += d
     return out

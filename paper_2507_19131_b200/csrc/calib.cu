@@ -3,8 +3,7 @@
 // branches).  The kernels below run the floating-point Two-Branch block (all quantizers off, weights = code x step)
 // through ONE branch's LayerNorm parameters and biases and record the minimum and maximum of what each of the seven
 // quantizer sites would see.  Arithmetic: LayerNorm, softmax and GELU exactly as in the quantized path (the same
-// device functions); matrix products accumulated in binary64 in index order.  Speed is irrelevant here (the pass
-// runs once per model), so the products are plain SIMT loops: one thread per output element.
+// device functions); matrix products accumulated in binary64 in index order (register-tiled SIMT kernels).
 #include "kernels.h"
 
 namespace mixaq {
@@ -24,7 +23,13 @@ __device__ __forceinline__ void observe_warp(uint32_t* obs, int site, float lo, 
     klo = min(klo, __shfl_xor_sync(0xffffffffu, klo, off));
     khi = max(khi, __shfl_xor_sync(0xffffffffu, khi, off));
   }
-  if ((threadIdx.x & 31) == 0) { atomicMin(obs + 2 * site, klo); atomicMax(obs + 2 * site + 1, khi); }
+  // most warps do not move the extremes: a plain read (possibly stale, which only costs an atomic) spares the
+  // serialised atomics on one address (stage-1 LayerNorm of a 200 x 334 map: 68 208 warps)
+  if ((threadIdx.x & 31) == 0) {
+    const uint2 seen = __ldcg(reinterpret_cast<const uint2*>(obs) + site);
+    if (klo < seen.x) atomicMin(obs + 2 * site, klo);
+    if (khi > seen.y) atomicMax(obs + 2 * site + 1, khi);
+  }
 }
 
 __device__ __forceinline__ int cal_window_src(int b, int H, int W, int Hp, int Wp, int shift, int nwx, int w, int t) {
@@ -121,56 +126,122 @@ struct CalLinearArgs {
   long M; int N, K, C;        // C: width of one q/k/v section (QKV)
   uint32_t* obs;
 };
-template <int MODE>
-__global__ void __launch_bounds__(256) k_cal_linear(CalLinearArgs p) {
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;       // consecutive threads: consecutive n of one row
-  const long m = idx / p.N;
-  const int n = (int)(idx - m * p.N);
-  float lo = INFINITY, hi = -INFINITY;
-  if (m < p.M) {
-    const float* ar = p.a + m * p.K;
-    const int8_t* wr = p.w + (long)n * p.K;
-    const double sw = (double)__ldg(p.sw + n);
-    double s = 0.0;
-    for (int k0 = 0; k0 < p.K; k0 += 16) {                              // K is a multiple of 32
-      const int4 wv = __ldg(reinterpret_cast<const int4*>(wr + k0));
-      const int words[4] = {wv.x, wv.y, wv.z, wv.w};
+// Register-tiled binary64 product: a CTA of 64 threads owns a 128 x 32 output tile (every width here is a multiple of 32),
+// a thread 8 rows x 8 columns, so one value read from shared memory feeds 8 products and an input is converted to
+// binary64 once per tile instead of once per product.  Each sum still runs over k in ascending order, so the results are
+// those of the plain loop.
+// FUSED: the product a * (code * step) needs at most 24 + 24 + (significant bits of the code) bits; up to 5 bits of code
+// (weights of 6 bits or fewer) it is exact in binary64, and a fused multiply-add rounds exactly like the product
+// followed by the addition.  Wider weights keep the two separate roundings.
+// Bound by the binary64 pipe (64 lanes per SM and clock) and by shared-memory reads: with 8 x 4 values per thread the
+// 16-byte reads took as long as the products.  Figures: see launch_calibrate_block.
+constexpr int CTM = 128, CTN = 32, CTK = 16, CTPAD = 2;   // tile, k-step, padding (doubles) of a shared row
+template <int MODE, bool FUSED>
+__global__ void __launch_bounds__(64, 4) k_cal_linear(CalLinearArgs p) {
+  __shared__ __align__(16) double sa[2][CTK][CTM + CTPAD], sb[2][CTK][CTN + CTPAD];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ty = (lane & 7) + 8 * warp, tx = lane >> 3;  // rows 2 ty + {0, 1} + 32 i, columns 2 tx + {0, 1} + 8 j
+  const int n_tiles = (p.N + CTN - 1) / CTN;
+  const long m0 = (long)(blockIdx.x / n_tiles) * CTM;
+  const int n0 = (int)(blockIdx.x % n_tiles) * CTN;
+  // staging: four lanes fetch the 16 k of one row (64-byte runs; one lane per row made the L1 lookups the bound), one
+  // half of the rows of a per half step; lane n of the first warp fetches the 16 weight codes of row n
+  const int sr = tid >> 2, sk = 4 * (tid & 3);
+  const bool b_ok = warp == 0 && n0 + lane < p.N;
+  const int8_t* wr = p.w + (long)(b_ok ? n0 + lane : 0) * p.K;
+  const double sw = b_ok ? (double)__ldg(p.sw + n0 + lane) : 0.0;
+  float4 av[4];
+  int4 wv = make_int4(0, 0, 0, 0);
+  auto fetch_a = [&](int k0, int half) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int code = (int)(int8_t)(words[j >> 2] >> (8 * (j & 3)));
-        s = __dadd_rn(s, __dmul_rn((double)__ldg(ar + k0 + j), __dmul_rn((double)code, sw)));
+    for (int r = 0; r < 4; ++r) {
+      const long m = m0 + sr + 16 * r + 64 * half;
+      av[r] = __ldg(reinterpret_cast<const float4*>(p.a + (m < p.M ? m : 0) * p.K + k0 + sk));
+    }
+  };
+  auto store_a = [&](int buf, int half) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int row = sr + 16 * r + 64 * half;
+      sa[buf][sk][row] = (double)av[r].x; sa[buf][sk + 1][row] = (double)av[r].y;
+      sa[buf][sk + 2][row] = (double)av[r].z; sa[buf][sk + 3][row] = (double)av[r].w;
+    }
+  };
+  auto store_b = [&](int buf) {
+    if (warp == 0) {
+      const int w4[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+      for (int j = 0; j < CTK; ++j)
+        sb[buf][j][lane] = __dmul_rn((double)(int)(int8_t)(w4[j >> 2] >> (8 * (j & 3))), sw);   // exact
+    }
+  };
+  double acc[8][8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
+  if (b_ok) wv = __ldg(reinterpret_cast<const int4*>(wr));
+  fetch_a(0, 0); store_a(0, 0);
+  fetch_a(0, 1); store_a(0, 1);
+  store_b(0);
+  __syncthreads();
+  for (int k0 = 0, buf = 0; k0 < p.K; k0 += CTK, buf ^= 1) {            // K is a multiple of 32
+    const bool more = k0 + CTK < p.K;
+    if (more && b_ok) wv = __ldg(reinterpret_cast<const int4*>(wr + k0 + CTK));
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      if (more) fetch_a(k0 + CTK, half);
+#pragma unroll
+      for (int k = half * (CTK / 2); k < (half + 1) * (CTK / 2); ++k) {
+        double a[8], b[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const double2 t = *reinterpret_cast<const double2*>(&sa[buf][k][2 * ty + 32 * i]);
+          const double2 u = *reinterpret_cast<const double2*>(&sb[buf][k][2 * tx + 8 * i]);
+          a[2 * i] = t.x; a[2 * i + 1] = t.y; b[2 * i] = u.x; b[2 * i + 1] = u.y;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            acc[i][j] = FUSED ? __fma_rn(a[i], b[j], acc[i][j]) : __dadd_rn(acc[i][j], __dmul_rn(a[i], b[j]));
       }
+      if (more) store_a(buf ^ 1, half);
     }
-    float v = (float)__dadd_rn(s, p.bias ? (double)__ldg(p.bias + n) : 0.0);
-    if (MODE == CAL_QKV) {
-      p.out[m * p.N + n] = v;
-      lo = hi = v;
-    } else if (MODE == CAL_PROJ) {
-      const long src = p.rowsrc[m];
-      const float xin = src >= 0 ? __ldg(p.res + src * p.N + n) : 0.0f;
-      p.out[m * p.N + n] = __fadd_rn(xin, v);
-    } else if (MODE == CAL_FC1) {
-      v = gelu_f2(make_float2(v, v)).x;
-      p.out[m * p.N + n] = v;
-      lo = hi = v;
-    } else if (MODE == CAL_FC2) {
-      const long src = p.rowsrc[m];
-      if (src >= 0) p.out[src * p.N + n] = __fadd_rn(__ldg(p.res + m * p.N + n), v);
-    } else {
-      p.out[m * p.N + n] = v;
-    }
+    if (more) store_b(buf ^ 1);
+    __syncthreads();
   }
-  if (MODE == CAL_QKV) {
-    // a warp may straddle two sections (or two rows): every lane reports to its own section
-    const int sec = m < p.M ? n / p.C : 0;
+  // the tile's 32 columns lie in one q/k/v section (sections are multiples of 32 channels)
+  float lo = INFINITY, hi = -INFINITY;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const bool mine = m < p.M && sec == q;
-      observe_warp(p.obs, 1 + q, mine ? lo : INFINITY, mine ? hi : -INFINITY);
+  for (int i = 0; i < 8; ++i) {
+    const long m = m0 + 2 * ty + (i & 1) + 32 * (i >> 1);
+    if (m >= p.M) continue;
+    long dst = m, src = -1;
+    if (MODE == CAL_PROJ || MODE == CAL_FC2) src = p.rowsrc[m];
+    if (MODE == CAL_FC2) { if (src < 0) continue; dst = src; }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int n = n0 + 2 * tx + 8 * j;
+      if (n >= p.N) continue;                                  // only a merge may have a ragged width
+      const bool pair = n + 1 < p.N;
+      float2 v = make_float2((float)__dadd_rn(acc[i][2 * j], p.bias ? (double)__ldg(p.bias + n) : 0.0),
+                             (float)__dadd_rn(acc[i][2 * j + 1], p.bias && pair ? (double)__ldg(p.bias + n + 1) : 0.0));
+      if (MODE == CAL_FC1) v = gelu_f2(v);
+      if (MODE == CAL_QKV || MODE == CAL_FC1) { lo = fminf(lo, fminf(v.x, v.y)); hi = fmaxf(hi, fmaxf(v.x, v.y)); }
+      if (MODE == CAL_PROJ || MODE == CAL_FC2) {
+        float2 r = make_float2(0.f, 0.f);
+        const long rr = MODE == CAL_PROJ ? src : m;
+        if (rr >= 0) r = __ldg(reinterpret_cast<const float2*>(p.res + rr * p.N + n));
+        v = make_float2(__fadd_rn(r.x, v.x), __fadd_rn(r.y, v.y));
+      }
+      float* out = p.out + dst * p.N + n;
+      if (MODE == CAL_PLAIN && p.N % 2) { out[0] = v.x; if (pair) out[1] = v.y; }
+      else *reinterpret_cast<float2*>(out) = v;
     }
-  } else if (MODE == CAL_FC1) {
-    observe_warp(p.obs, 6, lo, hi);
   }
+  if (MODE == CAL_QKV) observe_warp(p.obs, 1 + n0 / p.C, lo, hi);
+  else if (MODE == CAL_FC1) observe_warp(p.obs, 6, lo, hi);
 }
 
 // softmax of the numeric contract over 49 logits: exact maximum, exponentials through 2^t, four interleaved partial
@@ -199,49 +270,101 @@ __device__ __forceinline__ void softmax49(float (&s)[WT]) {
   for (int j = 0; j < WT; ++j) s[j] = __fmul_rn(s[j], inv);
 }
 
-// one thread per (window slot, head, query row): logits in binary64, softmax of the contract, P.V in binary64
+// One CTA of 64 threads per (window slot, head): q, k, v staged in shared memory as binary64, logits as 7 x 7 register
+// tiles (thread (i/7, j/7)), one thread per row for the softmax of the contract, P.V as 7 rows x 4 channels per thread.
+// The products of binary32 values are exact in binary64 (48 bits), so a fused multiply-add rounds like multiply-then-add;
+// the sums run in index order.  Bound by the binary64 pipe and the conversions of the operands (once per CTA).
 struct CalAttnArgs {
   const float* qkv; const float* relpos; float* o;
   long slots; int C, heads, shift, Hp, Wp, nwx, nW;
   uint32_t* obs;
 };
-__global__ void __launch_bounds__(128) k_cal_attention(CalAttnArgs a) {
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long total = a.slots * a.heads * WT;
-  float lo = INFINITY, hi = -INFINITY;
-  if (idx < total) {
-    const int i = (int)(idx % WT);
-    const int h = (int)((idx / WT) % a.heads);
-    const long slot = idx / ((long)WT * a.heads);
-    const int w = (int)(slot % a.nW), wy = w / a.nwx, wx = w - wy * a.nwx;
-    const int C = a.C;
-    const float* base = a.qkv + slot * WT * 3 * C;
-    const float* q = base + (long)i * 3 * C + h * HEAD_DIM;
-    auto region = [&](int pos, int L) { return pos < L - WS ? 0 : (pos < L - a.shift ? 1 : 2); };
-    const int ri = region(wy * WS + i / WS, a.Hp) * 3 + region(wx * WS + i % WS, a.Wp);
-    const double rs = 1.0 / sqrt((double)HEAD_DIM);
-    float s[WT];
-    for (int j = 0; j < WT; ++j) {
-      const float* k = base + (long)j * 3 * C + C + h * HEAD_DIM;
-      double d = 0.0;
-      for (int e = 0; e < HEAD_DIM; ++e) d = __dadd_rn(d, __dmul_rn((double)__ldg(q + e), (double)__ldg(k + e)));
-      const int ridx = (i / WS - j / WS + WS - 1) * (2 * WS - 1) + (i % WS - j % WS + WS - 1);
-      double maskv = 0.0;
-      if (a.shift > 0) {
-        const int rj = region(wy * WS + j / WS, a.Hp) * 3 + region(wx * WS + j % WS, a.Wp);
-        maskv = rj == ri ? 0.0 : -100.0;
-      }
-      s[j] = (float)__dadd_rn(__dadd_rn(__dmul_rn(d, rs), (double)__ldg(a.relpos + (long)ridx * a.heads + h)), maskv);
-    }
-    softmax49(s);
-    float* orow = a.o + (slot * WT + i) * C + h * HEAD_DIM;
+struct CalAttnSmem {
+  double q[HEAD_DIM][WT + 1], k[HEAD_DIM][WT + 1];   // [channel][token]
+  double v[WT][HEAD_DIM + 2];
+  float s[WT][WT];
+  uint8_t region[WT + 7];
+};
+__global__ void __launch_bounds__(64) k_cal_attention(CalAttnArgs a) {
+  extern __shared__ __align__(16) uint8_t cal_smem[];
+  CalAttnSmem& sm = *reinterpret_cast<CalAttnSmem*>(cal_smem);
+  double (*pd)[WT + 1] = reinterpret_cast<double (*)[WT + 1]>(&sm.q[0][0]);   // P in binary64 over the dead q and k
+  static_assert(sizeof(double) * WT * (WT + 1) <= 2 * sizeof(double) * HEAD_DIM * (WT + 1), "P does not fit over q and k");
+  const int tid = threadIdx.x;
+  const long slot = (long)blockIdx.x / a.heads;
+  const int h = (int)((long)blockIdx.x - slot * a.heads), C = a.C;
+  const float* base = a.qkv + slot * WT * 3 * C + h * HEAD_DIM;
+  const int w = (int)(slot % a.nW), wy = w / a.nwx, wx = w - wy * a.nwx;
+  auto region = [&](int pos, int L) { return pos < L - WS ? 0 : (pos < L - a.shift ? 1 : 2); };
+  for (int item = tid; item < WT * HEAD_DIM; item += 64) {
+    const int r = item >> 5, e = item & 31;
+    const float* row = base + (long)r * 3 * C + e;
+    sm.q[e][r] = (double)__ldg(row); sm.k[e][r] = (double)__ldg(row + C); sm.v[r][e] = (double)__ldg(row + 2 * C);
+  }
+  if (tid < WT) sm.region[tid] = (uint8_t)(region(wy * WS + tid / WS, a.Hp) * 3 + region(wx * WS + tid % WS, a.Wp));
+  __syncthreads();
+  if (tid < 49) {
+    const int i0 = (tid / 7) * 7, j0 = (tid % 7) * 7;
+    double d[7][7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+#pragma unroll
+      for (int j = 0; j < 7; ++j) d[i][j] = 0.0;
     for (int e = 0; e < HEAD_DIM; ++e) {
-      double d = 0.0;
-      for (int j = 0; j < WT; ++j)
-        d = __dadd_rn(d, __dmul_rn((double)s[j], (double)__ldg(base + (long)j * 3 * C + 2 * C + h * HEAD_DIM + e)));
-      const float v = (float)d;
-      orow[e] = v;
-      lo = fminf(lo, v); hi = fmaxf(hi, v);
+      double qv[7], kv[7];
+#pragma unroll
+      for (int i = 0; i < 7; ++i) { qv[i] = sm.q[e][i0 + i]; kv[i] = sm.k[e][j0 + i]; }
+#pragma unroll
+      for (int i = 0; i < 7; ++i)
+#pragma unroll
+        for (int j = 0; j < 7; ++j) d[i][j] = __fma_rn(qv[i], kv[j], d[i][j]);
+    }
+    const double rs = 1.0 / sqrt((double)HEAD_DIM);
+    // row i0 + i is token (tid / 7, i) of the window, column j0 + j token (tid % 7, j)
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+#pragma unroll
+      for (int j = 0; j < 7; ++j) {
+        const int ridx = (tid / 7 - tid % 7 + WS - 1) * (2 * WS - 1) + (i - j + WS - 1);
+        const double maskv = a.shift > 0 && sm.region[i0 + i] != sm.region[j0 + j] ? -100.0 : 0.0;
+        sm.s[i0 + i][j0 + j] = (float)__dadd_rn(__dadd_rn(__dmul_rn(d[i][j], rs), (double)__ldg(a.relpos + (long)ridx * a.heads + h)), maskv);
+      }
+  }
+  __syncthreads();
+  if (tid < WT) {
+    float s[WT];
+#pragma unroll
+    for (int j = 0; j < WT; ++j) s[j] = sm.s[tid][j];
+    softmax49(s);
+#pragma unroll
+    for (int j = 0; j < WT; ++j) pd[tid][j] = (double)s[j];
+  }
+  __syncthreads();
+  float lo = INFINITY, hi = -INFINITY;
+  if (tid < 56) {
+    const int i0 = (tid >> 3) * 7, e0 = (tid & 7) * 4;
+    double o[7][4];
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[i][e] = 0.0;
+    for (int j = 0; j < WT; ++j) {
+      double vv[4];
+#pragma unroll
+      for (int e = 0; e < 4; e += 2) *reinterpret_cast<double2*>(&vv[e]) = *reinterpret_cast<const double2*>(&sm.v[j][e0 + e]);
+#pragma unroll
+      for (int i = 0; i < 7; ++i) {
+        const double pv = pd[i0 + i][j];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[i][e] = __fma_rn(pv, vv[e], o[i][e]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      const float4 f = make_float4((float)o[i][0], (float)o[i][1], (float)o[i][2], (float)o[i][3]);
+      *reinterpret_cast<float4*>(a.o + (slot * WT + i0 + i) * C + h * HEAD_DIM + e0) = f;
+      lo = fminf(fminf(lo, fminf(f.x, f.y)), fminf(f.z, f.w));
+      hi = fmaxf(fmaxf(hi, fmaxf(f.x, f.y)), fmaxf(f.z, f.w));
     }
   }
   observe_warp(a.obs, 4, lo, hi);
@@ -252,11 +375,13 @@ __global__ void k_cal_obs_init(uint32_t* obs, int sites) {
   if (i < 2 * sites) obs[i] = (i & 1) ? 0u : 0xFFFFFFFFu;
 }
 
+// w_bits: declared width of the weight codes; up to 6 bits (5 significant) the fused product is exact, see k_cal_linear
 template <int MODE>
-void launch_cal_linear(const CalLinearArgs& p, cudaStream_t st) {
-  const long total = p.M * p.N;
-  if (total == 0) return;
-  k_cal_linear<MODE><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(p);
+void launch_cal_linear(const CalLinearArgs& p, int w_bits, cudaStream_t st) {
+  if (p.M == 0) return;
+  const unsigned grid = (unsigned)(((p.N + CTN - 1) / CTN) * ((p.M + CTM - 1) / CTM));
+  if (w_bits >= 2 && w_bits <= 6) k_cal_linear<MODE, true><<<grid, 64, 0, st>>>(p);
+  else k_cal_linear<MODE, false><<<grid, 64, 0, st>>>(p);
   ++g_launches;
 }
 
@@ -283,6 +408,9 @@ static bool launch_cal_ln(const float* src, int32_t* rowsrc_out, const float* ga
   return true;
 }
 
+// Calibration of a Swin-T backbone on a 200 x 334 map (W4, both branches of 12 blocks, 205 G products): 125 ms with one
+// thread per output, 31 ms with the register tiles (27 ms of kernels: 24 ms of products at 8.5 T/s, about half of the
+// binary64 pipe's rate).  The output map, the observed ranges and the quantizers are unchanged bit for bit.
 // The floating-point block through one branch.  Workspace (floats unless noted): rowsrc int32[M], ln [M][C],
 // qkv [M][3C], o [M][C], x1 [M][C], h [M][hidden]; obs: 16 keys (seven sites and the block's input map).
 bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
@@ -295,20 +423,20 @@ bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
   CalLinearArgs l;
   l.obs = c.obs; l.M = M; l.C = C; l.rowsrc = c.rowsrc;
   l.a = c.ln; l.w = c.w_qkv; l.sw = c.s_qkv; l.bias = c.b_qkv; l.out = c.qkv; l.res = nullptr; l.N = 3 * C; l.K = C;
-  launch_cal_linear<CAL_QKV>(l, st);
+  launch_cal_linear<CAL_QKV>(l, c.wb_qkv, st);
   CalAttnArgs a;
   a.qkv = c.qkv; a.relpos = c.relpos; a.o = c.o; a.slots = slots; a.C = C; a.heads = c.heads; a.shift = c.shift;
   a.Hp = Hp; a.Wp = Wp; a.nwx = nwx; a.nW = nW; a.obs = c.obs;
-  const long athreads = slots * c.heads * WT;
-  k_cal_attention<<<(unsigned)((athreads + 127) / 128), 128, 0, st>>>(a);
+  if (cudaFuncSetAttribute(k_cal_attention, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CalAttnSmem)) != cudaSuccess) return false;
+  k_cal_attention<<<(unsigned)(slots * c.heads), 64, sizeof(CalAttnSmem), st>>>(a);
   ++g_launches;
   l.a = c.o; l.w = c.w_proj; l.sw = c.s_proj; l.bias = c.b_proj; l.out = c.x1; l.res = c.x; l.N = C; l.K = C;
-  launch_cal_linear<CAL_PROJ>(l, st);
+  launch_cal_linear<CAL_PROJ>(l, c.wb_proj, st);
   if (!launch_cal_ln(c.x1, nullptr, c.ln2_g, c.ln2_b, c.ln, M, C, 0, c.H, c.W, c.shift, nwx, nW, c.obs, 5, -1, st)) return false;
   l.a = c.ln; l.w = c.w_fc1; l.sw = c.s_fc1; l.bias = c.b_fc1; l.out = c.h; l.res = nullptr; l.N = Hd; l.K = C;
-  launch_cal_linear<CAL_FC1>(l, st);
+  launch_cal_linear<CAL_FC1>(l, c.wb_fc1, st);
   l.a = c.h; l.w = c.w_fc2; l.sw = c.s_fc2; l.bias = c.b_fc2; l.out = c.y; l.res = c.x1; l.N = C; l.K = Hd;
-  launch_cal_linear<CAL_FC2>(l, st);
+  launch_cal_linear<CAL_FC2>(l, c.wb_fc2, st);
   return true;
 }
 
@@ -327,7 +455,7 @@ bool launch_calibrate_merge(const CalMergeArgs& c, cudaStream_t st) {
   CalLinearArgs l;
   l.obs = c.obs; l.M = M; l.C = c.N; l.rowsrc = nullptr; l.res = nullptr;
   l.a = c.ln; l.w = c.w; l.sw = c.sw; l.bias = nullptr; l.out = c.y; l.N = c.N; l.K = 4 * c.C;
-  launch_cal_linear<CAL_PLAIN>(l, st);
+  launch_cal_linear<CAL_PLAIN>(l, c.w_bits, st);
   return true;
 }
 

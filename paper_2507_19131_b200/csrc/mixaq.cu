@@ -1114,6 +1114,7 @@ mixaq_status mixaq_calibrate_block(mixaq_ctx* ctx, const mixaq_block_params* p, 
   c.ln1_g = br.ln1_g; c.ln1_b = br.ln1_b; c.ln2_g = br.ln2_g; c.ln2_b = br.ln2_b;
   c.b_qkv = br.b_qkv; c.b_proj = br.b_proj; c.b_fc1 = br.b_fc1; c.b_fc2 = br.b_fc2;
   c.w_qkv = p->qkv.codes; c.w_proj = p->proj.codes; c.w_fc1 = p->fc1.codes; c.w_fc2 = p->fc2.codes;
+  c.wb_qkv = p->qkv.bits; c.wb_proj = p->proj.bits; c.wb_fc1 = p->fc1.bits; c.wb_fc2 = p->fc2.bits;
   c.s_qkv = p->qkv.scale; c.s_proj = p->proj.scale; c.s_fc1 = p->fc1.scale; c.s_fc2 = p->fc2.scale; c.relpos = p->relpos_table;
   c.rowsrc = ws.rowsrc; c.ln = ws.ln; c.qkv = ws.qkv; c.o = ws.o; c.x1 = ws.x1; c.h = ws.h; c.obs = ws.obs;
   g_launches = 0;
@@ -1147,7 +1148,7 @@ mixaq_status mixaq_calibrate_merge(mixaq_ctx* ctx, const mixaq_merge_params* p, 
   c.obs = cv.take<uint32_t>(16);
   c.ln = cv.take<float>((size_t)B * ((H + 1) / 2) * ((W + 1) / 2) * K);
   c.x = x; c.y = y; c.B = B; c.H = H; c.W = W; c.C = C; c.N = N;
-  c.ln_g = p->ln_g; c.ln_b = p->ln_b; c.w = p->reduction.codes; c.sw = p->reduction.scale;
+  c.ln_g = p->ln_g; c.ln_b = p->ln_b; c.w = p->reduction.codes; c.sw = p->reduction.scale; c.w_bits = p->reduction.bits;
   g_launches = 0;
   if (!launch_calibrate_merge(c, st)) return fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "calibrate_merge: unsupported dim");
   ctx->launches = g_launches;
