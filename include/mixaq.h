@@ -256,9 +256,9 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
 /* mixaq_backbone_forward replays a CUDA graph when it is called again with exactly the same arguments (same
  * parameter structs byte for byte, pointers, sizes, ratios, workspace and stream): the first such call captures the
  * launches on `cuda_stream`, later calls cost one graph launch on the host.  The data behind the pointers may
- * change freely between calls.  Captured graphs are kept per context (16 at most) until mixaq_destroy.  Caching
- * needs a stream that can be captured: calls on the legacy default stream (NULL), calls made while the caller is
- * capturing the stream itself launch their kernels directly.  A call between mixaq_profile_begin/end is captured
+ * change freely between calls.  Captured graphs are kept per context (16 at most) until mixaq_destroy.  A call on the
+ * legacy default stream (NULL), which cannot be captured, is recorded on a stream of the context's own and its graph
+ * launched on the legacy stream; a call made while the caller is capturing the stream itself launches its kernels directly.  A call between mixaq_profile_begin/end is captured
  * together with its event records, launched once and not cached.
  * enabled = 0 switches the cache off and drops the stored graphs; it is on by default. */
 mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled);

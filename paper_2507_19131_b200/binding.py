@@ -135,7 +135,8 @@ def branch_counts(H: int, W: int, low_ratio: float, prune_ratio: float = 0.0, wi
 
 
 def _stream_ptr() -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle of torch's current stream (building a Stream object for it costs more than a launch)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -530,10 +531,9 @@ def backbone_forward(ctx: Context, dbb: DeviceBackbone, x0: torch.Tensor, low_ra
     """mixaq_backbone_forward.  Returns the per-stage output tensors owned by `dbb` (overwritten by the next call)."""
     assert x0.is_cuda and x0.dtype == torch.float32 and x0.is_contiguous()
     assert tuple(x0.shape[:3]) == (dbb.B, dbb.H0, dbb.W0)
-    lr = (C.c_float * dbb.npairs)(*[float(r) for r in low_ratios][:dbb.npairs])
-    pr = None
-    if prune_ratios is not None:
-        pr = (C.c_float * dbb.npairs)(*[float(r) for r in prune_ratios][:dbb.npairs])
+    n = dbb.npairs
+    lr = (C.c_float * n)(*low_ratios[:n])
+    pr = (C.c_float * n)(*prune_ratios[:n]) if prune_ratios is not None else None
     st = lib().mixaq_backbone_forward(ctx.h, C.byref(dbb.s), _ptr(x0), dbb.out_ptrs, dbb.B, dbb.H0, dbb.W0, lr, pr,
                                       _ptr(dbb.ws), C.c_size_t(dbb.ws.numel()), _stream_ptr())
     ctx.check(st, "backbone_forward")

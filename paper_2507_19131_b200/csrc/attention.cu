@@ -74,6 +74,7 @@ __device__ __forceinline__ uint32_t squeeze_pairs(uint32_t t) {
 // TAPS: the debug taps (softmax output, P codes, P.V accumulators) are compiled in only for calls that ask for them
 template <bool SHIFTED, bool TAPS>
 __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
+  griddep_launch();
   __shared__ __align__(16) WarpSmem sm;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
   const long row_bytes = (long)3 * C * cbits / 8;
   const int zq = br.q.zp, zk = br.k.zp, zv = br.v.zp;
 
+  griddep_wait();
   // ---- stage q, k (rows) and v (transposed, permuted) of this head, one code per byte: 3 x 64 row items ----
   int wy = 0, wx = 0;
   if (SHIFTED) { const int w = br.win[slot]; wy = w / a.nwx; wx = w - wy * a.nwx; }
@@ -316,11 +318,11 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   const unsigned grid = (unsigned)problems;
   const bool taps = a.br[0].tap_p || a.br[0].tap_pv || a.br[0].tap_probs || a.br[1].tap_p || a.br[1].tap_pv || a.br[1].tap_probs;
   if (a.shift > 0) {
-    if (taps) k_attention<true, true><<<grid, ATT_WARPS * 32, 0, st>>>(a);
-    else      k_attention<true, false><<<grid, ATT_WARPS * 32, 0, st>>>(a);
+    if (taps) launch_pdl(k_attention<true, true>, dim3(grid), ATT_WARPS * 32, 0, st, a);
+    else      launch_pdl(k_attention<true, false>, dim3(grid), ATT_WARPS * 32, 0, st, a);
   } else {
-    if (taps) k_attention<false, true><<<grid, ATT_WARPS * 32, 0, st>>>(a);
-    else      k_attention<false, false><<<grid, ATT_WARPS * 32, 0, st>>>(a);
+    if (taps) launch_pdl(k_attention<false, true>, dim3(grid), ATT_WARPS * 32, 0, st, a);
+    else      launch_pdl(k_attention<false, false>, dim3(grid), ATT_WARPS * 32, 0, st, a);
   }
   ++g_launches;
 }

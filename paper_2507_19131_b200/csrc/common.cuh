@@ -11,6 +11,15 @@ constexpr int WS = 7;         // window side
 constexpr int WT = 49;        // tokens per window
 constexpr int HEAD_DIM = 32;
 
+// Programmatic dependent launch.  Every kernel of a forward is launched so that its CTAs may start while the kernel before it
+// in the stream still runs (launch_pdl in kernels.h): griddep_launch() lets the next kernel start, griddep_wait() returns when the kernel before
+// has finished and its writes are visible.  Before the wait a kernel may only read what no kernel of the forward writes
+// (weights, derived tables, its parameters) and must not write global memory.  The kernels that can come first in a call
+// (energy, window score, stem, merge gather) let their successor start only after their own wait: whatever the caller's
+// stream did before the call (preparing the tables, say) is then complete for every kernel of the call.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 struct AQ {                   // activation quantizer in kernel-friendly form
   float scale, inv_scale, zpf, qmaxf;
   int zp, bits;
@@ -45,8 +54,7 @@ __device__ __forceinline__ float2 exp2_core2(float2 t) {
 }
 
 // GELU(v) = max(v,0) - a*Phi(-a), a = min(|v|, 5); log2 Phi(-a) is a degree-7 polynomial on [0,5].
-__device__ __forceinline__ float2 gelu_f2(float2 v) {
-  const float2 a = make_float2(fminf(fabsf(v.x), 5.0f), fminf(fabsf(v.y), 5.0f));
+__device__ __forceinline__ float2 gelu_log2_tail2(float2 a) {      // log2 Phi(-a) on [0, 5]
   float2 q = f2(__uint_as_float(0xb5d6f9e3u));
   q = __ffma2_rn(q, a, f2(__uint_as_float(0x38729e20u)));
   q = __ffma2_rn(q, a, f2(__uint_as_float(0xba6dcc74u)));
@@ -54,7 +62,11 @@ __device__ __forceinline__ float2 gelu_f2(float2 v) {
   q = __ffma2_rn(q, a, f2(__uint_as_float(0xbd5c93e3u)));
   q = __ffma2_rn(q, a, f2(__uint_as_float(0xbeeac5d4u)));
   q = __ffma2_rn(q, a, f2(__uint_as_float(0xbf935b8fu)));
-  q = __ffma2_rn(q, a, f2(__uint_as_float(0xbf7fffbeu)));
+  return __ffma2_rn(q, a, f2(__uint_as_float(0xbf7fffbeu)));
+}
+__device__ __forceinline__ float2 gelu_f2(float2 v) {
+  const float2 a = make_float2(fminf(fabsf(v.x), 5.0f), fminf(fabsf(v.y), 5.0f));
+  const float2 q = gelu_log2_tail2(a);
   const float2 h = __fmul2_rn(a, exp2_core2(q));
   return sub2(make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f)), h);
 }
@@ -65,6 +77,13 @@ __device__ __forceinline__ void quant_magic2(float2 x, float inv_scale, float lo
   t = make_float2(fminf(fmaxf(t.x, lo), hi), fminf(fmaxf(t.y, lo), hi));
   t = __fadd2_rn(t, f2(12582912.0f));
   m0 = __float_as_uint(t.x); m1 = __float_as_uint(t.y);
+}
+
+// 2^t by the special-function unit (relative error at most 2^-22), for values that are checked before they decide a code
+__device__ __forceinline__ float ex2_approx(float t) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+  return r;
 }
 
 // q = clamp(rne(x*inv_scale) + zp, 0, qmax), evaluated without a rounding or conversion instruction:
@@ -87,28 +106,50 @@ __device__ __forceinline__ uint32_t pack_const(int zp, int bits) {
   const uint32_t k = (uint32_t)zp - kMagicBits;
   return k * (bits == 8 ? 0x01010101u : (bits == 4 ? 0x11111111u : 0x55555555u));
 }
-// NC (16 or 32) consecutive codes of one row, given as magic patterns, packed and stored with one or two vector
-// stores (dst is NC*BITS/8-byte aligned).
-template <int BITS, int NC>
-__device__ __forceinline__ void store_magic(uint8_t* dst, const uint32_t (&m)[NC], uint32_t kpack) {
-  constexpr int PER = 32 / BITS, WORDS = NC / PER;   // codes per word, words
-  uint32_t w[WORDS];
+// Four unclamped codes to one word, one per byte, clamped to [0, 2^bits - 1]: m holds the rounding patterns
+// 0x4B400000 + n, and (m << SH) + bias is (n + zp) << SH for bias = (zp - 0x4B400000) << SH, SH = 8 - bits.  The
+// saturating byte conversion then clamps both ends at once: codes above the range become 255, whose top `bits` bits are
+// all ones.  1.5 instructions per code against 3 for two binary32 clamps and a shifted add.  For bits < 8 the codes come
+// out in the top bits of their bytes.
+template <int SH>
+__device__ __forceinline__ uint32_t sat_pack4(uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3, uint32_t bias) {
+  uint32_t d;
+  asm("{\n\t.reg .b32 t;\n\t"
+      "cvt.pack.sat.u8.s32.b32 t, %4, %3, 0;\n\t"
+      "cvt.pack.sat.u8.s32.b32 %0, %2, %1, t;\n\t}"
+      : "=r"(d) : "r"((m0 << SH) + bias), "r"((m1 << SH) + bias), "r"((m2 << SH) + bias), "r"((m3 << SH) + bias));
+  return d;
+}
+// Stores 32 codes of one row (eight words of sat_pack4): one code per byte (cbits = 8, codes of `bits` bits) or packed at
+// cbits = bits = 4 or 2.  dst is 4 * cbits bytes aligned.
+__device__ __forceinline__ void store_sat32(uint8_t* dst, uint32_t (&w)[8], int bits, int cbits) {
+  if (cbits == 8) {
+    if (bits < 8) {
+      const int sh = 8 - bits;
+      const uint32_t mask = bits == 4 ? 0x0F0F0F0Fu : 0x03030303u;
 #pragma unroll
-  for (int i = 0; i < WORDS; ++i) {
-    uint32_t v = kpack;
+      for (int i = 0; i < 8; ++i) w[i] = (w[i] >> sh) & mask;
+    }
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  } else if (cbits == 4) {
+    // bytes 0 and 1 of a word hold codes 0 and 1 in their high nibbles: the pair is (byte 0 >> 4) | (byte 1 & 0xF0)
+    uint32_t n[8];
 #pragma unroll
-    for (int e = 0; e < PER; ++e) v += m[PER * i + e] << (BITS * e);
-    w[i] = v;
-  }
-  if (WORDS == 8) {
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4 % WORDS], w[5 % WORDS], w[6 % WORDS], w[7 % WORDS]);
-  } else if (WORDS == 4) {
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1 % WORDS], w[2 % WORDS], w[3 % WORDS]);
-  } else if (WORDS == 2) {
-    reinterpret_cast<uint2*>(dst)[0] = make_uint2(w[0], w[1 % WORDS]);
+    for (int i = 0; i < 8; ++i) n[i] = ((w[i] >> 4) & 0x000F000Fu) | ((w[i] >> 8) & 0x00F000F0u);
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(__byte_perm(n[0], n[1], 0x6420), __byte_perm(n[2], n[3], 0x6420),
+                                                  __byte_perm(n[4], n[5], 0x6420), __byte_perm(n[6], n[7], 0x6420));
   } else {
-    reinterpret_cast<uint32_t*>(dst)[0] = w[0];
+    // four codes in the top two bits of four bytes to one byte
+    uint32_t n[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t t = ((w[i] >> 6) & 0x00030003u) | ((w[i] >> 12) & 0x000C000Cu);     // codes 0, 1 and codes 2, 3
+      n[i] = t | (t >> 12);
+    }
+    reinterpret_cast<uint2*>(dst)[0] =
+        make_uint2(__byte_perm(__byte_perm(n[0], n[1], 0x0040), __byte_perm(n[2], n[3], 0x0040), 0x5410),
+                   __byte_perm(__byte_perm(n[4], n[5], 0x0040), __byte_perm(n[6], n[7], 0x0040), 0x5410));
   }
 }
 

@@ -1,25 +1,42 @@
 // Fused epilogues of the integer GEMMs (MixA-Q Section 3.2: shared integer weights, per-branch step sizes,
 // zero points and biases).  One epilogue warp owns 32 rows (one TMEM lane quarter, one row per thread) and every
-// c_step-th 16-column chunk of the tile (the warps that share a lane quarter deal the chunks round-robin):
-//   acc_raw[n] = sum_k a[m][k] * w[n][k]   with UNSIGNED activation codes a;
-//   acc[n]     = acc_raw[n] - z_a * sum_k w[n][k]                (zero-point correction, exact in int32)
+// c_step-th 32-column chunk of the tile (the warps that share a lane quarter deal the chunks round-robin):
+//   raw[n] = sum_k a[m][k] * w[n][k]                   with UNSIGNED activation codes a;
+//   acc[n] = raw[n] - z_a * sum_k w[n][k]              (zero-point correction, exact in int32)
 //   v[n]       = fma((float)acc[n], s_a*s_w[n], bias[n])
-// The per-column constants (zc, mult, bias) of the warp's columns sit in shared memory; every lane reads the same
+// The per-column constants (pre, mult, bias) sit in shared memory; every lane reads the same
 // column, so the reads are broadcasts.
 #pragma once
 #include "kernels.h"
+#include <type_traits>
 
 namespace mixaq {
 
-constexpr int EPI_NC = 16;                             // columns per chunk
-constexpr int EPI_STAGE_FLOATS = 32 * EPI_NC;          // per-warp transposition tile of the binary32 epilogues
+constexpr int CODE_NC = 32, F32_NC = 16;               // columns per chunk of the code and of the binary32 epilogues
+constexpr int EPI_STAGE_FLOATS = 32 * F32_NC;          // per-warp transposition tile of the binary32 epilogues
 
-struct ColConsts {                                     // shared-memory arrays indexed by the warp's local column
-  const int32_t* zc; const float* mult; const float* bias;
+struct ColConsts {                                     // shared-memory arrays indexed by the column within the tile
+  const int32_t* pre; const float* mult; const float* bias;
 };
 
-// Asynchronous TMEM load of 16 columns (one row per thread); the registers are valid after tmem_ld_wait().
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, int32_t (&r)[16]) {
+// Asynchronous TMEM load of 8 / 16 / 32 columns (one row per thread); the registers are valid after tmem_ld_wait().
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, int32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, int32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, int32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -29,11 +46,23 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, int32_t (&r)[16]
 }
 // Waits for every TMEM load issued so far.  The registers pass through the statement as in-out operands so that
 // no use of them can be scheduled ahead of the wait.
+__device__ __forceinline__ void tmem_ld_wait(int32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+        "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+        "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+      :: "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait(int32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
       : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
         "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
       :: "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(int32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]) :: "memory");
 }
 
 // asynchronous 16-byte copy global -> shared (no register staging); groups complete in order
@@ -45,19 +74,26 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 constexpr int RES_SLOTS = 4;                           // residual chunks a warp keeps in flight (32 x 16 floats each)
 
-// zero-point correction + dequantization of one chunk; lc0 = first column of the chunk in the warp's constants
-template <int MODE, bool TAPS>
-__device__ __forceinline__ void dequant16(const GemmBranch& br, int N, long m, bool row_ok, int n0, int lc0,
-                                          const ColConsts& cc, const int32_t (&acc_raw)[16], float (&v)[16]) {
+// raw + pre[n] is 0x4B400000 + acc: the zero point is taken out, and while |acc| < 2^22 (IN_RANGE) those bits ARE the
+// binary32 number 1.5 * 2^23 + acc, so one packed subtraction converts two of them.
+template <bool IN_RANGE>
+__device__ __forceinline__ float2 acc_to_float2(int32_t a, int32_t b) {
+  if (IN_RANGE) return __fadd2_rn(make_float2(__int_as_float(a), __int_as_float(b)), f2(-12582912.0f));
+  return make_float2(__int2float_rn(a - (int32_t)kMagicBits), __int2float_rn(b - (int32_t)kMagicBits));
+}
+// dequantization of NC columns; lc0 = first column in the warp's constants, n0 = its global index
+template <int MODE, bool TAPS, bool IN_RANGE, int NC>
+__device__ __forceinline__ void dequant(const GemmBranch& br, int N, long m, bool row_ok, int n0, int lc0, const ColConsts& cc,
+                                        const int32_t* acc, float (&v)[NC]) {
   if (TAPS && br.tap_acc && row_ok) {
 #pragma unroll
-    for (int i = 0; i < EPI_NC; ++i) br.tap_acc[m * N + n0 + i] = acc_raw[i] - cc.zc[lc0 + i];
+    for (int i = 0; i < NC; ++i) br.tap_acc[m * N + n0 + i] = acc[i] + cc.pre[lc0 + i] - (int32_t)kMagicBits;
   }
 #pragma unroll
-  for (int i4 = 0; i4 < EPI_NC / 4; ++i4) {
-    const int4 z4 = *reinterpret_cast<const int4*>(cc.zc + lc0 + 4 * i4);
+  for (int i4 = 0; i4 < NC / 4; ++i4) {
+    const int4 p4 = *reinterpret_cast<const int4*>(cc.pre + lc0 + 4 * i4);
+    const int pp[4] = {p4.x, p4.y, p4.z, p4.w};
     const float4 m4 = *reinterpret_cast<const float4*>(cc.mult + lc0 + 4 * i4);
-    const int zz[4] = {z4.x, z4.y, z4.z, z4.w};
     const float mm[4] = {m4.x, m4.y, m4.z, m4.w};
     float bb[4] = {0.f, 0.f, 0.f, 0.f};
     if (MODE != EPI_MERGE) {
@@ -68,7 +104,7 @@ __device__ __forceinline__ void dequant16(const GemmBranch& br, int N, long m, b
 #pragma unroll
     for (int j = 0; j < 4; j += 2) {
       const int i = 4 * i4 + j;
-      const float2 f = make_float2(__int2float_rn(acc_raw[i] - zz[j]), __int2float_rn(acc_raw[i + 1] - zz[j + 1]));
+      const float2 f = acc_to_float2<IN_RANGE>(acc[i] + pp[j], acc[i + 1] + pp[j + 1]);
       const float2 r = MODE == EPI_MERGE ? __fmul2_rn(f, make_float2(mm[j], mm[j + 1]))
                                          : __ffma2_rn(f, make_float2(mm[j], mm[j + 1]), make_float2(bb[j], bb[j + 1]));
       v[i] = r.x; v[i + 1] = r.y;
@@ -76,76 +112,168 @@ __device__ __forceinline__ void dequant16(const GemmBranch& br, int N, long m, b
   }
 }
 
+// ---- quantizers of the code outputs ------------------------------------------------------------------------------------
+// Both leave rne(x * inv_scale) (FC1: + zp) in the low 16 bits of every pattern, unclamped; sat_pack4 adds, clamps and
+// packs.  They need |x * inv_scale| < 2^15, which `in_range` of the caller guarantees (vbound + |bias|, times inv_scale);
+// launches for which that cannot be shown take the exact functions with their binary32 clamps.
+constexpr float kPatternRange = 30000.0f;
+
+// QKV: t = x * inv_scale rounded, then the rounding add.  A packed multiply feeding a packed add would be contracted into
+// one rounding; the multiply is therefore written as fma(x, inv_scale, -0) (same value) with a -0 the compiler cannot see.
+__device__ __forceinline__ void quant_pattern2(float2 x, float inv_scale, float neg_zero, uint32_t& m0, uint32_t& m1) {
+  const float2 t = __fadd2_rn(__ffma2_rn(x, f2(inv_scale), f2(neg_zero)), f2(12582912.0f));
+  m0 = __float_as_uint(t.x); m1 = __float_as_uint(t.y);
+}
+// FC1: code of GELU(v) from the special-function exponential instead of the contract's polynomial (a third of the
+// packed operations).  The value can differ from the contract's in the last bits, so `dist` collects the largest distance
+// to the nearest integer; where it comes within the error bound of one half (see gelu_threshold) the caller recomputes.
+// The zero point is part of the rounding constant; at exact ties that changes the parity rule, and ties are recomputed.
+__device__ __forceinline__ void gelu_pattern2(float2 v, float inv_scale, float magic_zp, float& dist, uint32_t& m0, uint32_t& m1) {
+  const float2 a = make_float2(fminf(fabsf(v.x), 5.0f), fminf(fabsf(v.y), 5.0f));
+  const float2 q = gelu_log2_tail2(a);
+  const float2 h = __fmul2_rn(a, make_float2(ex2_approx(q.x), ex2_approx(q.y)));
+  const float2 g = sub2(make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f)), h);
+  const float2 t = __fmul2_rn(g, f2(inv_scale));
+  const float2 r = __fadd2_rn(t, f2(magic_zp));
+  const float2 d = sub2(t, __fadd2_rn(r, f2(-magic_zp)));
+  dist = fmaxf(fmaxf(dist, fabsf(d.x)), fabsf(d.y));
+  m0 = __float_as_uint(r.x); m1 = __float_as_uint(r.y);
+}
+// Error of t = g * inv_scale between the two evaluations: both exponentials are within 2^-22 of 2^q, h = a 2^q <= 0.17, so
+// h differs by at most 0.17 * 2^-21 + one rounding < 1.0e-7; the roundings of g and t add |t| * 2^-22, and |t| <= qmax + 1
+// for every t that is not clamped anyway.
+__device__ __forceinline__ float gelu_threshold(float inv_scale, float qmaxf) {
+  return 0.5f - __fmaf_rn(inv_scale, 1.1e-7f, (qmaxf + 1.0f) * 2.4e-7f);
+}
+
+// What a warp's epilogue needs of its branch, read once per branch (the parameters sit in constant memory, and a tile used
+// to read them again field by field).
+struct EpiBranch {
+  int M, bits, cbits;                                      // code outputs: width of the codes, bits a stored code takes
+  uint8_t* out_codes; float* out_f; const float* res; const int32_t* rowsrc;
+  long row_bytes;                                          // code outputs: bytes of an output row
+  float qmaxf;                                             // largest code
+  __device__ __forceinline__ EpiBranch(const GemmBranch& b, int N)
+      : M(b.M), bits(b.q0.bits), cbits(b.out_bits), out_codes(b.out_codes), out_f(b.out_f), res(b.res), rowsrc(b.rowsrc),
+        row_bytes((long)N * b.out_bits / 8), qmaxf(b.q0.qmaxf) {}
+};
+
 // The warp's part of one output tile.  taddr: TMEM address of (the warp's lane quarter, the tile's first column);
 // n_tile0: global index of that column; the warp owns the tile's chunks c_first, c_first + c_step, ... < c_total
-// (its constants are stored densely: chunk number j of the warp at local column 16 j);
+// cc: the constants of the tile's columns;
+// in_range: the code outputs of the tile's columns cannot leave the pattern's range (see quant_pattern2);
 // acc_ready(): waits (bounded) for the tile's accumulator, false when the CTA is giving up.
 template <int MODE, bool TAPS, class WaitFn>
-__device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, int N, int C, long row0, int lane, int n_tile0,
+__device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const EpiBranch& eb, int N, int C, long row0, int lane, int n_tile0,
                                                    int c_first, int c_step, int c_total, const ColConsts& cc,
-                                                   uint32_t taddr_tile, float* stage, WaitFn acc_ready,
+                                                   uint32_t taddr_tile, float* stage, bool in_range, float neg_zero, WaitFn acc_ready,
                                                    float* res_ring = nullptr /* per warp: RES_SLOTS x 32 x 16 floats */) {
   const long m = row0 + lane;
-  const bool row_ok = m < br.M;
+  const bool row_ok = m < eb.M;
+  constexpr int NC = MODE == EPI_QKV || MODE == EPI_FC1 ? CODE_NC : F32_NC;
   const int n_chunks = c_first < c_total ? (c_total - c_first + c_step - 1) / c_step : 0;
-  const int n_first = n_tile0 + c_first * EPI_NC;          // global column of the warp's first chunk
-  const int col_step = c_step * EPI_NC;                    // distance between consecutive chunks of the warp
-  const uint32_t taddr = taddr_tile + (uint32_t)(c_first * EPI_NC);
+  const int n_first = n_tile0 + c_first * NC;              // global column of the warp's first chunk
+  const int col_step = c_step * NC;                        // distance between consecutive chunks of the warp
+  const uint32_t taddr = taddr_tile + (uint32_t)(c_first * NC);
 
   if (MODE == EPI_QKV || MODE == EPI_FC1) {
-    // ---- code outputs: every thread quantizes and packs the 16 codes of its own row ----
+    // ---- code outputs: every thread quantizes and packs the 32 codes of its own row ----
+    // a tile lies within one of the q, k, v sections (pick_bn), so its quantizer is the tile's
+    const AQ& q = MODE == EPI_FC1 || n_tile0 < C ? br.q0 : (n_tile0 < 2 * C ? br.q1 : br.q2);
+    const float inv_scale = q.inv_scale, zpf = q.zpf;
+    const int cbits = eb.cbits, bits = eb.bits;
+    const uint32_t zbias = (MODE == EPI_FC1 ? 0u : (uint32_t)q.zp) - kMagicBits;
+    const float magic_zp = 12582912.0f + zpf;                              // FC1
+    const float thr = gelu_threshold(inv_scale, eb.qmaxf);                 // FC1
+    // this thread's output position of the warp's first chunk
+    uint8_t* out_ptr = eb.out_codes + m * eb.row_bytes + n_first * cbits / 8;
+    const int out_step = col_step * cbits / 8;
     if (!acc_ready()) return false;
-    const int bits = br.out_bits;
-    // this thread's output position of the warp's first chunk; packing constants of the (up to three) quantizers
-    uint8_t* out_ptr = br.out_codes + m * ((long)N * bits / 8) + (long)n_first * bits / 8;
-    const int out_step = col_step * bits / 8;
-    const uint32_t kp0 = pack_const(br.q0.zp, bits);
-    const uint32_t kp1 = MODE == EPI_QKV ? pack_const(br.q1.zp, bits) : kp0;
-    const uint32_t kp2 = MODE == EPI_QKV ? pack_const(br.q2.zp, bits) : kp0;
-    const int n_k = C, n_v = 2 * C;                      // first columns of the k and v sections (QKV)
-    auto chunk = [&](int ch, const int32_t (&acc)[EPI_NC]) {
-      const int n0 = n_first + ch * col_step;
-      float v[EPI_NC];
-      dequant16<MODE, TAPS>(br, N, m, row_ok, n0, ch * EPI_NC, cc, acc, v);
-      AQ q = br.q0;
-      uint32_t kp = kp0;
-      if (MODE == EPI_QKV) { if (n0 >= n_v) { q = br.q2; kp = kp2; } else if (n0 >= n_k) { q = br.q1; kp = kp1; } }
-      uint32_t c[EPI_NC];
-      const float q_lo = -q.zpf, q_hi = q.qmaxf - q.zpf;
+    // the quantizer's width as a constant (a shift in the packing)
+    auto walk = [&](auto bits_tag, auto range_tag) {
+      constexpr int SH = 8 - decltype(bits_tag)::value;
+      constexpr bool IN_RANGE = decltype(range_tag)::value;
+      // eight columns by the contract's own operations (values out of range, or too close to a rounding boundary)
+      auto exact8 = [&](int col, const int32_t* acc, uint32_t& w0, uint32_t& w1) {
+        float v[8];
+        uint32_t c[8];
+        dequant<MODE, TAPS, IN_RANGE, 8>(br, N, m, row_ok, n_tile0 + col, col, cc, acc, v);
 #pragma unroll
-      for (int i = 0; i < EPI_NC; i += 2) {
-        float2 g = make_float2(v[i], v[i + 1]);
-        if (MODE == EPI_FC1) g = gelu_f2(g);
-        quant_magic2(g, q.inv_scale, q_lo, q_hi, c[i], c[i + 1]);
-      }
-      if (row_ok) {
-        uint8_t* dst = out_ptr + ch * out_step;
-        if (bits == 8) store_magic<8, EPI_NC>(dst, c, kp);
-        else if (bits == 4) store_magic<4, EPI_NC>(dst, c, kp);
-        else store_magic<2, EPI_NC>(dst, c, kp);
+        for (int i = 0; i < 8; i += 2) {
+          const float2 x = make_float2(v[i], v[i + 1]);
+          quant_magic2(MODE == EPI_FC1 ? gelu_f2(x) : x, inv_scale, -zpf, eb.qmaxf - zpf, c[i], c[i + 1]);
+        }
+        const uint32_t zb = (uint32_t)q.zp - kMagicBits;
+        w0 = sat_pack4<SH>(c[0], c[1], c[2], c[3], zb << SH);
+        w1 = sat_pack4<SH>(c[4], c[5], c[6], c[7], zb << SH);
+      };
+      // 32 columns at a time, without a branch between them: the dependent chain of a value is about twenty operations
+      // long, and with four warps per scheduler only independent values hide its latency
+#pragma unroll 1
+      for (int ch = 0; ch < n_chunks; ++ch) {
+        const uint32_t ta = taddr + (uint32_t)(ch * col_step);
+        const int col = c_first * CODE_NC + ch * col_step;
+        int32_t acc[CODE_NC];
+        uint32_t w[8];
+        tmem_ld(ta, acc);
+        tmem_ld_wait(acc);
+        float dist[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          if (!IN_RANGE) { exact8(col + 8 * g, acc + 8 * g, w[2 * g], w[2 * g + 1]); continue; }
+          float v[8];
+          uint32_t c[8];
+          dequant<MODE, TAPS, IN_RANGE, 8>(br, N, m, row_ok, n_tile0 + col + 8 * g, col + 8 * g, cc, acc + 8 * g, v);
+          dist[g] = 0.0f;
+#pragma unroll
+          for (int i = 0; i < 8; i += 2) {
+            if (MODE == EPI_FC1) gelu_pattern2(make_float2(v[i], v[i + 1]), inv_scale, magic_zp, dist[g], c[i], c[i + 1]);
+            else quant_pattern2(make_float2(v[i], v[i + 1]), inv_scale, neg_zero, c[i], c[i + 1]);
+          }
+          w[2 * g] = sat_pack4<SH>(c[0], c[1], c[2], c[3], zbias << SH);
+          w[2 * g + 1] = sat_pack4<SH>(c[4], c[5], c[6], c[7], zbias << SH);
+        }
+        if (MODE == EPI_FC1 && IN_RANGE) {
+          // some value of the warp too close to a rounding boundary (a sixth of the chunks at A8): its eight columns again
+          const bool near = fmaxf(fmaxf(dist[0], dist[1]), fmaxf(dist[2], dist[3])) >= thr;
+          if (__any_sync(0xffffffffu, near)) {
+#pragma unroll 1
+            for (int g = 0; g < 4; ++g) {
+              const float d = g == 0 ? dist[0] : g == 1 ? dist[1] : g == 2 ? dist[2] : dist[3];
+              if (!__any_sync(0xffffffffu, d >= thr)) continue;
+              int32_t again[8];
+              uint32_t w0, w1;
+              tmem_ld(ta + (uint32_t)(8 * g), again);
+              tmem_ld_wait(again);
+              exact8(col + 8 * g, again, w0, w1);
+              w[0] = g == 0 ? w0 : w[0]; w[1] = g == 0 ? w1 : w[1];
+              w[2] = g == 1 ? w0 : w[2]; w[3] = g == 1 ? w1 : w[3];
+              w[4] = g == 2 ? w0 : w[4]; w[5] = g == 2 ? w1 : w[5];
+              w[6] = g == 3 ? w0 : w[6]; w[7] = g == 3 ? w1 : w[7];
+            }
+          }
+        }
+        if (row_ok) store_sat32(out_ptr + ch * out_step, w, bits, cbits);
       }
     };
-    // the TMEM load of the next chunk is in flight while this chunk is computed
-    // (one copy of the chunk body keeps the loop inside the instruction cache: the prefetched registers are moved)
-    int32_t acc[EPI_NC], nxt[EPI_NC];
-    if (n_chunks > 0) tmem_ld16_issue(taddr, nxt);
-#pragma unroll 1
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      tmem_ld_wait(nxt);
-#pragma unroll
-      for (int i = 0; i < EPI_NC; ++i) acc[i] = nxt[i];
-      if (ch + 1 < n_chunks) tmem_ld16_issue(taddr + (uint32_t)((ch + 1) * col_step), nxt);
-      chunk(ch, acc);
-    }
+    auto walk_bits = [&](auto range_tag) {
+      if (bits == 8) walk(std::integral_constant<int, 8>{}, range_tag);
+      else if (bits == 4) walk(std::integral_constant<int, 4>{}, range_tag);
+      else walk(std::integral_constant<int, 2>{}, range_tag);
+    };
+    if (in_range) walk_bits(std::true_type{}); else walk_bits(std::false_type{});
     return true;
   }
 
   // ---- binary32 outputs (proj: x1 = x_window + out; fc2: y = x1 + out scattered to the token's own position;
-  //      merge: out).  Each chunk is transposed through shared memory so that global accesses are 64-byte runs
-  //      (4 lanes per row, 8 rows per instruction). ----
+  //      merge: out).  The raw sums of a 16-column chunk are transposed through shared memory so that global accesses are
+  //      64-byte runs (4 lanes per row, 8 rows per instruction), and a lane then needs the constants of 4 columns only:
+  //      these launches are bound by the load/store pipe, and constants read per row and column were a third of its work.
+  //      (32-column chunks with 128-byte runs: 86 against 68 us for a proj of 296 450 rows of 128 channels -- half the
+  //      chunks in flight per warp, and the addresses of eight rows spill.) ----
   const int cj = lane & 3, rsub = lane >> 2;
   long src_mine = -1;
-  if (MODE != EPI_MERGE && row_ok) src_mine = br.rowsrc[m];
+  if (MODE != EPI_MERGE && row_ok) src_mine = eb.rowsrc[m];
   // this lane's four (row, 16-byte piece) positions of the warp's first chunk: residual source and output, NULL: none
   const float* res_ptr[4];
   float* dst_ptr[4];
@@ -154,13 +282,13 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, int N, 
     const int r = 8 * i + rsub;
     const long mr = row0 + r;
     const long s = __shfl_sync(0xffffffffu, src_mine, r);
-    const bool ok = mr < br.M;
+    const bool ok = mr < eb.M;
     long res_row, dst_row;               // row offsets (in elements), -1: none
     if (MODE == EPI_PROJ)     { res_row = (ok && s >= 0) ? s * N : -1;  dst_row = ok ? mr * N : -1; }
     else if (MODE == EPI_FC2) { res_row = (ok && s >= 0) ? mr * N : -1; dst_row = (ok && s >= 0) ? s * N : -1; }
     else                      { res_row = -1;                            dst_row = ok ? mr * N : -1; }
-    res_ptr[i] = (MODE != EPI_MERGE && res_row >= 0) ? br.res + res_row + n_first + 4 * cj : nullptr;
-    dst_ptr[i] = dst_row >= 0 ? br.out_f + dst_row + n_first + 4 * cj : nullptr;
+    res_ptr[i] = (MODE != EPI_MERGE && res_row >= 0) ? eb.res + res_row + n_first + 4 * cj : nullptr;
+    dst_ptr[i] = dst_row >= 0 ? eb.out_f + dst_row + n_first + 4 * cj : nullptr;
   }
   // The residual rows come into shared memory by asynchronous copies, RES_SLOTS chunks ahead of their use: the copies
   // of a whole tile are in flight while the accumulator is still being computed, and they cost no registers.
@@ -173,7 +301,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, int N, 
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int r = 8 * i + rsub;
-        float* dst = slot + r * EPI_NC + 4 * (cj ^ ((r >> 1) & 3));
+        float* dst = slot + r * F32_NC + 4 * (cj ^ ((r >> 1) & 3));
         if (res_ptr[i]) cp_async16(dst, res_ptr[i] + ch * col_step);
         else *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);   // a pad token's residual input is zero
       }
@@ -185,47 +313,55 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, int N, 
     for (int ch = 0; ch < RES_SLOTS; ++ch) fetch(ch);
   }
   if (!acc_ready()) { cp_async_wait<0>(); return false; }
-  auto chunk = [&](int ch, const int32_t (&acc)[EPI_NC]) {
-    const int n0 = n_first + ch * col_step;
-    float v[EPI_NC];
-    dequant16<MODE, TAPS>(br, N, m, row_ok, n0, ch * EPI_NC, cc, acc, v);
-    // row `lane`, logical 16-byte piece j is stored at piece j ^ ((lane >> 1) & 3): conflict-free both ways
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      *reinterpret_cast<float4*>(stage + lane * EPI_NC + 4 * (j ^ ((lane >> 1) & 3))) =
-          make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-    if (MODE != EPI_MERGE) cp_async_wait<RES_SLOTS - 1>();     // this lane's copies of chunk ch have landed
-    __syncwarp();
-    const float* slot = res_ring + (ch % RES_SLOTS) * EPI_STAGE_FLOATS;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = 8 * i + rsub;
-      const int off = r * EPI_NC + 4 * (cj ^ ((r >> 1) & 3));
-      const float4 a = *reinterpret_cast<const float4*>(stage + off);
-      if (dst_ptr[i]) {
-        float4 o = a;
-        if (MODE != EPI_MERGE) {
-          const float4 rr = *reinterpret_cast<const float4*>(slot + off);
-          const float2 lo = __fadd2_rn(make_float2(rr.x, rr.y), make_float2(a.x, a.y));
-          const float2 hi = __fadd2_rn(make_float2(rr.z, rr.w), make_float2(a.z, a.w));
-          o = make_float4(lo.x, lo.y, hi.x, hi.y);
-        }
-        *reinterpret_cast<float4*>(dst_ptr[i] + ch * col_step) = o;
-      }
-    }
-    __syncwarp();
-    if (MODE != EPI_MERGE) fetch(ch + RES_SLOTS);              // the slot just read is free again
-  };
-  int32_t acc[EPI_NC], nxt[EPI_NC];
-  if (n_chunks > 0) tmem_ld16_issue(taddr, nxt);
+  auto walk = [&](auto range_tag) {
+    constexpr bool IN_RANGE = decltype(range_tag)::value;
+    int32_t acc[F32_NC];
+    if (n_chunks > 0) tmem_ld(taddr, acc);
 #pragma unroll 1
-  for (int ch = 0; ch < n_chunks; ++ch) {
-    tmem_ld_wait(nxt);
+    for (int ch = 0; ch < n_chunks; ++ch) {
+      const int lc = c_first * F32_NC + ch * col_step + 4 * cj;       // this lane's first column within the tile
+      tmem_ld_wait(acc);
+      // row `lane`, logical 16-byte piece j is stored at piece j ^ ((lane >> 1) & 3): conflict-free both ways
 #pragma unroll
-    for (int i = 0; i < EPI_NC; ++i) acc[i] = nxt[i];
-    if (ch + 1 < n_chunks) tmem_ld16_issue(taddr + (uint32_t)((ch + 1) * col_step), nxt);
-    chunk(ch, acc);
-  }
+      for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<int4*>(stage + lane * F32_NC + 4 * (j ^ ((lane >> 1) & 3))) =
+            make_int4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+      // the TMEM load of the next chunk is in flight while this chunk is finished
+      if (ch + 1 < n_chunks) tmem_ld(taddr + (uint32_t)((ch + 1) * col_step), acc);
+      const int4 p4 = *reinterpret_cast<const int4*>(cc.pre + lc);
+      const float4 m4 = *reinterpret_cast<const float4*>(cc.mult + lc);
+      float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (MODE != EPI_MERGE) b4 = *reinterpret_cast<const float4*>(cc.bias + lc);
+      if (MODE != EPI_MERGE) cp_async_wait<RES_SLOTS - 1>();     // this lane's copies of chunk ch have landed
+      __syncwarp();
+      const float* slot = res_ring + (ch % RES_SLOTS) * EPI_STAGE_FLOATS;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = 8 * i + rsub;
+        const int off = r * F32_NC + 4 * (cj ^ ((r >> 1) & 3));
+        const int4 a = *reinterpret_cast<const int4*>(stage + off);
+        if (TAPS && br.tap_acc && row0 + r < eb.M) {
+          int32_t* tp = br.tap_acc + (row0 + r) * N + n_tile0 + lc;
+          tp[0] = a.x + p4.x - (int32_t)kMagicBits; tp[1] = a.y + p4.y - (int32_t)kMagicBits;
+          tp[2] = a.z + p4.z - (int32_t)kMagicBits; tp[3] = a.w + p4.w - (int32_t)kMagicBits;
+        }
+        if (!dst_ptr[i]) continue;
+        const float2 f0 = acc_to_float2<IN_RANGE>(a.x + p4.x, a.y + p4.y), f1 = acc_to_float2<IN_RANGE>(a.z + p4.z, a.w + p4.w);
+        float2 lo, hi;
+        if (MODE == EPI_MERGE) {
+          lo = __fmul2_rn(f0, make_float2(m4.x, m4.y)); hi = __fmul2_rn(f1, make_float2(m4.z, m4.w));
+        } else {
+          const float4 rr = *reinterpret_cast<const float4*>(slot + off);
+          lo = __fadd2_rn(make_float2(rr.x, rr.y), __ffma2_rn(f0, make_float2(m4.x, m4.y), make_float2(b4.x, b4.y)));
+          hi = __fadd2_rn(make_float2(rr.z, rr.w), __ffma2_rn(f1, make_float2(m4.z, m4.w), make_float2(b4.z, b4.w)));
+        }
+        *reinterpret_cast<float4*>(dst_ptr[i] + ch * col_step) = make_float4(lo.x, lo.y, hi.x, hi.y);
+      }
+      __syncwarp();
+      if (MODE != EPI_MERGE) fetch(ch + RES_SLOTS);              // the slot just read is free again
+    }
+  };
+  if (in_range) walk(std::true_type{}); else walk(std::false_type{});
   if (MODE != EPI_MERGE) cp_async_wait<0>();                   // nothing of this tile is left in flight
   return true;
 }

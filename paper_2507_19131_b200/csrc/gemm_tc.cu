@@ -12,13 +12,24 @@
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
 //               the swizzled layout (rows whose byte pitch is no multiple of 16 cannot be described to the TMA
 //               unit and are read with plain loads instead);
-//   then        epilogue (12 warps for the code outputs, 8 for the binary32 outputs): tcgen05.ld (one row per thread, 16 columns per load) + the fused epilogue of the mode.
+//   then        epilogue (12 or 16 warps for the code outputs, 8 for the binary32 outputs): tcgen05.ld (one row per thread,
+//               16 or 32 columns per load) + the fused epilogue of the mode.
 // Every wait on an mbarrier is bounded; on expiry the CTA raises the status word, then waits (bounded again) for the
 // copies it has issued to land and for the MMAs it has issued to retire, frees its tensor memory and returns.
 #include <cuda.h>
 #include "gemm_epilogue.cuh"
 
 namespace mixaq {
+
+int sm_count() {
+  static int n = 0;
+  if (!n) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+      n = 148;
+  }
+  return n;
+}
 
 namespace {
 
@@ -28,21 +39,36 @@ constexpr int UMMA_K = 32;         // codes per tcgen05.mma kind::i8
 constexpr int A_STAGE_BYTES = BM * BK;
 // warps 2..5 expand sub-byte codes (two warps left the long-K main loops of 4-bit tiles waiting for the expansion;
 // eight cost more registers than they return)
-__host__ __device__ constexpr int unpack_warps(int mode) { return 4; }
-// epilogue warps: 12 for the arithmetic-bound code epilogues, 8 for the binary32 ones
-__host__ __device__ constexpr int epi_warps(int mode) { return (mode == EPI_QKV || mode == EPI_FC1) ? 12 : 8; }
+constexpr int UNPACK_WARPS = 4;
+// Epilogue warps.  Binary32 outputs: 8.  Code outputs: 12, or 16 where every CTA has many row tiles: whole tiles are then
+// dealt to groups of warps (see pick_tiling) and the launch is bound by throughput (C = 128 at 2 x 384 x 384 tokens: fc1 165
+// us with 12, 155 with 16); below that the shorter tile latency of 12 warps with more registers wins (C = 384 at 50 x 84: fc1
+// 18.7 against 21.5).
+constexpr int F32_WARPS = 8, CODE_WARPS = 12, CODE_WARPS_MANY = 16;
+constexpr int MANY_ROW_TILES = 8;              // row tiles per SM from which CODE_WARPS_MANY is used
+__host__ __device__ constexpr int num_threads(int warps) { return 32 * (2 + UNPACK_WARPS + warps); }
 constexpr int MAX_BN = 256;
-constexpr int EPI_WARP_COLS = MAX_BN / 2;      // most columns one epilogue warp handles per tile (two warps per lane quarter)
+__host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
 constexpr int MAX_RING = 6;
+constexpr int TMEM_COLS = 512;                 // one CTA per SM: it takes all of the tensor memory
+constexpr int MAX_ACC = 4;                     // accumulators in it, as far as the tile width allows
 constexpr uint32_t MAX_POLLS = 1u << 22;       // tries per wait
+constexpr uint32_t MAX_SUSPENDED_POLLS = 1u << 16;   // tries that may each suspend the thread for up to 20 us
 
 struct TcParams {
   GemmArgs g;
-  int tiles_m0;          // 128-row tiles of the first (high) branch
-  int total_tiles, n_tiles, BN, k_blocks, ring, tmem_cols;
-  int packed_bytes;      // bytes of the packed staging slot of a stage (0: no branch stages packed rows by TMA)
-  int res_bytes;         // bytes of the residual rings (proj, fc2: RES_SLOTS chunks per epilogue warp; else 0)
-  int tma_packed[2];     // branch i stages its bit-packed rows by TMA (tmA_i then describes the packed matrix)
+  int tiles_m0, tiles_m;   // 128-row tiles of the first (high) branch, of both
+  int n_tiles, BN, k_blocks, ring;
+  int step_m, step_n;      // a CTA walks over the tiles (row tile major) gridDim.x at a time: the step as (row, column) tiles
+  // The epilogue warps of a lane quarter form `groups` groups; group g takes the CTA's tiles g, g + groups, ... (gstep: that
+  // stride as (row, column) tiles), and the `split` warps of a group deal a tile's chunks among themselves.
+  int groups, split, gstep_m, gstep_n;
+  int const_cols;          // columns whose constants a CTA keeps in shared memory: BN where it stays on one column tile, else N
+  int last_step;           // number of the CTA's last tile is the largest blockIdx.x + i * gridDim.x <= last_step
+  int n_acc, acc_stride;   // accumulators in tensor memory and the columns between them
+  int packed_bytes;        // bytes of the packed staging slot of a stage (0: no branch stages packed rows by TMA)
+  int res_bytes;           // bytes of the residual rings (proj, fc2: RES_SLOTS chunks per epilogue warp; else 0)
+  int tma_packed[2];       // branch i stages its bit-packed rows by TMA (tmA_i then describes the packed matrix)
   int* status;
 };
 
@@ -50,15 +76,16 @@ struct TcParams {
 struct SmemLayout {
   int stage_bytes, ring_bytes, consts_off, stage_off, res_off, bars_off, total;
 };
-__host__ __device__ inline SmemLayout smem_layout(int BN, int ring, int packed_bytes, int res_bytes, int NUM_EPI_WARPS) {
+constexpr int NUM_BARS = 4 * MAX_RING + 2 * MAX_ACC + 2;        // full, empty, raw, unpacked; accumulator full, empty; constants, drain
+__host__ __device__ inline SmemLayout smem_layout(int BN, int ring, int packed_bytes, int res_bytes, int const_cols, int mode, int warps) {
   SmemLayout L;
   L.stage_bytes = A_STAGE_BYTES + BN * BK + packed_bytes;
   L.ring_bytes = ring * L.stage_bytes;
-  L.consts_off = L.ring_bytes;                                  // per epilogue warp (zc, mult, bias) x 128 columns
-  L.stage_off = L.consts_off + NUM_EPI_WARPS * 3 * EPI_WARP_COLS * 4;   // per epilogue warp 32 x 16 floats
-  L.res_off = L.stage_off + NUM_EPI_WARPS * EPI_STAGE_FLOATS * 4;       // residual rings of the binary32 epilogues
+  L.consts_off = L.ring_bytes;                                  // (pre, mult, bias) of const_cols columns
+  L.stage_off = L.consts_off + 3 * const_cols * 4;    // binary32 epilogues: a 32 x 16 chunk per warp
+  L.res_off = L.stage_off + (code_mode(mode) ? 0 : warps * EPI_STAGE_FLOATS * 4);   // and their residual rings
   L.bars_off = L.res_off + res_bytes;
-  L.total = L.bars_off + (3 * MAX_RING + 5) * 8 + 16;   // + the drain barrier; then TMEM base, abort flag, fill count
+  L.total = L.bars_off + NUM_BARS * 8 + 16;                     // then TMEM base, abort flag, constants-out-of-range flag
   return L;
 }
 
@@ -84,11 +111,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait.  Returns false when the limit ran out or another thread of the CTA already gave up.
+__device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
+  return ok != 0;
+}
+// Bounded wait.  Returns false when the limit ran out or another thread of the CTA already gave up (looked at now and
+// then only).  The waits that are not on a tile's critical path give the hardware a suspend time: the polls of the TMA and
+// MMA threads took up to a tenth of the issue slots of their schedulers.
+template <bool LATENCY = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t it = 0; it < MAX_POLLS; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
+  if (mbar_try_wait(bar, parity)) return true;
+  for (uint32_t it = 1; it < (LATENCY ? MAX_POLLS : MAX_SUSPENDED_POLLS); ++it) {
+    if (LATENCY ? mbar_try_wait(bar, parity) : mbar_try_wait_hint(bar, parity)) return true;
+    if ((it & 15u) == 0u && *abort_flag) return false;
   }
   *abort_flag = 1;
   return false;
@@ -121,46 +161,63 @@ __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-struct TileCoord { int mt, nt; bool is_hi; };
-__device__ __forceinline__ TileCoord decode_tile(const TcParams& p, int t) {
-  TileCoord c;
-  c.nt = t % p.n_tiles;
-  c.mt = t / p.n_tiles;
-  c.is_hi = c.mt < p.tiles_m0;
-  if (!c.is_hi) c.mt -= p.tiles_m0;
-  return c;
-}
+
+// The tiles of a CTA, without a division per tile: tile number blockIdx.x, + gridDim.x, ..., row tile major.  The high
+// branch's row tiles come first, so every role runs one loop per branch and keeps the branch's constants in registers.
+struct TileWalk {
+  int mt, nt;
+  __device__ __forceinline__ explicit TileWalk(const TcParams& p) : mt((int)blockIdx.x / p.n_tiles), nt((int)blockIdx.x - mt * p.n_tiles) {}
+  __device__ __forceinline__ void advance(int dm, int dn, int n_tiles) {
+    mt += dm; nt += dn;
+    if (nt >= n_tiles) { nt -= n_tiles; ++mt; }
+  }
+  __device__ __forceinline__ void next(const TcParams& p) { advance(p.step_m, p.step_n, p.n_tiles); }
+};
+// Position in the ring of stages (or of accumulators): slot and parity of the current pass.
+struct RingPos {
+  int slot = 0; uint32_t pass = 0;
+  __device__ __forceinline__ void next(int n) { if (++slot == n) { slot = 0; pass ^= 1u; } }
+};
 
 // TAPS: the accumulator tap is compiled in only for calls that ask for it
-template <int MODE, bool TAPS>
-__global__ void __launch_bounds__(32 * (2 + unpack_warps(MODE) + epi_warps(MODE)), 1)
+//
+// The loops of the two single threads (TMA, MMA) bound a tile as much as the epilogue does: a thread on its own issues an
+// instruction every 5 to 10 cycles, so the slot and phase divisions and the branch look-ups that used to sit in them cost
+// 1 100 cycles per k-block (stage-1 QKV at 200 x 334 tokens: 17 us of launch without any epilogue work).
+template <int MODE, bool TAPS, int EW>
+__global__ void __launch_bounds__(num_threads(EW), 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
-          const __grid_constant__ CUtensorMap tmB, const TcParams p) {
+          const __grid_constant__ CUtensorMap tmB, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;                 // swizzled tiles need 1024-byte alignment
   uint8_t* smem = smem_raw + (base - raw);
-  const SmemLayout L = smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, epi_warps(MODE));
+  const SmemLayout L = smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW);
   const int stage_bytes = L.stage_bytes;
-  int32_t* s_consts = reinterpret_cast<int32_t*>(smem + L.consts_off);
-  float* s_stage = reinterpret_cast<float*>(smem + L.stage_off);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars_off);
   const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8u * MAX_RING, bar_raw = bar_empty + 8u * MAX_RING;
-  const uint32_t bar_tfull = bar_raw + 8u * MAX_RING, bar_tempty = bar_tfull + 16u, bar_drain = bar_tempty + 16u;
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 3 * MAX_RING + 5);
+  const uint32_t bar_unp = bar_raw + 8u * MAX_RING, bar_tfull = bar_unp + 8u * MAX_RING;
+  const uint32_t bar_tempty = bar_tfull + 8u * MAX_ACC, bar_consts = bar_tempty + 8u * MAX_ACC, bar_drain = bar_consts + 8u;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  volatile int* fills_issued = reinterpret_cast<volatile int*>(tmem_holder + 2);   // k-blocks the TMA thread has issued
-  int my_arrivals = 0;                       // unpack warps: k-blocks this warp has arrived for on the full barriers
+  volatile int* beyond_flag = reinterpret_cast<volatile int*>(tmem_holder + 2);
+  // TMA thread: stages that hold a fill, and the phase of the last one, on the full and on the packed-rows barrier
+  // (bit s of each; read by the give-up path only)
+  uint32_t full_used = 0, full_phase = 0, raw_used = 0, raw_phase = 0;
 
-  constexpr int NUM_EPI_WARPS = epi_warps(MODE);
-  constexpr int NUM_UNPACK_WARPS = unpack_warps(MODE), NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
+  constexpr int NUM_EPI_WARPS = EW;
+  constexpr int NUM_UNPACK_WARPS = UNPACK_WARPS, NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
   constexpr int FIRST_EPI_WARP = 2 + NUM_UNPACK_WARPS;
   constexpr int UNPACK_ITEMS = BM * (BK / UMMA_K) / NUM_UNPACK_THREADS;   // (row, 32-code group) items per thread and stage
-  constexpr int EPI_SPLIT = NUM_EPI_WARPS / 4;   // warps that share a TMEM lane quarter deal its chunks round-robin
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int K = p.g.K;
-  const int acc_stride = p.tmem_cols >> 1;                     // TMEM columns between the two accumulators
 
+  // Every launch starts with a cold constant cache, and the roles below would miss on one parameter after the other
+  // (1 800 cycles until the first copy was issued): the warps touch the lines of the parameter block side by side.
+  {
+    const int word = (warp * 16) % (int)(sizeof(TcParams) / 4);
+    const int touched = reinterpret_cast<const int*>(&p)[word];
+    asm volatile("" ::"r"(touched));
+  }
   if (tid == 32) {
     // the descriptors are fetched while the barriers are set up
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
@@ -169,108 +226,152 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   }
   if (tid == 0) {
     for (int s = 0; s < p.ring; ++s) {
-      mbar_init(bar_full + 8u * s, 1u + NUM_UNPACK_WARPS);      // TMA thread + one arrival per unpack warp
+      mbar_init(bar_full + 8u * s, 1u);                         // TMA thread; the operand bytes of the stage
       mbar_init(bar_empty + 8u * s, 1u);                        // tcgen05.commit
-      mbar_init(bar_raw + 8u * s, 1u);                          // TMA thread: "the unpack warps may touch stage s"
+      mbar_init(bar_raw + 8u * s, 1u);                          // TMA thread (+ bytes): packed rows are there
+      mbar_init(bar_unp + 8u * s, NUM_UNPACK_WARPS);            // unpack warps: the activation tile is expanded
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < p.n_acc; ++a) {
       mbar_init(bar_tfull + 8u * a, 1u);                        // tcgen05.commit of the tile's last MMA
-      mbar_init(bar_tempty + 8u * a, NUM_EPI_WARPS);            // one arrival per epilogue warp
+      mbar_init(bar_tempty + 8u * a, 4u * (uint32_t)p.split);   // one arrival per epilogue warp of a group
     }
+    mbar_init(bar_consts, NUM_EPI_WARPS);                       // constants of a branch: loaded / no longer in use
+    *beyond_flag = 0;
     mbar_init(bar_drain, 1u);                                   // tcgen05.commit of the give-up path
     *abort_flag = 0;
-    *fills_issued = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {
+  if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(smem_u32(tmem_holder)), "r"((uint32_t)p.tmem_cols) : "memory");
+                 ::"r"(smem_u32(tmem_holder)), "r"((uint32_t)TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_holder;
+  griddep_launch();
 
   if (warp == 0) {
     // ---- TMA producer ----
     if (lane == 0) {
-      int it = 0;                                               // running k-block counter over all tiles of this CTA
+      TileWalk w(p);
+      RingPos rp;
       bool ok = true;
-      for (int t = blockIdx.x; t < p.total_tiles && ok; t += gridDim.x) {
-        const TileCoord tc = decode_tile(p, t);
-        const GemmBranch& br = tc.is_hi ? p.g.br[0] : p.g.br[1];
-        const bool packed = br.a_bits != 8;
-        const bool stage_packed = packed && p.tma_packed[tc.is_hi ? 0 : 1];
-        const CUtensorMap* tmA = tc.is_hi ? &tmA0 : &tmA1;
-        const uint32_t tx = (uint32_t)(p.BN * BK) + (packed ? 0u : (uint32_t)A_STAGE_BYTES);
-        const int pk_row = BK * br.a_bits / 8;                  // packed bytes per row and k-block
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-          const int s = it % p.ring;
-          if (it >= p.ring && !mbar_wait(bar_empty + 8u * s, ((it / p.ring) - 1) & 1, abort_flag)) { ok = false; break; }
-          const uint32_t sa = base + (uint32_t)s * stage_bytes, sb = sa + A_STAGE_BYTES, sp = sb + (uint32_t)(p.BN * BK);
-          mbar_arrive_expect_tx(bar_full + 8u * s, tx);
-          tma_load_2d(sb, &tmB, kb * BK, tc.nt * p.BN, bar_full + 8u * s);
-          if (!packed) tma_load_2d(sa, tmA, kb * BK, tc.mt * BM, bar_full + 8u * s);
-          if (stage_packed) {
-            mbar_arrive_expect_tx(bar_raw + 8u * s, (uint32_t)(pk_row * BM));
-            tma_load_2d(sp, tmA, kb * pk_row, tc.mt * BM, bar_raw + 8u * s);
-          } else {
-            mbar_arrive(bar_raw + 8u * s);
+      const uint32_t b_bytes = (uint32_t)(p.BN * BK);
+      bool waited = false;                                      // for the kernel that writes the activations (weights do not wait)
+      const int k_blocks = p.k_blocks, ring = p.ring, BN = p.BN;
+      for (int b = 0; b < 2 && ok; ++b) {
+        const int m_first = b == 0 ? 0 : p.tiles_m0, m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
+        if (w.mt >= m_end) continue;
+        const int abits = p.g.br[b].a_bits;
+        const bool packed = abits != 8, stage_packed = packed && p.tma_packed[b];
+        const CUtensorMap* tmA = b == 0 ? &tmA0 : &tmA1;
+        const uint32_t tx = b_bytes + (packed ? 0u : (uint32_t)A_STAGE_BYTES);
+        const int pk_row = BK * abits / 8;                      // packed bytes per row and k-block
+        for (; w.mt < m_end && ok; w.next(p)) {
+          const int m_row = (w.mt - m_first) * BM, n_row = w.nt * BN;
+          for (int kb = 0; kb < k_blocks; ++kb, rp.next(ring)) {
+            const uint32_t o = 8u * (uint32_t)rp.slot, bit = 1u << rp.slot;
+            if ((full_used & bit) && !mbar_wait(bar_empty + o, rp.pass ^ 1u, abort_flag)) { ok = false; break; }
+            const uint32_t sa = base + (uint32_t)(rp.slot * stage_bytes), sb = sa + A_STAGE_BYTES;
+            mbar_arrive_expect_tx(bar_full + o, tx);
+            full_used |= bit;
+            full_phase = rp.pass ? full_phase | bit : full_phase & ~bit;
+            tma_load_2d(sb, &tmB, kb * BK, n_row, bar_full + o);
+            if (!waited) { griddep_wait(); waited = true; }
+            if (!packed) {
+              tma_load_2d(sa, tmA, kb * BK, m_row, bar_full + o);
+            } else {
+              raw_phase = (raw_used & bit) ? raw_phase ^ bit : raw_phase & ~bit;
+              raw_used |= bit;
+              if (stage_packed) {
+                mbar_arrive_expect_tx(bar_raw + o, (uint32_t)(pk_row * BM));
+                tma_load_2d(sb + b_bytes, tmA, kb * pk_row, m_row, bar_raw + o);
+              } else {
+                mbar_arrive(bar_raw + o);
+              }
+            }
           }
         }
       }
-      *fills_issued = it;                                       // read by the give-up path only
     }
     __syncwarp();
   } else if (warp == 1) {
     // ---- MMA issuer ----
     if (lane == 0) {
       const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      int it = 0, lt = 0;
+      const uint64_t adesc0 = smem_desc_sw128(base), bdesc0 = smem_desc_sw128(base + A_STAGE_BYTES);
+      const uint32_t stage16 = (uint32_t)stage_bytes >> 4;      // stage pitch in descriptor units
+      const int k_blocks = p.k_blocks, ring = p.ring, n_acc = p.n_acc;
+      const int last_steps = (p.g.K - (k_blocks - 1) * BK) / UMMA_K;      // MMAs of the last k-block (4 in the others)
+      TileWalk w(p);
+      RingPos rp, ap;
+      uint32_t acc_used = 0, unp_next = 0;                      // bit s of unp_next: parity of stage s' next expansion
       bool ok = true;
-      for (int t = blockIdx.x; t < p.total_tiles && ok; t += gridDim.x, ++lt) {
-        const int a = lt & 1;
-        // wait until the epilogue has drained this accumulator (its use two tiles ago)
-        if (lt >= 2 && !mbar_wait(bar_tempty + 8u * a, ((lt >> 1) - 1) & 1, abort_flag)) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d_tmem = tmem_base + (uint32_t)(a * acc_stride);
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-          const int s = it % p.ring;
-          if (!mbar_wait(bar_full + 8u * s, (it / p.ring) & 1, abort_flag)) { ok = false; break; }
+      for (int b = 0; b < 2 && ok; ++b) {
+        const int m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
+        if (w.mt >= m_end) continue;
+        const bool packed = p.g.br[b].a_bits != 8;
+        for (; w.mt < m_end && ok; w.next(p), ap.next(n_acc)) {
+          // wait until the epilogue has drained this accumulator (its previous use)
+          if ((acc_used >> ap.slot & 1u) && !mbar_wait(bar_tempty + 8u * ap.slot, ap.pass ^ 1u, abort_flag)) { ok = false; break; }
+          acc_used |= 1u << ap.slot;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sa = base + (uint32_t)s * stage_bytes, sb = sa + A_STAGE_BYTES;
-          const uint64_t adesc = smem_desc_sw128(sa), bdesc = smem_desc_sw128(sb);
-          const int ksteps = min(BK, K - kb * BK) / UMMA_K;
-          for (int kk = 0; kk < ksteps; ++kk)
-            mma_i8(d_tmem, adesc + (uint64_t)(kk * (UMMA_K >> 4)), bdesc + (uint64_t)(kk * (UMMA_K >> 4)), idesc,
-                   (kb > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(bar_empty + 8u * s);          // frees the ring slot when these MMAs have read it
+          const uint32_t d_tmem = tmem_base + (uint32_t)(ap.slot * p.acc_stride);
+          for (int kb = 0; kb < k_blocks; ++kb, rp.next(ring)) {
+            const uint32_t o = 8u * (uint32_t)rp.slot;
+            if (!mbar_wait(bar_full + o, rp.pass, abort_flag)) { ok = false; break; }
+            if (packed) {
+              if (!mbar_wait(bar_unp + o, (unp_next >> rp.slot) & 1u, abort_flag)) { ok = false; break; }
+              unp_next ^= 1u << rp.slot;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t so = (uint64_t)((uint32_t)rp.slot * stage16);
+            const uint64_t adesc = adesc0 + so, bdesc = bdesc0 + so;
+            const int steps = kb == k_blocks - 1 ? last_steps : BK / UMMA_K;
+#pragma unroll
+            for (int kk = 0; kk < BK / UMMA_K; ++kk)
+              if (kk < steps)
+                mma_i8(d_tmem, adesc + (uint64_t)(kk * (UMMA_K >> 4)), bdesc + (uint64_t)(kk * (UMMA_K >> 4)), idesc,
+                       kk > 0 ? 1u : (uint32_t)(kb > 0));
+            mma_commit(bar_empty + o);               // frees the ring slot when these MMAs have read it
+          }
+          if (ok) mma_commit(bar_tfull + 8u * ap.slot);    // accumulator complete
         }
-        if (ok) mma_commit(bar_tfull + 8u * a);    // accumulator complete
       }
     }
     __syncwarp();
   } else if (warp < FIRST_EPI_WARP) {
     // ---- unpack producers: bit-packed rows -> one code per byte, written in the swizzled layout ----
     const int ptid = tid - 64;                   // 0 .. NUM_UNPACK_THREADS-1
-    int it = 0;
+    TileWalk w(p);
+    int slot = 0;
+    uint32_t raw_next = 0;                       // bit s: parity of stage s' next packed fill
     bool ok = true;
-    for (int t = blockIdx.x; t < p.total_tiles && ok; t += gridDim.x) {
-      const TileCoord tc = decode_tile(p, t);
-      const GemmBranch& br = tc.is_hi ? p.g.br[0] : p.g.br[1];
-      const int abits = br.a_bits;
-      const bool packed = abits != 8;
-      const bool staged = packed && p.tma_packed[tc.is_hi ? 0 : 1];
+    for (int b = 0; b < 2 && ok; ++b) {
+      const int m_first = b == 0 ? 0 : p.tiles_m0, m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
+      if (w.mt >= m_end) continue;
+      const int abits = p.g.br[b].a_bits;
+      if (abits == 8) {                          // nothing to expand: skip the stages of these tiles
+        int tiles = 0;
+        for (; w.mt < m_end; w.next(p)) ++tiles;
+        slot = (slot + tiles * p.k_blocks) % p.ring;
+        continue;
+      }
+      const bool staged = p.tma_packed[b];
+      if (!staged) griddep_wait();               // these warps read the rows themselves
+      const uint8_t* a = p.g.br[b].a;
+      const int M = p.g.br[b].M, K = p.g.K;
       const long row_bytes = (long)K * abits / 8;
-      const long m0 = (long)tc.mt * BM;
       const int grp_bytes = UMMA_K * abits / 8;                 // packed bytes of one 32-code group
-      for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-        const int s = it % p.ring;
-        // the TMA thread arrives on raw[s] once it owns the stage (and, when staged, the packed bytes have landed)
-        if (!mbar_wait(bar_raw + 8u * s, (it / p.ring) & 1, abort_flag)) { ok = false; break; }
-        if (packed) {
-          uint8_t* sa = smem + (size_t)s * stage_bytes;
+      for (; w.mt < m_end && ok; w.next(p)) {
+        const long m0 = (long)(w.mt - m_first) * BM;
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          // the TMA thread arrives on raw[s] once it owns the stage (and, when staged, the packed bytes have landed)
+          if (!mbar_wait(bar_raw + 8u * slot, (raw_next >> slot) & 1u, abort_flag)) { ok = false; break; }
+          raw_next ^= 1u << slot;
+          uint8_t* sa = smem + (size_t)slot * stage_bytes;
           const uint8_t* sp = sa + A_STAGE_BYTES + p.BN * BK;
           const int kgroups = min(BK, K - kb * BK) / UMMA_K;
           // item i of this thread: row r = item / 4, 32-code group kg = item % 4, item = ptid + NUM_UNPACK_THREADS * i
@@ -278,82 +379,101 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
           for (int i = 0; i < UNPACK_ITEMS; ++i) {
             const int item = ptid + NUM_UNPACK_THREADS * i;
             const int r = item >> 2, kg = item & 3;
-            uint32_t w[8];
+            uint32_t c[8];
             bool have = true;
             if (staged) {
               // rows and columns outside the matrix were zero-filled by the TMA unit
-              load_codes_32(sp + item * grp_bytes, abits, w);
+              load_codes_32(sp + item * grp_bytes, abits, c);
             } else {
-              have = kg < kgroups && m0 + r < br.M;
-              if (have) load_codes_32(br.a + (m0 + r) * row_bytes + (long)(kb * BK + kg * UMMA_K) * abits / 8, abits, w);
+              have = kg < kgroups && m0 + r < M;
+              if (have) load_codes_32(a + (m0 + r) * row_bytes + (long)(kb * BK + kg * UMMA_K) * abits / 8, abits, c);
             }
             if (have) {
               uint8_t* rowp = sa + (r >> 3) * 1024 + (r & 7) * 128;
               const int c0 = (2 * kg) ^ (r & 7), c1 = (2 * kg + 1) ^ (r & 7);
-              *reinterpret_cast<uint4*>(rowp + c0 * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-              *reinterpret_cast<uint4*>(rowp + c1 * 16) = make_uint4(w[4], w[5], w[6], w[7]);
+              *reinterpret_cast<uint4*>(rowp + c0 * 16) = make_uint4(c[0], c[1], c[2], c[3]);
+              *reinterpret_cast<uint4*>(rowp + c1 * 16) = make_uint4(c[4], c[5], c[6], c[7]);
             }
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // make the writes visible to the MMA proxy
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_unp + 8u * slot);
+          if (++slot == p.ring) slot = 0;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_full + 8u * s);
       }
     }
-    my_arrivals = it;
     __syncwarp();
   } else {
-    // ---- epilogue warps: warp e reads TMEM lanes 32*(e%4).. and takes every EPI_SPLIT-th 16-column chunk ----
-    const int e = warp - FIRST_EPI_WARP, q = warp & 3, sub = e >> 2;   // any 4 consecutive warps cover the 4 lane quarters
-    float* stage = s_stage + e * EPI_STAGE_FLOATS;
+    // ---- epilogue warps: warp e reads TMEM lanes 32*(e%4).. of its group's tiles, every split-th chunk ----
+    const int e = warp - FIRST_EPI_WARP, q = warp & 3;         // any 4 consecutive warps cover the 4 lane quarters
+    const int split = p.split, groups = p.groups, group = (e >> 2) / split, sub = (e >> 2) - group * split;
+    float* stage = reinterpret_cast<float*>(smem + L.stage_off) + e * EPI_STAGE_FLOATS;
     float* res_ring = reinterpret_cast<float*>(smem + L.res_off) + e * RES_SLOTS * EPI_STAGE_FLOATS;
-    int32_t* c_zc = s_consts + e * 3 * EPI_WARP_COLS;
-    float* c_mult = reinterpret_cast<float*>(c_zc + EPI_WARP_COLS);
-    float* c_bias = c_mult + EPI_WARP_COLS;
-    const int c_total = p.BN / EPI_NC;                         // BN is a multiple of 32
-    int lt = 0, consts_key = -1;
-    // the tile walk without a division per tile: (row tile, column tile) advance by gridDim.x tiles at a time
-    const int step_m = (int)gridDim.x / p.n_tiles, step_n = (int)gridDim.x % p.n_tiles;
-    int w_mt = (int)blockIdx.x / p.n_tiles, w_nt = (int)blockIdx.x % p.n_tiles;
-    for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++lt) {
-      TileCoord tc;
-      tc.nt = w_nt; tc.mt = w_mt; tc.is_hi = w_mt < p.tiles_m0;
-      if (!tc.is_hi) tc.mt -= p.tiles_m0;
-      w_mt += step_m; w_nt += step_n;
-      if (w_nt >= p.n_tiles) { w_nt -= p.n_tiles; ++w_mt; }
-      const GemmBranch& br = tc.is_hi ? p.g.br[0] : p.g.br[1];
-      const int a = lt & 1;
-      const int n_tile0 = tc.nt * p.BN;
-      // per-column constants of this warp's chunks, densely in the warp's own shared-memory slot; they depend on
-      // the branch and the column tile only, and the grid is sized so that a CTA keeps its column tile
-      // (no CTA-wide barrier: the only waits of this kernel are the bounded mbarrier waits)
-      const int key = tc.nt * 2 + (tc.is_hi ? 1 : 0);
-      if (key != consts_key) {
-        consts_key = key;
-        __syncwarp();
-        for (int c = sub, j = 0; c < c_total; c += EPI_SPLIT, ++j) {
-          if (lane < EPI_NC) {
-            const int n = n_tile0 + c * EPI_NC + lane;
-            c_zc[j * EPI_NC + lane] = __ldg(br.zc + n);
-            c_mult[j * EPI_NC + lane] = __ldg(br.mult + n);
-            if (MODE != EPI_MERGE) c_bias[j * EPI_NC + lane] = __ldg(br.bias + n);
-          }
-        }
-        __syncwarp();
-      }
-      ColConsts cc; cc.zc = c_zc; cc.mult = c_mult; cc.bias = c_bias;
-      const long row0 = (long)tc.mt * BM + q * 32;
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * acc_stride);
-      auto acc_ready = [&]() -> bool {
-        if (!mbar_wait(bar_tfull + 8u * a, (lt >> 1) & 1, abort_flag)) return false;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        return true;
-      };
-      if (!epilogue_warp_tile<MODE, TAPS>(br, p.g.N, p.g.C, row0, lane, n_tile0, sub, EPI_SPLIT, c_total, cc, taddr, stage,
-                                    acc_ready, res_ring)) break;
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    int32_t* c_pre = reinterpret_cast<int32_t*>(smem + L.consts_off);
+    float* c_mult = reinterpret_cast<float*>(c_pre + p.const_cols);
+    float* c_bias = c_mult + p.const_cols;
+    const int c_total = p.BN / (code_mode(MODE) ? CODE_NC : F32_NC);   // BN is a multiple of 32
+    const uint32_t tmem_q = tmem_base + ((uint32_t)(q * 32) << 16);
+    TileWalk w(p);
+    for (int g = 0; g < group; ++g) w.next(p);
+    auto step = [&](TileWalk& t) { t.advance(p.gstep_m, p.gstep_n, p.n_tiles); };
+    const int first_mt = (int)blockIdx.x / p.n_tiles;
+    int acc = group;
+    uint32_t acc_pass = 0;
+    bool ok = true;
+    // The per-column constants of a branch, for all columns the CTA can meet, are loaded once by all epilogue warps (a tile
+    // that fetched its own waited 600 cycles per chunk for the dependent loads).  The waits are the bounded mbarrier waits.
+    const int const_first = p.const_cols == p.BN ? (int)(blockIdx.x % (unsigned)p.n_tiles) * p.BN : 0;
+    const int last_mt = (int)(blockIdx.x + (unsigned)(p.last_step - (int)blockIdx.x) / gridDim.x * gridDim.x) / p.n_tiles;
+    uint32_t consts_pass = 0;
+    bool waited = false;
+    bool in_range = false;                                     // the patterns of these columns stay in range
+    auto all_warps = [&]() -> bool {
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_tempty + 8u * a);
+      if (lane == 0) mbar_arrive(bar_consts);
+      const bool done = mbar_wait(bar_consts, consts_pass, abort_flag);
+      consts_pass ^= 1u;
+      return done;
+    };
+    for (int b = 0; b < 2 && ok; ++b) {
+      const int m_first = b == 0 ? 0 : p.tiles_m0, m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
+      if (first_mt >= m_end || last_mt < m_first) continue;     // the CTA has no tile of this branch
+      const GemmBranch& br = p.g.br[b];
+      const EpiBranch eb(br, p.g.N);
+      if (b == 1 && first_mt < p.tiles_m0 && !all_warps()) { ok = false; break; }      // everybody is done with the first branch's
+      bool fits = true;
+      for (int i = e * 32 + lane; i < p.const_cols; i += NUM_EPI_WARPS * 32) {
+        const int n = const_first + i;
+        const float bias = MODE != EPI_MERGE ? __ldg(br.bias + n) : 0.0f, bound = __ldg(br.bound + n);
+        c_pre[i] = __ldg(br.pre + n);
+        c_mult[i] = __ldg(br.mult + n);
+        c_bias[i] = bias;
+        const float inv = !code_mode(MODE) ? 0.0f : MODE == EPI_FC1 || n < p.g.C ? br.q0.inv_scale : (n < 2 * p.g.C ? br.q1.inv_scale : br.q2.inv_scale);
+        fits &= code_mode(MODE) ? (bound + fabsf(bias)) * inv < kPatternRange : bound < INFINITY;
+      }
+      if (!fits) *beyond_flag = b + 1;                          // (a branch out of range takes the next one along: it is only slower)
+      if (!all_warps()) { ok = false; break; }
+      if (!waited) { griddep_wait(); waited = true; }           // residuals, row indices and outputs belong to earlier kernels
+      in_range = *beyond_flag == 0;
+      for (; w.mt < m_end; step(w)) {
+        const int n_tile0 = w.nt * p.BN;
+        const int c0 = n_tile0 - const_first;
+        const ColConsts cc = {c_pre + c0, c_mult + c0, c_bias + c0};
+        const long row0 = (long)(w.mt - m_first) * BM + q * 32;
+        auto acc_ready = [&]() -> bool {
+          if (!mbar_wait<true>(bar_tfull + 8u * acc, acc_pass, abort_flag)) return false;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          return true;
+        };
+        if (!epilogue_warp_tile<MODE, TAPS>(br, eb, p.g.N, p.g.C, row0, lane, n_tile0, sub, split, c_total, cc,
+                                            tmem_q + (uint32_t)(acc * p.acc_stride), stage, in_range, p.g.neg_zero,
+                                            acc_ready, res_ring)) { ok = false; break; }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tempty + 8u * acc);
+        acc += groups;
+        if (acc >= p.n_acc) { acc = group; acc_pass ^= 1u; }
+      }
     }
   }
 
@@ -361,14 +481,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   __syncthreads();
   if (*abort_flag) {
     // A wait ran out.  Before the CTA may exit, the copies already issued must have landed in its shared memory and
-    // the MMAs already issued must have retired.  (1) Every unpack warp arrives, on the full barrier of each k-block
-    // that was issued but that it had not reached, so that those phases can complete once their bytes are there
-    // (the ring admits at most one such k-block per stage).  (2) The MMA thread commits what it has issued to a
-    // barrier of its own.  (3) One thread waits, bounded, for the phase of the LAST fill of every stage, on the
-    // packed-rows barrier and on the full barrier, and for the MMA commit.
-    const int issued = *fills_issued;
-    if (warp >= 2 && warp < FIRST_EPI_WARP && lane == 0)
-      for (int j = my_arrivals; j < issued; ++j) mbar_arrive(bar_full + 8u * (uint32_t)(j % p.ring));
+    // the MMAs already issued must have retired.  (1) The MMA thread commits what it has issued to a barrier of its
+    // own.  (2) The TMA thread waits, bounded, for the phase of the last fill of every stage, on the full barrier and on
+    // the packed-rows barrier (both complete by the copies alone), and for that commit.
     if (tid == 32) mma_commit(bar_drain);
     __syncthreads();
     if (tid == 0) {
@@ -377,18 +492,15 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         for (uint32_t it = 0; it < (1u << 20); ++it) if (mbar_try_wait(bar, parity)) return;
       };
       for (int s = 0; s < p.ring; ++s) {
-        const int fills = issued > s ? (issued - s + p.ring - 1) / p.ring : 0;     // k-blocks j < issued with j % ring == s
-        if (fills == 0) continue;
-        const uint32_t parity = (uint32_t)(fills - 1) & 1u;
-        drain(bar_raw + 8u * s, parity);
-        drain(bar_full + 8u * s, parity);
+        if (full_used >> s & 1u) drain(bar_full + 8u * s, full_phase >> s & 1u);
+        if (raw_used >> s & 1u) drain(bar_raw + 8u * s, raw_phase >> s & 1u);
       }
       drain(bar_drain, 0u);
     }
     __syncthreads();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
   }
 }
 
@@ -424,44 +536,52 @@ bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t row_bytes
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int num_sms() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-      n = 148;
-  }
-  return n;
-}
 
-// Tile width: a multiple of 32 (epilogue groups) that divides N, at most 256; among those, the one that needs the
-// fewest "waves x (columns per tile + fixed per-tile work)" on this many SMs.
-int pick_bn(int N, int m_tiles, int sms) {
-  int best = 0; long best_cost = 0;
+// Tile width and the epilogue's division of labour.  The width is a multiple of 32 that divides `unit` (N; for QKV the
+// width C of a section, so that a tile has one quantizer), at most 256.  The epilogue bounds every shape here; in units of
+// 32 columns a warp needs (columns / 32 of its tile share + about 0.6 of fixed work) per tile, and `groups` tiles are in
+// work at once.  Many tiles per CTA: whole tiles per warp (groups = accumulators), the fixed work is paid once per tile;
+// few: all warps share a tile, its latency counts.
+#ifndef GMAX
+#define GMAX 4
+#endif
+struct Tiling { int bn, n_acc, groups, split; };
+Tiling pick_tiling(int unit, int N, int m_tiles, int k_blocks, int sms, int warps, int chunk) {
+  Tiling best = {0, 0, 0, 0};
+  double best_cost = 0.0;
+  const int per_quarter = warps / 4;
   for (int bn = 32; bn <= MAX_BN; bn += 32) {
-    if (N % bn) continue;
-    const long tiles = (long)m_tiles * (N / bn);
-    const long waves = (tiles + sms - 1) / sms;
-    const long cost = waves * (bn + 48);
-    if (!best || cost <= best_cost) { best = bn; best_cost = cost; }
+    if (unit % bn) continue;
+    const int n_acc = bn <= TMEM_COLS / 4 ? 4 : 2;
+    const long tiles = (long)m_tiles * (N / bn), per_cta = (tiles + sms - 1) / sms;
+    for (int groups = 1; groups <= per_quarter && groups <= n_acc && groups <= GMAX; groups *= 2) {
+      if (per_quarter % groups) continue;
+      const int split = per_quarter / groups;
+      const double chunks = (bn / chunk + split - 1) / split * (chunk / 32.0);
+      const long rounds = (per_cta + groups - 1) / groups;
+      const double cost = rounds * (chunks + 0.6) + 0.03 * k_blocks * per_cta;
+      if (!best.bn || cost <= best_cost) { best = {bn, n_acc, groups, split}; best_cost = cost; }
+    }
   }
   return best;
 }
 
-template <int MODE>
+template <int MODE, int EW>
 bool launch_mode(const GemmArgs& g, int* status, cudaStream_t st) {
   TcParams p;
   p.g = g; p.status = status;
+  p.g.neg_zero = -0.0f;
   const int t0 = (g.br[0].M + BM - 1) / BM, t1 = (g.br[1].M + BM - 1) / BM;
   if (t0 + t1 == 0) return true;
   if (g.N % 32 || g.K % UMMA_K) return false;
-  const int sms = num_sms();
-  p.tiles_m0 = t0;
-  p.BN = pick_bn(g.N, t0 + t1, sms);
-  if (p.BN == 0) return false;
-  p.n_tiles = g.N / p.BN;
-  p.total_tiles = (t0 + t1) * p.n_tiles;
+  const int sms = sm_count();
+  p.tiles_m0 = t0; p.tiles_m = t0 + t1;
   p.k_blocks = (g.K + BK - 1) / BK;
+  const Tiling tl = pick_tiling(MODE == EPI_QKV ? g.C : g.N, g.N, t0 + t1, p.k_blocks, sms, EW, code_mode(MODE) ? CODE_NC : F32_NC);
+  if (tl.bn == 0) return false;
+  p.BN = tl.bn; p.n_acc = tl.n_acc; p.groups = tl.groups; p.split = tl.split;
+  p.n_tiles = g.N / p.BN;
+  const int total_tiles = (t0 + t1) * p.n_tiles;
   // packed branches whose row pitch the TMA unit accepts (a multiple of 16 bytes) are staged by TMA
   p.packed_bytes = 0;
   for (int i = 0; i < 2; ++i) {
@@ -469,11 +589,8 @@ bool launch_mode(const GemmArgs& g, int* status, cudaStream_t st) {
     p.tma_packed[i] = g.br[i].M > 0 && bits != 8 && ((long)g.K * bits / 8) % 16 == 0;
     if (p.tma_packed[i]) p.packed_bytes = BM * (BK / 2);        // room for the widest packed format (4 bit)
   }
-  p.res_bytes = (g.mode == EPI_PROJ || g.mode == EPI_FC2) ? epi_warps(g.mode) * RES_SLOTS * EPI_STAGE_FLOATS * 4 : 0;
-  p.ring = MAX_RING;
-  while (p.ring > 2 && smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, epi_warps(MODE)).total + 1024 > 220 * 1024) --p.ring;
-  p.tmem_cols = 32;
-  while (p.tmem_cols < 2 * p.BN) p.tmem_cols <<= 1;
+  p.res_bytes = (g.mode == EPI_PROJ || g.mode == EPI_FC2) ? EW * RES_SLOTS * EPI_STAGE_FLOATS * 4 : 0;
+  p.acc_stride = p.BN;
   CUtensorMap mA[2], mB;
   memset(mA, 0, sizeof(mA));
   for (int i = 0; i < 2; ++i) {
@@ -488,19 +605,25 @@ bool launch_mode(const GemmArgs& g, int* status, cudaStream_t st) {
     if (!ok) return false;
   }
   if (!make_map(&mB, g.w, (uint64_t)g.N, (uint64_t)g.K, (uint32_t)p.BN)) return false;
-  const size_t smem = (size_t)smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, epi_warps(MODE)).total + 1024 /*alignment slack*/;
-  if (smem > 227 * 1024) return false;
   // a grid that is a multiple of the number of column tiles keeps every CTA on one column tile (t mod n_tiles);
   // taken only where it does not cost a wave of tiles
-  int grid = p.total_tiles < sms ? p.total_tiles : sms;
-  if (grid > p.n_tiles && grid < p.total_tiles) {
+  int grid = total_tiles < sms ? total_tiles : sms;
+  if (grid > p.n_tiles && grid < total_tiles) {
     const int g2 = grid - grid % p.n_tiles;
-    if ((p.total_tiles + g2 - 1) / g2 == (p.total_tiles + grid - 1) / grid) grid = g2;
+    if ((total_tiles + g2 - 1) / g2 == (total_tiles + grid - 1) / grid) grid = g2;
   }
+  p.step_m = grid / p.n_tiles; p.step_n = grid % p.n_tiles;
+  p.gstep_m = grid * p.groups / p.n_tiles; p.gstep_n = grid * p.groups % p.n_tiles;
+  p.const_cols = p.step_n == 0 || total_tiles == grid ? p.BN : g.N;
+  p.last_step = total_tiles - 1;
+  p.ring = MAX_RING;
+  while (p.ring > 2 && smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW).total + 1024 > 220 * 1024) --p.ring;
+  const size_t smem = (size_t)smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW).total + 1024 /*alignment slack*/;
+  if (smem > 227 * 1024) return false;
   if (g.br[0].tap_acc || g.br[1].tap_acc)
-    k_gemm_tc<MODE, true><<<grid, 32 * (2 + unpack_warps(MODE) + epi_warps(MODE)), smem, st>>>(mA[0], mA[1], mB, p);
+    launch_pdl(k_gemm_tc<MODE, true, EW>, dim3(grid), num_threads(EW), smem, st, mA[0], mA[1], mB, p);
   else
-    k_gemm_tc<MODE, false><<<grid, 32 * (2 + unpack_warps(MODE) + epi_warps(MODE)), smem, st>>>(mA[0], mA[1], mB, p);
+    launch_pdl(k_gemm_tc<MODE, false, EW>, dim3(grid), num_threads(EW), smem, st, mA[0], mA[1], mB, p);
   ++g_launches;
   return true;
 }
@@ -602,7 +725,7 @@ __global__ void __launch_bounds__(128, 1) k_mma_peak(int groups, unsigned long l
 
 // ns_out: one entry per SM (device memory).  Returns the grid size, 0 on failure.
 int launch_mma_peak(int kind, int groups, unsigned long long* ns_out, int* status, cudaStream_t st) {
-  const int sms = num_sms();
+  const int sms = sm_count();
   const size_t smem = A_STAGE_BYTES + MAX_BN * BK + 1024 + 64;
   if (kind == 0) {
     if (cudaFuncSetAttribute(k_mma_peak<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
@@ -621,27 +744,27 @@ int launch_mma_peak(int kind, int groups, unsigned long long* ns_out, int* statu
 // One-time set-up per device context (kept out of the launch path so that launches can be stream-captured):
 // opt-in to large dynamic shared memory for every epilogue mode, resolve the tensor-map encoder, read the SM count.
 bool gemm_init() {
-  bool ok = encode_fn() != nullptr && num_sms() > 0;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_QKV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_QKV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_PROJ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_PROJ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_FC1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_FC1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_FC2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_FC2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_MERGE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_gemm_tc<EPI_MERGE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
+  bool ok = encode_fn() != nullptr && sm_count() > 0;
+  auto big_smem = [&](auto kernel) { ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess; };
+  big_smem(k_gemm_tc<EPI_QKV, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_QKV, true, CODE_WARPS>);
+  big_smem(k_gemm_tc<EPI_QKV, false, CODE_WARPS_MANY>); big_smem(k_gemm_tc<EPI_QKV, true, CODE_WARPS_MANY>);
+  big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS>);
+  big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS_MANY>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS_MANY>);
+  big_smem(k_gemm_tc<EPI_PROJ, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_PROJ, true, F32_WARPS>);
+  big_smem(k_gemm_tc<EPI_FC2, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_FC2, true, F32_WARPS>);
+  big_smem(k_gemm_tc<EPI_MERGE, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_MERGE, true, F32_WARPS>);
   return ok;
 }
 
 bool launch_gemm(const GemmArgs& g, cudaStream_t st) {
+  const long row_tiles = (long)(g.br[0].M + BM - 1) / BM + (g.br[1].M + BM - 1) / BM;
+  const bool many = row_tiles >= (long)MANY_ROW_TILES * sm_count();
   switch (g.mode) {
-    case EPI_QKV:   return launch_mode<EPI_QKV>(g, g.status, st);
-    case EPI_PROJ:  return launch_mode<EPI_PROJ>(g, g.status, st);
-    case EPI_FC1:   return launch_mode<EPI_FC1>(g, g.status, st);
-    case EPI_FC2:   return launch_mode<EPI_FC2>(g, g.status, st);
-    case EPI_MERGE: return launch_mode<EPI_MERGE>(g, g.status, st);
+    case EPI_QKV:   return many ? launch_mode<EPI_QKV, CODE_WARPS_MANY>(g, g.status, st) : launch_mode<EPI_QKV, CODE_WARPS>(g, g.status, st);
+    case EPI_FC1:   return many ? launch_mode<EPI_FC1, CODE_WARPS_MANY>(g, g.status, st) : launch_mode<EPI_FC1, CODE_WARPS>(g, g.status, st);
+    case EPI_PROJ:  return launch_mode<EPI_PROJ, F32_WARPS>(g, g.status, st);
+    case EPI_FC2:   return launch_mode<EPI_FC2, F32_WARPS>(g, g.status, st);
+    case EPI_MERGE: return launch_mode<EPI_MERGE, F32_WARPS>(g, g.status, st);
   }
   return false;
 }

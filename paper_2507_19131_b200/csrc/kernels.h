@@ -10,6 +10,22 @@ namespace mixaq {
 // contexts from different threads do not disturb each other's counts
 extern thread_local int g_launches;
 
+// Launch with programmatic stream serialization (see griddep_wait): the kernel has to call griddep_wait() itself before it
+// touches what earlier kernels wrote.  In a 224 x 224 Swin-T forward the launches are 5 us each of which 2 to 3 are start-up.
+#ifndef PDLN
+#define PDLN 1
+#endif
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = &attr; cfg.numAttrs = PDLN;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- selection ------------------------------------------------------------------------------
 void launch_energy(const float* x, int32_t* energy, long ntok, int C, float inv_scale, cudaStream_t st);
 
@@ -69,8 +85,9 @@ struct GemmBranch {
   const uint8_t* a;          // [M][K*a_bits/8] packed unsigned codes
   int M, a_bits;
   const float* mult;         // [N]  s_a * s_w[n]
-  const int32_t* zc;         // [N]  z_a * sum_k w[n][k]
+  const int32_t* pre;        // [N]  0x4B400000 - z_a * sum_k w[n][k]
   const float* bias;         // [N]  (nullable for EPI_MERGE)
+  const float* bound;        // [N]  largest |acc * mult| the channel can reach (see k_prepare_linear)
   AQ q0, q1, q2;             // output quantizers (QKV: q,k,v; FC1: q0)
   int out_bits;
   uint8_t* out_codes;        // QKV, FC1: [M][N*out_bits/8]
@@ -83,14 +100,17 @@ struct GemmArgs {
   const int8_t* w;           // [N][K]
   int N, K, C;               // C: channels per q/k/v section (EPI_QKV)
   int mode;
+  float neg_zero;        // -0.0f, from the host so that the compiler cannot see it (see quant_pattern2)
   int* status;           // device status word (raised when a bounded wait runs out)
   GemmBranch br[2];
 };
 bool launch_gemm(const GemmArgs& g, cudaStream_t st);
+int sm_count();                                          // of the current device (read once)
 void launch_wait_probe(int* status, cudaStream_t st);   // self-test of the bounded wait (it must run out)
 // tensor-core issue-rate microbenchmark (kind 0: i8, 1: f8f6f4/E4M3); ns per SM into ns_out; returns the grid size
 int launch_mma_peak(int kind, int groups, unsigned long long* ns_out, int* status, cudaStream_t st);
 bool gemm_init();   // once per device context, before the first launch
+bool ln_init();     // the same for the LayerNorm kernels
 
 // ---- fused window attention ----------------------------------------------------------------------
 struct AttnBranch {
@@ -135,8 +155,8 @@ bool launch_calibrate_merge(const CalMergeArgs& c, cudaStream_t st);
 float cal_key_to_float(uint32_t key);
 
 // ---- preparation -----------------------------------------------------------------------------------
-void launch_prepare_linear(const int8_t* w, const float* sw, int N, int K, float sa, int za, float* mult,
-                           int32_t* zc, cudaStream_t st);
+void launch_prepare_linear(const int8_t* w, const float* sw, int N, int K, float sa, int za, int bits, float* mult,
+                           int32_t* pre, float* bound, cudaStream_t st);
 void launch_prepare_relbias(const float* table, int heads, float* out, cudaStream_t st);
 
 }  // namespace mixaq

@@ -108,13 +108,14 @@ extern "C" mixaq_status mixaq_merge_forward_static(mixaq_ctx* ctx, const mixaq_m
   mg.B = B; mg.H = H; mg.W = W; mg.C = C;
   launch_merge_gather(mg, st);
   float* mult = reinterpret_cast<float*>(p->prepared);
-  int32_t* zc = reinterpret_cast<int32_t*>(static_cast<char*>(p->prepared) + round256((size_t)N * 4));
+  int32_t* pre = reinterpret_cast<int32_t*>(static_cast<char*>(p->prepared) + round256((size_t)N * 4));
+  float* bound = reinterpret_cast<float*>(static_cast<char*>(p->prepared) + 2 * round256((size_t)N * 4));
   GemmArgs ga;
   ga.status = ctx_status_word(ctx);
   ga.w = p->reduction.codes; ga.N = N; ga.K = K; ga.C = N; ga.mode = EPI_MERGE;
   for (int i = 0; i < 2; ++i) {
     memset(&ga.br[i], 0, sizeof(GemmBranch));
-    ga.br[i].a_bits = bits; ga.br[i].mult = mult; ga.br[i].zc = zc;
+    ga.br[i].a_bits = bits; ga.br[i].mult = mult; ga.br[i].pre = pre; ga.br[i].bound = bound;
   }
   ga.br[0].a = scratch; ga.br[0].M = M; ga.br[0].out_f = y;
   if (!launch_gemm(ga, st)) {

@@ -35,6 +35,7 @@ struct mixaq_ctx {
   bool guards;                         // fill the guard zones of the workspace before a forward, compare them after it
   bool nvtx;                           // name every kernel family, stage and block with an NVTX range (host side)
   bool allow_elevation;                // backbone: every pair uses its own ratios even if an earlier pair of the stage had larger ones
+  cudaStream_t capture_stream;         // forwards on a stream that cannot be captured (the legacy default one) are recorded here
   std::vector<GraphEntry> graphs;
   std::vector<ProfRec> prof;          // event pairs recorded since mixaq_profile_begin
   std::vector<cudaEvent_t> pool;      // events ready for reuse
@@ -194,13 +195,15 @@ mixaq_status validate_block(mixaq_ctx* ctx, const mixaq_block_params* p, bool ne
 
 // layout of a block's prepared buffer
 struct Prepared {
-  float* mult[4][2]; int32_t* zc[4][2]; float* relbias; size_t bytes;
+  float* mult[4][2]; int32_t* pre[4][2]; float* bound[4][2]; float* relbias; size_t bytes;
 };
 Prepared carve_prepared(const mixaq_block_params* p, void* base) {
   Prepared r; Carver c(base, false);
   const int N[4] = {3 * p->dim, p->dim, p->hidden, p->dim};
   for (int l = 0; l < 4; ++l)
-    for (int b = 0; b < 2; ++b) { r.mult[l][b] = c.take<float>(N[l]); r.zc[l][b] = c.take<int32_t>(N[l]); }
+    for (int b = 0; b < 2; ++b) {
+      r.mult[l][b] = c.take<float>(N[l]); r.pre[l][b] = c.take<int32_t>(N[l]); r.bound[l][b] = c.take<float>(N[l]);
+    }
   r.relbias = c.take<float>((size_t)p->heads * 4 * 7 * 32 * 4);   // fragment order, see k_prepare_relbias
   r.bytes = c.off;
   return r;
@@ -270,10 +273,10 @@ SelectArgs make_select_args(const SelWs& sel, const int32_t* energy, int B, int 
   return sa;
 }
 
-void fill_gemm_branch(GemmBranch& g, const uint8_t* a, int M, int a_bits, const float* mult, const int32_t* zc,
-                      const float* bias) {
+void fill_gemm_branch(GemmBranch& g, const uint8_t* a, int M, int a_bits, const float* mult, const int32_t* pre,
+                      const float* bound, const float* bias) {
   memset(&g, 0, sizeof(g));
-  g.a = a; g.M = M; g.a_bits = a_bits; g.mult = mult; g.zc = zc; g.bias = bias;
+  g.a = a; g.M = M; g.a_bits = a_bits; g.mult = mult; g.pre = pre; g.bound = bound; g.bias = bias;
 }
 
 }  // namespace
@@ -299,9 +302,9 @@ mixaq_status mixaq_create(mixaq_ctx** out, int device) {
   if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return MIXAQ_CUDA_ERROR; }
   mixaq_ctx* c = new (std::nothrow) mixaq_ctx();
   if (!c) return MIXAQ_INTERNAL;
-  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false;
+  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr;
   if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess || cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess ||
-      !gemm_init()) {
+      !gemm_init() || !ln_init()) {
     cudaGetLastError(); if (c->d_status) cudaFree(c->d_status); delete c; return MIXAQ_CUDA_ERROR;
   }
   *out = c;
@@ -311,6 +314,7 @@ mixaq_status mixaq_create(mixaq_ctx** out, int device) {
 mixaq_status mixaq_destroy(mixaq_ctx* ctx) {
   if (!ctx) return MIXAQ_INVALID_ARG;
   if (ctx->d_status) cudaFree(ctx->d_status);
+  if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
   for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
   for (cudaGraphExec_t g : ctx->prof_execs) cudaGraphExecDestroy(g);
   for (auto& r : ctx->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
@@ -432,7 +436,7 @@ mixaq_status mixaq_block_prepare(mixaq_ctx* ctx, const mixaq_block_params* p, vo
     const mixaq_aq* in[4] = {&br.qkv_in, &br.proj_in, &br.fc1_in, &br.fc2_in};
     for (int l = 0; l < 4; ++l)
       launch_prepare_linear(L[l]->codes, L[l]->scale, L[l]->out_features, L[l]->in_features, in[l]->scale,
-                            in[l]->zero_point, pr.mult[l][b], pr.zc[l][b], st);
+                            in[l]->zero_point, in[l]->bits, pr.mult[l][b], pr.pre[l][b], pr.bound[l][b], st);
   }
   launch_prepare_relbias(p->relpos_table, p->heads, pr.relbias, st);
   return check_cuda(ctx, "block_prepare");
@@ -440,7 +444,7 @@ mixaq_status mixaq_block_prepare(mixaq_ctx* ctx, const mixaq_block_params* p, vo
 
 size_t mixaq_merge_prepared_bytes(const mixaq_merge_params* p) {
   if (!p || p->reduction.out_features <= 0) return 0;
-  return align_up((size_t)p->reduction.out_features * 4) * 2;
+  return align_up((size_t)p->reduction.out_features * 4) * 3;
 }
 
 mixaq_status mixaq_merge_prepare(mixaq_ctx* ctx, const mixaq_merge_params* p, void* cuda_stream) {
@@ -448,9 +452,10 @@ mixaq_status mixaq_merge_prepare(mixaq_ctx* ctx, const mixaq_merge_params* p, vo
   if (!p->prepared || !p->reduction.codes || !p->reduction.scale) return fail(ctx, MIXAQ_INVALID_ARG, "merge params incomplete");
   Carver c(p->prepared, false);
   float* mult = c.take<float>(p->reduction.out_features);
-  int32_t* zc = c.take<int32_t>(p->reduction.out_features);
+  int32_t* pre = c.take<int32_t>(p->reduction.out_features);
+  float* bound = c.take<float>(p->reduction.out_features);
   launch_prepare_linear(p->reduction.codes, p->reduction.scale, p->reduction.out_features, p->reduction.in_features,
-                        p->in.scale, p->in.zero_point, mult, zc, (cudaStream_t)cuda_stream);
+                        p->in.scale, p->in.zero_point, p->in.bits, mult, pre, bound, (cudaStream_t)cuda_stream);
   return check_cuda(ctx, "merge_prepare");
 }
 
@@ -501,7 +506,12 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   g_launches = 0;
 
   // 1. scores and selection
-  const SelWs& sel = presel ? *presel : ws.sel;
+  SelWs sel = presel ? *presel : ws.sel;
+  if (sel_out && !presel) {                  // the selection kernels write the caller's buffers themselves
+    if (sel_out->cls) sel.cls = sel_out->cls;
+    if (sel_out->order) sel.order = sel_out->order;
+    if (sel_out->score) sel.score = sel_out->score;
+  }
   if (!presel) {
     const int32_t* energy = opts ? opts->energy : nullptr;
     if (!energy) { PROF(PC_ENERGY); launch_energy(x, ws.energy, (long)B * H * W, C, p->score_inv_scale, st); energy = ws.energy; }
@@ -509,10 +519,6 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
     { PROF(PC_SELECT); launch_select(&sa, 1, st); }
   }
   if (sel_out) {
-    const size_t n = (size_t)B * g.nW;
-    if (sel_out->cls)   cudaMemcpyAsync(sel_out->cls, sel.cls, n, cudaMemcpyDeviceToDevice, st);
-    if (sel_out->order) cudaMemcpyAsync(sel_out->order, sel.order, n * 4, cudaMemcpyDeviceToDevice, st);
-    if (sel_out->score) cudaMemcpyAsync(sel_out->score, sel.score, n * 8, cudaMemcpyDeviceToDevice, st);
     if (sel_out->idx_hi || sel_out->idx_lo || sel_out->idx_pr) {
       int32_t* const lists[3] = {sel_out->idx_hi, sel_out->idx_lo, sel_out->idx_pr};
       const int cnt[3] = {g.n_hi, g.n_lo, g.n_pr};
@@ -540,7 +546,7 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   ga.status = ctx->d_status;
   ga.w = p->qkv.codes; ga.N = 3 * C; ga.K = C; ga.C = C; ga.mode = EPI_QKV;
   for (int i = 0; i < 2; ++i) {
-    fill_gemm_branch(ga.br[i], ws.a[i], M[i], cb[i], pr.mult[0][i], pr.zc[0][i], brp[i]->b_qkv);
+    fill_gemm_branch(ga.br[i], ws.a[i], M[i], cb[i], pr.mult[0][i], pr.pre[0][i], pr.bound[0][i], brp[i]->b_qkv);
     ga.br[i].q0 = to_aq(brp[i]->q); ga.br[i].q1 = to_aq(brp[i]->k); ga.br[i].q2 = to_aq(brp[i]->v);
     ga.br[i].out_bits = cb[i]; ga.br[i].out_codes = ws.qkv[i];
     ga.br[i].tap_acc = tp[i] ? tp[i]->qkv_acc : nullptr;
@@ -566,7 +572,7 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   // 5. proj GEMM + attention residual -> x1
   ga.w = p->proj.codes; ga.N = C; ga.K = C; ga.mode = EPI_PROJ;
   for (int i = 0; i < 2; ++i) {
-    fill_gemm_branch(ga.br[i], ws.o[i], M[i], cb[i], pr.mult[1][i], pr.zc[1][i], brp[i]->b_proj);
+    fill_gemm_branch(ga.br[i], ws.o[i], M[i], cb[i], pr.mult[1][i], pr.pre[1][i], pr.bound[1][i], brp[i]->b_proj);
     ga.br[i].out_f = ws.x1[i]; ga.br[i].res = x; ga.br[i].rowsrc = sel.rowsrc[i];
     ga.br[i].tap_acc = tp[i] ? tp[i]->proj_acc : nullptr;
   }
@@ -582,7 +588,7 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   // 7. fc1 GEMM + GELU + requantize
   ga.w = p->fc1.codes; ga.N = Hd; ga.K = C; ga.mode = EPI_FC1;
   for (int i = 0; i < 2; ++i) {
-    fill_gemm_branch(ga.br[i], ws.f1[i], M[i], cb[i], pr.mult[2][i], pr.zc[2][i], brp[i]->b_fc1);
+    fill_gemm_branch(ga.br[i], ws.f1[i], M[i], cb[i], pr.mult[2][i], pr.pre[2][i], pr.bound[2][i], brp[i]->b_fc1);
     ga.br[i].q0 = to_aq(brp[i]->fc2_in); ga.br[i].out_bits = cb[i]; ga.br[i].out_codes = ws.f2[i];
     ga.br[i].tap_acc = tp[i] ? tp[i]->fc1_acc : nullptr;
   }
@@ -591,7 +597,7 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   // 8. fc2 GEMM + residual + scatter (reverse shift, crop)
   ga.w = p->fc2.codes; ga.N = C; ga.K = Hd; ga.mode = EPI_FC2;
   for (int i = 0; i < 2; ++i) {
-    fill_gemm_branch(ga.br[i], ws.f2[i], M[i], cb[i], pr.mult[3][i], pr.zc[3][i], brp[i]->b_fc2);
+    fill_gemm_branch(ga.br[i], ws.f2[i], M[i], cb[i], pr.mult[3][i], pr.pre[3][i], pr.bound[3][i], brp[i]->b_fc2);
     ga.br[i].out_f = y; ga.br[i].res = ws.x1[i]; ga.br[i].rowsrc = sel.rowsrc[i];
     ga.br[i].tap_acc = tp[i] ? tp[i]->fc2_acc : nullptr;
   }
@@ -657,13 +663,14 @@ mixaq_status mixaq_merge_forward(mixaq_ctx* ctx, const mixaq_merge_params* p, co
   { PROF(PC_MERGE_GATHER); launch_merge_gather(mg, st); }
   Carver c(p->prepared, false);
   float* mult = c.take<float>(N);
-  int32_t* zc = c.take<int32_t>(N);
+  int32_t* pre = c.take<int32_t>(N);
+  float* bound = c.take<float>(N);
   GemmArgs ga;
   ga.status = ctx->d_status;
   ga.w = p->reduction.codes; ga.N = N; ga.K = K; ga.C = N; ga.mode = EPI_MERGE;
-  fill_gemm_branch(ga.br[0], (const uint8_t*)workspace, M, p->in.bits, mult, zc, nullptr);
+  fill_gemm_branch(ga.br[0], (const uint8_t*)workspace, M, p->in.bits, mult, pre, bound, nullptr);
   ga.br[0].out_f = y;
-  fill_gemm_branch(ga.br[1], nullptr, 0, p->in.bits, mult, zc, nullptr);
+  fill_gemm_branch(ga.br[1], nullptr, 0, p->in.bits, mult, pre, bound, nullptr);
   { PROF(PC_MERGE_GEMM); if (!launch_gemm(ga, st)) return fail(ctx, MIXAQ_INTERNAL, "GEMM launch set-up failed (tensor map / tile shape)"); }
   ctx->launches = g_launches;
   return check_cuda(ctx, "merge_forward");
@@ -761,8 +768,17 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
 
   // Replay as a CUDA graph when an identical call was captured before.  The key is made of every value that
   // shapes the launches: the fields of the HOST parameter structs, ratios, pointers, sizes and the stream.
-  bool use_graph = ctx->graph_cache && st != nullptr && st != cudaStreamLegacy;
-  if (use_graph) {
+  bool use_graph = ctx->graph_cache;
+  // The legacy default stream cannot be captured, but a graph can be launched on it: such calls are recorded on a stream
+  // of the context's own (stage1_pair and Swin-T calls on it were bound by one host launch per kernel).
+  const cudaStream_t user_stream = st;
+  if (use_graph && (st == nullptr || st == cudaStreamLegacy)) {
+    if (ctx->profiling) use_graph = false;       // profiled as stream launches
+    else if (!ctx->capture_stream && cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError(); ctx->capture_stream = nullptr; use_graph = false;
+    } else st = ctx->capture_stream;
+  }
+  if (use_graph && user_stream == st) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) { cudaGetLastError(); use_graph = false; }
   }
@@ -815,16 +831,17 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
     put(low_ratio_per_pair, sizeof(float) * npairs);
     const char has_prune = prune_ratio_per_pair ? 1 : 0; put(&has_prune, 1);
     if (prune_ratio_per_pair) put(prune_ratio_per_pair, sizeof(float) * npairs);
-    put(&workspace, sizeof(workspace)); put(&workspace_bytes, sizeof(workspace_bytes)); put(&st, sizeof(st));
+    put(&workspace, sizeof(workspace)); put(&workspace_bytes, sizeof(workspace_bytes)); put(&user_stream, sizeof(user_stream));
     const char elev = (ctx->allow_elevation ? 1 : 0) | (ctx->reverse_selection ? 2 : 0); put(&elev, 1);
     for (auto& g : ctx->graphs)
       if (g.key == key) {
-        if (cudaGraphLaunch(g.exec, st) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
+        if (cudaGraphLaunch(g.exec, user_stream) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
         ctx->launches = g.launches;
         return MIXAQ_OK;
       }
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); use_graph = false; }
   }
+  if (!use_graph) st = user_stream;
 
   mixaq_status result = MIXAQ_OK;
   int total = 0, H = H0, W = W0, blk = 0;
@@ -915,7 +932,7 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
       if (ctx->graphs.size() >= 16) { cudaGraphExecDestroy(ctx->graphs.front().exec); ctx->graphs.erase(ctx->graphs.begin()); }
       ctx->graphs.push_back({key, exec, total});
     }
-    if (cudaGraphLaunch(exec, st) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
+    if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
   }
   if (result != MIXAQ_OK) return result;
   ctx->launches = total;
@@ -926,11 +943,11 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
 // stem and output norms
 namespace {
 constexpr int EMBED_K = 48, EMBED_KP = 64;     // patch vector, padded to a multiple of 32 codes
-struct EmbedPrepared { int8_t* w; float* mult; int32_t* zc; size_t bytes; };
+struct EmbedPrepared { int8_t* w; float* mult; int32_t* pre; float* bound; size_t bytes; };
 EmbedPrepared carve_embed(const mixaq_embed_params* p, void* base) {
   EmbedPrepared r; Carver c(base, false);
   const int N = p->proj.out_features;
-  r.w = c.take<int8_t>((size_t)N * EMBED_KP); r.mult = c.take<float>(N); r.zc = c.take<int32_t>(N);
+  r.w = c.take<int8_t>((size_t)N * EMBED_KP); r.mult = c.take<float>(N); r.pre = c.take<int32_t>(N); r.bound = c.take<float>(N);
   r.bytes = c.off;
   return r;
 }
@@ -953,7 +970,7 @@ mixaq_status mixaq_embed_prepare(mixaq_ctx* ctx, const mixaq_embed_params* p, vo
   EmbedPrepared pr = carve_embed(p, p->prepared);
   const int N = p->proj.out_features;
   launch_pad_weights(p->proj.codes, N, EMBED_K, EMBED_KP, pr.w, st);
-  launch_prepare_linear(pr.w, p->proj.scale, N, EMBED_KP, p->in.scale, p->in.zero_point, pr.mult, pr.zc, st);
+  launch_prepare_linear(pr.w, p->proj.scale, N, EMBED_KP, p->in.scale, p->in.zero_point, p->in.bits, pr.mult, pr.pre, pr.bound, st);
   return check_cuda(ctx, "embed_prepare");
 }
 
@@ -987,9 +1004,9 @@ mixaq_status mixaq_embed_forward(mixaq_ctx* ctx, const mixaq_embed_params* p, co
   GemmArgs ga;
   ga.status = ctx->d_status;
   ga.w = pr.w; ga.N = N; ga.K = EMBED_KP; ga.C = N; ga.mode = EPI_MERGE;      // dequantize only: acc * mult
-  fill_gemm_branch(ga.br[0], codes, (int)toks, 8, pr.mult, pr.zc, nullptr);
+  fill_gemm_branch(ga.br[0], codes, (int)toks, 8, pr.mult, pr.pre, pr.bound, nullptr);
   ga.br[0].out_f = t;
-  fill_gemm_branch(ga.br[1], nullptr, 0, 8, pr.mult, pr.zc, nullptr);
+  fill_gemm_branch(ga.br[1], nullptr, 0, 8, pr.mult, pr.pre, pr.bound, nullptr);
   if (!launch_gemm(ga, st)) return fail(ctx, MIXAQ_INTERNAL, "GEMM launch set-up failed (tensor map / tile shape)");
   if (!launch_bias_ln(t, p->bias, p->ln_g, p->ln_b, x0, (long)toks, N, st)) return fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "embed: unsupported C0");
   ctx->launches = g_launches;

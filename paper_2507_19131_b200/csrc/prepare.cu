@@ -4,17 +4,29 @@
 
 namespace mixaq {
 
-// one warp per output channel: zc[n] = z_a * sum_k w[n][k];  mult[n] = s_a * s_w[n]
+// one warp per output channel: mult[n] = s_a * s_w[n];
+// pre[n] = 0x4B400000 - z_a * sum_k w[n][k], what the GEMM's epilogue adds to the raw sums (see acc_to_float2);
+// bound[n]: no dequantized sum |mult * acc| exceeds it (|a - z_a| <= qmax_a, so |acc| <= qmax_a * sum_k |w[n][k]|), or
+// infinity where |acc| could reach the 2^22 that this leaves room for.
 __global__ void __launch_bounds__(256) k_prepare_linear(const int8_t* __restrict__ w, const float* __restrict__ sw,
-                                                        int N, int K, float sa, int za, float* mult, int32_t* zc) {
+                                                        int N, int K, float sa, int za, int qmax, float* mult, int32_t* pre,
+                                                        float* bound) {
   int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
   if (n >= N) return;
-  int s = 0;
-  for (int k = lane; k < K; k += 32) s += (int)w[(long)n * K + k];
+  int s = 0, sabs = 0;
+  for (int k = lane; k < K; k += 32) { const int c = (int)w[(long)n * K + k]; s += c; sabs += c < 0 ? -c : c; }
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if (lane == 0) { zc[n] = za * s; mult[n] = __fmul_rn(sa, sw[n]); }
+  for (int off = 16; off >= 1; off >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, off);
+    sabs += __shfl_xor_sync(0xffffffffu, sabs, off);
+  }
+  if (lane == 0) {
+    pre[n] = (int32_t)(kMagicBits - (uint32_t)(za * s));
+    mult[n] = __fmul_rn(sa, sw[n]);
+    const long most = (long)qmax * sabs;
+    bound[n] = most < (1L << 22) - 16 ? fabsf(mult[n]) * (float)most * 1.0001f : INFINITY;
+  }
 }
 
 // Relative-position bias in the order the attention kernel's accumulator fragments want it:
@@ -37,9 +49,9 @@ __global__ void k_prepare_relbias(const float* __restrict__ table, int heads, fl
   out[idx] = v;
 }
 
-void launch_prepare_linear(const int8_t* w, const float* sw, int N, int K, float sa, int za, float* mult,
-                           int32_t* zc, cudaStream_t st) {
-  k_prepare_linear<<<(N + 7) / 8, 256, 0, st>>>(w, sw, N, K, sa, za, mult, zc);
+void launch_prepare_linear(const int8_t* w, const float* sw, int N, int K, float sa, int za, int bits, float* mult,
+                           int32_t* pre, float* bound, cudaStream_t st) {
+  k_prepare_linear<<<(N + 7) / 8, 256, 0, st>>>(w, sw, N, K, sa, za, (1 << bits) - 1, mult, pre, bound);
   ++g_launches;
 }
 

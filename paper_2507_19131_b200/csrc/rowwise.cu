@@ -12,6 +12,8 @@ namespace mixaq {
 // (gamma, beta, quantizer) are fetched once per warp and no per-row selection is left in the loop.
 template <int NPL, int R>
 __global__ void __launch_bounds__(256) k_ln_quant(LnBranch hi, LnBranch lo, int blocks_hi) {
+  griddep_launch();
+  griddep_wait();
   const int C = NPL * 32;
   const int lane = threadIdx.x & 31;
   const bool is_hi = (int)blockIdx.x < blocks_hi;
@@ -62,57 +64,13 @@ __global__ void __launch_bounds__(256) k_ln_quant(LnBranch hi, LnBranch lo, int 
 // between lanes followed by a tree inside the lane -- the same additions in the same order.
 // MERGE: the rows are the output tokens of a patch merging: channel group i of a row comes from input neighbour
 // i / (NG/4) (order (0,0), (1,0), (0,1), (1,1)); neighbours outside the map are zeros that take part in the LayerNorm.
-template <int NG, int G, bool MERGE>
-__global__ void __launch_bounds__(256, (NG * (32 / G) > 24 ? 2 : 4)) k_ln_quant_g(LnBranch hi, LnBranch lo, int blocks_hi) {
-  constexpr int C = NG * 32, P = 32 / G, ROWS = 32 / G;     // channels, partials per lane, rows per warp
-  constexpr int VEC = P >= 4 ? 4 : 2;                       // floats per load
-  static_assert(P >= 2 && (!MERGE || NG % 4 == 0), "unsupported lane split");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = lane % G, rw = lane / G;
-  const bool is_hi = (int)blockIdx.x < blocks_hi;
-  const LnBranch& br = is_hi ? hi : lo;
-  const int M = br.M;
-  const int blk = is_hi ? blockIdx.x : blockIdx.x - blocks_hi;
-  const int m0 = (blk * 8 + warp) * ROWS;
-  if (m0 >= M) return;
-  const int m = m0 + rw;
+// Normalisation, quantizer and packing of the rows a warp holds in the multi-lane layout (x: this lane's channels of row m,
+// groups of P at channel 32 i + P j; pad: the row is a pad token, zero after the normalisation).
+template <int NG, int G>
+__device__ __forceinline__ void ln_g_finish(const LnBranch& br, const float (&x)[NG][32 / G], int m, bool pad, int j) {
+  constexpr int C = NG * 32, P = 32 / G, VEC = P >= 4 ? 4 : 2;
   const AQ q = br.q;
-  const int bits = q.bits;
-  long srow = -1;
-  if (m < M) srow = (MERGE || !br.rowsrc) ? (long)m : (long)br.rowsrc[m];
-  // source rows: one (gather / plain) or the four input neighbours (merge); -1: zeros
-  long nsrc[MERGE ? 4 : 1];
-  if (MERGE) {
-    const int H2 = (br.mgH + 1) / 2, W2 = (br.mgW + 1) / 2;
-    const int mm = m < M ? m : 0;
-    const int b = mm / (H2 * W2), r2 = mm - b * (H2 * W2), y2 = r2 / W2, x2 = r2 - y2 * W2;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const int yy = 2 * y2 + (g & 1), xx = 2 * x2 + (g >> 1);
-      nsrc[MERGE ? g : 0] = (m < M && yy < br.mgH && xx < br.mgW) ? ((long)b * br.mgH + yy) * br.mgW + xx : -1;
-    }
-  } else {
-    nsrc[0] = srow;
-  }
-  float x[NG][P];
-#pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    constexpr int GPN = MERGE ? NG / 4 : NG;                 // channel groups per source row
-    const long sr = nsrc[MERGE ? i / GPN : 0];
-    const float* src = br.src + (sr < 0 ? 0 : sr) * (GPN * 32) + 32 * (i % GPN) + P * j;
-#pragma unroll
-    for (int v = 0; v < P / VEC; ++v) {
-      if (VEC == 4) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (sr >= 0) a = __ldg(reinterpret_cast<const float4*>(src) + v);
-        x[i][4 * v] = a.x; x[i][4 * v + 1] = a.y; x[i][4 * v + 2] = a.z; x[i][4 * v + 3] = a.w;
-      } else {
-        float2 a = make_float2(0.f, 0.f);
-        if (sr >= 0) a = __ldg(reinterpret_cast<const float2*>(src) + v);
-        x[i][2 * v] = a.x; x[i][2 * v + 1] = a.y;
-      }
-    }
-  }
+  const int bits = q.bits, M = br.M;
   // partial sums in channel order, then the butterfly: lanes first (offsets 16 .. P), then inside the lane
   auto reduce32 = [&](float (&p)[P]) -> float {
 #pragma unroll
@@ -189,7 +147,7 @@ __global__ void __launch_bounds__(256, (NG * (32 / G) > 24 ? 2 : 4)) k_ln_quant_
           }
         }
       }
-      if (srow < 0) { w0 = zw0; w1 = zw1; }
+      if (pad) { w0 = zw0; w1 = zw1; }
       // P codes of BITS bits: P*BITS/8 whole bytes (the launcher only picks G with P*BITS >= 8)
       uint8_t* dst = out + 32 * i * BITS / 8;
       constexpr int NBYTES = P * BITS / 8;
@@ -204,10 +162,133 @@ __global__ void __launch_bounds__(256, (NG * (32 / G) > 24 ? 2 : 4)) k_ln_quant_
   else finish(std::integral_constant<int, 2>{});
 }
 
+template <int NG, int G, bool MERGE>
+__global__ void __launch_bounds__(256, (NG * (32 / G) > 24 ? 2 : 4)) k_ln_quant_g(LnBranch hi, LnBranch lo, int blocks_hi) {
+  if (!MERGE) griddep_launch();
+  griddep_wait();
+  if (MERGE) griddep_launch();                               // opens a stage, see griddep_wait
+  constexpr int P = 32 / G, ROWS = 32 / G;                  // partials per lane, rows per warp
+  constexpr int VEC = P >= 4 ? 4 : 2;                       // floats per load
+  static_assert(P >= 2 && (!MERGE || NG % 4 == 0), "unsupported lane split");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = lane % G, rw = lane / G;
+  const bool is_hi = (int)blockIdx.x < blocks_hi;
+  const LnBranch& br = is_hi ? hi : lo;
+  const int M = br.M;
+  const int blk = is_hi ? blockIdx.x : blockIdx.x - blocks_hi;
+  const int m0 = (blk * 8 + warp) * ROWS;
+  if (m0 >= M) return;
+  const int m = m0 + rw;
+  long srow = -1;
+  if (m < M) srow = (MERGE || !br.rowsrc) ? (long)m : (long)br.rowsrc[m];
+  // source rows: one (gather / plain) or the four input neighbours (merge); -1: zeros
+  long nsrc[MERGE ? 4 : 1];
+  if (MERGE) {
+    const int H2 = (br.mgH + 1) / 2, W2 = (br.mgW + 1) / 2;
+    const int mm = m < M ? m : 0;
+    const int b = mm / (H2 * W2), r2 = mm - b * (H2 * W2), y2 = r2 / W2, x2 = r2 - y2 * W2;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int yy = 2 * y2 + (g & 1), xx = 2 * x2 + (g >> 1);
+      nsrc[MERGE ? g : 0] = (m < M && yy < br.mgH && xx < br.mgW) ? ((long)b * br.mgH + yy) * br.mgW + xx : -1;
+    }
+  } else {
+    nsrc[0] = srow;
+  }
+  float x[NG][P];
+#pragma unroll
+  for (int i = 0; i < NG; ++i) {
+    constexpr int GPN = MERGE ? NG / 4 : NG;                 // channel groups per source row
+    const long sr = nsrc[MERGE ? i / GPN : 0];
+    const float* src = br.src + (sr < 0 ? 0 : sr) * (GPN * 32) + 32 * (i % GPN) + P * j;
+#pragma unroll
+    for (int v = 0; v < P / VEC; ++v) {
+      if (VEC == 4) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (sr >= 0) a = __ldg(reinterpret_cast<const float4*>(src) + v);
+        x[i][4 * v] = a.x; x[i][4 * v + 1] = a.y; x[i][4 * v + 2] = a.z; x[i][4 * v + 3] = a.w;
+      } else {
+        float2 a = make_float2(0.f, 0.f);
+        if (sr >= 0) a = __ldg(reinterpret_cast<const float2*>(src) + v);
+        x[i][2 * v] = a.x; x[i][2 * v + 1] = a.y;
+      }
+    }
+  }
+  ln_g_finish<NG, G>(br, x, m, srow < 0, j);
+}
+
+// The same for batches that keep every SM busy for a while: persistent warps walk over row groups and fetch STAGES groups
+// ahead by asynchronous copies into shared memory, every thread into slots that it alone reads back (no barrier).  The plain
+// kernel alternates between waiting for its loads and computing: 3.6 TB/s at 296 450 rows of 128 channels (45 to 50 us); see
+// launch_ln_quant for what this one reaches.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t smem_dst, const void* src) {
+  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_dst), "l"(src), "n"(BYTES) : "memory");
+}
+constexpr int LN_STAGES = 3, LN_STREAM_CTAS = 2;
+template <int NG, int G> constexpr int ln_stream_smem() { return LN_STAGES * NG * (32 / G) * 256 * 4; }
+template <int NG, int G>
+__global__ void __launch_bounds__(256, LN_STREAM_CTAS) k_ln_stream(LnBranch hi, LnBranch lo, int groups_hi, int groups) {
+  constexpr int C = NG * 32, P = 32 / G, ROWS = 32 / G, VEC = P >= 4 ? 4 : 2, NV = NG * P / VEC;
+  extern __shared__ __align__(16) float ring[];
+  griddep_launch();
+  const int lane = threadIdx.x & 31, j = lane % G, rw = lane / G;
+  const int step = gridDim.x * 8;
+  const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * (VEC * 4);
+  int it = blockIdx.x * 8 + (threadIdx.x >> 5);
+  griddep_wait();
+  // source row of this lane's row of a group: -1 pad token, -2 beyond the batch
+  auto source = [&](int g) -> int {
+    if (g >= groups) return -2;
+    const bool is_hi = g < groups_hi;
+    const int m = (is_hi ? g : g - groups_hi) * ROWS + rw;
+    const int32_t* rs = is_hi ? hi.rowsrc : lo.rowsrc;
+    if (m >= (is_hi ? hi.M : lo.M)) return -2;
+    return rs ? __ldg(rs + m) : m;
+  };
+  auto fetch = [&](int g, int srow, int stage) {
+    if (srow >= 0) {
+      const float* src = (g < groups_hi ? hi.src : lo.src) + (long)srow * C + P * j;
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        cp_async<VEC * 4>(slot0 + (uint32_t)((stage * NV + v) * 256 * VEC * 4), src + 32 * (v / (P / VEC)) + VEC * (v % (P / VEC)));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int src[LN_STAGES + 1];
+#pragma unroll
+  for (int s = 0; s <= LN_STAGES; ++s) src[s] = source(it + s * step);
+#pragma unroll
+  for (int s = 0; s < LN_STAGES; ++s) fetch(it + s * step, src[s], s);
+  int stage = 0;
+  for (; it < groups; it += step) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(LN_STAGES - 1) : "memory");
+    float x[NG][P];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const float* sl = ring + ((stage * NV + v) * 256 + threadIdx.x) * VEC;
+      float* d = &x[v / (P / VEC)][VEC * (v % (P / VEC))];
+      if (VEC == 4) { const float4 a = *reinterpret_cast<const float4*>(sl); d[0] = a.x; d[1] = a.y; d[2 % P] = a.z; d[3 % P] = a.w; }
+      else { const float2 a = *reinterpret_cast<const float2*>(sl); d[0] = a.x; d[1] = a.y; }
+    }
+    const int mine = src[0];
+#pragma unroll
+    for (int s = 0; s < LN_STAGES; ++s) src[s] = src[s + 1];
+    fetch(it + LN_STAGES * step, src[LN_STAGES - 1], stage);           // into the slots just read
+    src[LN_STAGES] = source(it + (LN_STAGES + 1) * step);
+    stage = stage + 1 == LN_STAGES ? 0 : stage + 1;
+    const bool is_hi = it < groups_hi;
+    ln_g_finish<NG, G>(is_hi ? hi : lo, x, (is_hi ? it : it - groups_hi) * ROWS + rw, mine < 0, j);
+  }
+}
+
 // patch merging: token (b, y2, x2) of the output gathers (2y2+dy, 2x2+dx) for (dy,dx) = (0,0),(1,0),(0,1),(1,1)
 // in this order along the channel axis; neighbours outside the map are zeros (they do take part in the LN).
 template <int NPL>   // NPL = 4C/32
 __global__ void __launch_bounds__(256) k_merge_gather(MergeGatherArgs a) {
+  griddep_wait();
+  griddep_launch();
   const int K = NPL * 32;
   const int C = K / 4;
   int H2 = (a.H + 1) / 2, W2 = (a.W + 1) / 2;
@@ -239,6 +320,8 @@ __global__ void __launch_bounds__(256) k_merge_gather(MergeGatherArgs a) {
 
 __global__ void __launch_bounds__(256) k_copy_rows(const float* __restrict__ x, float* __restrict__ y,
                                                    const int32_t* __restrict__ rowsrc, int M, int C) {
+  griddep_launch();
+  griddep_wait();
   int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
   if (row >= M) return;
@@ -247,12 +330,12 @@ __global__ void __launch_bounds__(256) k_copy_rows(const float* __restrict__ x, 
   for (int c = lane; c < C; c += 32) y[s * C + c] = __ldg(x + s * C + c);
 }
 
-#define MIXAQ_NPL_CASE(n, KERNEL, ...) case n: KERNEL<n><<<grid, 256, 0, st>>>(__VA_ARGS__); break;
+#define MIXAQ_NPL_CASE(n, KERNEL, ...) case n: launch_pdl(KERNEL<n>, dim3(grid), 256, 0, st, __VA_ARGS__); break;
 template <int NPL, int R>
 void launch_ln_r(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
   const int rows_per_block = 8 * R;
   const int bh = (hi.M + rows_per_block - 1) / rows_per_block, bl = (lo.M + rows_per_block - 1) / rows_per_block;
-  k_ln_quant<NPL, R><<<bh + bl, 256, 0, st>>>(hi, lo, bh);
+  launch_pdl(k_ln_quant<NPL, R>, dim3(bh + bl), 256, 0, st, hi, lo, bh);
 }
 // rows per warp: more rows amortise the per-warp constants and the divisions, but small problems need the warps
 template <int NPL, int RMAX>
@@ -269,7 +352,29 @@ template <int NG, int G, bool MERGE = false>
 void launch_ln_g(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
   const int rpb = 8 * (32 / G);                              // rows per block: 8 warps x 32/G rows
   const int bh = (hi.M + rpb - 1) / rpb, bl = (lo.M + rpb - 1) / rpb;
-  k_ln_quant_g<NG, G, MERGE><<<bh + bl, 256, 0, st>>>(hi, lo, bh);
+  launch_pdl(k_ln_quant_g<NG, G, MERGE>, dim3(bh + bl), 256, 0, st, hi, lo, bh);
+}
+
+// elements per SM from which the streaming LayerNorm is used: four row groups of 8 x 128 channels for each of its 16 warps
+#ifndef LN_STREAM_MIN
+#define LN_STREAM_MIN 65536
+#endif
+template <int NG, int G>
+void launch_ln_stream(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
+  constexpr int rows = 32 / G;
+  const int gh = (hi.M + rows - 1) / rows, gl = (lo.M + rows - 1) / rows;
+  const int want = (gh + gl + 7) / 8, most = LN_STREAM_CTAS * sm_count();
+  launch_pdl(k_ln_stream<NG, G>, dim3(want < most ? want : most), 256, ln_stream_smem<NG, G>(), st, hi, lo, gh, gh + gl);
+}
+
+// once per device context: opt-in to the large rings
+bool ln_init() {
+  bool ok = true;
+  auto big = [&](auto kernel, int bytes) { ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
+  big(k_ln_stream<3, 4>, ln_stream_smem<3, 4>()); big(k_ln_stream<4, 4>, ln_stream_smem<4, 4>());
+  big(k_ln_stream<6, 8>, ln_stream_smem<6, 8>()); big(k_ln_stream<8, 8>, ln_stream_smem<8, 8>());
+  big(k_ln_stream<12, 16>, ln_stream_smem<12, 16>()); big(k_ln_stream<16, 16>, ln_stream_smem<16, 16>());
+  return ok;
 }
 
 void launch_ln_quant(const LnBranch& hi, const LnBranch& lo, int C, cudaStream_t st) {
@@ -278,6 +383,19 @@ void launch_ln_quant(const LnBranch& hi, const LnBranch& lo, int C, cudaStream_t
   const int rows = hi.M + lo.M;
   const int min_bits = hi.M > 0 && lo.M > 0 ? (hi.q.bits < lo.q.bits ? hi.q.bits : lo.q.bits) : (hi.M > 0 ? hi.q.bits : lo.q.bits);
   bool done = false;
+  // streaming kernel: from four row groups per warp of the persistent grid on
+  const long elems = (long)rows * C;
+  if (elems >= (long)LN_STREAM_MIN * sm_count()) {
+    done = true;
+    if (C == 96) launch_ln_stream<3, 4>(hi, lo, st);
+    else if (C == 128) launch_ln_stream<4, 4>(hi, lo, st);
+    else if (C == 192 && min_bits * 4 >= 8) launch_ln_stream<6, 8>(hi, lo, st);
+    else if (C == 256 && min_bits * 4 >= 8) launch_ln_stream<8, 8>(hi, lo, st);
+    else if (C == 384 && min_bits * 2 >= 8) launch_ln_stream<12, 16>(hi, lo, st);
+    else if (C == 512 && min_bits * 2 >= 8) launch_ln_stream<16, 16>(hi, lo, st);
+    else done = false;
+    if (done) { ++g_launches; return; }
+  }
   if (rows >= 8192) {
     done = true;
     if (C == 32) launch_ln_g<1, 4>(hi, lo, st);
@@ -330,7 +448,7 @@ void launch_merge_gather(const MergeGatherArgs& a, cudaStream_t st) {
 
 void launch_copy_rows(const float* x, float* y, const int32_t* rowsrc, int M, int C, cudaStream_t st) {
   if (M == 0) return;
-  k_copy_rows<<<(M + 7) / 8, 256, 0, st>>>(x, y, rowsrc, M, C);
+  launch_pdl(k_copy_rows, dim3((M + 7) / 8), 256, 0, st, x, y, rowsrc, M, C);
   ++g_launches;
 }
 

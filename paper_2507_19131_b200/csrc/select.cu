@@ -15,6 +15,8 @@ __device__ __forceinline__ int score_code_sq(float v, float inv) {
 }
 __global__ void __launch_bounds__(256) k_energy(const float* __restrict__ x, int32_t* __restrict__ energy,
                                                 long ntok, int C, float inv) {
+  griddep_wait();
+  griddep_launch();
   const long tok = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   const int sub = threadIdx.x & 7;
   int e = 0;
@@ -49,6 +51,8 @@ constexpr int MAX_SELECT_BATCH = 24;
 struct SelectBatch { SelectArgs a[MAX_SELECT_BATCH]; };
 
 __global__ void __launch_bounds__(256) k_window_score(const __grid_constant__ SelectBatch batch) {
+  griddep_wait();
+  griddep_launch();
   const SelectArgs& a = batch.a[blockIdx.y];
   int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
@@ -70,6 +74,8 @@ __global__ void __launch_bounds__(256) k_window_score(const __grid_constant__ Se
 // and the lanes then write the batch bookkeeping of the window's slot (49 source-token indices) together.
 constexpr int RANK_WARPS = 8;
 __global__ void __launch_bounds__(RANK_WARPS * 32) k_rank_emit(const __grid_constant__ SelectBatch batch) {
+  griddep_launch();
+  griddep_wait();
   extern __shared__ long long s_score[];
   const SelectArgs& a = batch.a[blockIdx.z];
   const int b = blockIdx.y;
@@ -130,7 +136,7 @@ void launch_class_lists(const uint8_t* cls, int B, int nW, int32_t* const out[3]
 }
 
 void launch_energy(const float* x, int32_t* energy, long ntok, int C, float inv_scale, cudaStream_t st) {
-  k_energy<<<(unsigned)((ntok * 8 + 255) / 256), 256, 0, st>>>(x, energy, ntok, C, inv_scale);
+  launch_pdl(k_energy, dim3((unsigned)((ntok * 8 + 255) / 256)), 256, 0, st, x, energy, ntok, C, inv_scale);
   ++g_launches;
 }
 
@@ -143,10 +149,10 @@ void launch_select(const SelectArgs* args, int count, cudaStream_t st) {
     for (int i = n; i < MAX_SELECT_BATCH; ++i) batch.a[i] = args[first];
     const SelectArgs& a = args[first];
     const int nwin = a.B * a.nW;
-    k_window_score<<<dim3((nwin + 7) / 8, n), 256, 0, st>>>(batch);
+    launch_pdl(k_window_score, dim3((nwin + 7) / 8, n), 256, 0, st, batch);
     ++g_launches;
     dim3 grid((a.nW + RANK_WARPS - 1) / RANK_WARPS, a.B, n);
-    k_rank_emit<<<grid, RANK_WARPS * 32, (size_t)a.nW * sizeof(long long), st>>>(batch);
+    launch_pdl(k_rank_emit, grid, RANK_WARPS * 32, (size_t)a.nW * sizeof(long long), st, batch);
     ++g_launches;
   }
 }

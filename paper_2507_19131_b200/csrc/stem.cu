@@ -10,6 +10,8 @@ namespace mixaq {
 // to 64 codes (the integer GEMM wants K a multiple of 32; the padded weight columns are zero): the ky == 0 thread
 // clears them.
 __global__ void __launch_bounds__(256) k_patch_gather(PatchGatherArgs a) {
+  griddep_wait();
+  griddep_launch();
   const int H = (a.Hi + 3) / 4, W = (a.Wi + 3) / 4;
   const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long tok = idx >> 2;
@@ -38,6 +40,8 @@ template <int NPL>
 __global__ void __launch_bounds__(256) k_bias_ln(const float* __restrict__ x, const float* __restrict__ bias,
                                                  const float* __restrict__ gamma, const float* __restrict__ beta,
                                                  float* __restrict__ y, long rows) {
+  griddep_wait();
+  griddep_launch();
   const int C = NPL * 32;
   const long row = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -68,11 +72,11 @@ __global__ void k_pad_weights(const int8_t* __restrict__ w, int N, int K, int Kp
 
 void launch_patch_gather(const PatchGatherArgs& a, cudaStream_t st) {
   const long threads = (long)a.B * ((a.Hi + 3) / 4) * ((a.Wi + 3) / 4) * 4;
-  k_patch_gather<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(a);
+  launch_pdl(k_patch_gather, dim3((unsigned)((threads + 255) / 256)), 256, 0, st, a);
   ++g_launches;
 }
 
-#define MIXAQ_BLN_CASE(n) case n: k_bias_ln<n><<<grid, 256, 0, st>>>(x, bias, gamma, beta, y, rows); break;
+#define MIXAQ_BLN_CASE(n) case n: launch_pdl(k_bias_ln<n>, dim3(grid), 256, 0, st, x, bias, gamma, beta, y, rows); break;
 bool launch_bias_ln(const float* x, const float* bias, const float* gamma, const float* beta, float* y, long rows,
                     int C, cudaStream_t st) {
   if (rows <= 0) return true;
