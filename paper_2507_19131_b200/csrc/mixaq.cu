@@ -36,6 +36,7 @@ struct mixaq_ctx {
   bool nvtx;                           // name every kernel family, stage and block with an NVTX range (host side)
   bool allow_elevation;                // backbone: every pair uses its own ratios even if an earlier pair of the stage had larger ones
   cudaStream_t capture_stream;         // forwards on a stream that cannot be captured (the legacy default one) are recorded here
+  cudaStream_t side_stream; cudaEvent_t fork, join;   // output norms run beside the next stage inside a captured forward
   std::vector<GraphEntry> graphs;
   std::vector<ProfRec> prof;          // event pairs recorded since mixaq_profile_begin
   std::vector<cudaEvent_t> pool;      // events ready for reuse
@@ -302,7 +303,7 @@ mixaq_status mixaq_create(mixaq_ctx** out, int device) {
   if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return MIXAQ_CUDA_ERROR; }
   mixaq_ctx* c = new (std::nothrow) mixaq_ctx();
   if (!c) return MIXAQ_INTERNAL;
-  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr;
+  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr; c->side_stream = nullptr; c->fork = c->join = nullptr;
   if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess || cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess ||
       !gemm_init() || !ln_init()) {
     cudaGetLastError(); if (c->d_status) cudaFree(c->d_status); delete c; return MIXAQ_CUDA_ERROR;
@@ -315,6 +316,7 @@ mixaq_status mixaq_destroy(mixaq_ctx* ctx) {
   if (!ctx) return MIXAQ_INVALID_ARG;
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
+  if (ctx->side_stream) { cudaStreamDestroy(ctx->side_stream); cudaEventDestroy(ctx->fork); cudaEventDestroy(ctx->join); }
   for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
   for (cudaGraphExec_t g : ctx->prof_execs) cudaGraphExecDestroy(g);
   for (auto& r : ctx->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
@@ -843,6 +845,17 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
   }
   if (!use_graph) st = user_stream;
 
+  // Inside a captured forward the output norms leave the chain: nothing waits for them but the end of the forward.
+  bool side = use_graph && !prof_graph && norms;
+  if (side && !ctx->side_stream) {
+    if (cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess) { ctx->side_stream = nullptr; side = false; }
+    else if (cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) != cudaSuccess ||
+             cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming) != cudaSuccess) {
+      cudaStreamDestroy(ctx->side_stream); ctx->side_stream = nullptr; side = false;
+    }
+    if (!side) cudaGetLastError();
+  }
+
   mixaq_status result = MIXAQ_OK;
   int total = 0, H = H0, W = W0, blk = 0;
   const float* cur = x0;
@@ -909,11 +922,14 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
     if (result == MIXAQ_OK && norms) {
       PROF(PC_OUT_NORM);
       g_launches = 0;
-      if (!launch_bias_ln(out_s, nullptr, p->out_norm_g[s], p->out_norm_b[s], stage_out[s], (long)B * H * W, b0->dim, st))
+      if (side) { cudaEventRecord(ctx->fork, st); cudaStreamWaitEvent(ctx->side_stream, ctx->fork, 0); }
+      if (!launch_bias_ln(out_s, nullptr, p->out_norm_g[s], p->out_norm_b[s], stage_out[s], (long)B * H * W, b0->dim,
+                          side ? ctx->side_stream : st))
         result = fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "output norm: unsupported width");
       total += g_launches;
     }
   }
+  if (side) { cudaEventRecord(ctx->join, ctx->side_stream); cudaStreamWaitEvent(st, ctx->join, 0); }
   if (use_graph) {
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(st, &graph);

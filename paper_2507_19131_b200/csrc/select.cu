@@ -69,6 +69,30 @@ __global__ void __launch_bounds__(256) k_window_score(const __grid_constant__ Se
   if (lane == 0) a.score[gw] = s;
 }
 
+// Rank of window w among the scores of its image, and the bookkeeping of its slot (by one warp)
+__device__ __forceinline__ void emit_window(const SelectArgs& a, int b, int w, const long long* s_score, int lane, int Hp, int Wp) {
+  const long long mine = s_score[w];
+  int cnt = 0;
+  if (!a.reverse) {
+    for (int v = lane; v < a.nW; v += 32) { long long o = s_score[v]; cnt += (o > mine) || (o == mine && v < w); }
+  } else {
+    for (int v = lane; v < a.nW; v += 32) { long long o = s_score[v]; cnt += (o < mine) || (o == mine && v < w); }
+  }
+  const int rank = __reduce_add_sync(0xffffffffu, cnt);
+  const int c = rank < a.n_hi ? 0 : (rank < a.n_hi + a.n_lo ? 1 : 2);
+  int32_t* dst; long slot;
+  if (c == 0)      { slot = (long)b * a.n_hi + rank;                     dst = a.rowsrc_hi; }
+  else if (c == 1) { slot = (long)b * a.n_lo + (rank - a.n_hi);          dst = a.rowsrc_lo; }
+  else             { slot = (long)b * a.n_pr + (rank - a.n_hi - a.n_lo); dst = a.rowsrc_pr; }
+  if (lane == 0) {
+    a.order[(long)b * a.nW + rank] = w;
+    a.cls[(long)b * a.nW + w] = (uint8_t)c;
+    if (c == 0) a.win_hi[slot] = w;
+    else if (c == 1) a.win_lo[slot] = w;
+  }
+  for (int t = lane; t < WT; t += 32) dst[slot * WT + t] = window_src(b, a.H, a.W, Hp, Wp, a.shift, a.nwx, w, t);
+}
+
 // Rank by counting: rank(w) = #{v : v precedes w in (score desc, index asc)}; ranks are a permutation.
 // One warp per window: the lanes split the windows to compare against, the counts are summed over the warp,
 // and the lanes then write the batch bookkeeping of the window's slot (49 source-token indices) together.
@@ -85,27 +109,32 @@ __global__ void __launch_bounds__(RANK_WARPS * 32) k_rank_emit(const __grid_cons
   const int lane = threadIdx.x & 31;
   const int w = blockIdx.x * RANK_WARPS + (threadIdx.x >> 5);
   if (w >= a.nW) return;
-  const long long mine = s_score[w];
-  int cnt = 0;
-  if (!a.reverse) {
-    for (int v = lane; v < a.nW; v += 32) { long long o = s_score[v]; cnt += (o > mine) || (o == mine && v < w); }
-  } else {
-    for (int v = lane; v < a.nW; v += 32) { long long o = s_score[v]; cnt += (o < mine) || (o == mine && v < w); }
-  }
-  const int rank = __reduce_add_sync(0xffffffffu, cnt);
-  const int c = rank < a.n_hi ? 0 : (rank < a.n_hi + a.n_lo ? 1 : 2);
+  emit_window(a, b, w, s_score, lane, (a.H + WS - 1) / WS * WS, (a.W + WS - 1) / WS * WS);
+}
+
+// Score, rank and bookkeeping of one (image, block) in one CTA, for images of few windows: there the two kernels above are
+// launch latency (3 us each at 64 windows), and one CTA needs no exchange through global memory.  (At 96 windows one CTA
+// already takes longer than the two launches: 10 against 6 us.)
+constexpr int SMALL_WINDOWS = 64, SMALL_WARPS = 32;
+__global__ void __launch_bounds__(SMALL_WARPS * 32) k_select_small(const __grid_constant__ SelectBatch batch) {
+  __shared__ long long s_score[SMALL_WINDOWS];
+  griddep_wait();
+  griddep_launch();
+  const SelectArgs& a = batch.a[blockIdx.y];
+  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int Hp = (a.H + WS - 1) / WS * WS, Wp = (a.W + WS - 1) / WS * WS;
-  int32_t* dst; long slot;
-  if (c == 0)      { slot = (long)b * a.n_hi + rank;                     dst = a.rowsrc_hi; }
-  else if (c == 1) { slot = (long)b * a.n_lo + (rank - a.n_hi);          dst = a.rowsrc_lo; }
-  else             { slot = (long)b * a.n_pr + (rank - a.n_hi - a.n_lo); dst = a.rowsrc_pr; }
-  if (lane == 0) {
-    a.order[(long)b * a.nW + rank] = w;
-    a.cls[(long)b * a.nW + w] = (uint8_t)c;
-    if (c == 0) a.win_hi[slot] = w;
-    else if (c == 1) a.win_lo[slot] = w;
+  for (int w = warp; w < a.nW; w += SMALL_WARPS) {
+    long long s = 0;
+    for (int t = lane; t < WT; t += 32) {
+      const int src = window_src(b, a.H, a.W, Hp, Wp, a.shift, a.nwx, w, t);
+      if (src >= 0) s += a.energy[src];
+    }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) { s_score[w] = s; a.score[(long)b * a.nW + w] = s; }
   }
-  for (int t = lane; t < WT; t += 32) dst[slot * WT + t] = window_src(b, a.H, a.W, Hp, Wp, a.shift, a.nwx, w, t);
+  __syncthreads();
+  for (int w = warp; w < a.nW; w += SMALL_WARPS) emit_window(a, b, w, s_score, lane, Hp, Wp);
 }
 
 // One warp per (image, class): walks the windows in ascending index, 32 at a time, and appends the members of its class
@@ -148,6 +177,11 @@ void launch_select(const SelectArgs* args, int count, cudaStream_t st) {
     for (int i = 0; i < n; ++i) batch.a[i] = args[first + i];
     for (int i = n; i < MAX_SELECT_BATCH; ++i) batch.a[i] = args[first];
     const SelectArgs& a = args[first];
+    if (a.nW <= SMALL_WINDOWS) {
+      launch_pdl(k_select_small, dim3(a.B, n), SMALL_WARPS * 32, 0, st, batch);
+      ++g_launches;
+      continue;
+    }
     const int nwin = a.B * a.nW;
     launch_pdl(k_window_score, dim3((nwin + 7) / 8, n), 256, 0, st, batch);
     ++g_launches;
