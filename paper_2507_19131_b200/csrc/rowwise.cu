@@ -371,9 +371,8 @@ void launch_ln_stream(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
 bool ln_init() {
   bool ok = true;
   auto big = [&](auto kernel, int bytes) { ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
-  big(k_ln_stream<3, 4>, ln_stream_smem<3, 4>()); big(k_ln_stream<4, 4>, ln_stream_smem<4, 4>());
+  big(k_ln_stream<3, 8>, ln_stream_smem<3, 8>()); big(k_ln_stream<4, 8>, ln_stream_smem<4, 8>());
   big(k_ln_stream<6, 8>, ln_stream_smem<6, 8>()); big(k_ln_stream<8, 8>, ln_stream_smem<8, 8>());
-  big(k_ln_stream<12, 16>, ln_stream_smem<12, 16>()); big(k_ln_stream<16, 16>, ln_stream_smem<16, 16>());
   return ok;
 }
 
@@ -387,12 +386,10 @@ void launch_ln_quant(const LnBranch& hi, const LnBranch& lo, int C, cudaStream_t
   const long elems = (long)rows * C;
   if (elems >= (long)LN_STREAM_MIN * sm_count()) {
     done = true;
-    if (C == 96) launch_ln_stream<3, 4>(hi, lo, st);
-    else if (C == 128) launch_ln_stream<4, 4>(hi, lo, st);
-    else if (C == 192 && min_bits * 4 >= 8) launch_ln_stream<6, 8>(hi, lo, st);
-    else if (C == 256 && min_bits * 4 >= 8) launch_ln_stream<8, 8>(hi, lo, st);
-    else if (C == 384 && min_bits * 2 >= 8) launch_ln_stream<12, 16>(hi, lo, st);
-    else if (C == 512 && min_bits * 2 >= 8) launch_ln_stream<16, 16>(hi, lo, st);
+    if (C == 96) launch_ln_stream<3, 8>(hi, lo, st);
+    else if (C == 128) launch_ln_stream<4, 8>(hi, lo, st);
+    else if (C == 192) launch_ln_stream<6, 8>(hi, lo, st);
+    else if (C == 256) launch_ln_stream<8, 8>(hi, lo, st);
     else done = false;
     if (done) { ++g_launches; return; }
   }
