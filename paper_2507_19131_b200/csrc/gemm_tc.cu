@@ -40,18 +40,19 @@ constexpr int A_STAGE_BYTES = BM * BK;
 // warps 2..5 expand sub-byte codes (two warps left the long-K main loops of 4-bit tiles waiting for the expansion;
 // eight cost more registers than they return)
 constexpr int UNPACK_WARPS = 4;
-// Epilogue warps.  Binary32 outputs: 8.  Code outputs: 12, or 16 where every CTA has many row tiles: whole tiles are then
-// dealt to groups of warps (see pick_tiling) and the launch is bound by throughput (C = 128 at 2 x 384 x 384 tokens: fc1 165
-// us with 12, 155 with 16); below that the shorter tile latency of 12 warps with more registers wins (C = 384 at 50 x 84: fc1
-// 18.7 against 21.5).
+// Epilogue warps.  Binary32 outputs: 8.  Code outputs: 12; fc1, whose GELU makes it the longest, 16 where every SM has two row
+// tiles or more: whole tiles are then dealt to groups of warps (see pick_tiling) and the launch is bound by throughput (C = 256
+// at 2 x 192 x 192 tokens: 93 us with 16, 97 with 12; C = 96 at 16 x 56 x 56: 30.4 and 32.5); below that the shorter tile
+// latency of 12 warps with more registers wins (C = 384 at 16 x 14 x 14: 14.4 us against 16.1).  QKV, with less work per
+// element, is faster with 12 everywhere (C = 128 at 2 x 384 x 384: 63 us against 68).
 constexpr int F32_WARPS = 8, CODE_WARPS = 12, CODE_WARPS_MANY = 16;
-constexpr int MANY_ROW_TILES = 8;              // row tiles per SM from which CODE_WARPS_MANY is used
+constexpr int MANY_ROW_TILES = 2;              // row tiles per SM from which fc1 has CODE_WARPS_MANY
 __host__ __device__ constexpr int num_threads(int warps) { return 32 * (2 + UNPACK_WARPS + warps); }
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
 constexpr int MAX_RING = 6;
 constexpr int TMEM_COLS = 512;                 // one CTA per SM: it takes all of the tensor memory
-constexpr int MAX_ACC = 4;                     // accumulators in it, as far as the tile width allows
+constexpr int MAX_ACC = 6;                     // accumulators in it, as far as the tile width allows
 constexpr uint32_t MAX_POLLS = 1u << 22;       // tries per wait
 constexpr uint32_t MAX_SUSPENDED_POLLS = 1u << 16;   // tries that may each suspend the thread for up to 20 us
 
@@ -538,28 +539,32 @@ bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t row_bytes
 
 
 // Tile width and the epilogue's division of labour.  The width is a multiple of 32 that divides `unit` (N; for QKV the
-// width C of a section, so that a tile has one quantizer), at most 256.  The epilogue bounds every shape here; in units of
-// 32 columns a warp needs (columns / 32 of its tile share + about 0.6 of fixed work) per tile, and `groups` tiles are in
-// work at once.  Many tiles per CTA: whole tiles per warp (groups = accumulators), the fixed work is paid once per tile;
-// few: all warps share a tile, its latency counts.
-#ifndef GMAX
-#define GMAX 4
-#endif
+// width C of a section, so that a tile has one quantizer), at most 256.  Cost in units of an epilogue warp's 32 columns
+// (about 0.6 us): a tile takes `mma` to multiply and each of its warps `epi` to convert, `groups` tiles are converted at
+// once while the next ones are multiplied, and the first tiles have nothing to hide behind.  A wide tile reads its rows
+// fewer times and pays the fixed part of the epilogue once for more columns; narrow ones spread a small problem over the
+// SMs.  The constants are a fit to the times of all (width, groups) at 13 shapes from 768 x 7 x 7 to 128 x 2 x 384 x 384; the
+// choice is within 5 % of the fastest at each of them, where a cost without the overlap was up to 30 % off (fc2 with
+// C = 1024 at 2 x 48 x 48: 50 us at the width of 256 it chose, 40 at 128).
 struct Tiling { int bn, n_acc, groups, split; };
 Tiling pick_tiling(int unit, int N, int m_tiles, int k_blocks, int sms, int warps, int chunk) {
   Tiling best = {0, 0, 0, 0};
   double best_cost = 0.0;
   const int per_quarter = warps / 4;
+  const double fixed = chunk == CODE_NC ? 0.5 : 2.5;
   for (int bn = 32; bn <= MAX_BN; bn += 32) {
     if (unit % bn) continue;
-    const int n_acc = bn <= TMEM_COLS / 4 ? 4 : 2;
+    const int fit = TMEM_COLS / bn < MAX_ACC ? TMEM_COLS / bn : MAX_ACC;
     const long tiles = (long)m_tiles * (N / bn), per_cta = (tiles + sms - 1) / sms;
-    for (int groups = 1; groups <= per_quarter && groups <= n_acc && groups <= GMAX; groups *= 2) {
+    const double mma = k_blocks * (0.26 + 0.16 * (bn / 32));
+    for (int groups = 1; groups <= per_quarter && groups <= fit; ++groups) {
       if (per_quarter % groups) continue;
+      const int n_acc = fit / groups * groups;                // a group keeps to its own accumulators
       const int split = per_quarter / groups;
-      const double chunks = (bn / chunk + split - 1) / split * (chunk / 32.0);
+      const double epi = (bn / chunk + split - 1) / split * (chunk / 32.0) + fixed;
       const long rounds = (per_cta + groups - 1) / groups;
-      const double cost = rounds * (chunks + 0.6) + 0.03 * k_blocks * per_cta;
+      const double first = per_cta < groups ? per_cta * mma : groups * mma;
+      const double cost = fmax(first + rounds * epi, per_cta * mma + epi);
       if (!best.bn || cost <= best_cost) { best = {bn, n_acc, groups, split}; best_cost = cost; }
     }
   }
@@ -747,7 +752,6 @@ bool gemm_init() {
   bool ok = encode_fn() != nullptr && sm_count() > 0;
   auto big_smem = [&](auto kernel) { ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess; };
   big_smem(k_gemm_tc<EPI_QKV, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_QKV, true, CODE_WARPS>);
-  big_smem(k_gemm_tc<EPI_QKV, false, CODE_WARPS_MANY>); big_smem(k_gemm_tc<EPI_QKV, true, CODE_WARPS_MANY>);
   big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS>);
   big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS_MANY>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS_MANY>);
   big_smem(k_gemm_tc<EPI_PROJ, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_PROJ, true, F32_WARPS>);
@@ -760,7 +764,7 @@ bool launch_gemm(const GemmArgs& g, cudaStream_t st) {
   const long row_tiles = (long)(g.br[0].M + BM - 1) / BM + (g.br[1].M + BM - 1) / BM;
   const bool many = row_tiles >= (long)MANY_ROW_TILES * sm_count();
   switch (g.mode) {
-    case EPI_QKV:   return many ? launch_mode<EPI_QKV, CODE_WARPS_MANY>(g, g.status, st) : launch_mode<EPI_QKV, CODE_WARPS>(g, g.status, st);
+    case EPI_QKV:   return launch_mode<EPI_QKV, CODE_WARPS>(g, g.status, st);
     case EPI_FC1:   return many ? launch_mode<EPI_FC1, CODE_WARPS_MANY>(g, g.status, st) : launch_mode<EPI_FC1, CODE_WARPS>(g, g.status, st);
     case EPI_PROJ:  return launch_mode<EPI_PROJ, F32_WARPS>(g, g.status, st);
     case EPI_FC2:   return launch_mode<EPI_FC2, F32_WARPS>(g, g.status, st);

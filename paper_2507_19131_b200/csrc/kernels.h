@@ -12,9 +12,6 @@ extern thread_local int g_launches;
 
 // Launch with programmatic stream serialization (see griddep_wait): the kernel has to call griddep_wait() itself before it
 // touches what earlier kernels wrote.  In a 224 x 224 Swin-T forward the launches are 5 us each of which 2 to 3 are start-up.
-#ifndef PDLN
-#define PDLN 1
-#endif
 template <class... P, class... A>
 inline void launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -22,7 +19,7 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t s
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cfg.attrs = &attr; cfg.numAttrs = PDLN;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

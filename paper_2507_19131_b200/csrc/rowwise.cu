@@ -356,9 +356,7 @@ void launch_ln_g(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
 }
 
 // elements per SM from which the streaming LayerNorm is used: four row groups of 8 x 128 channels for each of its 16 warps
-#ifndef LN_STREAM_MIN
-#define LN_STREAM_MIN 65536
-#endif
+constexpr long LN_STREAM_MIN = 65536;
 template <int NG, int G>
 void launch_ln_stream(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
   constexpr int rows = 32 / G;
@@ -384,7 +382,7 @@ void launch_ln_quant(const LnBranch& hi, const LnBranch& lo, int C, cudaStream_t
   bool done = false;
   // streaming kernel: from four row groups per warp of the persistent grid on
   const long elems = (long)rows * C;
-  if (elems >= (long)LN_STREAM_MIN * sm_count()) {
+  if (elems >= LN_STREAM_MIN * sm_count()) {
     done = true;
     if (C == 96) launch_ln_stream<3, 8>(hi, lo, st);
     else if (C == 128) launch_ln_stream<4, 8>(hi, lo, st);
