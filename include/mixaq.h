@@ -258,8 +258,11 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
  * launches on `cuda_stream`, later calls cost one graph launch on the host.  The data behind the pointers may
  * change freely between calls.  Captured graphs are kept per context (16 at most) until mixaq_destroy.  A call on the
  * legacy default stream (NULL), which cannot be captured, is recorded on a stream of the context's own and its graph
- * launched on the legacy stream; a call made while the caller is capturing the stream itself launches its kernels directly.  A call between mixaq_profile_begin/end is captured
- * together with its event records, launched once and not cached.
+ * launched on the legacy stream; a call made while the caller is capturing the stream itself launches its kernels
+ * directly.  A backbone forward between mixaq_profile_begin/end is captured together with its event records, launched once
+ * and not cached; a block forward there launches its kernels directly.
+ * mixaq_block_forward (without taps) does the same from the second call with the same arguments on; it keeps 8 graphs,
+ * and stops recording new ones while those it has are not replayed.
  * enabled = 0 switches the cache off and drops the stored graphs; it is on by default. */
 mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled);
 

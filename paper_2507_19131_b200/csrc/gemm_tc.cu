@@ -556,7 +556,8 @@ Tiling pick_tiling(int unit, int N, int m_tiles, int k_blocks, int sms, int warp
     if (unit % bn) continue;
     const int fit = TMEM_COLS / bn < MAX_ACC ? TMEM_COLS / bn : MAX_ACC;
     const long tiles = (long)m_tiles * (N / bn), per_cta = (tiles + sms - 1) / sms;
-    const double mma = k_blocks * (0.26 + 0.16 * (bn / 32));
+    // a launch that leaves SMs idle has more of the L2 for each tile: width then costs less
+    const double mma = k_blocks * (0.26 + 0.16 * (bn / 32) * (tiles < sms ? (double)tiles / sms : 1.0));
     for (int groups = 1; groups <= per_quarter && groups <= fit; ++groups) {
       if (per_quarter % groups) continue;
       const int n_acc = fit / groups * groups;                // a group keeps to its own accumulators

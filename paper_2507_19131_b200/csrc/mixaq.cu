@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -20,8 +21,31 @@ thread_local int g_launches = 0;
 using namespace mixaq;
 
 struct ProfRec { int cat; cudaEvent_t e0, e1; };
-// One captured backbone forward: the exact bytes of every argument that shaped it, and the instantiated graph.
+// One captured forward: the exact bytes of every argument that shaped it, and the instantiated graph.
 struct GraphEntry { std::string key; cudaGraphExec_t exec; int launches; };
+// Writes such a key, field by field: the structs contain padding bytes whose content the caller does not control.
+struct KeyWriter {
+  std::string& key;
+  void put(const void* ptr, size_t n) { key.append((const char*)ptr, n); }
+  template <class T> void val(const T& v) { put(&v, sizeof(v)); }
+  void aq(const mixaq_aq& q) { val(q.bits); val(q.scale); val(q.inv_scale); val(q.zero_point); }
+  void linear(const mixaq_linear& l) { val(l.codes); val(l.scale); val(l.out_features); val(l.in_features); val(l.bits); }
+  void branch(const mixaq_branch& b) {
+    const float* ptrs[8] = {b.ln1_g, b.ln1_b, b.ln2_g, b.ln2_b, b.b_qkv, b.b_proj, b.b_fc1, b.b_fc2};
+    put(ptrs, sizeof(ptrs));
+    aq(b.qkv_in); aq(b.q); aq(b.k); aq(b.v); aq(b.proj_in); aq(b.fc1_in); aq(b.fc2_in);
+    val(b.bits);
+  }
+  void block(const mixaq_block_params& q) {
+    const int dims[5] = {q.dim, q.heads, q.window, q.shift, q.hidden};
+    put(dims, sizeof(dims));
+    linear(q.qkv); linear(q.proj); linear(q.fc1); linear(q.fc2);
+    val(q.relpos_table);
+    branch(q.hi); branch(q.lo);
+    val(q.score_inv_scale); val(q.prepared); val(q.byte_codes);
+  }
+};
+constexpr size_t MAX_BACKBONE_GRAPHS = 16, MAX_BLOCK_GRAPHS = 8, MAX_BLOCK_KEYS = 8;
 struct mixaq_ctx {
   int device;
   int* d_status;
@@ -37,7 +61,11 @@ struct mixaq_ctx {
   bool allow_elevation;                // backbone: every pair uses its own ratios even if an earlier pair of the stage had larger ones
   cudaStream_t capture_stream;         // forwards on a stream that cannot be captured (the legacy default one) are recorded here
   cudaStream_t side_stream; cudaEvent_t fork, join;   // output norms run beside the next stage inside a captured forward
-  std::vector<GraphEntry> graphs;
+  std::mutex graph_lock;               // for what follows and the two streams above
+  std::vector<GraphEntry> graphs;      // of backbone forwards
+  std::vector<GraphEntry> block_graphs;
+  std::vector<std::string> block_keys; // block calls seen once, the oldest first
+  long block_captures, block_replays;
   std::vector<ProfRec> prof;          // event pairs recorded since mixaq_profile_begin
   std::vector<cudaEvent_t> pool;      // events ready for reuse
 };
@@ -303,7 +331,7 @@ mixaq_status mixaq_create(mixaq_ctx** out, int device) {
   if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return MIXAQ_CUDA_ERROR; }
   mixaq_ctx* c = new (std::nothrow) mixaq_ctx();
   if (!c) return MIXAQ_INTERNAL;
-  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr; c->side_stream = nullptr; c->fork = c->join = nullptr;
+  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr; c->side_stream = nullptr; c->fork = c->join = nullptr; c->block_captures = c->block_replays = 0;
   if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess || cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess ||
       !gemm_init() || !ln_init()) {
     cudaGetLastError(); if (c->d_status) cudaFree(c->d_status); delete c; return MIXAQ_CUDA_ERROR;
@@ -318,6 +346,7 @@ mixaq_status mixaq_destroy(mixaq_ctx* ctx) {
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
   if (ctx->side_stream) { cudaStreamDestroy(ctx->side_stream); cudaEventDestroy(ctx->fork); cudaEventDestroy(ctx->join); }
   for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
+  for (auto& g : ctx->block_graphs) cudaGraphExecDestroy(g.exec);
   for (cudaGraphExec_t g : ctx->prof_execs) cudaGraphExecDestroy(g);
   for (auto& r : ctx->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
   for (auto e : ctx->pool) cudaEventDestroy(e);
@@ -632,8 +661,82 @@ mixaq_status mixaq_block_forward(mixaq_ctx* ctx, const mixaq_block_params* p, co
                                  const mixaq_select_opts* opts, const mixaq_selection* sel_out,
                                  void* workspace, size_t workspace_bytes, const mixaq_taps* taps,
                                  void* cuda_stream) {
-  return block_forward_impl(ctx, p, x, y, B, H, W, low_ratio, prune_ratio, opts, sel_out, workspace, workspace_bytes,
-                            taps, nullptr, cuda_stream);
+  const cudaStream_t user_stream = (cudaStream_t)cuda_stream;
+  auto forward = [&](cudaStream_t st) {
+    return block_forward_impl(ctx, p, x, y, B, H, W, low_ratio, prune_ratio, opts, sel_out, workspace, workspace_bytes,
+                              taps, nullptr, st);
+  };
+  // A call repeated with the same arguments replays a graph: issuing its eleven launches and their tensor maps takes the
+  // host longer than a small block takes the GPU (C = 96 at 56 x 56: 55 us a call before, 41 now; C = 384 at 50 x 84 with
+  // pruning, bound by the GPU but for the gaps between stream launches: 78 and 69).  The buffers of a block call change from call to call more often than a
+  // backbone's, so a graph is recorded at the SECOND call with a key, and no further ones once they are not being replayed
+  // (recording costs the host about as much as ten calls).
+  if (!ctx || !p || taps || !ctx->graph_cache || ctx->profiling || ctx->guards || ctx->nvtx) return forward(user_stream);
+  const bool legacy = user_stream == nullptr || user_stream == cudaStreamLegacy;   // cannot be captured itself
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (!legacy && (cudaStreamIsCapturing(user_stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) {
+    cudaGetLastError();
+    return forward(user_stream);
+  }
+  std::string key;
+  key.reserve(1024);
+  KeyWriter k{key};
+  k.val(x); k.val(y); k.val(workspace); k.val(workspace_bytes); k.val(user_stream);
+  const int32_t* energy = opts ? opts->energy : nullptr;
+  const int dims[5] = {B, H, W, opts ? opts->reverse : 0, sel_out ? 1 : 0};
+  k.put(dims, sizeof(dims));
+  k.val(energy); k.val(low_ratio); k.val(prune_ratio);
+  if (sel_out) {
+    const void* ptrs[6] = {sel_out->cls, sel_out->order, sel_out->score, sel_out->idx_hi, sel_out->idx_lo, sel_out->idx_pr};
+    k.put(ptrs, sizeof(ptrs));
+  }
+  k.block(*p);
+  std::lock_guard<std::mutex> lock(ctx->graph_lock);
+  for (auto& g : ctx->block_graphs)
+    if (g.key == key) {
+      if (cudaGraphLaunch(g.exec, user_stream) != cudaSuccess) return check_cuda(ctx, "block_forward (graph launch)");
+      ctx->launches = g.launches;
+      ++ctx->block_replays;
+      return MIXAQ_OK;
+    }
+  size_t at = 0;
+  while (at < ctx->block_keys.size() && ctx->block_keys[at] != key) ++at;
+  const bool seen = at < ctx->block_keys.size();
+  bool record = seen && ctx->block_captures <= (long)MAX_BLOCK_GRAPHS + ctx->block_replays / 32;
+  if (record && legacy && !ctx->capture_stream &&
+      cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    ctx->capture_stream = nullptr; record = false;
+  }
+  const cudaStream_t st = legacy ? ctx->capture_stream : user_stream;
+  if (record && cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) record = false;
+  if (!record) {
+    cudaGetLastError();
+    const mixaq_status result = forward(user_stream);
+    if (result == MIXAQ_OK && !seen) {
+      if (ctx->block_keys.size() >= MAX_BLOCK_KEYS) ctx->block_keys.erase(ctx->block_keys.begin());
+      ctx->block_keys.push_back(std::move(key));
+    }
+    return result;
+  }
+  const mixaq_status result = forward(st);
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  const bool recorded = cudaStreamEndCapture(st, &graph) == cudaSuccess && graph && result == MIXAQ_OK &&
+                        cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
+  if (graph) cudaGraphDestroy(graph);
+  ++ctx->block_captures;
+  if (!recorded) {
+    cudaGetLastError();
+    return result != MIXAQ_OK ? result : forward(user_stream);
+  }
+  ctx->block_keys.erase(ctx->block_keys.begin() + at);
+  if (ctx->block_graphs.size() >= MAX_BLOCK_GRAPHS) {
+    cudaGraphExecDestroy(ctx->block_graphs.front().exec);
+    ctx->block_graphs.erase(ctx->block_graphs.begin());
+  }
+  ctx->block_graphs.push_back({std::move(key), exec, ctx->launches});
+  if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, "block_forward (graph launch)");
+  return MIXAQ_OK;
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -771,6 +874,8 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
   // Replay as a CUDA graph when an identical call was captured before.  The key is made of every value that
   // shapes the launches: the fields of the HOST parameter structs, ratios, pointers, sizes and the stream.
   bool use_graph = ctx->graph_cache;
+  std::unique_lock<std::mutex> lock(ctx->graph_lock, std::defer_lock);
+  if (use_graph) lock.lock();
   // The legacy default stream cannot be captured, but a graph can be launched on it: such calls are recorded on a stream
   // of the context's own (stage1_pair and Swin-T calls on it were bound by one host launch per kernel).
   const cudaStream_t user_stream = st;
@@ -792,39 +897,21 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); use_graph = false; }
     else ctx->prof_capture = true;
   } else if (use_graph) {
-    // field by field: the structs contain padding bytes whose content the caller does not control
-    auto put = [&key](const void* ptr, size_t n) { key.append((const char*)ptr, n); };
-    auto put_aq = [&](const mixaq_aq& q) { put(&q.bits, 4); put(&q.scale, 4); put(&q.inv_scale, 4); put(&q.zero_point, 4); };
-    auto put_lin = [&](const mixaq_linear& l) {
-      put(&l.codes, sizeof(l.codes)); put(&l.scale, sizeof(l.scale)); put(&l.out_features, 4); put(&l.in_features, 4); put(&l.bits, 4);
-    };
-    auto put_branch = [&](const mixaq_branch& b) {
-      const float* ptrs[8] = {b.ln1_g, b.ln1_b, b.ln2_g, b.ln2_b, b.b_qkv, b.b_proj, b.b_fc1, b.b_fc2};
-      put(ptrs, sizeof(ptrs));
-      put_aq(b.qkv_in); put_aq(b.q); put_aq(b.k); put_aq(b.v); put_aq(b.proj_in); put_aq(b.fc1_in); put_aq(b.fc2_in);
-      put(&b.bits, 4);
-    };
+    KeyWriter k{key};
+    auto put = [&k](const void* ptr, size_t n) { k.put(ptr, n); };
     const int npairs = (nblk + 1) / 2;
     put(&p->num_stages, sizeof(int)); put(p->depths, sizeof(int) * p->num_stages);
-    for (int b = 0; b < nblk; ++b) {
-      const mixaq_block_params& q = p->blocks[b];
-      const int dims[5] = {q.dim, q.heads, q.window, q.shift, q.hidden};
-      put(dims, sizeof(dims));
-      put_lin(q.qkv); put_lin(q.proj); put_lin(q.fc1); put_lin(q.fc2);
-      put(&q.relpos_table, sizeof(q.relpos_table));
-      put_branch(q.hi); put_branch(q.lo);
-      put(&q.score_inv_scale, 4); put(&q.prepared, sizeof(q.prepared)); put(&q.byte_codes, 4);
-    }
+    for (int b = 0; b < nblk; ++b) k.block(p->blocks[b]);
     for (int m = 0; m + 1 < p->num_stages; ++m) {
       const mixaq_merge_params& q = p->merges[m];
-      put(&q.ln_g, sizeof(q.ln_g)); put(&q.ln_b, sizeof(q.ln_b)); put_aq(q.in); put_lin(q.reduction);
+      put(&q.ln_g, sizeof(q.ln_g)); put(&q.ln_b, sizeof(q.ln_b)); k.aq(q.in); k.linear(q.reduction);
       put(&q.prepared, sizeof(q.prepared));
     }
     const char has_embed = p->embed ? 1 : 0, has_norms = norms ? 1 : 0;
     put(&has_embed, 1); put(&has_norms, 1);
     if (p->embed) {
       const mixaq_embed_params& q = *p->embed;
-      put(&q.ln_g, sizeof(q.ln_g)); put(&q.ln_b, sizeof(q.ln_b)); put(&q.bias, sizeof(q.bias)); put_aq(q.in); put_lin(q.proj);
+      put(&q.ln_g, sizeof(q.ln_g)); put(&q.ln_b, sizeof(q.ln_b)); put(&q.bias, sizeof(q.bias)); k.aq(q.in); k.linear(q.proj);
       put(&q.prepared, sizeof(q.prepared));
     }
     if (norms) { put(p->out_norm_g, sizeof(float*) * p->num_stages); put(p->out_norm_b, sizeof(float*) * p->num_stages); }
@@ -945,7 +1032,7 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
     if (prof_graph && ctx->profiling) {
       ctx->prof_execs.push_back(exec);
     } else {
-      if (ctx->graphs.size() >= 16) { cudaGraphExecDestroy(ctx->graphs.front().exec); ctx->graphs.erase(ctx->graphs.begin()); }
+      if (ctx->graphs.size() >= MAX_BACKBONE_GRAPHS) { cudaGraphExecDestroy(ctx->graphs.front().exec); ctx->graphs.erase(ctx->graphs.begin()); }
       ctx->graphs.push_back({key, exec, total});
     }
     if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
@@ -1089,10 +1176,14 @@ mixaq_status mixaq_set_window_elevation(mixaq_ctx* ctx, int allow) {
 
 mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled) {
   if (!ctx) return MIXAQ_INVALID_ARG;
+  std::lock_guard<std::mutex> lock(ctx->graph_lock);
   ctx->graph_cache = enabled != 0;
   if (!enabled) {
-    for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
-    ctx->graphs.clear();
+    for (auto* cache : {&ctx->graphs, &ctx->block_graphs}) {
+      for (auto& g : *cache) cudaGraphExecDestroy(g.exec);
+      cache->clear();
+    }
+    ctx->block_keys.clear();
   }
   return MIXAQ_OK;
 }
