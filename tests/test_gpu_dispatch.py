@@ -1,0 +1,86 @@
+"""The size, width and value ranges between which the library chooses another kernel or another branch of one, at their
+edges: each against the CPU oracle, bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2507_19131_b200 import synth  # noqa: E402
+from test_gpu_parity import F32, ctx, dev, mq, run_block_case  # noqa: E402,F401
+
+
+@pytest.mark.parametrize("dim,H,W,bits", [(96, 312, 319, (8, 4)), (128, 270, 278, (4, 2)), (192, 221, 230, (8, 2)),
+                                          (256, 194, 196, (8, 4))])
+def test_streaming_layer_norm_just_above_its_threshold(orc, mq, ctx, dim, H, W, bits):
+    """Ragged maps with a few windows more than the streaming kernel's lower limit; row counts that are no multiple of
+    the rows of a warp, in both branches."""
+    blk = synth.make_block(np.random.default_rng(dim), dim, dim // 32, 3, 4, *bits)
+    run_block_case(orc, mq, ctx, blk, synth.input_student_t(dim, 1, H, W, dim), 0.35, taps=False)
+
+
+@pytest.mark.parametrize("H,W", [(7, 7), (56, 56), (34, 90), (63, 49)])
+def test_window_selection_around_64_windows(orc, mq, ctx, H, W):
+    """1, 64 (one launch), 65 and 63 windows per image, with ties, in every order of two ratios."""
+    blk = synth.make_block(np.random.default_rng(H), 32, 1, 3, 8, 8, 4)
+    x = np.round(synth.input_student_t(W, 3, H, W, 32))
+    for low, prune, rev in [(0.5, 0.0, False), (0.25, 0.25, True)]:
+        run_block_case(orc, mq, ctx, blk, x, low, prune, reverse=rev, taps=False)
+
+
+@pytest.mark.parametrize("dim,windows", [(32, (27, 28)), (32, (28, 28)), (64, (28, 28)), (96, (28, 28)), (1024, (1, 2))])
+def test_gemm_tilings_around_their_limits(orc, mq, ctx, dim, windows):
+    """Row tiles just below and above the limit of the 16 epilogue warps, tile widths 32 to 256, more accumulators than
+    tiles, remainders in the last row tile of both branches."""
+    blk = synth.make_block(np.random.default_rng(dim), dim, dim // 32, 0, 4, 8, 4, share_bias=False)
+    x = synth.input_student_t(dim, 1, 7 * windows[0], 7 * windows[1] - 2, dim)
+    run_block_case(orc, mq, ctx, blk, x, 0.55, taps=False)
+
+
+@pytest.mark.parametrize("dim,sign", [(128, 1), (128, -1), (192, 1), (384, -1), (384, 0)])
+def test_gemm_accumulators_beyond_the_bias_trick(orc, mq, ctx, dim, sign):
+    """Weights of full magnitude: sums of 128 products of 255 x 127 stay below 2^22, from 192 on they may not, and the
+    epilogues then convert them with integer instructions."""
+    rng = np.random.default_rng(dim + sign)
+    blk = synth.make_block(rng, dim, dim // 32, 3, 8, 8, 4)
+    for lin in (blk.qkv, blk.proj, blk.fc1, blk.fc2):
+        lin.codes[:] = 127 * (sign if sign else rng.choice([-1, 1], size=lin.codes.shape))
+        lin.scale[:] = (lin.scale * F32(0.05)).astype(F32)
+    run_block_case(orc, mq, ctx, blk, synth.input_blobs(dim, 1, 17, 23, dim, bg_std=0.5, gain=4.0), 0.4)
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_block_graphs_follow_data_buffers_and_switch(orc, mq, ctx, own_stream):
+    """Repeated block calls (recorded at the second, replayed from the third) see fresh data; more sets of buffers than
+    graphs are kept, and the switch that turns them off, change nothing."""
+    blk = synth.make_block(np.random.default_rng(3), 64, 2, 3, 4, 8, 4)
+    xs = [synth.input_blobs(s, 1, 15, 22, 64, bg_std=0.5, gain=4.0) for s in range(3)]
+    want = [orc.block_forward(blk, x, 0.5, 0.25).y for x in xs]
+    stream = torch.cuda.Stream() if own_stream else torch.cuda.default_stream()
+    with torch.cuda.stream(stream):
+        db = mq.DeviceBlock(ctx, blk)
+        pairs = [(dev(xs[0]), torch.empty(xs[0].shape, device="cuda")) for _ in range(10)]
+        for step in range(6):
+            if step == 4:
+                ctx.set_graph_cache(False)
+            for xd, yd in pairs:
+                xd.copy_(torch.from_numpy(xs[step % 3]))
+                yd.zero_()
+                mq.block_forward(ctx, db, xd, 0.5, 0.25, y=yd)
+                stream.synchronize()
+                assert np.array_equal(yd.cpu().numpy(), want[step % 3]), f"step {step}"
+        ctx.set_graph_cache(True)
+
+
+@pytest.mark.parametrize("w_bits,H,W,dim", [(8, 9, 15, 96), (6, 8, 16, 32), (2, 12, 11, 128)])
+def test_calibration_products_by_weight_width(orc, mq, ctx, w_bits, H, W, dim):
+    """Weights whose products are fused (2 to 6 bits) and are not (8), at row counts around a tile of 128."""
+    blk = synth.make_block(np.random.default_rng(w_bits), dim, dim // 32, 3, w_bits, 8, 4)
+    x = synth.input_blobs(5, 1, H, W, dim, bg_std=0.5, gain=3.0)
+    params = mq._Dev(ctx.device)                                  # keeps the uploads alive
+    bs = mq.fill_block_struct(params, blk)
+    y, got = mq.calibrate_block(ctx, bs, 0, dev(x))
+    want_y, want = orc.block_observe_fp(blk, "hi", x)
+    assert np.array_equal(y.cpu().numpy(), want_y)
+    for site, span in want.items():
+        assert got[site] == span, site
