@@ -219,23 +219,23 @@ __global__ void __launch_bounds__(256, (NG * (32 / G) > 24 ? 2 : 4)) k_ln_quant_
 
 // The same for batches that keep every SM busy for a while: persistent warps walk over row groups and fetch STAGES groups
 // ahead by asynchronous copies into shared memory, every thread into slots that it alone reads back (no barrier).  The plain
-// kernel alternates between waiting for its loads and computing: 3.6 TB/s at 296 450 rows of 128 channels (45 to 50 us); see
-// launch_ln_quant for what this one reaches.
-template <int BYTES>
-__device__ __forceinline__ void cp_async(uint32_t smem_dst, const void* src) {
-  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(src) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_dst), "l"(src), "n"(BYTES) : "memory");
+// kernel alternates between waiting for its loads and computing: 45 to 50 us at 296 450 rows of 128 channels (180 MB, 3.6 to 4
+// TB/s), this one 40 (4.5 TB/s); 148 225 rows of 256 channels 26 and 21.5.  Eight lanes per row: with 16 the shuffles cost more
+// (50 us), with 4 the chain of a lane (59).
+__device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(src) : "memory");
 }
 constexpr int LN_STAGES = 3, LN_STREAM_CTAS = 2;
 template <int NG, int G> constexpr int ln_stream_smem() { return LN_STAGES * NG * (32 / G) * 256 * 4; }
 template <int NG, int G>
 __global__ void __launch_bounds__(256, LN_STREAM_CTAS) k_ln_stream(LnBranch hi, LnBranch lo, int groups_hi, int groups) {
-  constexpr int C = NG * 32, P = 32 / G, ROWS = 32 / G, VEC = P >= 4 ? 4 : 2, NV = NG * P / VEC;
+  constexpr int C = NG * 32, P = 32 / G, ROWS = 32 / G;
+  static_assert(P == 4, "one 16-byte copy per channel group");
   extern __shared__ __align__(16) float ring[];
   griddep_launch();
   const int lane = threadIdx.x & 31, j = lane % G, rw = lane / G;
   const int step = gridDim.x * 8;
-  const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * (VEC * 4);
+  const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * 16;
   int it = blockIdx.x * 8 + (threadIdx.x >> 5);
   griddep_wait();
   // source row of this lane's row of a group: -1 pad token, -2 beyond the batch
@@ -251,8 +251,7 @@ __global__ void __launch_bounds__(256, LN_STREAM_CTAS) k_ln_stream(LnBranch hi, 
     if (srow >= 0) {
       const float* src = (g < groups_hi ? hi.src : lo.src) + (long)srow * C + P * j;
 #pragma unroll
-      for (int v = 0; v < NV; ++v)
-        cp_async<VEC * 4>(slot0 + (uint32_t)((stage * NV + v) * 256 * VEC * 4), src + 32 * (v / (P / VEC)) + VEC * (v % (P / VEC)));
+      for (int v = 0; v < NG; ++v) cp_async_16(slot0 + (uint32_t)((stage * NG + v) * 256 * 16), src + 32 * v);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -266,11 +265,9 @@ __global__ void __launch_bounds__(256, LN_STREAM_CTAS) k_ln_stream(LnBranch hi, 
     asm volatile("cp.async.wait_group %0;" ::"n"(LN_STAGES - 1) : "memory");
     float x[NG][P];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const float* sl = ring + ((stage * NV + v) * 256 + threadIdx.x) * VEC;
-      float* d = &x[v / (P / VEC)][VEC * (v % (P / VEC))];
-      if (VEC == 4) { const float4 a = *reinterpret_cast<const float4*>(sl); d[0] = a.x; d[1] = a.y; d[2 % P] = a.z; d[3 % P] = a.w; }
-      else { const float2 a = *reinterpret_cast<const float2*>(sl); d[0] = a.x; d[1] = a.y; }
+    for (int v = 0; v < NG; ++v) {
+      const float4 a = *reinterpret_cast<const float4*>(ring + ((stage * NG + v) * 256 + threadIdx.x) * 4);
+      x[v][0] = a.x; x[v][1] = a.y; x[v][2] = a.z; x[v][3] = a.w;
     }
     const int mine = src[0];
 #pragma unroll
@@ -355,7 +352,8 @@ void launch_ln_g(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
   launch_pdl(k_ln_quant_g<NG, G, MERGE>, dim3(bh + bl), 256, 0, st, hi, lo, bh);
 }
 
-// elements per SM from which the streaming LayerNorm is used: four row groups of 8 x 128 channels for each of its 16 warps
+// elements per SM from which the streaming LayerNorm is used: below, its 16 warps have fewer than eight groups of 4 rows x 128
+// channels each, and the set-up of the persistent grid costs what the overlap gives
 constexpr long LN_STREAM_MIN = 65536;
 template <int NG, int G>
 void launch_ln_stream(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
