@@ -178,11 +178,13 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
         uint32_t xlo = 0, xhi = 0;
         if (SHIFTED) { const uint32_t ri = sm.reg[i] * 0x11111111u; xlo = regj_lo ^ ri; xhi = regj_hi ^ ri; }
         // the two columns a lane holds per key tile are handled as a pair (packed binary32 arithmetic, lane-wise
-        // the same operations as the scalar contract)
-        float2 lg[7];
-        float mx = -3.0e38f;
+        // the same operations as the scalar contract).  Key columns 49..55 do not exist: of tile 6 a lane computes one
+        // column, and lane t = 0 alone uses it (as a pair it took a seventh of the softmax; Swin-B at 2 x 1536 x 1536, of
+        // which the attention is a fifth, went from 6117 to 6056 us).
+        float2 lg[6];
+        float mx = -3.0e38f, last;
 #pragma unroll
-        for (int nt = 0; nt < 7; ++nt) {
+        for (int nt = 0; nt < 6; ++nt) {
           const float4 rb = __ldg(relf + (mt * 7 + nt) * 32);
           const float2 sf = make_float2(__int2float_rn(c[nt][2 * r] + rqi + ckj[nt][0]),
                                         __int2float_rn(c[nt][2 * r + 1] + rqi + ckj[nt][1]));
@@ -193,66 +195,72 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
             v = __fadd2_rn(v, make_float2(x0 != 0 ? -100.0f : 0.0f, x1 != 0 ? -100.0f : 0.0f));
           }
           lg[nt] = v;
-          // key columns 49..55 do not exist: of tile 6 only column 0 of lane t = 0
-          if (nt < 6 || t == 0) mx = fmaxf(mx, v.x);
-          if (nt < 6) mx = fmaxf(mx, v.y);
+          mx = fmaxf(fmaxf(mx, v.x), v.y);
+        }
+        {
+          const float2 rb = __ldg(reinterpret_cast<const float2*>(relf + (mt * 7 + 6) * 32) + r);
+          last = __fmaf_rn(__int2float_rn(c[6][2 * r] + rqi + ckj[6][0]), alpha, rb.x);
+          if (SHIFTED) last = __fadd_rn(last, ((xhi >> 16) & 15u) != 0 ? -100.0f : 0.0f);
+          if (t == 0) mx = fmaxf(mx, last);
         }
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         // exponentials and this lane's partial sum in column order (the partial of index t of the contract)
         float part = 0.0f;
 #pragma unroll
-        for (int nt = 0; nt < 7; ++nt) {
+        for (int nt = 0; nt < 6; ++nt) {
           float2 tt = __fmul2_rn(sub2(lg[nt], f2(mx)), f2(kLog2e));
           tt = make_float2(fmaxf(tt.x, -125.0f), fmaxf(tt.y, -125.0f));
-          float2 e = exp2_core2(tt);
-          if (!(nt < 6 || t == 0)) e.x = 0.0f;
-          if (!(nt < 6)) e.y = 0.0f;
+          const float2 e = exp2_core2(tt);
           lg[nt] = e;
           part = __fadd_rn(__fadd_rn(part, e.x), e.y);
         }
+        last = exp2_core1(fmaxf(__fmul_rn(__fsub_rn(last, mx), kLog2e), -125.0f));
+        if (t != 0) last = 0.0f;
+        part = __fadd_rn(part, last);
         const float s1 = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, 1));
         const float sum = __fadd_rn(s1, __shfl_xor_sync(0xffffffffu, s1, 2));
         const float inv = __fdiv_rn(1.0f, sum);
         // P codes: clamp(rne(p * pmax), 0, pmax); byte u of A register (ks, r [+2]) is tile 4ks + [2 +] (u>>1), column u&1.
         // The clamp never acts: 0 <= e_j <= sum, so p * pmax lies in [0, pmax * (1 + 2^-22)] and rounds into 0 .. pmax;
-        // it is left out.  The rounded values stay in their "1.5 * 2^23 + code" patterns: the patterns are added into
-        // the A registers shifted into place and the bias they carry is taken out once per register.
-        uint32_t acc_pa[4] = {0u, 0u, 0u, 0u};
+        // it is left out.  The code is the low byte of the rounded value's "1.5 * 2^23 + code" pattern.
+        uint32_t code[14];
         uint32_t ps_raw = 0u;
+        // two roundings (product, then the add that rounds to an integer).  The products are scalar multiplies: a packed
+        // multiply feeding a packed add gets contracted into one fused operation, which rounds once and differs at exact .5 ties
 #pragma unroll
         for (int nt = 0; nt < 7; ++nt) {
-          const float2 pr = __fmul2_rn(lg[nt], f2(inv));          // the softmax output itself
+          const float2 pr = nt < 6 ? __fmul2_rn(lg[nt < 6 ? nt : 0], f2(inv)) : make_float2(__fmul_rn(last, inv), 0.0f);   // the softmax output
           if (TAPS && br.tap_probs) {
             const int j0 = 8 * nt + 2 * t;
             float* tp = br.tap_probs + (((long)slot * a.heads + h) * WT + i) * WT;
             if (i < WT && j0 < WT) tp[j0] = pr.x;
             if (i < WT && j0 + 1 < WT) tp[j0 + 1] = pr.y;
           }
-          // two roundings (product, then the add that rounds to an integer).  The products are scalar multiplies: a
-          // packed multiply feeding a packed add gets contracted into one fused operation, which rounds once and
-          // differs at exact .5 ties
-          const float2 tq = __fadd2_rn(make_float2(__fmul_rn(pr.x, pmaxf), __fmul_rn(pr.y, pmaxf)), f2(12582912.0f));
-          const uint32_t pat[2] = {__float_as_uint(tq.x), __float_as_uint(tq.y)};
-          const int ks = nt >> 2, sub = nt & 3;
+          if (nt < 6) {
+            const float2 tq = __fadd2_rn(make_float2(__fmul_rn(pr.x, pmaxf), __fmul_rn(pr.y, pmaxf)), f2(12582912.0f));
+            code[2 * nt] = __float_as_uint(tq.x);
+            code[2 * nt + 1] = __float_as_uint(tq.y);
+            ps_raw += code[2 * nt] + code[2 * nt + 1];
+          } else {
+            code[12] = __float_as_uint(__fadd_rn(__fmul_rn(pr.x, pmaxf), 12582912.0f));
+            code[13] = kMagicBits;
+            ps_raw += code[12];
+          }
+          if (TAPS && br.tap_p) {
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            ps_raw += pat[u];
-            acc_pa[2 * ks + (sub >> 1)] += pat[u] << (8 * (2 * (sub & 1) + u));
-            if (TAPS && br.tap_p) {
+            for (int u = 0; u < 2; ++u) {
               const int j = 8 * nt + 2 * t + u;
-              if (i < WT && j < WT) br.tap_p[(((long)slot * a.heads + h) * WT + i) * WT + j] = (uint8_t)(pat[u] - kMagicBits);
+              if (i < WT && j < WT) br.tap_p[(((long)slot * a.heads + h) * WT + i) * WT + j] = (uint8_t)(code[2 * nt + u] - kMagicBits);
             }
           }
         }
-        // register (ks, half): four patterns (three for ks = 1, half = 1: tiles 4..6 only); the low byte of a pattern's
-        // bias 0x4B400000 is zero, so shifted into a byte lane it only reaches higher bytes, which the sum drops
-        // beyond bit 31: bias of a register = sum over its lanes of (0x4B400000 << 8 lane) mod 2^32
-        constexpr uint32_t kBias4 = kMagicBits + (kMagicBits << 8) + (kMagicBits << 16) + (kMagicBits << 24);
-        constexpr uint32_t kBias2 = kMagicBits + (kMagicBits << 8);
-        pa[0][r] = acc_pa[0] - kBias4;  pa[0][r + 2] = acc_pa[1] - kBias4;
-        pa[1][r] = acc_pa[2] - kBias4;  pa[1][r + 2] = acc_pa[3] - kBias2;
-        int ps = (int)(ps_raw - 14u * kMagicBits);
+        auto join = [](uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3) {
+          return __byte_perm(__byte_perm(a0, a1, 0x0040), __byte_perm(a2, a3, 0x0040), 0x5410);
+        };
+        pa[0][r] = join(code[0], code[1], code[2], code[3]);  pa[0][r + 2] = join(code[4], code[5], code[6], code[7]);
+        pa[1][r] = join(code[8], code[9], code[10], code[11]);  pa[1][r + 2] = code[12] & 0xFFu;
+        int ps = (int)(ps_raw - 13u * kMagicBits);
         ps += __shfl_xor_sync(0xffffffffu, ps, 1);
         ps += __shfl_xor_sync(0xffffffffu, ps, 2);
         psum[r] = ps;

@@ -54,6 +54,18 @@ __device__ __forceinline__ float2 exp2_core2(float2 t) {
                      __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(r.y) << 23)));
 }
 
+__device__ __forceinline__ float exp2_core1(float t) {             // one lane of exp2_core2
+  const float r = __fadd_rn(t, 12582912.0f);
+  const float f = __fsub_rn(t, __fadd_rn(r, -12582912.0f));
+  float p = __uint_as_float(0x3aafc47du);
+  p = __fmaf_rn(p, f, __uint_as_float(0x3c1e883du));
+  p = __fmaf_rn(p, f, __uint_as_float(0x3d635716u));
+  p = __fmaf_rn(p, f, __uint_as_float(0x3e75fc83u));
+  p = __fmaf_rn(p, f, __uint_as_float(0x3f317219u));
+  p = __fmaf_rn(p, f, __uint_as_float(0x3f800001u));
+  return __uint_as_float(__float_as_uint(p) + (__float_as_uint(r) << 23));
+}
+
 // GELU(v) = max(v,0) - a*Phi(-a), a = min(|v|, 5); log2 Phi(-a) is a degree-7 polynomial on [0,5].
 __device__ __forceinline__ float2 gelu_log2_tail2(float2 a) {      // log2 Phi(-a) on [0, 5]
   float2 q = f2(__uint_as_float(0xb5d6f9e3u));
