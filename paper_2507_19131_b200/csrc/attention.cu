@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
   const float pmaxf = (float)pmax;
   const AQ oq = br.o;
   const float kLog2e = 1.44269504088896340736f;
-  const float4* relf = reinterpret_cast<const float4*>(a.relbias) + (long)h * (4 * 7 * 32) + lane;
+  const float2* relf = reinterpret_cast<const float2*>(a.relbias) + (long)h * (4 * 7 * 64) + lane;
   const long m_base = (long)slot * WT;
   const long out_row_bytes = (long)C * cbits / 8;
 
@@ -185,10 +185,10 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
         float mx = -3.0e38f, last;
 #pragma unroll
         for (int nt = 0; nt < 6; ++nt) {
-          const float4 rb = __ldg(relf + (mt * 7 + nt) * 32);
+          const float2 rb = __ldg(relf + (mt * 7 + nt) * 64 + 32 * r);
           const float2 sf = make_float2(__int2float_rn(c[nt][2 * r] + rqi + ckj[nt][0]),
                                         __int2float_rn(c[nt][2 * r + 1] + rqi + ckj[nt][1]));
-          float2 v = __ffma2_rn(sf, f2(alpha), r == 0 ? make_float2(rb.x, rb.y) : make_float2(rb.z, rb.w));
+          float2 v = __ffma2_rn(sf, f2(alpha), rb);
           if (SHIFTED) {
             const uint32_t x0 = nt < 4 ? (xlo >> (4 * (2 * nt))) & 15u : (xhi >> (4 * (2 * (nt - 4)))) & 15u;
             const uint32_t x1 = nt < 4 ? (xlo >> (4 * (2 * nt + 1))) & 15u : (xhi >> (4 * (2 * (nt - 4) + 1))) & 15u;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
           mx = fmaxf(fmaxf(mx, v.x), v.y);
         }
         {
-          const float2 rb = __ldg(reinterpret_cast<const float2*>(relf + (mt * 7 + 6) * 32) + r);
+          const float2 rb = __ldg(relf + (mt * 7 + 6) * 64 + 32 * r);
           last = __fmaf_rn(__int2float_rn(c[6][2 * r] + rqi + ckj[6][0]), alpha, rb.x);
           if (SHIFTED) last = __fadd_rn(last, ((xhi >> 16) & 15u) != 0 ? -100.0f : 0.0f);
           if (t == 0) mx = fmaxf(mx, last);

@@ -30,13 +30,14 @@ __global__ void __launch_bounds__(256) k_prepare_linear(const int8_t* __restrict
 }
 
 // Relative-position bias in the order the attention kernel's accumulator fragments want it:
-// out[((h*4 + mt)*7 + nt)*32 + lane] = float4 of bias[h][i][j] at (i, j) = (16mt+g, 8nt+2t), (16mt+g, 8nt+2t+1),
-// (16mt+g+8, 8nt+2t), (16mt+g+8, 8nt+2t+1) with g = lane/4, t = lane%4; 0 outside the 49 x 49 table, where
+// out[(((h*4 + mt)*7 + nt)*2 + r)*32 + lane] = float2 of bias[h][i][j] at (i, j) = (16mt+g+8r, 8nt+2t), (16mt+g+8r, 8nt+2t+1)
+// with g = lane/4, t = lane%4, so that a warp reads a row half of a tile as 256 consecutive bytes; 0 outside the 49 x 49
+// table, where
 // bias[h][i][j] = table[((yi - yj + 6) * 13 + (xi - xj + 6)) * heads + h].
 __global__ void k_prepare_relbias(const float* __restrict__ table, int heads, float* out) {
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= heads * 4 * 7 * 32 * 4) return;
-  const int comp = idx & 3, lane = (idx >> 2) & 31;
+  const int comp = (idx & 1) | ((idx >> 6 & 1) << 1), lane = (idx >> 1) & 31;
   const int tile = idx >> 7;                       // (h*4 + mt)*7 + nt
   const int nt = tile % 7, mt = (tile / 7) & 3, h = tile / 28;
   const int i = 16 * mt + (lane >> 2) + 8 * (comp >> 1);
