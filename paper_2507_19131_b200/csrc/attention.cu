@@ -90,39 +90,44 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 8) k_attention(AttnArgs a) {
   const int zq = br.q.zp, zk = br.k.zp, zv = br.v.zp;
 
   griddep_wait();
-  // ---- stage q, k (rows) and v (transposed, permuted) of this head, one code per byte: 3 x 64 row items ----
+  // ---- stage q, k (rows) and v (transposed, permuted) of this head, one code per byte: half a row per thread and matrix.
+  // Two neighbouring lanes share a row of q or k, so that a load instruction touches 16 rows instead of 32 (the rows lie
+  // 3C codes apart: the load/store pipe takes a cycle for each); v rows go to the warp that writes their bytes in order. ----
   int wy = 0, wx = 0;
   if (SHIFTED) { const int w = br.win[slot]; wy = w / a.nwx; wx = w - wy * a.nwx; }
-  for (int item = threadIdx.x; item < 3 * 64; item += ATT_WARPS * 32) {
-    const int sec = item >> 6, r = item & 63;
-    const uint8_t* src = br.qkv + ((long)slot * WT + r) * row_bytes + (long)(sec * C + h * HEAD_DIM) * cbits / 8;
-    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (r < WT) load_codes_32(src, cbits, w);
-    if (sec < 2) {
-      int s = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s = dp4a_uu(w[e], 0x01010101u, s);
-      if (sec == 0) {
-        *reinterpret_cast<uint4*>(&sm.q[r][0]) = make_uint4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<uint4*>(&sm.q[r][4]) = make_uint4(w[4], w[5], w[6], w[7]);
-        sm.rq[r] = r < WT ? -zk * s + HEAD_DIM * zq * zk : 0;
-        int reg = 0;
-        if (SHIFTED && r < WT) {
-          const int i = r / WS, j = r - i * WS;
-          reg = shift_region(wy * WS + i, a.Hp, a.shift) * 3 + shift_region(wx * WS + j, a.Wp, a.shift);
-        }
-        sm.reg[r] = (uint8_t)reg;
-      } else if (r < 56) {
-        *reinterpret_cast<uint4*>(&sm.k[r][0]) = make_uint4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<uint4*>(&sm.k[r][4]) = make_uint4(w[4], w[5], w[6], w[7]);
-        sm.ck[r] = -zq * s;
-      }
-    } else {
-      uint8_t* vtb = reinterpret_cast<uint8_t*>(&sm.vt[0][0]);
-      const int p = pos(r);
-#pragma unroll
-      for (int e = 0; e < 32; ++e) vtb[e * (VT_LD * 4) + p] = (uint8_t)(w[e >> 2] >> (8 * (e & 3)));
+  {
+    const int half_bytes = 16 * cbits / 8;
+    const uint8_t* head = br.qkv + (long)slot * WT * row_bytes + (long)(h * HEAD_DIM) * cbits / 8;
+    const long sec_bytes = (long)C * cbits / 8;
+    const int rq = threadIdx.x >> 1, hq = threadIdx.x & 1;       // q, k: row and half
+    const int rv = threadIdx.x & 63, hv = threadIdx.x >> 6;      // v
+    uint32_t wq[4] = {0, 0, 0, 0}, wk[4] = {0, 0, 0, 0}, wv[4] = {0, 0, 0, 0};
+    if (rq < WT) {
+      load_codes_16(head + rq * row_bytes + hq * half_bytes, cbits, wq);
+      load_codes_16(head + rq * row_bytes + sec_bytes + hq * half_bytes, cbits, wk);
     }
+    if (rv < WT) load_codes_16(head + rv * row_bytes + 2 * sec_bytes + hv * half_bytes, cbits, wv);
+    int s_q = 0, s_k = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { s_q = dp4a_uu(wq[e], 0x01010101u, s_q); s_k = dp4a_uu(wk[e], 0x01010101u, s_k); }
+    s_q += __shfl_xor_sync(0xffffffffu, s_q, 1);
+    s_k += __shfl_xor_sync(0xffffffffu, s_k, 1);
+    *reinterpret_cast<uint4*>(&sm.q[rq][4 * hq]) = make_uint4(wq[0], wq[1], wq[2], wq[3]);
+    if (rq < 56) *reinterpret_cast<uint4*>(&sm.k[rq][4 * hq]) = make_uint4(wk[0], wk[1], wk[2], wk[3]);
+    if (hq == 0) {
+      sm.rq[rq] = rq < WT ? -zk * s_q + HEAD_DIM * zq * zk : 0;
+      if (rq < 56) sm.ck[rq] = -zq * s_k;
+    } else {
+      int reg = 0;
+      if (SHIFTED && rq < WT) {
+        const int i = rq / WS, j = rq - i * WS;
+        reg = shift_region(wy * WS + i, a.Hp, a.shift) * 3 + shift_region(wx * WS + j, a.Wp, a.shift);
+      }
+      sm.reg[rq] = (uint8_t)reg;
+    }
+    uint8_t* vtb = reinterpret_cast<uint8_t*>(&sm.vt[0][0]) + 16 * hv * (VT_LD * 4) + pos(rv);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) vtb[e * (VT_LD * 4)] = (uint8_t)(wv[e >> 2] >> (8 * (e & 3)));
   }
   __syncthreads();
 

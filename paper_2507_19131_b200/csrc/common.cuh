@@ -276,5 +276,20 @@ __device__ __forceinline__ void load_codes_32(const uint8_t* src, int bits, uint
     expand_nibbles(spread_pairs(a.y >> 16), w[6], w[7]);
   }
 }
+// 16 codes, one per byte (the source aligned to their packed size)
+__device__ __forceinline__ void load_codes_16(const uint8_t* src, int bits, uint32_t (&w)[4]) {
+  if (bits == 8) {
+    const uint4 a = *reinterpret_cast<const uint4*>(src);
+    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+  } else if (bits == 4) {
+    const uint2 a = *reinterpret_cast<const uint2*>(src);
+    expand_nibbles(a.x, w[0], w[1]);
+    expand_nibbles(a.y, w[2], w[3]);
+  } else {
+    const uint32_t a = *reinterpret_cast<const uint32_t*>(src);
+    expand_nibbles(spread_pairs(a & 0xFFFFu), w[0], w[1]);
+    expand_nibbles(spread_pairs(a >> 16), w[2], w[3]);
+  }
+}
 
 }  // namespace mixaq
