@@ -137,7 +137,7 @@ typedef struct {
 
 /* ---- context ---- */
 /* Creates a context on `device` (makes it current).  Holds the status word, the captured graphs of
- * mixaq_backbone_forward and the profiling events. */
+ * repeated calls and the profiling events. */
 mixaq_status mixaq_create(mixaq_ctx** ctx, int device);
 mixaq_status mixaq_destroy(mixaq_ctx* ctx);
 /* Text of the last host-side error of this context (static storage, valid until the next call). */
@@ -253,16 +253,16 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
                                     const float* low_ratio_per_pair, const float* prune_ratio_per_pair /* nullable */,
                                     void* workspace, size_t workspace_bytes, void* cuda_stream);
 
-/* mixaq_backbone_forward replays a CUDA graph when it is called again with exactly the same arguments (same
- * parameter structs byte for byte, pointers, sizes, ratios, workspace and stream): the first such call captures the
- * launches on `cuda_stream`, later calls cost one graph launch on the host.  The data behind the pointers may
- * change freely between calls.  Captured graphs are kept per context (16 at most) until mixaq_destroy.  A call on the
- * legacy default stream (NULL), which cannot be captured, is recorded on a stream of the context's own and its graph
- * launched on the legacy stream; a call made while the caller is capturing the stream itself launches its kernels
- * directly.  A backbone forward between mixaq_profile_begin/end is captured together with its event records, launched once
- * and not cached; a block forward there launches its kernels directly.
- * mixaq_block_forward (without taps) does the same from the second call with the same arguments on; it keeps 8 graphs,
- * and stops recording new ones while those it has are not replayed.
+/* mixaq_backbone_forward and mixaq_block_forward (without taps) replay a CUDA graph when they are called again with exactly
+ * the same arguments (same parameter structs field by field, pointers, sizes, ratios, workspace and stream).  The first
+ * such call issues its kernels, the second is recorded, later ones cost one graph launch on the host.  The data behind the
+ * pointers may change freely between calls.  A context keeps 16 graphs of backbone calls and 8 of block calls, the least
+ * recently used leave; it remembers as many calls that are not recorded yet.  Recording costs the host several times what
+ * issuing a call does, so calls whose graphs are not replayed (rotating buffers, changing ratios) stop being recorded;
+ * a call repeated 32 times is recorded in any case.  A call on the legacy default stream (NULL), which cannot be captured,
+ * is recorded on a stream of the context's own and its graph launched on the legacy stream; a call made while the caller is
+ * capturing the stream itself issues its kernels.  A backbone forward between mixaq_profile_begin/end is captured together
+ * with its event records, launched once and not kept; a block forward there issues its kernels.
  * enabled = 0 switches the cache off and drops the stored graphs; it is on by default. */
 mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled);
 

@@ -3,6 +3,7 @@
 // Nothing here computes: every step of the path runs in the kernels.
 #include <nvtx3/nvToolsExt.h>
 #include "../../include/mixaq.h"
+#include "graph_cache.h"
 #include "kernels.h"
 #include <cmath>
 #include <cstdio>
@@ -21,9 +22,8 @@ thread_local int g_launches = 0;
 using namespace mixaq;
 
 struct ProfRec { int cat; cudaEvent_t e0, e1; };
-// One captured forward: the exact bytes of every argument that shaped it, and the instantiated graph.
-struct GraphEntry { std::string key; cudaGraphExec_t exec; int launches; };
-// Writes such a key, field by field: the structs contain padding bytes whose content the caller does not control.
+// Writes the key of a call (the exact bytes of every argument that shapes its launches) field by field: the structs contain
+// padding bytes whose content the caller does not control.
 struct KeyWriter {
   std::string& key;
   void put(const void* ptr, size_t n) { key.append((const char*)ptr, n); }
@@ -45,7 +45,7 @@ struct KeyWriter {
     val(q.score_inv_scale); val(q.prepared); val(q.byte_codes);
   }
 };
-constexpr size_t MAX_BACKBONE_GRAPHS = 16, MAX_BLOCK_GRAPHS = 8, MAX_BLOCK_KEYS = 8;
+constexpr size_t MAX_BACKBONE_GRAPHS = 16, MAX_BLOCK_GRAPHS = 8;     // kept, and calls remembered (see graph_cache.h)
 struct mixaq_ctx {
   int device;
   int* d_status;
@@ -62,10 +62,8 @@ struct mixaq_ctx {
   cudaStream_t capture_stream;         // forwards on a stream that cannot be captured (the legacy default one) are recorded here
   cudaStream_t side_stream; cudaEvent_t fork, join;   // output norms run beside the next stage inside a captured forward
   std::mutex graph_lock;               // for what follows and the two streams above
-  std::vector<GraphEntry> graphs;      // of backbone forwards
-  std::vector<GraphEntry> block_graphs;
-  std::vector<std::string> block_keys; // block calls seen once, the oldest first
-  long block_captures, block_replays;
+  GraphCache<cudaGraphExec_t> graphs{MAX_BACKBONE_GRAPHS, MAX_BACKBONE_GRAPHS};      // of backbone forwards
+  GraphCache<cudaGraphExec_t> block_graphs{MAX_BLOCK_GRAPHS, MAX_BLOCK_GRAPHS};
   std::vector<ProfRec> prof;          // event pairs recorded since mixaq_profile_begin
   std::vector<cudaEvent_t> pool;      // events ready for reuse
 };
@@ -331,7 +329,7 @@ mixaq_status mixaq_create(mixaq_ctx** out, int device) {
   if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return MIXAQ_CUDA_ERROR; }
   mixaq_ctx* c = new (std::nothrow) mixaq_ctx();
   if (!c) return MIXAQ_INTERNAL;
-  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr; c->side_stream = nullptr; c->fork = c->join = nullptr; c->block_captures = c->block_replays = 0;
+  c->device = device; c->launches = 0; c->err[0] = 0; c->d_status = nullptr; c->profiling = false; c->graph_cache = true; c->allow_elevation = false; c->reverse_selection = false; c->nvtx = false; c->prof_capture = false; c->guards = false; c->capture_stream = nullptr; c->side_stream = nullptr; c->fork = c->join = nullptr;
   if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess || cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess ||
       !gemm_init() || !ln_init()) {
     cudaGetLastError(); if (c->d_status) cudaFree(c->d_status); delete c; return MIXAQ_CUDA_ERROR;
@@ -345,8 +343,8 @@ mixaq_status mixaq_destroy(mixaq_ctx* ctx) {
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
   if (ctx->side_stream) { cudaStreamDestroy(ctx->side_stream); cudaEventDestroy(ctx->fork); cudaEventDestroy(ctx->join); }
-  for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
-  for (auto& g : ctx->block_graphs) cudaGraphExecDestroy(g.exec);
+  ctx->graphs.clear(cudaGraphExecDestroy);
+  ctx->block_graphs.clear(cudaGraphExecDestroy);
   for (cudaGraphExec_t g : ctx->prof_execs) cudaGraphExecDestroy(g);
   for (auto& r : ctx->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
   for (auto e : ctx->pool) cudaEventDestroy(e);
@@ -654,6 +652,56 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   return check_cuda(ctx, "block_forward");
 }
 
+// ---- graphs of whole calls ---------------------------------------------------------------------------------------------
+// the legacy default stream cannot be captured itself
+static bool is_legacy(cudaStream_t st) { return st == nullptr || st == cudaStreamLegacy; }
+static bool caller_is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (is_legacy(st) || (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)) return false;
+  cudaGetLastError();
+  return true;
+}
+// The call `forward(stream, recording)` with this key: replayed when it was recorded before, recorded (and launched) when
+// that is worth it, else issued on the caller's stream.  What a call costs (us, Swin-T forwards on the default stream,
+// waited for one by one; 224 x 224 image / 800 x 1333 map): 473 / 902 replayed, 514 / 939 issued, 1 026 / 1 341 recorded.
+// The caller holds graph_lock.
+template <class Forward>
+static mixaq_status replay_record_or_run(mixaq_ctx* ctx, GraphCache<cudaGraphExec_t>& cache, std::string&& key,
+                                         cudaStream_t user_stream, const char* what, Forward forward) {
+  if (const auto* g = cache.replay(key)) {
+    if (cudaGraphLaunch(g->exec, user_stream) != cudaSuccess) return check_cuda(ctx, what);
+    ctx->launches = g->launches;
+    return MIXAQ_OK;
+  }
+  bool record = cache.worth_recording(key);
+  if (record && is_legacy(user_stream) && !ctx->capture_stream &&
+      cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    ctx->capture_stream = nullptr; record = false;
+  }
+  const cudaStream_t st = is_legacy(user_stream) ? ctx->capture_stream : user_stream;
+  if (record && cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) record = false;
+  if (!record) {
+    cudaGetLastError();
+    const mixaq_status result = forward(user_stream, false);
+    if (result == MIXAQ_OK) cache.saw(std::move(key));
+    return result;
+  }
+  const mixaq_status result = forward(st, true);
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  const bool recorded = cudaStreamEndCapture(st, &graph) == cudaSuccess && graph && result == MIXAQ_OK &&
+                        cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
+  if (graph) cudaGraphDestroy(graph);
+  if (!recorded) {
+    cudaGetLastError();
+    cache.not_recorded(key);
+    return result != MIXAQ_OK ? result : forward(user_stream, false);
+  }
+  cache.recorded(std::move(key), exec, ctx->launches, cudaGraphExecDestroy);
+  if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, what);
+  return MIXAQ_OK;
+}
+
 extern "C" {
 
 mixaq_status mixaq_block_forward(mixaq_ctx* ctx, const mixaq_block_params* p, const float* x, float* y,
@@ -667,17 +715,10 @@ mixaq_status mixaq_block_forward(mixaq_ctx* ctx, const mixaq_block_params* p, co
                               taps, nullptr, st);
   };
   // A call repeated with the same arguments replays a graph: issuing its eleven launches and their tensor maps takes the
-  // host longer than a small block takes the GPU (C = 96 at 56 x 56: 55 us a call before, 41 now; C = 384 at 50 x 84 with
-  // pruning, bound by the GPU but for the gaps between stream launches: 78 and 69).  The buffers of a block call change from call to call more often than a
-  // backbone's, so a graph is recorded at the SECOND call with a key, and no further ones once they are not being replayed
-  // (recording costs the host about as much as ten calls).
+  // host longer than a small block takes the GPU (C = 96 at 56 x 56: 58 us a call without a replay, 40 with; C = 384 at
+  // 50 x 84 with pruning, bound by the GPU but for the gaps between stream launches: 72 and 66).
   if (!ctx || !p || taps || !ctx->graph_cache || ctx->profiling || ctx->guards || ctx->nvtx) return forward(user_stream);
-  const bool legacy = user_stream == nullptr || user_stream == cudaStreamLegacy;   // cannot be captured itself
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (!legacy && (cudaStreamIsCapturing(user_stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) {
-    cudaGetLastError();
-    return forward(user_stream);
-  }
+  if (caller_is_capturing(user_stream)) return forward(user_stream);
   std::string key;
   key.reserve(1024);
   KeyWriter k{key};
@@ -692,51 +733,8 @@ mixaq_status mixaq_block_forward(mixaq_ctx* ctx, const mixaq_block_params* p, co
   }
   k.block(*p);
   std::lock_guard<std::mutex> lock(ctx->graph_lock);
-  for (auto& g : ctx->block_graphs)
-    if (g.key == key) {
-      if (cudaGraphLaunch(g.exec, user_stream) != cudaSuccess) return check_cuda(ctx, "block_forward (graph launch)");
-      ctx->launches = g.launches;
-      ++ctx->block_replays;
-      return MIXAQ_OK;
-    }
-  size_t at = 0;
-  while (at < ctx->block_keys.size() && ctx->block_keys[at] != key) ++at;
-  const bool seen = at < ctx->block_keys.size();
-  bool record = seen && ctx->block_captures <= (long)MAX_BLOCK_GRAPHS + ctx->block_replays / 32;
-  if (record && legacy && !ctx->capture_stream &&
-      cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    ctx->capture_stream = nullptr; record = false;
-  }
-  const cudaStream_t st = legacy ? ctx->capture_stream : user_stream;
-  if (record && cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) record = false;
-  if (!record) {
-    cudaGetLastError();
-    const mixaq_status result = forward(user_stream);
-    if (result == MIXAQ_OK && !seen) {
-      if (ctx->block_keys.size() >= MAX_BLOCK_KEYS) ctx->block_keys.erase(ctx->block_keys.begin());
-      ctx->block_keys.push_back(std::move(key));
-    }
-    return result;
-  }
-  const mixaq_status result = forward(st);
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  const bool recorded = cudaStreamEndCapture(st, &graph) == cudaSuccess && graph && result == MIXAQ_OK &&
-                        cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
-  if (graph) cudaGraphDestroy(graph);
-  ++ctx->block_captures;
-  if (!recorded) {
-    cudaGetLastError();
-    return result != MIXAQ_OK ? result : forward(user_stream);
-  }
-  ctx->block_keys.erase(ctx->block_keys.begin() + at);
-  if (ctx->block_graphs.size() >= MAX_BLOCK_GRAPHS) {
-    cudaGraphExecDestroy(ctx->block_graphs.front().exec);
-    ctx->block_graphs.erase(ctx->block_graphs.begin());
-  }
-  ctx->block_graphs.push_back({std::move(key), exec, ctx->launches});
-  if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, "block_forward (graph launch)");
-  return MIXAQ_OK;
+  return replay_record_or_run(ctx, ctx->block_graphs, std::move(key), user_stream, "block_forward (graph launch)",
+                              [&](cudaStream_t st, bool) { return forward(st); });
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -825,6 +823,139 @@ BackboneWs carve_backbone(const mixaq_backbone_params* p, int B, int H0, int W0,
 }
 }  // namespace
 
+// ---- the walk over a backbone -------------------------------------------------------------------------------------------
+namespace {
+// a validated backbone call; H0 x W0 is the token map of stage 1, Hi x Wi the size that the caller gave
+struct BackboneCall {
+  const mixaq_backbone_params* p;
+  const float* x0; float* const* stage_out;
+  int B, H0, W0, Hi, Wi;
+  const float *low, *prune;              // per pair; prune nullable
+  BackboneWs ws;
+};
+
+// Issues every launch of the call on `st`.  recording: the stream is being captured into a graph that will be kept.
+mixaq_status issue_backbone(mixaq_ctx* ctx, const BackboneCall& c, bool recording, cudaStream_t st) {
+  const mixaq_backbone_params* p = c.p;
+  const BackboneWs& ws = c.ws;
+  const int B = c.B;
+  const bool norms = p->out_norm_g && p->out_norm_b;
+  // Inside a recorded forward the output norms leave the chain: nothing waits for them but the end of the forward.
+  bool side = recording && norms;
+  if (side && !ctx->side_stream) {
+    if (cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess) { ctx->side_stream = nullptr; side = false; }
+    else if (cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) != cudaSuccess ||
+             cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming) != cudaSuccess) {
+      cudaStreamDestroy(ctx->side_stream); ctx->side_stream = nullptr; side = false;
+    }
+    if (!side) cudaGetLastError();
+  }
+  mixaq_status result = MIXAQ_OK;
+  int total = 0, H = c.H0, W = c.W0, blk = 0;
+  const float* cur = c.x0;
+  // while profiling: a few event pairs with nothing between them, so that what a bracket itself adds to every kernel's
+  // time can be read off the same record
+  if (ctx->profiling) for (int i = 0; i < 4; ++i) { PROF(PC_BRACKET); }
+  if (p->embed) {
+    // image -> token map of stage 1 (patch embedding), inside the same captured graph
+    result = mixaq_embed_forward(ctx, p->embed, c.x0, ws.tokens, B, c.Hi, c.Wi, ws.embed, ws.embed_bytes, st);
+    total += ctx->launches;
+    cur = ws.tokens;
+  }
+  for (int s = 0; s < p->num_stages && result == MIXAQ_OK; ++s) {
+    NvtxScope stage_range(ctx, "stage", s + 1);
+    const int d = p->depths[s];
+    // with output norms the un-normalised map stays in the workspace (the next stage reads it) and the caller's
+    // buffer receives its LayerNorm
+    float* out_s = norms ? ws.raw[s] : c.stage_out[s];
+    if (s > 0) {
+      // the merge writes where the first block of the stage does NOT write
+      float* mdst = (d % 2 == 0) ? out_s : ws.scratch;
+      result = mixaq_merge_forward(ctx, &p->merges[s - 1], cur, mdst, B, H, W, ws.merge, ws.merge_bytes, st);
+      if (result != MIXAQ_OK) break;
+      total += ctx->launches;
+      cur = mdst; H = (H + 1) / 2; W = (W + 1) / 2;
+    }
+    // importance is scored once per stage, before its first block (Section 3.2): one energy map, and from it the
+    // window classes and batch bookkeeping of EVERY block of the stage (own shift, own pair's ratios) in one go
+    const mixaq_block_params* b0 = &p->blocks[blk];
+    { PROF(PC_ENERGY); launch_energy(cur, ws.energy, (long)B * H * W, b0->dim, b0->score_inv_scale, st); }
+    total += 1;
+    const size_t sel_stride = carve_sel(B, H, W, nullptr).bytes;
+    std::vector<SelWs> sels(d);
+    std::vector<SelectArgs> sargs(d);
+    // Windows keep their precision class within a stage (Section 4.4, "Windows Elevation"): unless elevation is
+    // allowed, a pair's effective ratios are the largest ratios of the stage's pairs so far.
+    std::vector<float> lr_eff(d), pr_eff(d);
+    float lmax = 0.f, pmax = 0.f;
+    for (int i = 0; i < d; ++i) {
+      float lr = c.low[(blk + i) / 2], pr = c.prune ? c.prune[(blk + i) / 2] : 0.f;
+      if (!ctx->allow_elevation) { lmax = std::max(lmax, lr); pmax = std::max(pmax, pr); lr = lmax; pr = pmax; }
+      lr_eff[i] = lr; pr_eff[i] = pr;
+    }
+    for (int i = 0; i < d; ++i) {
+      const float lr = lr_eff[i], pr = pr_eff[i];
+      Geometry g = geometry(H, W, lr, pr);
+      if ((size_t)g.nW * 8 > 48 * 1024) { result = fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "too many windows per image (max 6144)"); break; }
+      sels[i] = carve_sel(B, H, W, ws.sel + (size_t)i * sel_stride);
+      sargs[i] = make_select_args(sels[i], ws.energy, B, H, W, p->blocks[blk + i].shift, g, ctx->reverse_selection ? 1 : 0);
+    }
+    if (result != MIXAQ_OK) break;
+    g_launches = 0;
+    { PROF(PC_SELECT); launch_select(sargs.data(), d, st); }
+    total += g_launches;
+    for (int i = 0; i < d; ++i, ++blk) {
+      float* dst = ((d - 1 - i) % 2 == 0) ? out_s : ws.scratch;
+      NvtxScope block_range(ctx, "block", blk);
+      result = block_forward_impl(ctx, &p->blocks[blk], cur, dst, B, H, W, lr_eff[i], pr_eff[i], nullptr, nullptr,
+                                  ws.block, ws.block_bytes, nullptr, &sels[i], st);
+      if (result != MIXAQ_OK) break;
+      total += ctx->launches;
+      cur = dst;
+    }
+    if (result == MIXAQ_OK && norms) {
+      PROF(PC_OUT_NORM);
+      g_launches = 0;
+      if (side) { cudaEventRecord(ctx->fork, st); cudaStreamWaitEvent(ctx->side_stream, ctx->fork, 0); }
+      if (!launch_bias_ln(out_s, nullptr, p->out_norm_g[s], p->out_norm_b[s], c.stage_out[s], (long)B * H * W, b0->dim,
+                          side ? ctx->side_stream : st))
+        result = fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "output norm: unsupported width");
+      total += g_launches;
+    }
+  }
+  if (side) { cudaEventRecord(ctx->join, ctx->side_stream); cudaStreamWaitEvent(st, ctx->join, 0); }
+  if (result != MIXAQ_OK) return result;
+  ctx->launches = total;
+  return check_cuda(ctx, "backbone_forward");
+}
+
+// A profiled forward on a capturable stream is captured too, with the event records around its kernels as graph nodes,
+// launched once and not kept: the kernels are then timed as they run inside a graph, not with a stream launch between the
+// events.  On the legacy stream the launches are profiled as they are.
+mixaq_status profile_backbone(mixaq_ctx* ctx, const BackboneCall& c, cudaStream_t st) {
+  if (is_legacy(st) || cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    cudaGetLastError();
+    return issue_backbone(ctx, c, false, st);
+  }
+  ctx->prof_capture = true;
+  const mixaq_status result = issue_backbone(ctx, c, false, st);
+  ctx->prof_capture = false;
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  const cudaError_t e = cudaStreamEndCapture(st, &graph);
+  if (result != MIXAQ_OK) { if (graph) cudaGraphDestroy(graph); cudaGetLastError(); return result; }
+  if (e != cudaSuccess || !graph || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
+    if (graph) cudaGraphDestroy(graph);
+    return check_cuda(ctx, "backbone_forward (graph capture)") == MIXAQ_OK
+               ? fail(ctx, MIXAQ_CUDA_ERROR, "backbone_forward: graph capture failed") : MIXAQ_CUDA_ERROR;
+  }
+  cudaGraphDestroy(graph);
+  ctx->prof_execs.push_back(exec);
+  if (cudaGraphLaunch(exec, st) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
+  return MIXAQ_OK;
+}
+}  // namespace
+
 size_t mixaq_backbone_workspace_bytes(const mixaq_backbone_params* p, int B, int H0, int W0) {
   if (!p || !p->depths || !p->blocks || p->num_stages <= 0 || p->num_stages > 16 || B <= 0 || H0 <= 0 || W0 <= 0) return 0;
   if (p->num_stages > 1 && !p->merges) return 0;
@@ -869,177 +1000,39 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
   }
   BackboneWs ws = carve_backbone(p, B, H0, W0, Hi, Wi, workspace);
   if (ws.bytes > workspace_bytes) return fail(ctx, MIXAQ_WORKSPACE_TOO_SMALL, "backbone workspace too small");
-  cudaStream_t st = (cudaStream_t)cuda_stream;
+  const BackboneCall call = {p, x0, stage_out, B, H0, W0, Hi, Wi, low_ratio_per_pair, prune_ratio_per_pair, ws};
+  const cudaStream_t user_stream = (cudaStream_t)cuda_stream;
+  if (!ctx->graph_cache) return issue_backbone(ctx, call, false, user_stream);
+  std::lock_guard<std::mutex> lock(ctx->graph_lock);
+  if (caller_is_capturing(user_stream)) return issue_backbone(ctx, call, false, user_stream);
+  if (ctx->profiling) return profile_backbone(ctx, call, user_stream);
 
-  // Replay as a CUDA graph when an identical call was captured before.  The key is made of every value that
-  // shapes the launches: the fields of the HOST parameter structs, ratios, pointers, sizes and the stream.
-  bool use_graph = ctx->graph_cache;
-  std::unique_lock<std::mutex> lock(ctx->graph_lock, std::defer_lock);
-  if (use_graph) lock.lock();
-  // The legacy default stream cannot be captured, but a graph can be launched on it: such calls are recorded on a stream
-  // of the context's own (stage1_pair and Swin-T calls on it were bound by one host launch per kernel).
-  const cudaStream_t user_stream = st;
-  if (use_graph && (st == nullptr || st == cudaStreamLegacy)) {
-    if (ctx->profiling) use_graph = false;       // profiled as stream launches
-    else if (!ctx->capture_stream && cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaGetLastError(); ctx->capture_stream = nullptr; use_graph = false;
-    } else st = ctx->capture_stream;
-  }
-  if (use_graph && user_stream == st) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) { cudaGetLastError(); use_graph = false; }
-  }
-  // A profiled forward is captured too, with the event records around its kernels as graph nodes, launched once and
-  // not cached: the kernels are then timed as they run inside a graph, not with a stream launch between the events.
-  const bool prof_graph = use_graph && ctx->profiling;
   std::string key;
-  if (prof_graph) {
-    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); use_graph = false; }
-    else ctx->prof_capture = true;
-  } else if (use_graph) {
-    KeyWriter k{key};
-    auto put = [&k](const void* ptr, size_t n) { k.put(ptr, n); };
-    const int npairs = (nblk + 1) / 2;
-    put(&p->num_stages, sizeof(int)); put(p->depths, sizeof(int) * p->num_stages);
-    for (int b = 0; b < nblk; ++b) k.block(p->blocks[b]);
-    for (int m = 0; m + 1 < p->num_stages; ++m) {
-      const mixaq_merge_params& q = p->merges[m];
-      put(&q.ln_g, sizeof(q.ln_g)); put(&q.ln_b, sizeof(q.ln_b)); k.aq(q.in); k.linear(q.reduction);
-      put(&q.prepared, sizeof(q.prepared));
-    }
-    const char has_embed = p->embed ? 1 : 0, has_norms = norms ? 1 : 0;
-    put(&has_embed, 1); put(&has_norms, 1);
-    if (p->embed) {
-      const mixaq_embed_params& q = *p->embed;
-      put(&q.ln_g, sizeof(q.ln_g)); put(&q.ln_b, sizeof(q.ln_b)); put(&q.bias, sizeof(q.bias)); k.aq(q.in); k.linear(q.proj);
-      put(&q.prepared, sizeof(q.prepared));
-    }
-    if (norms) { put(p->out_norm_g, sizeof(float*) * p->num_stages); put(p->out_norm_b, sizeof(float*) * p->num_stages); }
-    put(&x0, sizeof(x0)); put(stage_out, sizeof(float*) * p->num_stages);
-    const int dims[5] = {B, H0, W0, Hi, Wi}; put(dims, sizeof(dims));
-    put(low_ratio_per_pair, sizeof(float) * npairs);
-    const char has_prune = prune_ratio_per_pair ? 1 : 0; put(&has_prune, 1);
-    if (prune_ratio_per_pair) put(prune_ratio_per_pair, sizeof(float) * npairs);
-    put(&workspace, sizeof(workspace)); put(&workspace_bytes, sizeof(workspace_bytes)); put(&user_stream, sizeof(user_stream));
-    const char elev = (ctx->allow_elevation ? 1 : 0) | (ctx->reverse_selection ? 2 : 0); put(&elev, 1);
-    for (auto& g : ctx->graphs)
-      if (g.key == key) {
-        if (cudaGraphLaunch(g.exec, user_stream) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
-        ctx->launches = g.launches;
-        return MIXAQ_OK;
-      }
-    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); use_graph = false; }
+  KeyWriter k{key};
+  const int npairs = (nblk + 1) / 2;
+  // what changes from call to call comes first: two keys that differ are then told apart by their first bytes
+  k.val(x0); k.put(stage_out, sizeof(float*) * p->num_stages);
+  k.val(workspace); k.val(workspace_bytes); k.val(user_stream);
+  const int dims[5] = {B, H0, W0, Hi, Wi};
+  k.put(dims, sizeof(dims));
+  k.put(low_ratio_per_pair, sizeof(float) * npairs);
+  const char flags = (p->embed ? 1 : 0) | (norms ? 2 : 0) | (prune_ratio_per_pair ? 4 : 0) | (ctx->allow_elevation ? 8 : 0) |
+                     (ctx->reverse_selection ? 16 : 0);
+  k.val(flags);
+  if (prune_ratio_per_pair) k.put(prune_ratio_per_pair, sizeof(float) * npairs);
+  k.val(p->num_stages); k.put(p->depths, sizeof(int) * p->num_stages);
+  for (int b = 0; b < nblk; ++b) k.block(p->blocks[b]);
+  for (int m = 0; m + 1 < p->num_stages; ++m) {
+    const mixaq_merge_params& q = p->merges[m];
+    k.val(q.ln_g); k.val(q.ln_b); k.aq(q.in); k.linear(q.reduction); k.val(q.prepared);
   }
-  if (!use_graph) st = user_stream;
-
-  // Inside a captured forward the output norms leave the chain: nothing waits for them but the end of the forward.
-  bool side = use_graph && !prof_graph && norms;
-  if (side && !ctx->side_stream) {
-    if (cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess) { ctx->side_stream = nullptr; side = false; }
-    else if (cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) != cudaSuccess ||
-             cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming) != cudaSuccess) {
-      cudaStreamDestroy(ctx->side_stream); ctx->side_stream = nullptr; side = false;
-    }
-    if (!side) cudaGetLastError();
-  }
-
-  mixaq_status result = MIXAQ_OK;
-  int total = 0, H = H0, W = W0, blk = 0;
-  const float* cur = x0;
-  // while profiling: a few event pairs with nothing between them, so that what a bracket itself adds to every kernel's
-  // time can be read off the same record
-  if (ctx->profiling) for (int i = 0; i < 4; ++i) { PROF(PC_BRACKET); }
   if (p->embed) {
-    // image -> token map of stage 1 (patch embedding), inside the same captured graph
-    result = mixaq_embed_forward(ctx, p->embed, x0, ws.tokens, B, Hi, Wi, ws.embed, ws.embed_bytes, st);
-    total += ctx->launches;
-    cur = ws.tokens;
+    const mixaq_embed_params& q = *p->embed;
+    k.val(q.ln_g); k.val(q.ln_b); k.val(q.bias); k.aq(q.in); k.linear(q.proj); k.val(q.prepared);
   }
-  for (int s = 0; s < p->num_stages && result == MIXAQ_OK; ++s) {
-    NvtxScope stage_range(ctx, "stage", s + 1);
-    const int d = p->depths[s];
-    // with output norms the un-normalised map stays in the workspace (the next stage reads it) and the caller's
-    // buffer receives its LayerNorm
-    float* out_s = norms ? ws.raw[s] : stage_out[s];
-    if (s > 0) {
-      // the merge writes where the first block of the stage does NOT write
-      float* mdst = (d % 2 == 0) ? out_s : ws.scratch;
-      result = mixaq_merge_forward(ctx, &p->merges[s - 1], cur, mdst, B, H, W, ws.merge, ws.merge_bytes, st);
-      if (result != MIXAQ_OK) break;
-      total += ctx->launches;
-      cur = mdst; H = (H + 1) / 2; W = (W + 1) / 2;
-    }
-    // importance is scored once per stage, before its first block (Section 3.2): one energy map, and from it the
-    // window classes and batch bookkeeping of EVERY block of the stage (own shift, own pair's ratios) in one go
-    const mixaq_block_params* b0 = &p->blocks[blk];
-    { PROF(PC_ENERGY); launch_energy(cur, ws.energy, (long)B * H * W, b0->dim, b0->score_inv_scale, st); }
-    total += 1;
-    const size_t sel_stride = carve_sel(B, H, W, nullptr).bytes;
-    std::vector<SelWs> sels(d);
-    std::vector<SelectArgs> sargs(d);
-    // Windows keep their precision class within a stage (Section 4.4, "Windows Elevation"): unless elevation is
-    // allowed, a pair's effective ratios are the largest ratios of the stage's pairs so far.
-    std::vector<float> lr_eff(d), pr_eff(d);
-    float lmax = 0.f, pmax = 0.f;
-    for (int i = 0; i < d; ++i) {
-      float lr = low_ratio_per_pair[(blk + i) / 2], pr = prune_ratio_per_pair ? prune_ratio_per_pair[(blk + i) / 2] : 0.f;
-      if (!ctx->allow_elevation) { lmax = std::max(lmax, lr); pmax = std::max(pmax, pr); lr = lmax; pr = pmax; }
-      lr_eff[i] = lr; pr_eff[i] = pr;
-    }
-    for (int i = 0; i < d; ++i) {
-      const float lr = lr_eff[i], pr = pr_eff[i];
-      Geometry g = geometry(H, W, lr, pr);
-      if ((size_t)g.nW * 8 > 48 * 1024) { result = fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "too many windows per image (max 6144)"); break; }
-      sels[i] = carve_sel(B, H, W, ws.sel + (size_t)i * sel_stride);
-      sargs[i] = make_select_args(sels[i], ws.energy, B, H, W, p->blocks[blk + i].shift, g, ctx->reverse_selection ? 1 : 0);
-    }
-    if (result != MIXAQ_OK) break;
-    g_launches = 0;
-    { PROF(PC_SELECT); launch_select(sargs.data(), d, st); }
-    total += g_launches;
-    for (int i = 0; i < d; ++i, ++blk) {
-      float* dst = ((d - 1 - i) % 2 == 0) ? out_s : ws.scratch;
-      NvtxScope block_range(ctx, "block", blk);
-      result = block_forward_impl(ctx, &p->blocks[blk], cur, dst, B, H, W, lr_eff[i], pr_eff[i], nullptr, nullptr,
-                                  ws.block, ws.block_bytes, nullptr, &sels[i], st);
-      if (result != MIXAQ_OK) break;
-      total += ctx->launches;
-      cur = dst;
-    }
-    if (result == MIXAQ_OK && norms) {
-      PROF(PC_OUT_NORM);
-      g_launches = 0;
-      if (side) { cudaEventRecord(ctx->fork, st); cudaStreamWaitEvent(ctx->side_stream, ctx->fork, 0); }
-      if (!launch_bias_ln(out_s, nullptr, p->out_norm_g[s], p->out_norm_b[s], stage_out[s], (long)B * H * W, b0->dim,
-                          side ? ctx->side_stream : st))
-        result = fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "output norm: unsupported width");
-      total += g_launches;
-    }
-  }
-  if (side) { cudaEventRecord(ctx->join, ctx->side_stream); cudaStreamWaitEvent(st, ctx->join, 0); }
-  if (use_graph) {
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamEndCapture(st, &graph);
-    ctx->prof_capture = false;
-    if (result != MIXAQ_OK) { if (graph) cudaGraphDestroy(graph); cudaGetLastError(); return result; }
-    cudaGraphExec_t exec = nullptr;
-    if (e != cudaSuccess || !graph || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      return check_cuda(ctx, "backbone_forward (graph capture)") == MIXAQ_OK
-                 ? fail(ctx, MIXAQ_CUDA_ERROR, "backbone_forward: graph capture failed") : MIXAQ_CUDA_ERROR;
-    }
-    cudaGraphDestroy(graph);
-    if (prof_graph && ctx->profiling) {
-      ctx->prof_execs.push_back(exec);
-    } else {
-      if (ctx->graphs.size() >= MAX_BACKBONE_GRAPHS) { cudaGraphExecDestroy(ctx->graphs.front().exec); ctx->graphs.erase(ctx->graphs.begin()); }
-      ctx->graphs.push_back({key, exec, total});
-    }
-    if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, "backbone_forward (graph launch)");
-  }
-  if (result != MIXAQ_OK) return result;
-  ctx->launches = total;
-  return check_cuda(ctx, "backbone_forward");
+  if (norms) { k.put(p->out_norm_g, sizeof(float*) * p->num_stages); k.put(p->out_norm_b, sizeof(float*) * p->num_stages); }
+  return replay_record_or_run(ctx, ctx->graphs, std::move(key), user_stream, "backbone_forward (graph launch)",
+                              [&](cudaStream_t st, bool recording) { return issue_backbone(ctx, call, recording, st); });
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -1179,11 +1172,8 @@ mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled) {
   std::lock_guard<std::mutex> lock(ctx->graph_lock);
   ctx->graph_cache = enabled != 0;
   if (!enabled) {
-    for (auto* cache : {&ctx->graphs, &ctx->block_graphs}) {
-      for (auto& g : *cache) cudaGraphExecDestroy(g.exec);
-      cache->clear();
-    }
-    ctx->block_keys.clear();
+    ctx->graphs.clear(cudaGraphExecDestroy);
+    ctx->block_graphs.clear(cudaGraphExecDestroy);
   }
   return MIXAQ_OK;
 }

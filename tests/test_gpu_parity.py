@@ -202,7 +202,7 @@ def test_backbone_tiny(orc, mq, ctx, prune):
 
 
 def test_backbone_graph_replay_reads_fresh_data(orc, mq, ctx):
-    """On a capturable stream the backbone call is captured once and replayed; replays must see new input data."""
+    """Repeated backbone calls are recorded once and replayed; replays must see new input data."""
     wl = synth.tiny_backbone(ratio=0.4, prune=0.2)
     dbb = mq.DeviceBackbone(ctx, wl.backbone, wl.B, wl.H, wl.W)
     xs = [wl.x, np.ascontiguousarray(wl.x[:, ::-1]), (wl.x * F32(0.5)).astype(F32)]
@@ -210,7 +210,7 @@ def test_backbone_graph_replay_reads_fresh_data(orc, mq, ctx):
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(side):
-        for i, x in enumerate(xs):                                # call 0 captures, calls 1 and 2 replay
+        for i, x in enumerate(xs):                                # issued, recorded, replayed
             xd.copy_(torch.from_numpy(x), non_blocking=False)
             got = mq.backbone_forward(ctx, dbb, xd, wl.low_ratios, wl.prune_ratios)
             side.synchronize()
@@ -233,11 +233,11 @@ def test_precision_classes_within_a_stage_and_the_elevation_switch(orc, mq):
         for allow in (False, True):
             c.set_window_elevation(allow)
             want = orc.backbone_forward(bb, x, ratios, prunes, allow_elevation=allow)[0]
-            got = mq.backbone_forward(c, dbb, dev(x), ratios, prunes)[0].cpu().numpy()       # default stream: direct launches
+            got = mq.backbone_forward(c, dbb, dev(x), ratios, prunes)[0].cpu().numpy()       # default stream, new buffer: issued
             assert np.array_equal(got, want), f"allow={allow}"
             with torch.cuda.stream(side):
                 xd = dev(x)
-                for _ in range(2):                                                             # capture, then replay
+                for _ in range(2):                                                             # issued, then recorded
                     got = mq.backbone_forward(c, dbb, xd, ratios, prunes)[0]
                 side.synchronize()
                 assert np.array_equal(got.cpu().numpy(), want), f"graph, allow={allow}"
@@ -274,8 +274,8 @@ def test_config2_stage1_pair_full_size(orc, mq, ctx):
 
 
 def _full_backbone_case(orc, mq, ctx, wl):
-    """Whole backbone at a benchmark configuration's full size, launched the way bench.py launches it (own stream, so
-    the second call replays the captured graph); every stage map against the oracle."""
+    """Whole backbone at a benchmark configuration's full size, launched the way bench.py launches it (own stream; the
+    second call runs as a recorded graph); every stage map against the oracle."""
     want = orc.backbone_forward(wl.backbone, wl.x, wl.low_ratios, wl.prune_ratios)
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
@@ -358,7 +358,7 @@ def test_image_to_normed_stage_maps_end_to_end(orc, mq, ctx):
 
 def test_image_to_normed_stage_maps_in_one_backbone_call(orc, mq, ctx):
     """The same chain through ONE mixaq_backbone_forward call (stem and output norms given in the backbone parameters),
-    on a capturable stream: first call captures the graph, second replays it."""
+    on a capturable stream: the first call issues its kernels, the second runs as a recorded graph."""
     wl = synth.tiny_backbone(ratio=0.4, prune=0.2)
     rng = np.random.default_rng(13)
     e = synth.make_embed(rng, wl.backbone.dims[0])

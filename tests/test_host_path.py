@@ -1,0 +1,165 @@
+"""The host side of the library (csrc/mixaq.cu) against a stand-in for the CUDA runtime and the kernel launchers
+(host_path/): which calls are recorded as graphs and replayed, and what happens when a call fails."""
+import ctypes as C
+import os
+import subprocess
+import threading
+
+import numpy as np
+import pytest
+
+from paper_2507_19131_b200 import binding as mq
+from paper_2507_19131_b200 import build as mq_build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+
+
+class Counts(C.Structure):
+    _fields_ = [(n, C.c_long) for n in ("captures", "instantiated", "live_graphs", "graph_launches", "direct", "captured",
+                                        "side_launches", "copies", "guard_launches", "violations")]
+
+
+class SelectArgs(C.Structure):
+    _fields_ = [(n, C.c_void_p) for n in ("energy", "score", "order", "cls", "rowsrc_hi", "rowsrc_lo", "rowsrc_pr", "win_hi", "win_lo")] + \
+               [(n, C.c_int) for n in ("B", "H", "W", "shift", "nwx", "nW", "n_hi", "n_lo", "n_pr", "reverse")]
+
+
+class Copy(C.Structure):
+    _fields_ = [("dst", C.c_void_p), ("src", C.c_void_p), ("bytes", C.c_size_t)]
+
+
+@pytest.fixture(scope="module")
+def L(tmp_path_factory):
+    if not os.path.exists(NVCC):
+        pytest.skip("no nvcc")
+    out = str(tmp_path_factory.mktemp("host_path") / "libhost.so")
+    flags = [f for f in mq_build.NVCC_FLAGS if f not in ("-O3", "-lineinfo")]
+    fake = os.path.join(HERE, "host_path")
+    subprocess.check_call([NVCC] + flags + ["-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", out, os.path.join(mq_build.CSRC, "mixaq.cu"),
+                                            os.path.join(fake, "fake_launch.cu"), os.path.join(fake, "fake_runtime.cpp"), "-ldl"])
+    lib = C.CDLL(out)
+    lib.mixaq_last_error.restype = C.c_char_p
+    for n in ("mixaq_block_workspace_bytes", "mixaq_backbone_workspace_bytes"):
+        getattr(lib, n).restype = C.c_size_t
+    return lib
+
+
+class Host:
+    """A context of the library over the stand-in, with parameters at made-up addresses."""
+    OWN = C.c_void_p(0x10)                        # a stream of the caller's
+    DEFAULT = C.c_void_p(None)
+
+    def __init__(self, L):
+        self.L, self.h, self.next = L, C.c_void_p(), 0x7000_0000_0000
+        for flag in ("fail_capture", "fail_instantiate", "fail_graph_launch"):
+            self.set(flag, 0)
+        L.fake_reset()
+        assert L.mixaq_create(C.byref(self.h), 0) == 0
+        self.keep = []
+
+    def set(self, flag, value):
+        C.c_int.in_dll(self.L, flag).value = value
+
+    @property
+    def counts(self):
+        return Counts.in_dll(self.L, "counts")
+
+    def addr(self, offset=0):
+        self.next += 1 << 24
+        return self.next + offset
+
+    def linear(self, o, i):
+        return mq.LinearS(self.addr(), self.addr(), o, i, 8)
+
+    def block(self, dim=32, shift=0):
+        s = mq.BlockS()
+        s.dim, s.heads, s.window, s.shift, s.hidden = dim, dim // 32, 7, shift, 4 * dim
+        s.qkv, s.proj, s.fc1, s.fc2 = self.linear(3 * dim, dim), self.linear(dim, dim), self.linear(4 * dim, dim), self.linear(dim, 4 * dim)
+        s.relpos_table, s.prepared, s.score_inv_scale = self.addr(), self.addr(), 20.0
+        for br, bits in ((s.hi, 8), (s.lo, 4)):
+            for n in ("ln1_g", "ln1_b", "ln2_g", "ln2_b", "b_qkv", "b_proj", "b_fc1", "b_fc2"):
+                setattr(br, n, self.addr())
+            for n in ("qkv_in", "q", "k", "v", "proj_in", "fc1_in", "fc2_in"):
+                setattr(br, n, mq.AQ(bits, 0.1, 10.0, 3))
+            br.bits = bits
+        return s
+
+    def backbone(self, norms=False):
+        blocks = (mq.BlockS * 2)(self.block(), self.block(shift=3))
+        depths = (C.c_int * 1)(2)
+        s = mq.BackboneS(1, depths, blocks, None, None, None, None)
+        if norms:
+            s.out_norm_g = (C.c_void_p * 1)(self.addr())
+            s.out_norm_b = (C.c_void_p * 1)(self.addr())
+        ws = self.L.mixaq_backbone_workspace_bytes(C.byref(s), 1, 14, 14)
+        return dict(s=s, ws=C.c_void_p(self.addr()), ws_bytes=C.c_size_t(ws), out=(C.c_void_p * 1)(self.addr()))
+
+    def run_backbone(self, b, x, stream=None, low=0.5):
+        return self.L.mixaq_backbone_forward(self.h, C.byref(b["s"]), C.c_void_p(x), b["out"], 1, 14, 14, (C.c_float * 1)(low), None,
+                                             b["ws"], b["ws_bytes"], stream if stream is not None else self.DEFAULT)
+
+    def run_block(self, s, x, y, ws, stream=None, sel=None, energy=None):
+        n = C.c_size_t(self.L.mixaq_block_workspace_bytes(C.byref(s), 1, 14, 14))
+        return self.L.mixaq_block_forward(self.h, C.byref(s), C.c_void_p(x), C.c_void_p(y), 1, 14, 14, C.c_float(0.5), C.c_float(0.25),
+                                          C.byref(mq.SelectOpts(energy, 0)), C.byref(sel) if sel is not None else None,
+                                          C.c_void_p(ws), n, None, stream if stream is not None else self.DEFAULT)
+
+    def close(self):
+        assert self.L.mixaq_destroy(self.h) == 0
+
+
+@pytest.fixture
+def host(L):
+    h = Host(L)
+    yield h
+    assert h.counts.violations == 0
+    h.close()
+    assert h.counts.live_graphs == 0
+
+
+@pytest.mark.parametrize("stream", [Host.DEFAULT, Host.OWN])
+def test_backbone_calls_are_recorded_at_the_second_call_and_then_replayed(host, stream):
+    b, xs = host.backbone(), [host.addr() for _ in range(16)]
+    for step in range(4):
+        for x in xs:
+            assert host.run_backbone(b, x, stream) == 0
+        assert host.counts.captures == host.counts.instantiated == (0 if step == 0 else 16)
+        assert host.counts.graph_launches == 16 * step
+    assert host.L.mixaq_last_launch_count(host.h) > 10
+
+
+@pytest.mark.parametrize("stream", [Host.DEFAULT, Host.OWN])
+def test_backbone_calls_that_never_repeat_soon_are_never_recorded(host, stream):
+    """More input buffers in rotation than graphs are kept, and new ratios on every call."""
+    b, xs = host.backbone(), [host.addr() for _ in range(32)]
+    for i in range(4 * 32):
+        assert host.run_backbone(b, xs[i % 32], stream) == 0
+    for i in range(64):
+        assert host.run_backbone(b, xs[0], stream, low=i / 64) == 0
+    assert host.counts.captures == 0 and host.counts.graph_launches == 0
+
+
+def calls_in_pairs(host, kind, n):
+    """Runs n calls of distinct arguments, each twice in a row."""
+    b, s, ws = host.backbone(), host.block(), host.addr()
+    for _ in range(n):
+        x, y = host.addr(), host.addr()
+        for _ in range(2):
+            assert (host.run_backbone(b, x) if kind == "backbone" else host.run_block(s, x, y, ws)) == 0
+
+
+@pytest.mark.parametrize("kind,budget", [("backbone", 16), ("block", 8)])
+def test_recordings_that_are_not_replayed_stop_and_a_steady_caller_still_gets_its_graph(host, kind, budget):
+    calls_in_pairs(host, kind, 5 * budget)
+    assert host.counts.captures == budget and host.counts.live_graphs == budget
+    b, s, ws, x, y = host.backbone(), host.block(), host.addr(), host.addr(), host.addr()
+    for i in range(40):
+        assert (host.run_backbone(b, x) if kind == "backbone" else host.run_block(s, x, y, ws)) == 0
+    assert host.counts.captures == budget + 1 and host.counts.live_graphs == budget
+    assert host.counts.graph_launches == budget + 40 - 31          # the pairs' second calls; recorded at the 32nd call
+    # replays earn further recordings, one for every 32
+    for i in range(64):
+        assert (host.run_backbone(b, x) if kind == "backbone" else host.run_block(s, x, y, ws)) == 0
+    calls_in_pairs(host, kind, 1)
+    assert host.counts.captures == budget + 2
