@@ -17,8 +17,10 @@
  *     DEVICE pointer owned by the caller.  The library never frees them and keeps none past the call, with
  *     one exception: `prepared` buffers are read by every later forward call that gets the same params.
  *   - Alignment: feature maps, weight codes and LayerNorm parameters 16 bytes; workspaces and `prepared` buffers
- *     256 bytes (what cudaMalloc and the usual framework allocators give).  Anything less is refused with
- *     MIXAQ_INVALID_ARG before a launch.
+ *     256 bytes (what cudaMalloc and the usual framework allocators give); every other array of 32-bit elements 4 bytes.
+ *     Anything less is refused with MIXAQ_INVALID_ARG before a launch.  Exceptions: the selection outputs cls, order and
+ *     score and the taps of codes and of x1 may sit at any address (an order or score buffer that is not aligned to its
+ *     elements is filled by a copy).
  *   - Feature maps are [B][H][W][C] binary32, channels contiguous.  C must be a multiple of 32, C/heads
  *     must be 32, window must be 7, hidden must be a multiple of 32.
  *   - Calls are asynchronous on `cuda_stream` (a cudaStream_t passed as void*); they allocate no device memory and do

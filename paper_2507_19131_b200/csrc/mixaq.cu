@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <new>
 #include <string>
@@ -92,6 +93,10 @@ inline size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 // to the TMA unit (16-byte aligned base); workspaces and prepared buffers are carved in 256-byte steps.  A pointer
 // that breaks this would fault on the device, so it is refused on the host.
 inline bool aligned_to(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
+inline bool all_aligned_to(size_t a, std::initializer_list<const void*> ptrs) {
+  for (const void* p : ptrs) if (!aligned_to(p, a)) return false;
+  return true;
+}
 
 // Every buffer carved out of a workspace is followed by a guard zone of GUARD_BYTES that no kernel has a reason to
 // touch.  With mixaq_set_workspace_guards the zones are filled with a pattern before a forward and compared after it.
@@ -208,6 +213,10 @@ mixaq_status validate_block(mixaq_ctx* ctx, const mixaq_block_params* p, bool ne
                          p->hi.ln1_g, p->hi.ln1_b, p->hi.ln2_g, p->hi.ln2_b, p->lo.ln1_g, p->lo.ln1_b, p->lo.ln2_g, p->lo.ln2_b};
     for (const void* q : q16)
       if (!aligned_to(q, 16)) return fail(ctx, MIXAQ_INVALID_ARG, "weight codes and LayerNorm parameters must be 16-byte aligned");
+    const bool words = all_aligned_to(4, {p->qkv.scale, p->proj.scale, p->fc1.scale, p->fc2.scale, p->relpos_table,
+                                          p->hi.b_qkv, p->hi.b_proj, p->hi.b_fc1, p->hi.b_fc2,
+                                          p->lo.b_qkv, p->lo.b_proj, p->lo.b_fc1, p->lo.b_fc2});
+    if (!words) return fail(ctx, MIXAQ_INVALID_ARG, "step sizes, biases and the relative-position table must be 4-byte aligned");
     if (p->prepared && !aligned_to(p->prepared, 256)) return fail(ctx, MIXAQ_INVALID_ARG, "prepared buffer must be 256-byte aligned");
   }
   if (p->byte_codes != 0 && p->byte_codes != 1) return fail(ctx, MIXAQ_INVALID_ARG, "byte_codes must be 0 or 1");
@@ -479,6 +488,8 @@ size_t mixaq_merge_prepared_bytes(const mixaq_merge_params* p) {
 mixaq_status mixaq_merge_prepare(mixaq_ctx* ctx, const mixaq_merge_params* p, void* cuda_stream) {
   if (!ctx || !p) return MIXAQ_INVALID_ARG;
   if (!p->prepared || !p->reduction.codes || !p->reduction.scale) return fail(ctx, MIXAQ_INVALID_ARG, "merge params incomplete");
+  if (!all_aligned_to(4, {p->prepared, p->reduction.scale}))
+    return fail(ctx, MIXAQ_INVALID_ARG, "merge: step sizes and prepared must be 4-byte aligned");
   Carver c(p->prepared, false);
   float* mult = c.take<float>(p->reduction.out_features);
   int32_t* pre = c.take<int32_t>(p->reduction.out_features);
@@ -504,6 +515,17 @@ size_t mixaq_block_workspace_bytes(const mixaq_block_params* p, int B, int H, in
 
 }  // extern "C"
 
+// What the kernels read or write through the optional arguments, by whole 32-bit elements.  (cls, order, score and the taps
+// that are filled by copies may sit at any address.)
+static bool optional_buffers_aligned(const mixaq_select_opts* opts, const mixaq_selection* sel, const mixaq_taps* taps) {
+  bool ok = !opts || aligned_to(opts->energy, 4);
+  if (sel) ok &= all_aligned_to(4, {sel->idx_hi, sel->idx_lo, sel->idx_pr});
+  if (taps)
+    for (const mixaq_branch_taps* t : {&taps->hi, &taps->lo})
+      ok &= all_aligned_to(4, {t->qkv_acc, t->probs, t->pv_acc, t->proj_acc, t->fc1_acc, t->fc2_acc});
+  return ok;
+}
+
 // `presel`: selection buffers already filled for this block (the backbone selects once per stage); NULL: select here.
 static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params* p, const float* x, float* y,
                                        int B, int H, int W, float low_ratio, float prune_ratio,
@@ -515,6 +537,8 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   if (s != MIXAQ_OK) return s;
   if (!x || !y || x == y) return fail(ctx, MIXAQ_INVALID_ARG, "x / y NULL or aliased");
   if (!aligned_to(x, 16) || !aligned_to(y, 16)) return fail(ctx, MIXAQ_INVALID_ARG, "x and y must be 16-byte aligned");
+  if (!optional_buffers_aligned(opts, sel_out, taps))
+    return fail(ctx, MIXAQ_INVALID_ARG, "energy, window lists, accumulator taps and softmax taps must be 4-byte aligned");
   if (B <= 0 || H <= 0 || W <= 0) return fail(ctx, MIXAQ_INVALID_ARG, "B, H, W must be positive");
   if (!(low_ratio >= 0.f && low_ratio <= 1.f) || !(prune_ratio >= 0.f && prune_ratio <= 1.f))
     return fail(ctx, MIXAQ_INVALID_ARG, "ratios must lie in [0, 1]");
@@ -536,10 +560,12 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
 
   // 1. scores and selection
   SelWs sel = presel ? *presel : ws.sel;
-  if (sel_out && !presel) {                  // the selection kernels write the caller's buffers themselves
+  if (sel_out && !presel) {
+    // the selection kernels write the caller's buffers themselves, whole elements at a time; a buffer whose address does
+    // not allow that is filled by a copy
     if (sel_out->cls) sel.cls = sel_out->cls;
-    if (sel_out->order) sel.order = sel_out->order;
-    if (sel_out->score) sel.score = sel_out->score;
+    if (sel_out->order && aligned_to(sel_out->order, alignof(int32_t))) sel.order = sel_out->order;
+    if (sel_out->score && aligned_to(sel_out->score, alignof(int64_t))) sel.score = sel_out->score;
   }
   if (!presel) {
     const int32_t* energy = opts ? opts->energy : nullptr;
@@ -548,6 +574,9 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
     { PROF(PC_SELECT); launch_select(&sa, 1, st); }
   }
   if (sel_out) {
+    const size_t n = (size_t)B * g.nW;
+    if (sel_out->order && sel.order != sel_out->order) cudaMemcpyAsync(sel_out->order, sel.order, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
+    if (sel_out->score && sel.score != sel_out->score) cudaMemcpyAsync(sel_out->score, sel.score, n * sizeof(int64_t), cudaMemcpyDeviceToDevice, st);
     if (sel_out->idx_hi || sel_out->idx_lo || sel_out->idx_pr) {
       int32_t* const lists[3] = {sel_out->idx_hi, sel_out->idx_lo, sel_out->idx_pr};
       const int cnt[3] = {g.n_hi, g.n_lo, g.n_pr};
@@ -1062,6 +1091,8 @@ size_t mixaq_embed_prepared_bytes(const mixaq_embed_params* p) {
 mixaq_status mixaq_embed_prepare(mixaq_ctx* ctx, const mixaq_embed_params* p, void* cuda_stream) {
   if (!ctx) return MIXAQ_INVALID_ARG;
   if (!embed_ok(p) || !p->prepared) return fail(ctx, MIXAQ_INVALID_ARG, "embed params incomplete (8-bit input, [C0][48] projection, C0 % 32 == 0)");
+  if (!all_aligned_to(4, {p->prepared, p->proj.scale}))
+    return fail(ctx, MIXAQ_INVALID_ARG, "embed: step sizes and prepared must be 4-byte aligned");
   cudaStream_t st = (cudaStream_t)cuda_stream;
   EmbedPrepared pr = carve_embed(p, p->prepared);
   const int N = p->proj.out_features;
@@ -1255,6 +1286,8 @@ mixaq_status mixaq_calibrate_merge(mixaq_ctx* ctx, const mixaq_merge_params* p, 
   const int K = p->reduction.in_features, N = p->reduction.out_features, C = K / 4;
   if (K % 4 || N <= 0 || !merge_dim_supported(C)) return fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "calibrate_merge: unsupported dims");
   if (!p->ln_g || !p->ln_b || !p->reduction.codes || !p->reduction.scale) return fail(ctx, MIXAQ_INVALID_ARG, "merge params incomplete");
+  if (!all_aligned_to(4, {p->ln_g, p->ln_b, p->reduction.scale}))
+    return fail(ctx, MIXAQ_INVALID_ARG, "calibrate_merge: LayerNorm parameters and step sizes must be 4-byte aligned");
   if (mixaq_calibrate_merge_workspace_bytes(p, B, H, W) > workspace_bytes) return fail(ctx, MIXAQ_WORKSPACE_TOO_SMALL, "calibrate_merge workspace");
   cudaStream_t st = (cudaStream_t)cuda_stream;
   Carver cv(workspace);

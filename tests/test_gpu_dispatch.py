@@ -84,3 +84,29 @@ def test_calibration_products_by_weight_width(orc, mq, ctx, w_bits, H, W, dim):
     assert np.array_equal(y.cpu().numpy(), want_y)
     for site, span in want.items():
         assert got[site] == span, site
+
+
+@pytest.mark.parametrize("H,W", [(21, 22), (63, 71)])
+def test_selection_outputs_at_odd_addresses(orc, mq, ctx, H, W):
+    """Class, order and score buffers that are not aligned to their elements, with both selection routes (12 windows: one
+    launch, 99: two), issued and as a recorded graph: as from aligned ones."""
+    import ctypes as C
+    blk = synth.make_block(np.random.default_rng(H), 32, 1, 3, 8, 8, 4)
+    x = dev(synth.input_blobs(W, 1, H, W, 32, bg_std=0.5, gain=4.0))
+    db = mq.DeviceBlock(ctx, blk)
+    want = mq.block_forward(ctx, db, x, 0.4, 0.2, selection=True)
+    n, y, ws = want.cls.numel(), torch.empty_like(x), db.workspace(1, H, W)
+    raw = {name: torch.zeros(off + n * size + 64, dtype=torch.uint8, device="cuda")
+           for name, off, size in (("cls", 3, 1), ("order", 2, 4), ("score", 4, 8))}
+    sel = mq.Selection(raw["cls"].data_ptr() + 3, raw["order"].data_ptr() + 2, raw["score"].data_ptr() + 4, None, None, None)
+    for _ in range(3):
+        for t in raw.values():
+            t.fill_(0xEE)
+        ctx.check(mq.lib().mixaq_block_forward(ctx.h, C.byref(db.s), mq._ptr(x), mq._ptr(y), 1, H, W, C.c_float(0.4), C.c_float(0.2), None,
+                                               C.byref(sel), mq._ptr(ws), C.c_size_t(ws.numel()), None, mq._stream_ptr()))
+        for name, off, ref in (("cls", 3, want.cls), ("order", 2, want.order), ("score", 4, want.scores)):
+            got = raw[name].cpu().numpy()
+            end = off + ref.numel() * ref.element_size()
+            assert got[off:end].tobytes() == ref.cpu().numpy().tobytes(), name
+            assert (got[:off] == 0xEE).all() and (got[end:] == 0xEE).all(), name
+        assert torch.equal(y, want.y)

@@ -163,3 +163,34 @@ def test_recordings_that_are_not_replayed_stop_and_a_steady_caller_still_gets_it
         assert (host.run_backbone(b, x) if kind == "backbone" else host.run_block(s, x, y, ws)) == 0
     calls_in_pairs(host, kind, 1)
     assert host.counts.captures == budget + 2
+
+
+@pytest.mark.parametrize("off_cls,off_order,off_score", [(0, 0, 0), (1, 0, 4), (3, 2, 0), (1, 1, 1), (0, 4, 8)])
+def test_selection_outputs_at_any_address(host, off_cls, off_order, off_score):
+    """The kernels only get buffers that whole elements can be written to; the others are filled by copies."""
+    s, x, y, ws = host.block(), host.addr(), host.addr(), host.addr()
+    sel = mq.Selection(host.addr(off_cls), host.addr(off_order), host.addr(off_score), host.addr(), host.addr(), host.addr())
+    assert host.run_block(s, x, y, ws, sel=sel) == 0
+    args, copies = SelectArgs.in_dll(host.L, "last_select"), (Copy * 16).in_dll(host.L, "last_copies")
+    late = {c.dst: (c.src, c.bytes) for c in copies[:host.counts.copies]}
+    assert args.cls == sel.cls
+    for name, size in (("order", 4), ("score", 8)):
+        want, got = getattr(sel, name), getattr(args, name)
+        assert got % size == 0
+        assert got == want if want % size == 0 else late.pop(want) == (got, 4 * size)      # 4 windows of a 14 x 14 map
+    assert not late
+
+
+def test_misaligned_arrays_are_refused_before_a_launch(host):
+    x, y, ws = host.addr(), host.addr(), host.addr()
+    sel = lambda **kw: mq.Selection(**{n: host.addr() for n in ("cls", "order", "score", "idx_hi", "idx_lo", "idx_pr")} | kw)  # noqa: E731
+    for name in ("idx_hi", "idx_lo", "idx_pr"):
+        assert host.run_block(host.block(), x, y, ws, sel=sel(**{name: host.addr(2)})) == -1
+    assert host.run_block(host.block(), x, y, ws, energy=host.addr(1)) == -1
+    for setter in (lambda s: setattr(s.qkv, "scale", host.addr(2)), lambda s: setattr(s.lo, "b_fc1", host.addr(1)),
+                   lambda s: setattr(s, "relpos_table", host.addr(3))):
+        s = host.block()
+        setter(s)
+        assert host.run_block(s, x, y, ws) == -1
+    assert b"aligned" in host.L.mixaq_last_error(host.h)
+    assert host.counts.direct == 0
