@@ -75,6 +75,14 @@ extern "C" mixaq_status mixaq_merge_forward_static(mixaq_ctx* ctx, const mixaq_m
     ctx_note(ctx, "merge_forward_static: merge params incomplete", 0);
     return MIXAQ_INVALID_ARG;
   }
+  // as in mixaq_merge_forward: the kernels use 16-byte accesses and the TMA unit, `prepared` is carved in 256-byte steps
+  const void* const q16[] = {x, y, p->reduction.codes, p->ln_g, p->ln_b};
+  bool aligned = reinterpret_cast<uintptr_t>(p->prepared) % 256 == 0;
+  for (const void* q : q16) aligned &= reinterpret_cast<uintptr_t>(q) % 16 == 0;
+  if (!aligned) {
+    ctx_note(ctx, "merge_forward_static: x, y, weights and LayerNorm parameters must be 16-byte aligned, prepared 256-byte", 0);
+    return MIXAQ_INVALID_ARG;
+  }
   const size_t toks = (size_t)B * ((H + 1) / 2) * ((W + 1) / 2);
   const size_t need = toks * (size_t)K * bits / 8;
   if (need > (size_t)MIXAQ_STATIC_SCRATCH_BYTES || toks > (size_t)0x7fffffff) {

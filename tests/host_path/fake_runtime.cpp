@@ -43,6 +43,8 @@ void enqueue(cudaStream_t st) {
 // ---- the runtime calls that csrc/mixaq.cu makes ----
 extern "C" {
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaGetSymbolAddress(void** p, const void*) { *p = reinterpret_cast<void*>(0x5000'0000'0000); return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t) { std::lock_guard<std::mutex> g(lock); *p = handle<void*>(); return cudaSuccess; }
 cudaError_t cudaFree(void*) { return cudaSuccess; }
@@ -126,5 +128,6 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t st) {
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 char __cudaInitModule(void**) { return 1; }
 }

@@ -1,4 +1,4 @@
-"""The host side of the library (csrc/mixaq.cu) against a stand-in for the CUDA runtime and the kernel launchers
+"""The host side of the library (csrc/mixaq.cu, csrc/merge_static.cu) against a stand-in for the CUDA runtime and the kernel launchers
 (host_path/): which calls are recorded as graphs and replayed, and what happens when a call fails."""
 import ctypes as C
 import os
@@ -36,7 +36,7 @@ def L(tmp_path_factory):
     out = str(tmp_path_factory.mktemp("host_path") / "libhost.so")
     flags = [f for f in mq_build.NVCC_FLAGS if f not in ("-O3", "-lineinfo")]
     fake = os.path.join(HERE, "host_path")
-    subprocess.check_call([NVCC] + flags + ["-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", out, os.path.join(mq_build.CSRC, "mixaq.cu"),
+    subprocess.check_call([NVCC] + flags + ["-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", out, os.path.join(mq_build.CSRC, "mixaq.cu"), os.path.join(mq_build.CSRC, "merge_static.cu"),
                                             os.path.join(fake, "fake_launch.cu"), os.path.join(fake, "fake_runtime.cpp"), "-ldl"])
     lib = C.CDLL(out)
     lib.mixaq_last_error.restype = C.c_char_p
@@ -194,3 +194,17 @@ def test_misaligned_arrays_are_refused_before_a_launch(host):
         assert host.run_block(s, x, y, ws) == -1
     assert b"aligned" in host.L.mixaq_last_error(host.h)
     assert host.counts.direct == 0
+
+
+def test_patch_merging_refuses_misaligned_buffers_with_and_without_a_workspace(host):
+    def merge(**off):
+        at = lambda n: host.addr(off.get(n, 0))                                              # noqa: E731
+        m = mq.MergeS(at("ln_g"), at("ln_b"), mq.AQ(8, 0.1, 10.0, 3), host.linear(64, 128), at("prepared"))
+        m.reduction.codes = at("codes")
+        x, y = C.c_void_p(at("x")), C.c_void_p(at("y"))
+        return (host.L.mixaq_merge_forward(host.h, C.byref(m), x, y, 1, 8, 8, C.c_void_p(host.addr()), C.c_size_t(1 << 20), None),
+                host.L.mixaq_merge_forward_static(host.h, C.byref(m), x, y, 1, 8, 8, None))
+    for off in (dict(x=4), dict(y=8), dict(codes=1), dict(ln_g=4), dict(ln_b=4), dict(prepared=16)):
+        assert merge(**off) == (-1, -1), off
+    assert host.counts.direct == 0
+    assert merge() == (0, 0) and host.counts.direct == 4
