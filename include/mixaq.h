@@ -23,8 +23,10 @@
  *     elements is filled by a copy).
  *   - Feature maps are [B][H][W][C] binary32, channels contiguous.  C must be a multiple of 32, C/heads
  *     must be 32, window must be 7, hidden must be a multiple of 32.
- *   - Calls are asynchronous on `cuda_stream` (a cudaStream_t passed as void*); they allocate no device memory and do
- *     not synchronise.  Errors found on the host are returned before anything is launched.
+ *   - Calls are asynchronous on `cuda_stream` (a cudaStream_t passed as void*); they do not synchronise, and they need no
+ *     device memory beyond the caller's.  Block and backbone calls may record CUDA graphs, for which the driver takes some
+ *     (see mixaq_set_graph_cache); where it cannot, they issue their kernels.  Errors found on the host are returned
+ *     before anything is launched.
  *   - Activation codes are unsigned, `bits` in {8, 4, 2}.  Sub-byte codes are stored bit-packed, little end
  *     first: element e of a row lives in byte e*bits/8 at bit (e*bits) mod 8.
  *   - There is no CPU fallback: without a CUDA device every entry point returns MIXAQ_CUDA_ERROR.

@@ -691,7 +691,8 @@ static bool caller_is_capturing(cudaStream_t st) {
   return true;
 }
 // The call `forward(stream, recording)` with this key: replayed when it was recorded before, recorded (and launched) when
-// that is worth it, else issued on the caller's stream.  What a call costs (us, Swin-T forwards on the default stream,
+// that is worth it and works, else issued on the caller's stream: recording takes device memory, which a call does not
+// otherwise need, so that it fails is no reason for the call to fail.  What a call costs (us, Swin-T forwards on the default stream,
 // waited for one by one; 224 x 224 image / 800 x 1333 map): 473 / 902 replayed, 514 / 939 issued, 1 026 / 1 341 recorded.
 // The caller holds graph_lock.
 template <class Forward>
@@ -721,14 +722,16 @@ static mixaq_status replay_record_or_run(mixaq_ctx* ctx, GraphCache<cudaGraphExe
   const bool recorded = cudaStreamEndCapture(st, &graph) == cudaSuccess && graph && result == MIXAQ_OK &&
                         cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
   if (graph) cudaGraphDestroy(graph);
-  if (!recorded) {
-    cudaGetLastError();
-    cache.not_recorded(key);
-    return result != MIXAQ_OK ? result : forward(user_stream, false);
+  if (recorded) {
+    if (cudaGraphLaunch(exec, user_stream) == cudaSuccess) {
+      cache.recorded(std::move(key), exec, ctx->launches, cudaGraphExecDestroy);
+      return MIXAQ_OK;
+    }
+    cudaGraphExecDestroy(exec);
   }
-  cache.recorded(std::move(key), exec, ctx->launches, cudaGraphExecDestroy);
-  if (cudaGraphLaunch(exec, user_stream) != cudaSuccess) return check_cuda(ctx, what);
-  return MIXAQ_OK;
+  cudaGetLastError();
+  cache.not_recorded(key);
+  return forward(user_stream, false);
 }
 
 extern "C" {

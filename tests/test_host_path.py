@@ -208,3 +208,23 @@ def test_patch_merging_refuses_misaligned_buffers_with_and_without_a_workspace(h
         assert merge(**off) == (-1, -1), off
     assert host.counts.direct == 0
     assert merge() == (0, 0) and host.counts.direct == 4
+
+
+@pytest.mark.parametrize("kind", ["backbone", "block"])
+@pytest.mark.parametrize("stream", [Host.DEFAULT, Host.OWN])
+@pytest.mark.parametrize("flag", ["fail_capture", "fail_instantiate", "fail_graph_launch"])
+def test_a_call_that_cannot_be_recorded_is_issued(host, kind, stream, flag):
+    """No memory for a graph, or a stream that cannot be captured just now: the call does its work, and is recorded later."""
+    b, s, x, y, ws = host.backbone(norms=True), host.block(), host.addr(), host.addr(), host.addr()
+    call = lambda: host.run_backbone(b, x, stream) if kind == "backbone" else host.run_block(s, x, y, ws, stream)   # noqa: E731
+    assert call() == 0
+    launches = host.counts.direct
+    host.set(flag, 1)
+    for i in range(2, 5):
+        assert call() == 0
+        assert host.counts.direct == i * launches and host.L.mixaq_last_launch_count(host.h) == launches
+    assert host.counts.graph_launches == 0 and host.counts.live_graphs == 0
+    host.set(flag, 0)
+    for _ in range(3):
+        assert call() == 0
+    assert host.counts.live_graphs == 1 and host.counts.graph_launches > 0
