@@ -285,7 +285,7 @@ mixaq_status mixaq_set_reverse_selection(mixaq_ctx* ctx, int reverse);
  * a 256-byte guard zone (always; the *_workspace_bytes figures include them).  enabled = 1: mixaq_block_forward (also
  * as part of mixaq_backbone_forward) writes a pattern into the zones of the block's workspace before its first kernel
  * and compares them after its last; a difference raises the status word (MIXAQ_WORKSPACE_OVERRUN from
- * mixaq_last_device_status).  Two small launches per block; off by default. */
+ * mixaq_last_device_status).  Two small launches per block; calls neither record nor replay graphs meanwhile; off by default. */
 mixaq_status mixaq_set_workspace_guards(mixaq_ctx* ctx, int enabled);
 /* Self-test of that check on a caller's buffer (>= 2 KiB of device memory): two 256-byte buffers are carved out of
  * it, their guard zones filled, and, with overrun = 1, one byte just past the second buffer is written (inside the
@@ -294,8 +294,7 @@ mixaq_status mixaq_selftest_workspace_guards(mixaq_ctx* ctx, void* buffer, size_
 
 /* NVTX ranges for external tracers (off by default): every kernel family launched through this context is wrapped in
  * a host-side range named like its profiling category, and mixaq_backbone_forward adds one range per stage and per
- * block.  The ranges mark where the launches are ISSUED: a forward that replays a cached graph issues none, so trace
- * with the graph cache off (mixaq_set_graph_cache) to see them. */
+ * block.  The ranges mark where the launches are ISSUED; calls neither record nor replay graphs meanwhile. */
 mixaq_status mixaq_set_nvtx(mixaq_ctx* ctx, int enabled);
 
 /* Number of kernel launches the last block / merge / backbone call of this context issued. */

@@ -1038,6 +1038,8 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
   std::lock_guard<std::mutex> lock(ctx->graph_lock);
   if (caller_is_capturing(user_stream)) return issue_backbone(ctx, call, false, user_stream);
   if (ctx->profiling) return profile_backbone(ctx, call, user_stream);
+  // guard zones and NVTX ranges are asked for on the calls that follow: a graph recorded before does not have them
+  if (ctx->guards || ctx->nvtx) return issue_backbone(ctx, call, false, user_stream);
 
   std::string key;
   KeyWriter k{key};

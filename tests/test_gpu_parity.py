@@ -401,7 +401,7 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(orc, mq):
 
 def test_workspace_guard_zones(orc, mq):
     """The guard zones behind every workspace buffer: untouched by a forward (block with all taps, and a small
-    backbone through its graph), and the check itself reports a byte written just past a buffer."""
+    backbone), and the check itself reports a byte written just past a buffer."""
     c = mq.Context(0)
     try:
         c.set_workspace_guards(True)

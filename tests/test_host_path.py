@@ -228,3 +228,23 @@ def test_a_call_that_cannot_be_recorded_is_issued(host, kind, stream, flag):
     for _ in range(3):
         assert call() == 0
     assert host.counts.live_graphs == 1 and host.counts.graph_launches > 0
+
+
+@pytest.mark.parametrize("kind", ["backbone", "block"])
+@pytest.mark.parametrize("stream", [Host.DEFAULT, Host.OWN])
+def test_guard_zones_and_ranges_apply_to_calls_that_were_recorded_before(host, kind, stream):
+    b, s, x, y, ws = host.backbone(), host.block(), host.addr(), host.addr(), host.addr()
+    call = lambda: host.run_backbone(b, x, stream) if kind == "backbone" else host.run_block(s, x, y, ws, stream)   # noqa: E731
+    for _ in range(3):
+        assert call() == 0
+    replayed, launches = host.counts.graph_launches, host.L.mixaq_last_launch_count(host.h)
+    blocks = 2 if kind == "backbone" else 1
+    host.L.mixaq_set_workspace_guards(host.h, 1)
+    assert call() == 0 and host.counts.guard_launches == 2 * blocks                 # filled, compared
+    host.L.mixaq_set_workspace_guards(host.h, 0)
+    host.L.mixaq_set_nvtx(host.h, 1)
+    direct = host.counts.direct
+    assert call() == 0 and host.counts.direct == direct + launches
+    host.L.mixaq_set_nvtx(host.h, 0)
+    assert host.counts.graph_launches == replayed
+    assert call() == 0 and host.counts.graph_launches == replayed + 1
