@@ -263,10 +263,10 @@ mixaq_status mixaq_backbone_forward(mixaq_ctx* ctx, const mixaq_backbone_params*
  * pointers may change freely between calls.  A context keeps 16 graphs of backbone calls and 8 of block calls, the least
  * recently used leave; it remembers as many calls that are not recorded yet.  Recording costs the host several times what
  * issuing a call does, so calls whose graphs are not replayed (rotating buffers, changing ratios) stop being recorded;
- * a call repeated 32 times is recorded in any case.  A call on the legacy default stream (NULL), which cannot be captured,
- * is recorded on a stream of the context's own and its graph launched on the legacy stream; a call made while the caller is
- * capturing the stream itself issues its kernels.  A backbone forward between mixaq_profile_begin/end is captured together
- * with its event records, launched once and not kept; a block forward there issues its kernels.
+ * a call repeated 32 times is recorded in any case.  Calls are recorded on a stream of the context's own and the graph
+ * is launched on the caller's; a call made while the caller is capturing the stream itself issues its kernels.  A
+ * backbone forward between mixaq_profile_begin/end is captured together with its event records, launched once and not
+ * kept; a block forward there issues its kernels.
  * enabled = 0 switches the cache off and drops the stored graphs; it is on by default. */
 mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled);
 

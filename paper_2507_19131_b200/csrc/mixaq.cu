@@ -60,7 +60,7 @@ struct mixaq_ctx {
   bool guards;                         // fill the guard zones of the workspace before a forward, compare them after it
   bool nvtx;                           // name every kernel family, stage and block with an NVTX range (host side)
   bool allow_elevation;                // backbone: every pair uses its own ratios even if an earlier pair of the stage had larger ones
-  cudaStream_t capture_stream;         // forwards on a stream that cannot be captured (the legacy default one) are recorded here
+  cudaStream_t capture_stream;         // calls are recorded here, not on the caller's stream (see replay_record_or_run)
   cudaStream_t side_stream; cudaEvent_t fork, join;   // output norms run beside the next stage inside a captured forward
   std::mutex graph_lock;               // for what follows and the two streams above
   GraphCache<cudaGraphExec_t> graphs{MAX_BACKBONE_GRAPHS, MAX_BACKBONE_GRAPHS};      // of backbone forwards
@@ -694,6 +694,8 @@ static bool caller_is_capturing(cudaStream_t st) {
 // that is worth it and works, else issued on the caller's stream: recording takes device memory, which a call does not
 // otherwise need, so that it fails is no reason for the call to fail.  What a call costs (us, Swin-T forwards on the default stream,
 // waited for one by one; 224 x 224 image / 800 x 1333 map): 473 / 902 replayed, 514 / 939 issued, 1 026 / 1 341 recorded.
+// Calls are recorded on a stream of the context's own: the legacy default stream cannot be captured, and while another one
+// is, it refuses what other threads put on it (a blocking one makes work on the default stream fail too).
 // The caller holds graph_lock.
 template <class Forward>
 static mixaq_status replay_record_or_run(mixaq_ctx* ctx, GraphCache<cudaGraphExec_t>& cache, std::string&& key,
@@ -704,22 +706,20 @@ static mixaq_status replay_record_or_run(mixaq_ctx* ctx, GraphCache<cudaGraphExe
     return MIXAQ_OK;
   }
   bool record = cache.worth_recording(key);
-  if (record && is_legacy(user_stream) && !ctx->capture_stream &&
-      cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+  if (record && !ctx->capture_stream && cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
     ctx->capture_stream = nullptr; record = false;
   }
-  const cudaStream_t st = is_legacy(user_stream) ? ctx->capture_stream : user_stream;
-  if (record && cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) record = false;
+  if (record && cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) record = false;
   if (!record) {
     cudaGetLastError();
     const mixaq_status result = forward(user_stream, false);
     if (result == MIXAQ_OK) cache.saw(std::move(key));
     return result;
   }
-  const mixaq_status result = forward(st, true);
+  const mixaq_status result = forward(ctx->capture_stream, true);
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  const bool recorded = cudaStreamEndCapture(st, &graph) == cudaSuccess && graph && result == MIXAQ_OK &&
+  const bool recorded = cudaStreamEndCapture(ctx->capture_stream, &graph) == cudaSuccess && graph && result == MIXAQ_OK &&
                         cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
   if (graph) cudaGraphDestroy(graph);
   if (recorded) {

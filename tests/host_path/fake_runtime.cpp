@@ -25,6 +25,7 @@ extern "C" {
 FakeCounts counts;
 int fail_capture, fail_instantiate, fail_graph_launch;      // the call fails while this is set
 FakeCopy last_copies[16];
+cudaStream_t capture_origins[16];                            // of the newest captures
 void fake_reset() { std::lock_guard<std::mutex> g(lock); const long live = counts.live_graphs; counts = FakeCounts(); counts.live_graphs = live; }
 }
 
@@ -93,7 +94,7 @@ cudaError_t cudaStreamBeginCapture(cudaStream_t st, cudaStreamCaptureMode) {
   if (capturing.count(st)) { ++counts.violations; return fail(cudaErrorIllegalState); }
   capturing[st] = {std::this_thread::get_id(), st};
   nodes[st] = 0;
-  ++counts.captures;
+  capture_origins[counts.captures++ % 16] = st;
   return cudaSuccess;
 }
 cudaError_t cudaStreamEndCapture(cudaStream_t st, cudaGraph_t* graph) {

@@ -248,3 +248,15 @@ def test_guard_zones_and_ranges_apply_to_calls_that_were_recorded_before(host, k
     host.L.mixaq_set_nvtx(host.h, 0)
     assert host.counts.graph_launches == replayed
     assert call() == 0 and host.counts.graph_launches == replayed + 1
+
+
+def test_recording_leaves_the_callers_stream_alone(host):
+    """A stream being captured refuses what other threads put on it, and a blocking one their work on the default stream
+    too: calls are recorded on a stream of the context's own."""
+    b, s, ws = host.backbone(norms=True), host.block(), host.addr()
+    for _ in range(3):
+        assert host.run_backbone(b, 0x7000_0000, Host.OWN) == 0
+        assert host.run_block(s, 0x7100_0000, 0x7200_0000, ws, Host.OWN) == 0
+    assert host.counts.captures == 2
+    origins = (C.c_void_p * 16).in_dll(host.L, "capture_origins")
+    assert all(o != Host.OWN.value for o in origins[:2])
