@@ -49,27 +49,108 @@ def test_gemm_accumulators_beyond_the_bias_trick(orc, mq, ctx, dim, sign):
     run_block_case(orc, mq, ctx, blk, synth.input_blobs(dim, 1, 17, 23, dim, bg_std=0.5, gain=4.0), 0.4)
 
 
+@pytest.mark.parametrize("pairs", [5, 10])
 @pytest.mark.parametrize("own_stream", [False, True])
-def test_block_graphs_follow_data_buffers_and_switch(orc, mq, ctx, own_stream):
+def test_block_graphs_follow_data_buffers_and_switch(orc, mq, pairs, own_stream):
     """Repeated block calls (recorded at the second, replayed from the third) see fresh data; more sets of buffers than
-    graphs are kept, and the switch that turns them off, change nothing."""
+    calls are remembered, and the switch that turns the graphs off, change nothing."""
     blk = synth.make_block(np.random.default_rng(3), 64, 2, 3, 4, 8, 4)
     xs = [synth.input_blobs(s, 1, 15, 22, 64, bg_std=0.5, gain=4.0) for s in range(3)]
     want = [orc.block_forward(blk, x, 0.5, 0.25).y for x in xs]
+    ctx = mq.Context(0)
     stream = torch.cuda.Stream() if own_stream else torch.cuda.default_stream()
     with torch.cuda.stream(stream):
         db = mq.DeviceBlock(ctx, blk)
-        pairs = [(dev(xs[0]), torch.empty(xs[0].shape, device="cuda")) for _ in range(10)]
+        bufs = [(dev(xs[0]), torch.empty(xs[0].shape, device="cuda")) for _ in range(pairs)]
         for step in range(6):
             if step == 4:
                 ctx.set_graph_cache(False)
-            for xd, yd in pairs:
+            for xd, yd in bufs:
                 xd.copy_(torch.from_numpy(xs[step % 3]))
                 yd.zero_()
                 mq.block_forward(ctx, db, xd, 0.5, 0.25, y=yd)
                 stream.synchronize()
                 assert np.array_equal(yd.cpu().numpy(), want[step % 3]), f"step {step}"
-        ctx.set_graph_cache(True)
+    ctx.close()
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_output_norms_of_recorded_calls_after_eviction(orc, mq, own_stream):
+    """Backbones with output norms (a branch of the graph) on 17 input buffers, one more than graphs are kept: the calls that
+    displace a graph, those that are displaced and those that stay give the oracle's maps."""
+    wl = synth.tiny_backbone(ratio=0.4, prune=0.2)
+    rng = np.random.default_rng(31)
+    norms = [((1.0 + 0.05 * rng.standard_normal(c)).astype(F32), (0.05 * rng.standard_normal(c)).astype(F32)) for c in wl.backbone.dims]
+    xs = [wl.x, np.ascontiguousarray(wl.x[:, ::-1])]
+    want = [[orc.layernorm(o, g, b) for o, (g, b) in zip(orc.backbone_forward(wl.backbone, x, wl.low_ratios, wl.prune_ratios), norms)]
+            for x in xs]
+    ctx = mq.Context(0)
+    stream = torch.cuda.Stream() if own_stream else torch.cuda.default_stream()
+    with torch.cuda.stream(stream):
+        dbb = mq.DeviceBackbone(ctx, wl.backbone, wl.B, wl.H, wl.W, norms=norms)
+        bufs = [dev(xs[0]) for _ in range(17)]
+
+        def call(i, which):
+            bufs[i].copy_(torch.from_numpy(xs[which]))
+            for o in dbb.outs:
+                o.zero_()
+            got = mq.backbone_forward(ctx, dbb, bufs[i], wl.low_ratios, wl.prune_ratios)
+            stream.synchronize()
+            for st, (g, w) in enumerate(zip(got, want[which])):
+                assert np.array_equal(g.cpu().numpy(), w), f"buffer {i}, stage {st}"
+        for step in range(3):                                   # issued, recorded, replayed
+            for i in range(16):
+                call(i, step % 2)
+        for step in range(24):                                  # 40 replays in all earn a further recording
+            call(0, step % 2)
+        for step in range(3):                                   # displaces the graph of buffer 1
+            call(16, step % 2)
+        for i in range(4):
+            call(i, 1)
+        assert ctx.device_status() == 0
+    ctx.close()
+
+
+def test_two_threads_share_a_context(orc, mq):
+    """Blocks and backbones from two threads, each on a stream of its own, through issue, recording and replay."""
+    import threading
+    wl = synth.tiny_backbone(ratio=0.4, prune=0.2)
+    blk = synth.make_block(np.random.default_rng(3), 64, 2, 3, 4, 8, 4)
+    rng = np.random.default_rng(32)
+    norms = [((1.0 + 0.05 * rng.standard_normal(c)).astype(F32), (0.05 * rng.standard_normal(c)).astype(F32)) for c in wl.backbone.dims]
+    xb = [wl.x, np.ascontiguousarray(wl.x[:, ::-1])]
+    xk = [synth.input_blobs(s, 1, 15, 22, 64, bg_std=0.5, gain=4.0) for s in range(2)]
+    want_b = [[orc.layernorm(o, g, b) for o, (g, b) in zip(orc.backbone_forward(wl.backbone, x, wl.low_ratios, wl.prune_ratios), norms)]
+              for x in xb]
+    want_k = [orc.block_forward(blk, x, 0.5, 0.25).y for x in xk]
+    ctx = mq.Context(0)
+    failed = []
+
+    def work(t):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                dbb, db = mq.DeviceBackbone(ctx, wl.backbone, wl.B, wl.H, wl.W, norms=norms), mq.DeviceBlock(ctx, blk)
+                bufs = [(dev(xb[0]), dev(xk[0]), torch.empty(xk[0].shape, device="cuda")) for _ in range(3)]
+                for step in range(15):
+                    which = (step + t) % 2
+                    x, k, y = bufs[step % 3]
+                    x.copy_(torch.from_numpy(xb[which])), k.copy_(torch.from_numpy(xk[which])), y.zero_()
+                    got = mq.backbone_forward(ctx, dbb, x, wl.low_ratios, wl.prune_ratios)
+                    mq.block_forward(ctx, db, k, 0.5, 0.25, y=y)
+                    stream.synchronize()
+                    assert all(np.array_equal(g.cpu().numpy(), w) for g, w in zip(got, want_b[which])), f"thread {t}, step {step}"
+                    assert np.array_equal(y.cpu().numpy(), want_k[which]), f"thread {t}, step {step}"
+        except BaseException as e:                              # noqa: BLE001
+            failed.append(e)
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed
+    assert ctx.device_status() == 0
+    ctx.close()
 
 
 @pytest.mark.parametrize("w_bits,H,W,dim", [(8, 9, 15, 96), (6, 8, 16, 32), (2, 12, 11, 128)])

@@ -250,6 +250,32 @@ def test_guard_zones_and_ranges_apply_to_calls_that_were_recorded_before(host, k
     assert call() == 0 and host.counts.graph_launches == replayed + 1
 
 
+def test_two_threads_share_a_context(host):
+    """Two threads, blocks and backbones on a stream of their own and on the default stream, new keys and old ones mixed:
+    recordings do not meet (the stand-in counts launches into another thread's capture and captures of a busy stream)."""
+    failed = []
+
+    def work(t):
+        h, b, s = host, made[t][0], made[t][1]
+        try:
+            for i in range(60):
+                stream = (Host.DEFAULT, C.c_void_p(0x20 + 0x10 * t))[i % 3 == 0]
+                assert h.run_backbone(b, xs[t][i // 4 % 5], stream) == 0
+                assert h.run_block(s, xs[t][5], xs[t][6 + i // 4 % 5], ws[t], stream) == 0
+        except BaseException as e:                                                               # noqa: BLE001
+            failed.append(e)
+    made = [(host.backbone(norms=True), host.block()) for _ in range(2)]
+    xs = [[host.addr() for _ in range(11)] for _ in range(2)]
+    ws = [host.addr() for _ in range(2)]
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+    assert host.counts.violations == 0 and host.counts.graph_launches > 0 and host.counts.side_launches > 0
+
+
 def test_recording_leaves_the_callers_stream_alone(host):
     """A stream being captured refuses what other threads put on it, and a blocking one their work on the default stream
     too: calls are recorded on a stream of the context's own."""
@@ -260,3 +286,19 @@ def test_recording_leaves_the_callers_stream_alone(host):
     assert host.counts.captures == 2
     origins = (C.c_void_p * 16).in_dll(host.L, "capture_origins")
     assert all(o != Host.OWN.value for o in origins[:2])
+
+
+@pytest.mark.parametrize("stream", [Host.DEFAULT, Host.OWN])
+def test_output_norms_run_beside_the_chain_also_after_eviction(host, stream):
+    """Every recording of an image backbone puts its norms on the side stream, also when earlier graphs have left."""
+    b = host.backbone(norms=True)
+    xs = [host.addr() for _ in range(17)]
+    for x in xs[:16] + [xs[0]] * 40:                           # replays that earn a further recording
+        for _ in range(2):
+            assert host.run_backbone(b, x, stream) == 0
+    for _ in range(2):
+        assert host.run_backbone(b, xs[16], stream) == 0       # displaces xs[1], the least recently used
+    assert (host.counts.captures, host.counts.live_graphs, host.counts.side_launches) == (17, 16, 17)
+    replayed = host.counts.graph_launches
+    assert host.run_backbone(b, xs[0], stream) == 0 and host.counts.graph_launches == replayed + 1
+    assert host.run_backbone(b, xs[1], stream) == 0 and host.counts.graph_launches == replayed + 1
