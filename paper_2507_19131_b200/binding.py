@@ -6,7 +6,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 from types import SimpleNamespace
-from typing import List, Optional, Sequence
+from typing import Iterable, List, Optional
 
 import numpy as np
 import torch
@@ -137,6 +137,11 @@ def branch_counts(H: int, W: int, low_ratio: float, prune_ratio: float = 0.0, wi
 def _stream_ptr() -> C.c_void_p:
     # the raw handle of torch's current stream (building a Stream object for it costs more than a launch)
     return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+
+
+def _ratios(values: Iterable[float], n: int):
+    """The first n ratios of any iterable as a C array (missing ones are 0)."""
+    return (C.c_float * n)(*[float(r) for r in values][:n])
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -526,14 +531,14 @@ class DeviceBackbone:
         self.npairs = (nb + 1) // 2
 
 
-def backbone_forward(ctx: Context, dbb: DeviceBackbone, x0: torch.Tensor, low_ratios: Sequence[float],
-                     prune_ratios: Optional[Sequence[float]] = None) -> List[torch.Tensor]:
+def backbone_forward(ctx: Context, dbb: DeviceBackbone, x0: torch.Tensor, low_ratios: Iterable[float],
+                     prune_ratios: Optional[Iterable[float]] = None) -> List[torch.Tensor]:
     """mixaq_backbone_forward.  Returns the per-stage output tensors owned by `dbb` (overwritten by the next call)."""
     assert x0.is_cuda and x0.dtype == torch.float32 and x0.is_contiguous()
     assert tuple(x0.shape[:3]) == (dbb.B, dbb.H0, dbb.W0)
     n = dbb.npairs
-    lr = (C.c_float * n)(*low_ratios[:n])
-    pr = (C.c_float * n)(*prune_ratios[:n]) if prune_ratios is not None else None
+    lr = _ratios(low_ratios, n)
+    pr = _ratios(prune_ratios, n) if prune_ratios is not None else None
     st = lib().mixaq_backbone_forward(ctx.h, C.byref(dbb.s), _ptr(x0), dbb.out_ptrs, dbb.B, dbb.H0, dbb.W0, lr, pr,
                                       _ptr(dbb.ws), C.c_size_t(dbb.ws.numel()), _stream_ptr())
     ctx.check(st, "backbone_forward")

@@ -95,3 +95,11 @@ def test_generators_are_seeded_and_shaped_like_the_workloads():
     assert np.abs(blk.qkv.codes).max() == 127 and blk.qkv.codes.shape == (288, 96)
     w4 = synth.make_linear(np.random.default_rng(0), 64, 32, 4)
     assert np.abs(w4.codes).max() == 7
+
+
+def test_ratios_come_from_any_iterable():
+    from paper_2507_19131_b200 import binding
+    want = [0.5, 0.25, 0.0]
+    for values in (want, tuple(want), (r for r in want), np.array(want, np.float32), dict(a=0.5, b=0.25, c=0.0).values(),
+                   want + [0.9], want[:2]):
+        assert list(binding._ratios(values, 3)) == want
