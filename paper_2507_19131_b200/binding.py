@@ -134,9 +134,15 @@ def branch_counts(H: int, W: int, low_ratio: float, prune_ratio: float = 0.0, wi
     return tuple(cnt)
 
 
+# The handle of torch's current stream without a Stream object around it, where this torch has the function (0.3 us a call
+# against 3.4: a block call's host work is 28 us); it is not part of torch's public interface.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr() -> C.c_void_p:
-    # the raw handle of torch's current stream (building a Stream object for it costs more than a launch)
-    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+    if _raw_stream is not None:
+        return C.c_void_p(_raw_stream(torch.cuda.current_device()))
+    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 def _ratios(values: Iterable[float], n: int):

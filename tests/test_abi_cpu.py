@@ -103,3 +103,13 @@ def test_ratios_come_from_any_iterable():
     for values in (want, tuple(want), (r for r in want), np.array(want, np.float32), dict(a=0.5, b=0.25, c=0.0).values(),
                    want + [0.9], want[:2]):
         assert list(binding._ratios(values, 3)) == want
+
+
+def test_the_current_stream_with_and_without_torchs_raw_handle(monkeypatch):
+    from paper_2507_19131_b200 import binding
+    monkeypatch.setattr(binding.torch.cuda, "current_device", lambda: 2)
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda *a: type("S", (), {"cuda_stream": 0x1230})())
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 0x4560 + device)
+    assert binding._stream_ptr().value == 0x4562
+    monkeypatch.setattr(binding, "_raw_stream", None)            # a torch without it
+    assert binding._stream_ptr().value == 0x1230
