@@ -112,18 +112,19 @@ __global__ void __launch_bounds__(RANK_WARPS * 32) k_rank_emit(const __grid_cons
   emit_window(a, b, w, s_score, lane, (a.H + WS - 1) / WS * WS, (a.W + WS - 1) / WS * WS);
 }
 
-// Score, rank and bookkeeping of one (image, block) in one CTA, for images of few windows: there the two kernels above are
-// launch latency (3 us each at 64 windows), and one CTA needs no exchange through global memory.  (At 96 windows one CTA
-// already takes longer than the two launches: 10 against 6 us.)
-constexpr int SMALL_WINDOWS = 64, SMALL_WARPS = 32;
-__global__ void __launch_bounds__(SMALL_WARPS * 32) k_select_small(const __grid_constant__ SelectBatch batch) {
+// Score, rank and bookkeeping of one (image, block) in one CTA with a warp per window, for images of at most 32 windows:
+// there the two kernels above are launch latency, and one CTA needs no exchange through global memory.  A whole block call
+// with one against two launches (us): 43.9 and 45.5 at 4 windows, 37.1 and 37.9 at 16, 36.2 and 36.9 at 25; with two windows
+// per warp it is the other way round, 38.9 and 37.4 at 36, 39.7 and 38.1 at 49, 41.1 and 39.0 at 64 windows.
+constexpr int SMALL_WINDOWS = 32;
+__global__ void __launch_bounds__(SMALL_WINDOWS * 32) k_select_small(const __grid_constant__ SelectBatch batch) {
   __shared__ long long s_score[SMALL_WINDOWS];
   griddep_wait();
   griddep_launch();
   const SelectArgs& a = batch.a[blockIdx.y];
-  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int Hp = (a.H + WS - 1) / WS * WS, Wp = (a.W + WS - 1) / WS * WS;
-  for (int w = warp; w < a.nW; w += SMALL_WARPS) {
+  if (w < a.nW) {
     long long s = 0;
     for (int t = lane; t < WT; t += 32) {
       const int src = window_src(b, a.H, a.W, Hp, Wp, a.shift, a.nwx, w, t);
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32) k_select_small(const __grid_
     if (lane == 0) { s_score[w] = s; a.score[(long)b * a.nW + w] = s; }
   }
   __syncthreads();
-  for (int w = warp; w < a.nW; w += SMALL_WARPS) emit_window(a, b, w, s_score, lane, Hp, Wp);
+  if (w < a.nW) emit_window(a, b, w, s_score, lane, Hp, Wp);
 }
 
 // One warp per (image, class): walks the windows in ascending index, 32 at a time, and appends the members of its class
@@ -178,7 +179,7 @@ void launch_select(const SelectArgs* args, int count, cudaStream_t st) {
     for (int i = n; i < MAX_SELECT_BATCH; ++i) batch.a[i] = args[first];
     const SelectArgs& a = args[first];
     if (a.nW <= SMALL_WINDOWS) {
-      launch_pdl(k_select_small, dim3(a.B, n), SMALL_WARPS * 32, 0, st, batch);
+      launch_pdl(k_select_small, dim3(a.B, n), SMALL_WINDOWS * 32, 0, st, batch);
       ++g_launches;
       continue;
     }

@@ -19,9 +19,9 @@ def test_streaming_layer_norm_just_above_its_threshold(orc, mq, ctx, dim, H, W, 
     run_block_case(orc, mq, ctx, blk, synth.input_student_t(dim, 1, H, W, dim), 0.35, taps=False)
 
 
-@pytest.mark.parametrize("H,W", [(7, 7), (56, 56), (34, 90), (63, 49)])
-def test_window_selection_around_64_windows(orc, mq, ctx, H, W):
-    """1, 64 (one launch), 65 and 63 windows per image, with ties, in every order of two ratios."""
+@pytest.mark.parametrize("H,W", [(7, 7), (28, 56), (76, 20), (21, 70), (56, 56), (34, 90), (63, 49)])
+def test_window_selection_by_window_count(orc, mq, ctx, H, W):
+    """1 and 32 windows per image (one launch), 33, 30 and 63 to 65, with ties, in every order of two ratios."""
     blk = synth.make_block(np.random.default_rng(H), 32, 1, 3, 8, 8, 4)
     x = np.round(synth.input_student_t(W, 3, H, W, 32))
     for low, prune, rev in [(0.5, 0.0, False), (0.25, 0.25, True)]:
