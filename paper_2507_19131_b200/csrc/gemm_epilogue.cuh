@@ -1,6 +1,7 @@
 // Fused epilogues of the integer GEMMs (MixA-Q Section 3.2: shared integer weights, per-branch step sizes,
 // zero points and biases).  One epilogue warp owns 32 rows (one TMEM lane quarter, one row per thread) and every
-// c_step-th 32-column chunk of the tile (the warps that share a lane quarter deal the chunks round-robin):
+// c_step-th chunk of the tile, 32 columns wide for the code outputs and 16 for the binary32 outputs (the warps of a group
+// that share a lane quarter deal the chunks round-robin):
 //   raw[n] = sum_k a[m][k] * w[n][k]                   with UNSIGNED activation codes a;
 //   acc[n] = raw[n] - z_a * sum_k w[n][k]              (zero-point correction, exact in int32)
 //   v[n]       = fma((float)acc[n], s_a*s_w[n], bias[n])
@@ -114,7 +115,7 @@ __device__ __forceinline__ void dequant(const GemmBranch& br, int N, long m, boo
 
 // ---- quantizers of the code outputs ------------------------------------------------------------------------------------
 // Both leave rne(x * inv_scale) (FC1: + zp) in the low 16 bits of every pattern, unclamped; sat_pack4 adds, clamps and
-// packs.  They need |x * inv_scale| < 2^15, which `in_range` of the caller guarantees (vbound + |bias|, times inv_scale);
+// packs.  They need |x * inv_scale| < 2^15, which `in_range` of the caller guarantees (the channel's bound + |bias|, times inv_scale);
 // launches for which that cannot be shown take the exact functions with their binary32 clamps.
 constexpr float kPatternRange = 30000.0f;
 
@@ -178,7 +179,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
 
   if (MODE == EPI_QKV || MODE == EPI_FC1) {
     // ---- code outputs: every thread quantizes and packs the 32 codes of its own row ----
-    // a tile lies within one of the q, k, v sections (pick_bn), so its quantizer is the tile's
+    // a tile lies within one of the q, k, v sections (its width divides a section's), so its quantizer is the tile's
     const AQ& q = MODE == EPI_FC1 || n_tile0 < C ? br.q0 : (n_tile0 < 2 * C ? br.q1 : br.q2);
     const float inv_scale = q.inv_scale, zpf = q.zpf;
     const int cbits = eb.cbits, bits = eb.bits;

@@ -6,8 +6,8 @@
 // Persistent, warp-specialised: one CTA per SM walks over the output tiles t = blockIdx.x, + gridDim.x, ...
 //   warp 0      TMA producer: weight tile and (8-bit branches) activation tile of every k-block into a ring of
 //               128-byte-swizzled K-major stages (cp.async.bulk.tensor, no multicast), completion on mbarriers;
-//   warp 1      MMA issuer: one thread feeds the tensor core; the accumulator alternates between two TMEM
-//               buffers so that the epilogue of tile i overlaps the loads and MMAs of tile i+1;
+//   warp 1      MMA issuer: one thread feeds the tensor core; the tiles take turns on up to six TMEM accumulators, so
+//               that the epilogue of a tile overlaps the loads and MMAs of the following ones;
 //   warps 2-5   unpack producers for 4-bit / 2-bit branches: the bit-packed rows of the k-block arrive by TMA in a
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
 //               the swizzled layout (rows whose byte pitch is no multiple of 16 cannot be described to the TMA
@@ -543,9 +543,11 @@ bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t row_bytes
 // (about 0.6 us): a tile takes `mma` to multiply and each of its warps `epi` to convert, `groups` tiles are converted at
 // once while the next ones are multiplied, and the first tiles have nothing to hide behind.  A wide tile reads its rows
 // fewer times and pays the fixed part of the epilogue once for more columns; narrow ones spread a small problem over the
-// SMs.  The constants are a fit to the times of all (width, groups) at 13 shapes from 768 x 7 x 7 to 128 x 2 x 384 x 384; the
-// choice is within 5 % of the fastest at each of them, where a cost without the overlap was up to 30 % off (fc2 with
-// C = 1024 at 2 x 48 x 48: 50 us at the width of 256 it chose, 40 at 128).
+// SMs.  The constants are a fit to the times of all (width, groups) at 13 shapes from 768 x 7 x 7 to 128 x 2 x 384 x 384.  Of
+// 80 shapes (four GEMMs of 20 maps from 7 x 7 to 2 x 384 x 384 tokens), all widths and groups of each timed, the choice is
+// within 5 % of the fastest at 73; the worst are proj with C = 192 at 16 x 28 x 28 (9.0 us at width 64, 7.5 at 192), QKV with
+// C = 768 at 4 x 32 x 32 (15.3 at 128, 13.4 at 256) and proj with C = 512 at 2 x 96 x 96 (23.9 at 256, 21.4 at 128).  A cost
+// without the overlap was up to 30 % off (fc2 with C = 1024 at 2 x 48 x 48: 50 us at the width of 256 it chose, 40 at 128).
 struct Tiling { int bn, n_acc, groups, split; };
 Tiling pick_tiling(int unit, int N, int m_tiles, int k_blocks, int sms, int warps, int chunk) {
   Tiling best = {0, 0, 0, 0};

@@ -378,7 +378,7 @@ void launch_ln_quant(const LnBranch& hi, const LnBranch& lo, int C, cudaStream_t
   const int rows = hi.M + lo.M;
   const int min_bits = hi.M > 0 && lo.M > 0 ? (hi.q.bits < lo.q.bits ? hi.q.bits : lo.q.bits) : (hi.M > 0 ? hi.q.bits : lo.q.bits);
   bool done = false;
-  // streaming kernel: from four row groups per warp of the persistent grid on
+  // streaming kernel: from eight row groups per warp of the persistent grid on
   const long elems = (long)rows * C;
   if (elems >= LN_STREAM_MIN * sm_count()) {
     done = true;
