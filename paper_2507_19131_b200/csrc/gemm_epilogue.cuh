@@ -115,8 +115,8 @@ __device__ __forceinline__ void dequant(const GemmBranch& br, int N, long m, boo
 
 // ---- quantizers of the code outputs ------------------------------------------------------------------------------------
 // Both leave rne(x * inv_scale) (FC1: + zp) in the low 16 bits of every pattern, unclamped; sat_pack4 adds, clamps and
-// packs.  They need |x * inv_scale| < 2^15, which `in_range` of the caller guarantees (the channel's bound + |bias|, times inv_scale);
-// launches for which that cannot be shown take the exact functions with their binary32 clamps.
+// packs.  They need |x * inv_scale| < 2^15, which `in_range` of the caller guarantees (the channel's bound + |bias|, times
+// inv_scale); launches for which that cannot be shown take the exact functions with their binary32 clamps.
 constexpr float kPatternRange = 30000.0f;
 
 // QKV: t = x * inv_scale rounded, then the rounding add.  A packed multiply feeding a packed add would be contracted into
