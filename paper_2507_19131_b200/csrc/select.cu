@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(RANK_WARPS * 32) k_rank_emit(const __grid_cons
 // Score, rank and bookkeeping of one (image, block) in one CTA with a warp per window, for images of at most 32 windows:
 // there the two kernels above are launch latency, and one CTA needs no exchange through global memory.  A whole block call
 // with one against two launches (us): 43.9 and 45.5 at 4 windows, 37.1 and 37.9 at 16, 36.2 and 36.9 at 25; with two windows
-// per warp it is the other way round, 38.9 and 37.4 at 36, 39.7 and 38.1 at 49, 41.1 and 39.0 at 64 windows.
+// per warp it is the other way round, 38.9 and 37.4 at 36, 39.7 and 38.1 at 49, 41.1 and 39.0 at 64 windows.  (Only for 16
+// images and the 18 blocks of a deep stage in one launch is the single kernel still 2 us faster up to 64 windows.)
 constexpr int SMALL_WINDOWS = 32;
 __global__ void __launch_bounds__(SMALL_WINDOWS * 32) k_select_small(const __grid_constant__ SelectBatch batch) {
   __shared__ long long s_score[SMALL_WINDOWS];
