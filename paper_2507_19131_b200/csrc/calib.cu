@@ -3,8 +3,9 @@
 // branches).  The kernels below run the floating-point Two-Branch block (all quantizers off, weights = code x step)
 // through ONE branch's LayerNorm parameters and biases and record the minimum and maximum of what each of the seven
 // quantizer sites would see.  Arithmetic: LayerNorm, softmax and GELU exactly as in the quantized path (the same
-// device functions); matrix products accumulated in binary64 in index order (register-tiled SIMT kernels).
+// device functions); matrix products on the integer tensor cores, to binary64 accuracy.
 #include "kernels.h"
+#include "tc_ptx.cuh"
 
 namespace mixaq {
 
@@ -116,132 +117,297 @@ __global__ void __launch_bounds__(256) k_cal_merge_ln(const float* __restrict__ 
   observe_warp(obs, 0, lo, hi);
 }
 
-// out[m][n] = (float)( sum_k a[m][k] * (w[n][k] * sw[n])  [binary64, k ascending]  + bias[n] ), then per mode:
+// ---- matrix products ----------------------------------------------------------------------------------------------------
+// out[m][n] = (float)( sum_k a[m][k] * w[n][k] * sw[n]  + bias[n] ) with the sum exact or rounded in binary64, then per mode:
 enum CalMode { CAL_QKV = 0, CAL_PROJ = 1, CAL_FC1 = 2, CAL_FC2 = 3, CAL_PLAIN = 4 };
 struct CalLinearArgs {
   const float* a; const int8_t* w; const float* sw; const float* bias;   // bias nullable
   float* out;                 // QKV, FC1, PLAIN: [M][N];  PROJ: x1 [M][N];  FC2: the output feature map
   const float* res;           // PROJ: input feature map (gathered through rowsrc);  FC2: x1 [M][N]
   const int32_t* rowsrc;      // PROJ, FC2
+  uint8_t* slices; int32_t* expo;   // workspace: [CAL_SLICES][M][K] bytes of the fixed-point rows, [M] their exponents
   long M; int N, K, C;        // C: width of one q/k/v section (QKV)
   uint32_t* obs;
+  int* status;
 };
-// Register-tiled binary64 product: a CTA of 64 threads owns a 128 x 32 output tile (every width here is a multiple of 32),
-// a thread 8 rows x 8 columns, so one value read from shared memory feeds 8 products and an input is converted to
-// binary64 once per tile instead of once per product.  Each sum still runs over k in ascending order, so the results are
-// those of the plain loop.
-// FUSED: the product a * (code * step) needs at most 24 + 24 + (significant bits of the code) bits; up to 5 bits of code
-// (weights of 6 bits or fewer) it is exact in binary64, and a fused multiply-add rounds exactly like the product
-// followed by the addition.  Wider weights keep the two separate roundings.
-// Bound by the binary64 pipe (64 lanes per SM and clock) and by shared-memory reads: with 8 x 4 values per thread the
-// 16-byte reads took as long as the products.  Figures: see launch_calibrate_block.
-constexpr int CTM = 128, CTN = 32, CTK = 16, CTPAD = 2;   // tile, k-step, padding (doubles) of a shared row
-template <int MODE, bool FUSED>
-__global__ void __launch_bounds__(64, 4) k_cal_linear(CalLinearArgs p) {
-  __shared__ __align__(16) double sa[2][CTK][CTM + CTPAD], sb[2][CTK][CTN + CTPAD];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ty = (lane & 7) + 8 * warp, tx = lane >> 3;  // rows 2 ty + {0, 1} + 32 i, columns 2 tx + {0, 1} + 8 j
-  const int n_tiles = (p.N + CTN - 1) / CTN;
-  const long m0 = (long)(blockIdx.x / n_tiles) * CTM;
-  const int n0 = (int)(blockIdx.x % n_tiles) * CTN;
-  // staging: four lanes fetch the 16 k of one row (64-byte runs; one lane per row made the L1 lookups the bound), one
-  // half of the rows of a per half step; lane n of the first warp fetches the 16 weight codes of row n
-  const int sr = tid >> 2, sk = 4 * (tid & 3);
-  const bool b_ok = warp == 0 && n0 + lane < p.N;
-  const int8_t* wr = p.w + (long)(b_ok ? n0 + lane : 0) * p.K;
-  const double sw = b_ok ? (double)__ldg(p.sw + n0 + lane) : 0.0;
-  float4 av[4];
-  int4 wv = make_int4(0, 0, 0, 0);
-  auto fetch_a = [&](int k0, int half) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const long m = m0 + sr + 16 * r + 64 * half;
-      av[r] = __ldg(reinterpret_cast<const float4*>(p.a + (m < p.M ? m : 0) * p.K + k0 + sk));
-    }
-  };
-  auto store_a = [&](int buf, int half) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = sr + 16 * r + 64 * half;
-      sa[buf][sk][row] = (double)av[r].x; sa[buf][sk + 1][row] = (double)av[r].y;
-      sa[buf][sk + 2][row] = (double)av[r].z; sa[buf][sk + 3][row] = (double)av[r].w;
-    }
-  };
-  auto store_b = [&](int buf) {
-    if (warp == 0) {
-      const int w4[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-      for (int j = 0; j < CTK; ++j)
-        sb[buf][j][lane] = __dmul_rn((double)(int)(int8_t)(w4[j >> 2] >> (8 * (j & 3))), sw);   // exact
-    }
-  };
-  double acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
-  if (b_ok) wv = __ldg(reinterpret_cast<const int4*>(wr));
-  fetch_a(0, 0); store_a(0, 0);
-  fetch_a(0, 1); store_a(0, 1);
-  store_b(0);
-  __syncthreads();
-  for (int k0 = 0, buf = 0; k0 < p.K; k0 += CTK, buf ^= 1) {            // K is a multiple of 32
-    const bool more = k0 + CTK < p.K;
-    if (more && b_ok) wv = __ldg(reinterpret_cast<const int4*>(wr + k0 + CTK));
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      if (more) fetch_a(k0 + CTK, half);
-#pragma unroll
-      for (int k = half * (CTK / 2); k < (half + 1) * (CTK / 2); ++k) {
-        double a[8], b[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const double2 t = *reinterpret_cast<const double2*>(&sa[buf][k][2 * ty + 32 * i]);
-          const double2 u = *reinterpret_cast<const double2*>(&sb[buf][k][2 * tx + 8 * i]);
-          a[2 * i] = t.x; a[2 * i + 1] = t.y; b[2 * i] = u.x; b[2 * i + 1] = u.y;
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            acc[i][j] = FUSED ? __fma_rn(a[i], b[j], acc[i][j]) : __dadd_rn(acc[i][j], __dmul_rn(a[i], b[j]));
-      }
-      if (more) store_a(buf ^ 1, half);
-    }
-    if (more) store_b(buf ^ 1);
-    __syncthreads();
+// The weights are whole numbers times a step per output channel, so the product runs on the integer tensor cores: every row of
+// `a` becomes 56-bit fixed point with the row's largest exponent (values down to 2^-31 of the largest keep all their bits, the
+// others are rounded at 2^-55 of it), cut into seven bytes, the top one signed.  Each byte plane times the weight codes is an
+// exact int32 sum; the seven sums are put together in integers and three binary64 values, so an output sees at most one rounding
+// of 2^-55 per input and a handful of binary64 roundings where the plain binary64 sum has two per product.
+// A Swin-T calibration on a 200 x 334 map: 23.4 ms of products on the binary64 pipe (8.5 T products/s, about half of its rate),
+// 5.8 ms here and 1.3 ms for the byte planes.
+constexpr int CAL_NOT_FINITE = 255;      // exponent field of a row that holds an infinity or a NaN
+
+// One warp per row: the largest exponent, then the byte planes (a row of one plane is K bytes).
+__global__ void __launch_bounds__(256) k_cal_split(const float* __restrict__ a, uint8_t* __restrict__ slices,
+                                                   int32_t* __restrict__ expo, long M, int K) {
+  const long m = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (m >= M) return;
+  const uint4* row = reinterpret_cast<const uint4*>(a + m * K);
+  uint32_t top = 0;
+  for (int i = lane; i < K / 4; i += 32) {
+    const uint4 v = __ldg(row + i);
+    top = max(max(top, max(v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu)), max(v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu));
   }
-  // the tile's 32 columns lie in one q/k/v section (sections are multiples of 32 channels)
-  float lo = INFINITY, hi = -INFINITY;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const long m = m0 + 2 * ty + (i & 1) + 32 * (i >> 1);
-    if (m >= p.M) continue;
-    long dst = m, src = -1;
-    if (MODE == CAL_PROJ || MODE == CAL_FC2) src = p.rowsrc[m];
-    if (MODE == CAL_FC2) { if (src < 0) continue; dst = src; }
+  const int E = max(1, (int)(__reduce_max_sync(0xffffffffu, top) >> 23));
+  if (lane == 0) expo[m] = E;
+  for (int i = lane; i < K / 4; i += 32) {
+    const uint4 v = __ldg(row + i);
+    const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+    uint32_t lo[4], hi[4];                                  // 56-bit two's complement: bytes 0-3 and 4-6
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + 2 * tx + 8 * j;
-      if (n >= p.N) continue;                                  // only a merge may have a ragged width
-      const bool pair = n + 1 < p.N;
-      float2 v = make_float2((float)__dadd_rn(acc[i][2 * j], p.bias ? (double)__ldg(p.bias + n) : 0.0),
-                             (float)__dadd_rn(acc[i][2 * j + 1], p.bias && pair ? (double)__ldg(p.bias + n + 1) : 0.0));
-      if (MODE == CAL_FC1) v = gelu_f2(v);
-      if (MODE == CAL_QKV || MODE == CAL_FC1) { lo = fminf(lo, fminf(v.x, v.y)); hi = fmaxf(hi, fmaxf(v.x, v.y)); }
-      if (MODE == CAL_PROJ || MODE == CAL_FC2) {
-        float2 r = make_float2(0.f, 0.f);
-        const long rr = MODE == CAL_PROJ ? src : m;
-        if (rr >= 0) r = __ldg(reinterpret_cast<const float2*>(p.res + rr * p.N + n));
-        v = make_float2(__fadd_rn(r.x, v.x), __fadd_rn(r.y, v.y));
-      }
-      float* out = p.out + dst * p.N + n;
-      if (MODE == CAL_PLAIN && p.N % 2) { out[0] = v.x; if (pair) out[1] = v.y; }
-      else *reinterpret_cast<float2*>(out) = v;
+      const int e = (in[j] >> 23) & 255;
+      const long long f = (in[j] & 0x7FFFFFu) | (e ? 0x800000u : 0u);
+      const int sh = (e ? e : 1) - E + 31;                  // at most 31
+      long long q = sh >= 0 ? f << sh : (sh < -25 ? 0 : (f + (1LL << (-sh - 1))) >> -sh);
+      if (in[j] >> 31) q = -q;
+      lo[j] = (uint32_t)q; hi[j] = (uint32_t)(q >> 32);
+    }
+#pragma unroll
+    for (int s = 0; s < CAL_SLICES; ++s) {
+      const uint32_t* x = s < 4 ? lo : hi;
+      const uint32_t sel = (uint32_t)(s & 3) | (uint32_t)((s & 3) + 4) << 4;
+      reinterpret_cast<uint32_t*>(slices + ((long)s * M + m) * K)[i] =
+          __byte_perm(__byte_perm(x[0], x[1], sel), __byte_perm(x[2], x[3], sel), 0x5410);
     }
   }
-  if (MODE == CAL_QKV) observe_warp(p.obs, 1 + n0 / p.C, lo, hi);
-  else if (MODE == CAL_FC1) observe_warp(p.obs, 6, lo, hi);
+}
+
+// Persistent, one CTA per SM: warp 0 TMA, warp 1 MMA, sixteen epilogue warps (a lane quarter and 16 columns each).
+// A 128 x 64 tile has seven accumulators of 64 TMEM columns, one per byte plane.  Per 128 codes of k the weight tile is loaded
+// once and met by the seven activation tiles, which are what the loads are made of (16 KB each against 140 cycles of MMA): the
+// width of 64 is the largest with which seven accumulators fit.  What bounds it up to K = 384 is the epilogue (seven TMEM loads,
+// eight binary64 operations and two conversions an output: 16 warps 5.8 ms, 8 warps with the loop unrolled 7.9), then the loads.  Sums of more than CAL_KCHUNK products, which int32 might not
+// hold, are drained in parts.
+constexpr int CG_BM = 128, CG_BN = 64, CG_BK = 128, CG_A_RING = 8, CG_B_RING = 4, CAL_KCHUNK = 32768;
+constexpr int CG_A_BYTES = CG_BM * CG_BK, CG_B_BYTES = CG_BN * CG_BK, CG_EPI_WARPS = 16, CG_THREADS = 32 * (2 + CG_EPI_WARPS);
+constexpr int CG_EPI_COLS = CG_BN / (CG_EPI_WARPS / 4);
+constexpr int CG_BARS = 2 * CG_A_RING + 2 * CG_B_RING + 3;
+constexpr int CG_COLS_OFF = CG_A_RING * CG_A_BYTES + CG_B_RING * CG_B_BYTES;             // constants of the epilogue warps' columns
+constexpr int CG_BARS_OFF = CG_COLS_OFF + CG_EPI_WARPS * CG_EPI_COLS * 16;
+constexpr int CG_SMEM = CG_BARS_OFF + CG_BARS * 8 + 16 + 1024;
+
+// The sum as it is written, for rows with infinities or NaNs: what follows from them is what the plain sum gives.
+__device__ __noinline__ float cal_plain_sum(const CalLinearArgs& p, long m, int n, double2 col) {
+  double s = 0.0;
+  for (int k = 0; k < p.K; ++k)
+    s = __dadd_rn(s, __dmul_rn((double)p.a[m * p.K + k], __dmul_rn((double)(int)p.w[(long)n * p.K + k], col.x)));
+  return (float)__dadd_rn(s, col.y);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(CG_THREADS, 1) k_cal_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                                                            const __grid_constant__ CalLinearArgs p, int n_tiles, int tiles) {
+  extern __shared__ uint8_t cg_raw[];
+  const uint32_t raw = smem_u32(cg_raw), base = (raw + 1023u) & ~1023u;
+  const uint32_t b_ring = base + CG_A_RING * CG_A_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(cg_raw + (base - raw) + CG_BARS_OFF);
+  const uint32_t a_full = smem_u32(bars), a_empty = a_full + 8u * CG_A_RING, b_full = a_empty + 8u * CG_A_RING;
+  const uint32_t b_empty = b_full + 8u * CG_B_RING, acc_full = b_empty + 8u * CG_B_RING, acc_empty = acc_full + 8u, drained = acc_full + 16u;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + CG_BARS);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t a_used = 0, a_phase = 0, b_used = 0, b_phase = 0;     // TMA thread: filled slots and the parity of their last fill
+  if (tid == 0) {
+    for (int i = 0; i < CG_BARS; ++i) {
+      const uint32_t bar = a_full + 8u * i;
+      mbar_init(bar, bar == acc_empty ? (uint32_t)CG_EPI_WARPS : 1u);
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = *tmem_holder;
+  const int K = p.K, n_chunks = (K + CAL_KCHUNK - 1) / CAL_KCHUNK;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      bool ok = true;
+      int as = 0, bs = 0;
+      uint32_t ap = 0, bp = 0;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        const int m0 = t / n_tiles * CG_BM, n0 = t % n_tiles * CG_BN;
+        for (int k0 = 0; k0 < K && ok; k0 += CG_BK) {
+          if ((b_used >> bs & 1u) && !mbar_wait(b_empty + 8u * bs, bp ^ 1u, abort_flag)) { ok = false; break; }
+          b_used |= 1u << bs; b_phase = (b_phase & ~(1u << bs)) | bp << bs;
+          mbar_arrive_expect_tx(b_full + 8u * bs, CG_B_BYTES);
+          tma_load_2d(b_ring + (uint32_t)(bs * CG_B_BYTES), &tmB, k0, n0, b_full + 8u * bs);
+          if (++bs == CG_B_RING) { bs = 0; bp ^= 1u; }
+          for (int s = 0; s < CAL_SLICES; ++s) {
+            if ((a_used >> as & 1u) && !mbar_wait(a_empty + 8u * as, ap ^ 1u, abort_flag)) { ok = false; break; }
+            a_used |= 1u << as; a_phase = (a_phase & ~(1u << as)) | ap << as;
+            mbar_arrive_expect_tx(a_full + 8u * as, CG_A_BYTES);
+            tma_load_2d(base + (uint32_t)(as * CG_A_BYTES), &tmA, k0, (int)(s * p.M) + m0, a_full + 8u * as);
+            if (++as == CG_A_RING) { as = 0; ap ^= 1u; }
+          }
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint64_t adesc0 = smem_desc_sw128(base), bdesc0 = smem_desc_sw128(b_ring);
+      bool ok = true, first = true;
+      int as = 0, bs = 0;
+      uint32_t ap = 0, bp = 0, ep = 0;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        for (int kc = 0; kc < K && ok; kc += CAL_KCHUNK) {
+          if (!first) { if (!mbar_wait(acc_empty, ep, abort_flag)) { ok = false; break; } ep ^= 1u; }
+          first = false;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const int k_end = min(K, kc + CAL_KCHUNK);
+          for (int k0 = kc; k0 < k_end && ok; k0 += CG_BK) {
+            if (!mbar_wait<true>(b_full + 8u * bs, bp, abort_flag)) { ok = false; break; }
+            const int steps = min(CG_BK, k_end - k0) / 32;
+            const uint64_t bdesc = bdesc0 + (uint64_t)(bs * (CG_B_BYTES >> 4));
+            for (int s = 0; s < CAL_SLICES; ++s) {
+              if (!mbar_wait<true>(a_full + 8u * as, ap, abort_flag)) { ok = false; break; }
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              // s32 += (byte plane: u8, the top one s8) x s8
+              const uint32_t idesc = (2u << 4) | ((s == CAL_SLICES - 1 ? 1u : 0u) << 7) | (1u << 10) | ((uint32_t)(CG_BN >> 3) << 17) | ((uint32_t)(CG_BM >> 4) << 24);
+              const uint64_t adesc = adesc0 + (uint64_t)(as * (CG_A_BYTES >> 4));
+              for (int kk = 0; kk < steps; ++kk)
+                mma_i8(tmem_base + (uint32_t)(s * CG_BN), adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), idesc, (uint32_t)(k0 > kc || kk > 0));
+              mma_commit(a_empty + 8u * as);
+              if (++as == CG_A_RING) { as = 0; ap ^= 1u; }
+            }
+            if (!ok) break;
+            mma_commit(b_empty + 8u * bs);
+            if (++bs == CG_B_RING) { bs = 0; bp ^= 1u; }
+          }
+          if (ok) mma_commit(acc_full);
+        }
+      }
+    }
+    __syncwarp();
+  } else {
+    // the warp's lane quarter (four consecutive warps cover the four) and CG_EPI_COLS columns
+    const int q = warp & 3, col0 = (warp - 2) / 4 * CG_EPI_COLS;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)col0;
+    double2* cols = reinterpret_cast<double2*>(cg_raw + (base - raw) + CG_COLS_OFF) + (warp - 2) * CG_EPI_COLS;   // (step, bias)
+    double part[CG_EPI_COLS];                                     // more than one chunk of k: the sums so far
+    uint32_t fp = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      const long m = (long)(t / n_tiles) * CG_BM + q * 32 + lane;
+      const int n0 = t % n_tiles * CG_BN + col0;
+      const bool row_ok = m < p.M;
+      const int E = row_ok ? __ldg(p.expo + m) : 1;
+      long src = -1, dst = m;
+      if (MODE == CAL_PROJ || MODE == CAL_FC2) src = row_ok ? (long)__ldg(p.rowsrc + m) : -1;
+      if (MODE == CAL_FC2) dst = src;
+      const long rr = MODE == CAL_PROJ ? src : m;                 // row of the residual, < 0: zero
+      const bool store = row_ok && (MODE != CAL_FC2 || src >= 0);
+      const double unit = __longlong_as_double((long long)(E - 181 + 1023) << 52);      // value of the lowest bit of the row
+      __syncwarp();
+      if (lane < CG_EPI_COLS) {
+        const int n = n0 + lane < p.N ? n0 + lane : 0;
+        cols[lane] = make_double2((double)__ldg(p.sw + n), p.bias ? (double)__ldg(p.bias + n) : 0.0);
+      }
+      __syncwarp();
+      float lo = INFINITY, hi = -INFINITY;
+      for (int c = 0; c < n_chunks; ++c) {
+        if (!mbar_wait(acc_full, fp, abort_flag)) { ok = false; break; }
+        fp ^= 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+        for (int g = 0; g < CG_EPI_COLS; g += 8) {
+          int32_t S[CAL_SLICES][8];
+#pragma unroll
+          for (int s = 0; s < CAL_SLICES; ++s) tmem_ld(taddr + (uint32_t)(s * CG_BN + g), S[s]);
+#pragma unroll
+          for (int s = 0; s < CAL_SLICES; ++s) tmem_ld_wait(S[s]);
+          if (g + 8 == CG_EPI_COLS) {                             // the accumulators are read: the next tile may start
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty);
+          }
+          float v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            // whole numbers below 2^51 become binary64 through the bit pattern of 1.5 * 2^52
+            constexpr long long kMagic64 = 0x4338000000000000LL;
+            const double h = __dadd_rn(__longlong_as_double((long long)S[6][j] * 65536 + ((long long)S[5][j] * 256 + (S[4][j] + kMagic64))), -6755399441055744.0);
+            const double mid = __dadd_rn(__longlong_as_double((long long)S[3][j] * 256 + (S[2][j] + kMagic64)), -6755399441055744.0);
+            const double l = __dadd_rn(__longlong_as_double((long long)S[1][j] * 256 + (S[0][j] + kMagic64)), -6755399441055744.0);
+            double d = __fma_rn(h, 4294967296.0, __fma_rn(mid, 65536.0, l));
+            if (n_chunks > 1) {
+              if (c > 0) d = __dadd_rn(d, part[g + j]);
+              part[g + j] = d;
+            }
+            const double2 cb = cols[g + j];
+            v[j] = (float)__dadd_rn(__dmul_rn(__dmul_rn(d, unit), cb.x), cb.y);
+          }
+          if (c + 1 < n_chunks) continue;
+          const int n = n0 + g;
+          if (__any_sync(0xffffffffu, E == CAL_NOT_FINITE)) {
+#pragma unroll 1
+            for (int j = 0; j < 8; ++j) {
+              const float f = E == CAL_NOT_FINITE && n + j < p.N ? cal_plain_sum(p, m, n + j, cols[g + j]) : 0.0f;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) if (i == j && E == CAL_NOT_FINITE) v[i] = f;
+            }
+          }
+          if (MODE == CAL_FC1) {
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) { const float2 a = gelu_f2(make_float2(v[j], v[j + 1])); v[j] = a.x; v[j + 1] = a.y; }
+          }
+          if ((MODE == CAL_QKV || MODE == CAL_FC1) && row_ok && n < p.N) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { lo = fminf(lo, v[j]); hi = fmaxf(hi, v[j]); }
+          }
+          if (!store || n >= p.N) continue;
+          float* out = p.out + dst * p.N + n;
+          if (MODE == CAL_PLAIN && p.N % 8) {                     // only a merge may have a ragged width
+#pragma unroll
+            for (int j = 0; j < 8; ++j) if (n + j < p.N) out[j] = v[j];
+            continue;
+          }
+          if ((MODE == CAL_PROJ || MODE == CAL_FC2) && rr >= 0) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(p.res + rr * p.N + n)), b = __ldg(reinterpret_cast<const float4*>(p.res + rr * p.N + n) + 1);
+            v[0] = __fadd_rn(a.x, v[0]); v[1] = __fadd_rn(a.y, v[1]); v[2] = __fadd_rn(a.z, v[2]); v[3] = __fadd_rn(a.w, v[3]);
+            v[4] = __fadd_rn(b.x, v[4]); v[5] = __fadd_rn(b.y, v[5]); v[6] = __fadd_rn(b.z, v[6]); v[7] = __fadd_rn(b.w, v[7]);
+          } else if (MODE == CAL_PROJ || MODE == CAL_FC2) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = __fadd_rn(0.0f, v[j]);
+          }
+          reinterpret_cast<float4*>(out)[0] = make_float4(v[0], v[1], v[2], v[3]);
+          reinterpret_cast<float4*>(out)[1] = make_float4(v[4], v[5], v[6], v[7]);
+        }
+      }
+      if (!ok) break;
+      // a warp's columns lie in one q/k/v section (sections are multiples of 32 channels)
+      if (MODE == CAL_QKV) { if (n0 < p.N) observe_warp(p.obs, 1 + n0 / p.C, lo, hi); }
+      else if (MODE == CAL_FC1) { if (n0 < p.N) observe_warp(p.obs, 6, lo, hi); }
+    }
+  }
+
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (*abort_flag) {
+    // a wait ran out: the copies and MMAs already issued have to end (bounded) before the CTA may exit
+    if (tid == 32) mma_commit(drained);
+    if (tid == 0) {
+      atomicExch(p.status, 1);
+      auto drain = [](uint32_t bar, uint32_t parity) {
+        for (uint32_t it = 0; it < (1u << 20); ++it) if (mbar_try_wait(bar, parity)) return;
+      };
+      for (int s = 0; s < CG_A_RING; ++s) if (a_used >> s & 1u) drain(a_full + 8u * s, a_phase >> s & 1u);
+      for (int s = 0; s < CG_B_RING; ++s) if (b_used >> s & 1u) drain(b_full + 8u * s, b_phase >> s & 1u);
+      drain(drained, 0u);
+    }
+    __syncthreads();
+  }
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
 }
 
 // softmax of the numeric contract over 49 logits: exact maximum, exponentials through 2^t, four interleaved partial
@@ -375,14 +541,18 @@ __global__ void k_cal_obs_init(uint32_t* obs, int sites) {
   if (i < 2 * sites) obs[i] = (i & 1) ? 0u : 0xFFFFFFFFu;
 }
 
-// w_bits: declared width of the weight codes; up to 6 bits (5 significant) the fused product is exact, see k_cal_linear
 template <int MODE>
-void launch_cal_linear(const CalLinearArgs& p, int w_bits, cudaStream_t st) {
-  if (p.M == 0) return;
-  const unsigned grid = (unsigned)(((p.N + CTN - 1) / CTN) * ((p.M + CTM - 1) / CTM));
-  if (w_bits >= 2 && w_bits <= 6) k_cal_linear<MODE, true><<<grid, 64, 0, st>>>(p);
-  else k_cal_linear<MODE, false><<<grid, 64, 0, st>>>(p);
-  ++g_launches;
+bool launch_cal_linear(const CalLinearArgs& p, cudaStream_t st) {
+  if (p.M == 0) return true;
+  if (cudaFuncSetAttribute(k_cal_gemm<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, CG_SMEM) != cudaSuccess) return false;
+  CUtensorMap mA, mB;
+  if (!make_map(&mA, p.slices, (uint64_t)CAL_SLICES * p.M, (uint64_t)p.K, CG_BM) || !make_map(&mB, p.w, (uint64_t)p.N, (uint64_t)p.K, CG_BN)) return false;
+  k_cal_split<<<(unsigned)((p.M + 7) / 8), 256, 0, st>>>(p.a, p.slices, p.expo, p.M, p.K);
+  const int n_tiles = (p.N + CG_BN - 1) / CG_BN;
+  const int tiles = (int)((p.M + CG_BM - 1) / CG_BM) * n_tiles, sms = sm_count();
+  k_cal_gemm<MODE><<<tiles < sms ? tiles : sms, CG_THREADS, CG_SMEM, st>>>(mA, mB, p, n_tiles, tiles);
+  g_launches += 2;
+  return true;
 }
 
 }  // namespace
@@ -408,11 +578,8 @@ static bool launch_cal_ln(const float* src, int32_t* rowsrc_out, const float* ga
   return true;
 }
 
-// Calibration of a Swin-T backbone on a 200 x 334 map (W4, both branches of 12 blocks, 205 G products): 125 ms with one
-// thread per output, 31 ms with the register tiles (27 ms of kernels: 24 ms of products at 8.5 T/s, about half of the
-// binary64 pipe's rate).  The output map, the observed ranges and the quantizers are unchanged bit for bit.
 // The floating-point block through one branch.  Workspace (floats unless noted): rowsrc int32[M], ln [M][C],
-// qkv [M][3C], o [M][C], x1 [M][C], h [M][hidden]; obs: 16 keys (seven sites and the block's input map).
+// qkv [M][3C], o [M][C], x1 [M][C], h [M][hidden], slices, expo; obs: 16 keys (seven sites and the block's input map).
 bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
   const int C = c.C, Hd = c.hidden;
   const int Hp = (c.H + WS - 1) / WS * WS, Wp = (c.W + WS - 1) / WS * WS, nwx = Wp / WS, nW = (Hp / WS) * nwx;
@@ -421,9 +588,9 @@ bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
   ++g_launches;
   if (!launch_cal_ln(c.x, c.rowsrc, c.ln1_g, c.ln1_b, c.ln, M, C, 1, c.H, c.W, c.shift, nwx, nW, c.obs, 0, 7, st)) return false;
   CalLinearArgs l;
-  l.obs = c.obs; l.M = M; l.C = C; l.rowsrc = c.rowsrc;
+  l.obs = c.obs; l.status = c.status; l.slices = c.slices; l.expo = c.expo; l.M = M; l.C = C; l.rowsrc = c.rowsrc;
   l.a = c.ln; l.w = c.w_qkv; l.sw = c.s_qkv; l.bias = c.b_qkv; l.out = c.qkv; l.res = nullptr; l.N = 3 * C; l.K = C;
-  launch_cal_linear<CAL_QKV>(l, c.wb_qkv, st);
+  if (!launch_cal_linear<CAL_QKV>(l, st)) return false;
   CalAttnArgs a;
   a.qkv = c.qkv; a.relpos = c.relpos; a.o = c.o; a.slots = slots; a.C = C; a.heads = c.heads; a.shift = c.shift;
   a.Hp = Hp; a.Wp = Wp; a.nwx = nwx; a.nW = nW; a.obs = c.obs;
@@ -431,12 +598,12 @@ bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
   k_cal_attention<<<(unsigned)(slots * c.heads), 64, sizeof(CalAttnSmem), st>>>(a);
   ++g_launches;
   l.a = c.o; l.w = c.w_proj; l.sw = c.s_proj; l.bias = c.b_proj; l.out = c.x1; l.res = c.x; l.N = C; l.K = C;
-  launch_cal_linear<CAL_PROJ>(l, c.wb_proj, st);
+  if (!launch_cal_linear<CAL_PROJ>(l, st)) return false;
   if (!launch_cal_ln(c.x1, nullptr, c.ln2_g, c.ln2_b, c.ln, M, C, 0, c.H, c.W, c.shift, nwx, nW, c.obs, 5, -1, st)) return false;
   l.a = c.ln; l.w = c.w_fc1; l.sw = c.s_fc1; l.bias = c.b_fc1; l.out = c.h; l.res = nullptr; l.N = Hd; l.K = C;
-  launch_cal_linear<CAL_FC1>(l, c.wb_fc1, st);
+  if (!launch_cal_linear<CAL_FC1>(l, st)) return false;
   l.a = c.h; l.w = c.w_fc2; l.sw = c.s_fc2; l.bias = c.b_fc2; l.out = c.y; l.res = c.x1; l.N = C; l.K = Hd;
-  launch_cal_linear<CAL_FC2>(l, c.wb_fc2, st);
+  if (!launch_cal_linear<CAL_FC2>(l, st)) return false;
   return true;
 }
 
@@ -453,9 +620,9 @@ bool launch_calibrate_merge(const CalMergeArgs& c, cudaStream_t st) {
   }
   ++g_launches;
   CalLinearArgs l;
-  l.obs = c.obs; l.M = M; l.C = c.N; l.rowsrc = nullptr; l.res = nullptr;
+  l.obs = c.obs; l.status = c.status; l.slices = c.slices; l.expo = c.expo; l.M = M; l.C = c.N; l.rowsrc = nullptr; l.res = nullptr;
   l.a = c.ln; l.w = c.w; l.sw = c.sw; l.bias = nullptr; l.out = c.y; l.N = c.N; l.K = 4 * c.C;
-  launch_cal_linear<CAL_PLAIN>(l, c.w_bits, st);
+  if (!launch_cal_linear<CAL_PLAIN>(l, st)) return false;
   return true;
 }
 

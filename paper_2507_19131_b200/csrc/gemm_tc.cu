@@ -16,7 +16,7 @@
 //               16 or 32 columns per load) + the fused epilogue of the mode.
 // Every wait on an mbarrier is bounded; on expiry the CTA raises the status word, then waits (bounded again) for the
 // copies it has issued to land and for the MMAs it has issued to retire, frees its tensor memory and returns.
-#include <cuda.h>
+#include "tc_ptx.cuh"
 #include "gemm_epilogue.cuh"
 
 namespace mixaq {
@@ -53,8 +53,6 @@ __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV 
 constexpr int MAX_RING = 6;
 constexpr int TMEM_COLS = 512;                 // one CTA per SM: it takes all of the tensor memory
 constexpr int MAX_ACC = 6;                     // accumulators in it, as far as the tile width allows
-constexpr uint32_t MAX_POLLS = 1u << 22;       // tries per wait
-constexpr uint32_t MAX_SUSPENDED_POLLS = 1u << 16;   // tries that may each suspend the thread for up to 20 us
 
 struct TcParams {
   GemmArgs g;
@@ -88,79 +86,6 @@ __host__ __device__ inline SmemLayout smem_layout(int BN, int ring, int packed_b
   L.bars_off = L.res_off + res_bytes;
   L.total = L.bars_off + NUM_BARS * 8 + 16;                     // then TMEM base, abort flag, constants-out-of-range flag
   return L;
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// One try (the hardware suspends the thread for a short, implementation-defined time while the phase is pending;
-// an explicit longer suspend hint measured slower: the waiters sit on the critical path of the small stages).
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
-  return ok != 0;
-}
-// Bounded wait.  Returns false when the limit ran out or another thread of the CTA already gave up (looked at now and
-// then only).  The waits that are not on a tile's critical path give the hardware a suspend time: the polls of the TMA and
-// MMA threads took up to a tenth of the issue slots of their schedulers.
-template <bool LATENCY = false>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait(bar, parity)) return true;
-  for (uint32_t it = 1; it < (LATENCY ? MAX_POLLS : MAX_SUSPENDED_POLLS); ++it) {
-    if (LATENCY ? mbar_try_wait(bar, parity) : mbar_try_wait_hint(bar, parity)) return true;
-    if ((it & 15u) == 0u && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;                    // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;          // stride byte offset
-  d |= (uint64_t)1 << 46;                    // descriptor version
-  d |= (uint64_t)2 << 61;                    // SWIZZLE_128B
-  return d;
-}
-
-__device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // The tiles of a CTA, without a division per tile: tile number blockIdx.x, + gridDim.x, ..., row tile major.  The high
@@ -506,38 +431,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 }
 
 // ---- host side -------------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-  }
-  return fn;
-}
-
-// 2-D byte matrix [rows][row_bytes] (bytes of a row contiguous), box = box_rows x box_bytes, zero fill outside.
-// swizzled: 128-byte swizzle for MMA operand tiles (box_bytes = 128); otherwise a plain row-major box.
-bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t row_bytes, uint32_t box_rows,
-              uint32_t box_bytes = BK, bool swizzled = true) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {row_bytes, rows};
-  cuuint64_t strides[1] = {row_bytes};
-  cuuint32_t box[2] = {box_bytes, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-
 // Tile width and the epilogue's division of labour.  The width is a multiple of 32 that divides `unit` (N; for QKV the
 // width C of a section, so that a tile has one quantizer), at most 256.  Cost in units of an epilogue warp's 32 columns
 // (about 0.6 us): a tile takes `mma` to multiply and each of its warps `epi` to convert, `groups` tiles are converted at

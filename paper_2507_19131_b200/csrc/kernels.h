@@ -136,19 +136,22 @@ struct CalBlockArgs {
   int B, H, W, C, heads, hidden, shift;
   const float *ln1_g, *ln1_b, *ln2_g, *ln2_b, *b_qkv, *b_proj, *b_fc1, *b_fc2;   // of the branch being calibrated
   const int8_t *w_qkv, *w_proj, *w_fc1, *w_fc2;
-  int wb_qkv, wb_proj, wb_fc1, wb_fc2;            // declared widths of the weight codes
   const float *s_qkv, *s_proj, *s_fc1, *s_fc2, *relpos;
   int32_t* rowsrc; float *ln, *qkv, *o, *x1, *h;  // workspace: [M], [M][C], [M][3C], [M][C], [M][C], [M][hidden]
+  uint8_t* slices; int32_t* expo;                 // workspace of the products: [7][M][max(C, hidden)] bytes, [M]
   uint32_t* obs;                                  // 16 order-preserving keys: min, max of the seven sites and of x
+  int* status;
 };
 bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st);
 struct CalMergeArgs {
   const float* x; float* y; int B, H, W, C, N;
-  const float *ln_g, *ln_b; const int8_t* w; const float* sw; int w_bits;
-  float* ln;                                      // workspace [M][4C]
+  const float *ln_g, *ln_b; const int8_t* w; const float* sw;
+  float* ln; uint8_t* slices; int32_t* expo;      // workspace [M][4C], [7][M][4C], [M]
   uint32_t* obs;                                  // 2 keys
+  int* status;
 };
 bool launch_calibrate_merge(const CalMergeArgs& c, cudaStream_t st);
+constexpr int CAL_SLICES = 7;                     // byte planes a calibration product cuts its input into
 float cal_key_to_float(uint32_t key);
 
 // ---- preparation -----------------------------------------------------------------------------------

@@ -1217,7 +1217,7 @@ mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled) {
 // -------------------------------------------------------------------------------------------------
 // calibration (Section 4.3)
 namespace {
-struct CalWs { int32_t* rowsrc; float *ln, *qkv, *o, *x1, *h; uint32_t* obs; size_t bytes; };
+struct CalWs { int32_t *rowsrc, *expo; float *ln, *qkv, *o, *x1, *h; uint8_t* slices; uint32_t* obs; size_t bytes; };
 CalWs carve_cal(const mixaq_block_params* p, int B, int H, int W, void* base) {
   CalWs w; Carver c(base);
   Geometry g = geometry(H, W, 0.f, 0.f);
@@ -1226,6 +1226,7 @@ CalWs carve_cal(const mixaq_block_params* p, int B, int H, int W, void* base) {
   w.rowsrc = c.take<int32_t>(M);
   w.ln = c.take<float>(M * p->dim); w.qkv = c.take<float>(M * 3 * p->dim); w.o = c.take<float>(M * p->dim);
   w.x1 = c.take<float>(M * p->dim); w.h = c.take<float>(M * p->hidden);
+  w.expo = c.take<int32_t>(M); w.slices = c.take<uint8_t>(CAL_SLICES * M * std::max(p->dim, p->hidden));
   w.bytes = c.off;
   return w;
 }
@@ -1264,9 +1265,9 @@ mixaq_status mixaq_calibrate_block(mixaq_ctx* ctx, const mixaq_block_params* p, 
   c.ln1_g = br.ln1_g; c.ln1_b = br.ln1_b; c.ln2_g = br.ln2_g; c.ln2_b = br.ln2_b;
   c.b_qkv = br.b_qkv; c.b_proj = br.b_proj; c.b_fc1 = br.b_fc1; c.b_fc2 = br.b_fc2;
   c.w_qkv = p->qkv.codes; c.w_proj = p->proj.codes; c.w_fc1 = p->fc1.codes; c.w_fc2 = p->fc2.codes;
-  c.wb_qkv = p->qkv.bits; c.wb_proj = p->proj.bits; c.wb_fc1 = p->fc1.bits; c.wb_fc2 = p->fc2.bits;
   c.s_qkv = p->qkv.scale; c.s_proj = p->proj.scale; c.s_fc1 = p->fc1.scale; c.s_fc2 = p->fc2.scale; c.relpos = p->relpos_table;
   c.rowsrc = ws.rowsrc; c.ln = ws.ln; c.qkv = ws.qkv; c.o = ws.o; c.x1 = ws.x1; c.h = ws.h; c.obs = ws.obs;
+  c.slices = ws.slices; c.expo = ws.expo; c.status = ctx->d_status;
   g_launches = 0;
   if (!launch_calibrate_block(c, st)) return fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "calibrate_block: unsupported dim");
   ctx->launches = g_launches;
@@ -1278,7 +1279,8 @@ mixaq_status mixaq_calibrate_block(mixaq_ctx* ctx, const mixaq_block_params* p, 
 size_t mixaq_calibrate_merge_workspace_bytes(const mixaq_merge_params* p, int B, int H, int W) {
   if (!p || B <= 0 || H <= 0 || W <= 0 || p->reduction.in_features <= 0) return 0;
   const size_t toks = (size_t)B * ((H + 1) / 2) * ((W + 1) / 2);
-  return carved_bytes(16 * sizeof(uint32_t)) + carved_bytes(toks * p->reduction.in_features * sizeof(float));
+  return carved_bytes(16 * sizeof(uint32_t)) + carved_bytes(toks * p->reduction.in_features * sizeof(float)) +
+         carved_bytes(toks * sizeof(int32_t)) + carved_bytes(CAL_SLICES * toks * p->reduction.in_features);
 }
 
 mixaq_status mixaq_calibrate_merge(mixaq_ctx* ctx, const mixaq_merge_params* p, const float* x, float* y,
@@ -1298,9 +1300,11 @@ mixaq_status mixaq_calibrate_merge(mixaq_ctx* ctx, const mixaq_merge_params* p, 
   Carver cv(workspace);
   CalMergeArgs c;
   c.obs = cv.take<uint32_t>(16);
-  c.ln = cv.take<float>((size_t)B * ((H + 1) / 2) * ((W + 1) / 2) * K);
+  const size_t toks = (size_t)B * ((H + 1) / 2) * ((W + 1) / 2);
+  c.ln = cv.take<float>(toks * K);
+  c.expo = cv.take<int32_t>(toks); c.slices = cv.take<uint8_t>(CAL_SLICES * toks * K);
   c.x = x; c.y = y; c.B = B; c.H = H; c.W = W; c.C = C; c.N = N;
-  c.ln_g = p->ln_g; c.ln_b = p->ln_b; c.w = p->reduction.codes; c.sw = p->reduction.scale; c.w_bits = p->reduction.bits;
+  c.ln_g = p->ln_g; c.ln_b = p->ln_b; c.w = p->reduction.codes; c.sw = p->reduction.scale; c.status = ctx->d_status;
   g_launches = 0;
   if (!launch_calibrate_merge(c, st)) return fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "calibrate_merge: unsupported dim");
   ctx->launches = g_launches;

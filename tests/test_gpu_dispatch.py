@@ -1,5 +1,7 @@
 """The size, width and value ranges between which the library chooses another kernel or another branch of one, at their
 edges: each against the CPU oracle, bit for bit."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -191,3 +193,59 @@ def test_selection_outputs_at_odd_addresses(orc, mq, ctx, H, W):
             assert got[off:end].tobytes() == ref.cpu().numpy().tobytes(), name
             assert (got[:off] == 0xEE).all() and (got[end:] == 0xEE).all(), name
         assert torch.equal(y, want.y)
+
+
+@pytest.mark.parametrize("N,dim", [(52, 32), (31, 32), (200, 64)])
+def test_calibration_products_of_rows_with_a_wide_range(orc, mq, ctx, N, dim):
+    """Rows whose values span 2^-45 to 1 of their largest (bits below 2^-55 of it are rounded away), ragged widths."""
+    rng = np.random.default_rng(N)
+    m = synth.make_merge(rng, dim, 8, 8)
+    m.red = synth.make_linear(rng, N, 4 * dim, 8)
+    m.ln_g = np.exp2(-rng.uniform(0, 45, 4 * dim)).astype(F32)
+    m.ln_b = np.zeros(4 * dim, F32)
+    x = synth.input_student_t(N, 1, 23, 27, dim)
+    params, xd = mq._Dev(ctx.device), dev(x)
+    ms, r = mq.fill_merge_struct(params, m), mq.RangeS()
+    y = torch.empty((1, 12, 14, N), device="cuda")                # (the binding allocates 2 * dim channels)
+    ws = torch.empty(mq.lib().mixaq_calibrate_merge_workspace_bytes(ctypes.byref(ms), 1, 23, 27), dtype=torch.uint8, device="cuda")
+    ctx.check(mq.lib().mixaq_calibrate_merge(ctx.h, ctypes.byref(ms), mq._ptr(xd), mq._ptr(y), 1, 23, 27, ctypes.byref(r), mq._ptr(ws),
+                                             ctypes.c_size_t(ws.numel()), mq._stream_ptr()))
+    want, span = orc.merge_observe_fp(m, x)
+    assert (r.lo, r.hi) == span
+    # per input at most 2^-55 of the row's largest value, the oracle's running sum 2^-53 of sum |a w| per term, one rounding
+    # to binary32 on either side
+    w = np.abs(m.red.codes.astype(np.float64) * m.red.scale[:, None]).sum(1)
+    top = max(abs(span[0]), abs(span[1]))
+    bound = 2.0 ** -23 * np.abs(want) + (2.0 ** -55 + 4 * dim * 2.0 ** -53) * top * w
+    assert (np.abs(y.cpu().numpy().astype(np.float64) - want) <= bound).all()
+    assert ctx.device_status() == 0
+
+
+def test_calibration_products_longer_than_an_int32_sum(orc, mq, ctx):
+    """fc2 over 32 896 hidden channels is drained from the accumulators in two parts."""
+    rng = np.random.default_rng(8)
+    blk = synth.make_block(rng, 32, 1, 0, 8, 8, 4)
+    blk.hidden = 32768 + 128
+    blk.fc1, blk.fc2 = synth.make_linear(rng, blk.hidden, 32, 8), synth.make_linear(rng, 32, blk.hidden, 8)
+    for br in (blk.hi, blk.lo):
+        br.b_fc1 = (0.02 * rng.standard_normal(blk.hidden)).astype(F32)
+    x = synth.input_blobs(5, 1, 7, 7, 32, bg_std=0.5, gain=3.0)
+    params = mq._Dev(ctx.device)
+    y, got = mq.calibrate_block(ctx, mq.fill_block_struct(params, blk), 0, dev(x))
+    want_y, want = orc.block_observe_fp(blk, "hi", x)
+    assert np.array_equal(y.cpu().numpy(), want_y)
+    assert all(got[site] == span for site, span in want.items())
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+def test_calibration_products_of_rows_that_are_not_finite(orc, mq, ctx, value):
+    """A token that is not finite reaches the rows of its window as the plain sums have it, and no others."""
+    blk = synth.make_block(np.random.default_rng(4), 64, 2, 0, 4, 8, 4)
+    x = synth.input_blobs(5, 1, 14, 21, 64, bg_std=0.5, gain=3.0)
+    x[0, 3, 4, 5] = value
+    params = mq._Dev(ctx.device)
+    y, _ = mq.calibrate_block(ctx, mq.fill_block_struct(params, blk), 0, dev(x))
+    want_y, _ = orc.block_observe_fp(blk, "hi", x)
+    assert np.isnan(want_y).any() and np.array_equal(np.isnan(y.cpu().numpy()), np.isnan(want_y))
+    finite = ~np.isnan(want_y)
+    assert np.array_equal(y.cpu().numpy()[finite], want_y[finite])
