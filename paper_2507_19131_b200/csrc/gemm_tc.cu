@@ -107,9 +107,9 @@ struct RingPos {
 
 // TAPS: the accumulator tap is compiled in only for calls that ask for it
 //
-// The loops of the two single threads (TMA, MMA) bound a tile as much as the epilogue does: a thread on its own issues an
-// instruction every 5 to 10 cycles, so the slot and phase divisions and the branch look-ups that used to sit in them cost
-// 1 100 cycles per k-block (stage-1 QKV at 200 x 334 tokens: 17 us of launch without any epilogue work).
+// The loops of the TMA and the MMA warp bound a tile as much as the epilogue does, so they hold no division, and the whole warp
+// walks through them with one elected lane issuing: in code that a single lane runs, an MMA of up to 64 columns takes 63 cycles to
+// issue (its operands go through the uniform registers one by one), elected in a converged warp 46 to 50.
 template <int MODE, bool TAPS, int EW>
 __global__ void __launch_bounds__(num_threads(EW), 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
@@ -127,9 +127,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
   volatile int* beyond_flag = reinterpret_cast<volatile int*>(tmem_holder + 2);
-  // TMA thread: stages that hold a fill, and the phase of the last one, on the full and on the packed-rows barrier
-  // (bit s of each; read by the give-up path only)
-  uint32_t full_used = 0, full_phase = 0, raw_used = 0, raw_phase = 0;
+  // TMA warp: fills of ring stages so far; stages that held packed rows and the phase of the last ones (bit s of each).  Read by
+  // the give-up path only.
+  uint32_t fills = 0, raw_used = 0, raw_phase = 0;
 
   constexpr int NUM_EPI_WARPS = EW;
   constexpr int NUM_UNPACK_WARPS = UNPACK_WARPS, NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
@@ -180,7 +180,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 
   if (warp == 0) {
     // ---- TMA producer ----
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       TileWalk w(p);
       RingPos rp;
       bool ok = true;
@@ -198,34 +199,36 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         for (; w.mt < m_end && ok; w.next(p)) {
           const int m_row = (w.mt - m_first) * BM, n_row = w.nt * BN;
           for (int kb = 0; kb < k_blocks; ++kb, rp.next(ring)) {
-            const uint32_t o = 8u * (uint32_t)rp.slot, bit = 1u << rp.slot;
-            if ((full_used & bit) && !mbar_wait(bar_empty + o, rp.pass ^ 1u, abort_flag)) { ok = false; break; }
+            const uint32_t o = 8u * (uint32_t)rp.slot;
+            if (!mbar_wait(bar_empty + o, rp.pass ^ 1u, abort_flag)) { ok = false; break; }    // (at once in the first pass)
             const uint32_t sa = base + (uint32_t)(rp.slot * stage_bytes), sb = sa + A_STAGE_BYTES;
-            mbar_arrive_expect_tx(bar_full + o, tx);
-            full_used |= bit;
-            full_phase = rp.pass ? full_phase | bit : full_phase & ~bit;
-            tma_load_2d(sb, &tmB, kb * BK, n_row, bar_full + o);
+            ++fills;
+            if (leader) {
+              mbar_arrive_expect_tx(bar_full + o, tx);
+              tma_load_2d(sb, &tmB, kb * BK, n_row, bar_full + o);
+            }
             if (!waited) { griddep_wait(); waited = true; }
-            if (!packed) {
-              tma_load_2d(sa, tmA, kb * BK, m_row, bar_full + o);
-            } else {
+            if (leader && !packed) tma_load_2d(sa, tmA, kb * BK, m_row, bar_full + o);
+            if (packed) {
+              const uint32_t bit = 1u << rp.slot;
               raw_phase = (raw_used & bit) ? raw_phase ^ bit : raw_phase & ~bit;
               raw_used |= bit;
-              if (stage_packed) {
+              if (leader && stage_packed) {
                 mbar_arrive_expect_tx(bar_raw + o, (uint32_t)(pk_row * BM));
                 tma_load_2d(sb + b_bytes, tmA, kb * pk_row, m_row, bar_raw + o);
-              } else {
+              } else if (leader) {
                 mbar_arrive(bar_raw + o);
               }
             }
+            __syncwarp();
           }
         }
       }
     }
-    __syncwarp();
   } else if (warp == 1) {
     // ---- MMA issuer ----
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       const uint64_t adesc0 = smem_desc_sw128(base), bdesc0 = smem_desc_sw128(base + A_STAGE_BYTES);
       const uint32_t stage16 = (uint32_t)stage_bytes >> 4;      // stage pitch in descriptor units
@@ -233,16 +236,15 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
       const int last_steps = (p.g.K - (k_blocks - 1) * BK) / UMMA_K;      // MMAs of the last k-block (4 in the others)
       TileWalk w(p);
       RingPos rp, ap;
-      uint32_t acc_used = 0, unp_next = 0;                      // bit s of unp_next: parity of stage s' next expansion
+      uint32_t unp_next = 0;                                    // bit s: parity of stage s' next expansion
       bool ok = true;
       for (int b = 0; b < 2 && ok; ++b) {
         const int m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
         if (w.mt >= m_end) continue;
         const bool packed = p.g.br[b].a_bits != 8;
         for (; w.mt < m_end && ok; w.next(p), ap.next(n_acc)) {
-          // wait until the epilogue has drained this accumulator (its previous use)
-          if ((acc_used >> ap.slot & 1u) && !mbar_wait(bar_tempty + 8u * ap.slot, ap.pass ^ 1u, abort_flag)) { ok = false; break; }
-          acc_used |= 1u << ap.slot;
+          // wait until the epilogue has drained this accumulator's previous use (at once in the first pass)
+          if (!mbar_wait(bar_tempty + 8u * ap.slot, ap.pass ^ 1u, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t d_tmem = tmem_base + (uint32_t)(ap.slot * p.acc_stride);
           for (int kb = 0; kb < k_blocks; ++kb, rp.next(ring)) {
@@ -256,18 +258,20 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
             const uint64_t so = (uint64_t)((uint32_t)rp.slot * stage16);
             const uint64_t adesc = adesc0 + so, bdesc = bdesc0 + so;
             const int steps = kb == k_blocks - 1 ? last_steps : BK / UMMA_K;
+            if (leader) {
 #pragma unroll
-            for (int kk = 0; kk < BK / UMMA_K; ++kk)
-              if (kk < steps)
-                mma_i8(d_tmem, adesc + (uint64_t)(kk * (UMMA_K >> 4)), bdesc + (uint64_t)(kk * (UMMA_K >> 4)), idesc,
-                       kk > 0 ? 1u : (uint32_t)(kb > 0));
-            mma_commit(bar_empty + o);               // frees the ring slot when these MMAs have read it
+              for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                if (kk < steps)
+                  mma_i8(d_tmem, adesc + (uint64_t)(kk * (UMMA_K >> 4)), bdesc + (uint64_t)(kk * (UMMA_K >> 4)), idesc,
+                         kk > 0 ? 1u : (uint32_t)(kb > 0));
+              mma_commit(bar_empty + o);             // frees the ring slot when these MMAs have read it
+              if (kb == k_blocks - 1) mma_commit(bar_tfull + 8u * ap.slot);    // accumulator complete
+            }
+            __syncwarp();
           }
-          if (ok) mma_commit(bar_tfull + 8u * ap.slot);    // accumulator complete
         }
       }
     }
-    __syncwarp();
   } else if (warp < FIRST_EPI_WARP) {
     // ---- unpack producers: bit-packed rows -> one code per byte, written in the swizzled layout ----
     const int ptid = tid - 64;                   // 0 .. NUM_UNPACK_THREADS-1
@@ -417,8 +421,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
       auto drain = [](uint32_t bar, uint32_t parity) {
         for (uint32_t it = 0; it < (1u << 20); ++it) if (mbar_try_wait(bar, parity)) return;
       };
-      for (int s = 0; s < p.ring; ++s) {
-        if (full_used >> s & 1u) drain(bar_full + 8u * s, full_phase >> s & 1u);
+      for (uint32_t s = 0; s < (uint32_t)p.ring; ++s) {
+        if (fills > s) drain(bar_full + 8u * s, (fills - 1u - s) / (uint32_t)p.ring & 1u);      // pass of the stage's last fill
         if (raw_used >> s & 1u) drain(bar_raw + 8u * s, raw_phase >> s & 1u);
       }
       drain(bar_drain, 0u);

@@ -21,6 +21,12 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// one lane of a converged warp; the compiler knows that the branch on it is taken by one lane
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
 // One try (the hardware suspends the thread for a short, implementation-defined time while the phase is pending;
 // an explicit longer suspend hint measured slower: the waiters sit on the critical path of the small stages).
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
