@@ -30,15 +30,15 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 constexpr int RES_SLOTS = 4;                           // residual chunks a warp keeps in flight (32 x 16 floats each)
 
-// raw + pre[n] is 0x4B400000 + acc: the zero point is taken out, and while |acc| < 2^22 (IN_RANGE) those bits ARE the
+// raw + pre[n] is 0x4B400000 + acc: the zero point is taken out, and while |acc| < 2^22 (NARROW) those bits ARE the
 // binary32 number 1.5 * 2^23 + acc, so one packed subtraction converts two of them.
-template <bool IN_RANGE>
+template <bool NARROW>
 __device__ __forceinline__ float2 acc_to_float2(int32_t a, int32_t b) {
-  if (IN_RANGE) return __fadd2_rn(make_float2(__int_as_float(a), __int_as_float(b)), f2(-12582912.0f));
+  if (NARROW) return __fadd2_rn(make_float2(__int_as_float(a), __int_as_float(b)), f2(-12582912.0f));
   return make_float2(__int2float_rn(a - (int32_t)kMagicBits), __int2float_rn(b - (int32_t)kMagicBits));
 }
 // dequantization of NC columns; lc0 = first column in the warp's constants, n0 = its global index
-template <int MODE, bool TAPS, bool IN_RANGE, int NC>
+template <int MODE, bool TAPS, bool NARROW, int NC>
 __device__ __forceinline__ void dequant(const GemmBranch& br, int N, long m, bool row_ok, int n0, int lc0, const ColConsts& cc,
                                         const int32_t* acc, float (&v)[NC]) {
   if (TAPS && br.tap_acc && row_ok) {
@@ -60,7 +60,7 @@ __device__ __forceinline__ void dequant(const GemmBranch& br, int N, long m, boo
 #pragma unroll
     for (int j = 0; j < 4; j += 2) {
       const int i = 4 * i4 + j;
-      const float2 f = acc_to_float2<IN_RANGE>(acc[i] + pp[j], acc[i + 1] + pp[j + 1]);
+      const float2 f = acc_to_float2<NARROW>(acc[i] + pp[j], acc[i + 1] + pp[j + 1]);
       const float2 r = MODE == EPI_MERGE ? __fmul2_rn(f, make_float2(mm[j], mm[j + 1]))
                                          : __ffma2_rn(f, make_float2(mm[j], mm[j + 1]), make_float2(bb[j], bb[j + 1]));
       v[i] = r.x; v[i + 1] = r.y;
@@ -89,17 +89,17 @@ __device__ __forceinline__ void gelu_pattern2(float2 v, float inv_scale, float m
   const float2 q = gelu_log2_tail2(a);
   const float2 h = __fmul2_rn(a, make_float2(ex2_approx(q.x), ex2_approx(q.y)));
   const float2 g = sub2(make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f)), h);
-  const float2 t = __fmul2_rn(g, f2(inv_scale));
-  const float2 r = __fadd2_rn(t, f2(magic_zp));
-  const float2 d = sub2(t, __fadd2_rn(r, f2(-magic_zp)));
+  const float2 r = __ffma2_rn(g, f2(inv_scale), f2(magic_zp));
+  const float2 n = __fadd2_rn(f2(magic_zp), make_float2(-r.x, -r.y));          // minus the rounded value, exactly
+  const float2 d = __ffma2_rn(g, f2(inv_scale), n);
   dist = fmaxf(fmaxf(dist, fabsf(d.x)), fabsf(d.y));
   m0 = __float_as_uint(r.x); m1 = __float_as_uint(r.y);
 }
-// Error of t = g * inv_scale between the two evaluations: both exponentials are within 2^-22 of 2^q, h = a 2^q <= 0.17, so
-// h differs by at most 0.17 * 2^-21 + one rounding < 1.0e-7; the roundings of g and t add |t| * 2^-22, and |t| <= qmax + 1
-// for every t that is not clamped anyway.
+// Distance of g * inv_scale from the contract's t: both exponentials are within 2^-22 of 2^q, h = a 2^q <= 0.17, so h differs
+// by at most 0.17 * 2^-21 + one rounding < 1.0e-7; g is rounded in both evaluations and t in the contract's, which adds
+// |t| * 3 * 2^-24, and |t| <= qmax + 1 for every t that is not clamped anyway; the distance itself is rounded by 2^-26.
 __device__ __forceinline__ float gelu_threshold(float inv_scale, float qmaxf) {
-  return 0.5f - __fmaf_rn(inv_scale, 1.1e-7f, (qmaxf + 1.0f) * 2.4e-7f);
+  return 0.5f - __fmaf_rn(inv_scale, 1.1e-7f, (qmaxf + 2.0f) * 1.8e-7f);
 }
 
 // What a warp's epilogue needs of its branch, read once per branch (the parameters sit in constant memory, and a tile used
@@ -117,12 +117,13 @@ struct EpiBranch {
 // The warp's part of one output tile.  taddr: TMEM address of (the warp's lane quarter, the tile's first column);
 // n_tile0: global index of that column; the warp owns the tile's chunks c_first, c_first + c_step, ... < c_total
 // cc: the constants of the tile's columns;
+// narrow: no sum of the tile's columns reaches 2^22 (see acc_to_float2);
 // in_range: the code outputs of the tile's columns cannot leave the pattern's range (see quant_pattern2);
 // acc_ready(): waits (bounded) for the tile's accumulator, false when the CTA is giving up.
 template <int MODE, bool TAPS, class WaitFn>
 __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const EpiBranch& eb, int N, int C, long row0, int lane, int n_tile0,
                                                    int c_first, int c_step, int c_total, const ColConsts& cc,
-                                                   uint32_t taddr_tile, float* stage, bool in_range, float neg_zero, WaitFn acc_ready,
+                                                   uint32_t taddr_tile, float* stage, bool narrow, bool in_range, float neg_zero, WaitFn acc_ready,
                                                    float* res_ring = nullptr /* per warp: RES_SLOTS x 32 x 16 floats */) {
   const long m = row0 + lane;
   const bool row_ok = m < eb.M;
@@ -146,40 +147,26 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
     const int out_step = col_step * cbits / 8;
     if (!acc_ready()) return false;
     // the quantizer's width as a constant (a shift in the packing)
-    auto walk = [&](auto bits_tag, auto range_tag) {
+    auto walk = [&](auto bits_tag) {
       constexpr int SH = 8 - decltype(bits_tag)::value;
-      constexpr bool IN_RANGE = decltype(range_tag)::value;
-      // eight columns by the contract's own operations (values out of range, or too close to a rounding boundary)
-      auto exact8 = [&](int col, const int32_t* acc, uint32_t& w0, uint32_t& w1) {
-        float v[8];
-        uint32_t c[8];
-        dequant<MODE, TAPS, IN_RANGE, 8>(br, N, m, row_ok, n_tile0 + col, col, cc, acc, v);
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-          const float2 x = make_float2(v[i], v[i + 1]);
-          quant_magic2(MODE == EPI_FC1 ? gelu_f2(x) : x, inv_scale, -zpf, eb.qmaxf - zpf, c[i], c[i + 1]);
-        }
-        const uint32_t zb = (uint32_t)q.zp - kMagicBits;
-        w0 = sat_pack4<SH>(c[0], c[1], c[2], c[3], zb << SH);
-        w1 = sat_pack4<SH>(c[4], c[5], c[6], c[7], zb << SH);
-      };
       // 32 columns at a time, without a branch between them: the dependent chain of a value is about twenty operations
-      // long, and with four warps per scheduler only independent values hide its latency
+      // long, and with four warps per scheduler only independent values hide its latency.  The accumulator comes in halves of 16
+      // columns, each requested a half ahead, the first one of the next chunk behind the second one of this.
+      int32_t first[CODE_NC / 2], second[CODE_NC / 2];
+      if (n_chunks > 0) tmem_ld(taddr, first);
 #pragma unroll 1
       for (int ch = 0; ch < n_chunks; ++ch) {
         const uint32_t ta = taddr + (uint32_t)(ch * col_step);
         const int col = c_first * CODE_NC + ch * col_step;
-        int32_t acc[CODE_NC];
         uint32_t w[8];
-        tmem_ld(ta, acc);
-        tmem_ld_wait(acc);
         float dist[4];
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-          if (!IN_RANGE) { exact8(col + 8 * g, acc + 8 * g, w[2 * g], w[2 * g + 1]); continue; }
+          if (g == 0) { tmem_ld_wait(first); tmem_ld(ta + CODE_NC / 2, second); }
+          if (g == 2) { tmem_ld_wait(second); if (ch + 1 < n_chunks) tmem_ld(ta + (uint32_t)col_step, first); }
           float v[8];
           uint32_t c[8];
-          dequant<MODE, TAPS, IN_RANGE, 8>(br, N, m, row_ok, n_tile0 + col + 8 * g, col + 8 * g, cc, acc + 8 * g, v);
+          dequant<MODE, TAPS, false, 8>(br, N, m, row_ok, n_tile0 + col + 8 * g, col + 8 * g, cc, (g < 2 ? first : second) + 8 * (g & 1), v);
           dist[g] = 0.0f;
 #pragma unroll
           for (int i = 0; i < 8; i += 2) {
@@ -189,35 +176,39 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
           w[2 * g] = sat_pack4<SH>(c[0], c[1], c[2], c[3], zbias << SH);
           w[2 * g + 1] = sat_pack4<SH>(c[4], c[5], c[6], c[7], zbias << SH);
         }
-        if (MODE == EPI_FC1 && IN_RANGE) {
-          // some value of the warp too close to a rounding boundary (a sixth of the chunks at A8): its eight columns again
-          const bool near = fmaxf(fmaxf(dist[0], dist[1]), fmaxf(dist[2], dist[3])) >= thr;
-          if (__any_sync(0xffffffffu, near)) {
+        // Eight columns again by the contract's own operations: where some value of the warp is too close to a rounding boundary
+        // (FC1, a sixth of the chunks at A8), and all of them where the patterns above do not hold
+        const bool near = MODE == EPI_FC1 && fmaxf(fmaxf(dist[0], dist[1]), fmaxf(dist[2], dist[3])) >= thr;
+        if (!in_range || (MODE == EPI_FC1 && __any_sync(0xffffffffu, near))) {
 #pragma unroll 1
-            for (int g = 0; g < 4; ++g) {
-              const float d = g == 0 ? dist[0] : g == 1 ? dist[1] : g == 2 ? dist[2] : dist[3];
-              if (!__any_sync(0xffffffffu, d >= thr)) continue;
-              int32_t again[8];
-              uint32_t w0, w1;
-              tmem_ld(ta + (uint32_t)(8 * g), again);
-              tmem_ld_wait(again);
-              exact8(col + 8 * g, again, w0, w1);
-              w[0] = g == 0 ? w0 : w[0]; w[1] = g == 0 ? w1 : w[1];
-              w[2] = g == 1 ? w0 : w[2]; w[3] = g == 1 ? w1 : w[3];
-              w[4] = g == 2 ? w0 : w[4]; w[5] = g == 2 ? w1 : w[5];
-              w[6] = g == 3 ? w0 : w[6]; w[7] = g == 3 ? w1 : w[7];
+          for (int g = 0; g < 4; ++g) {
+            const float d = g == 0 ? dist[0] : g == 1 ? dist[1] : g == 2 ? dist[2] : dist[3];
+            if (in_range && !__any_sync(0xffffffffu, d >= thr)) continue;
+            int32_t again[8];
+            tmem_ld(ta + (uint32_t)(8 * g), again);
+            tmem_ld_wait(again);
+            float v[8];
+            uint32_t c[8];
+            dequant<MODE, TAPS, false, 8>(br, N, m, row_ok, n_tile0 + col + 8 * g, col + 8 * g, cc, again, v);
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+              const float2 x = make_float2(v[i], v[i + 1]);
+              quant_magic2(MODE == EPI_FC1 ? gelu_f2(x) : x, inv_scale, -zpf, eb.qmaxf - zpf, c[i], c[i + 1]);
             }
+            const uint32_t zb = (uint32_t)q.zp - kMagicBits;
+            const uint32_t w0 = sat_pack4<SH>(c[0], c[1], c[2], c[3], zb << SH), w1 = sat_pack4<SH>(c[4], c[5], c[6], c[7], zb << SH);
+            w[0] = g == 0 ? w0 : w[0]; w[1] = g == 0 ? w1 : w[1];
+            w[2] = g == 1 ? w0 : w[2]; w[3] = g == 1 ? w1 : w[3];
+            w[4] = g == 2 ? w0 : w[4]; w[5] = g == 2 ? w1 : w[5];
+            w[6] = g == 3 ? w0 : w[6]; w[7] = g == 3 ? w1 : w[7];
           }
         }
         if (row_ok) store_sat32(out_ptr + ch * out_step, w, bits, cbits);
       }
     };
-    auto walk_bits = [&](auto range_tag) {
-      if (bits == 8) walk(std::integral_constant<int, 8>{}, range_tag);
-      else if (bits == 4) walk(std::integral_constant<int, 4>{}, range_tag);
-      else walk(std::integral_constant<int, 2>{}, range_tag);
-    };
-    if (in_range) walk_bits(std::true_type{}); else walk_bits(std::false_type{});
+    if (bits == 8) walk(std::integral_constant<int, 8>{});
+    else if (bits == 4) walk(std::integral_constant<int, 4>{});
+    else walk(std::integral_constant<int, 2>{});
     return true;
   }
 
@@ -269,8 +260,8 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
     for (int ch = 0; ch < RES_SLOTS; ++ch) fetch(ch);
   }
   if (!acc_ready()) { cp_async_wait<0>(); return false; }
-  auto walk = [&](auto range_tag) {
-    constexpr bool IN_RANGE = decltype(range_tag)::value;
+  auto walk = [&](auto narrow_tag) {
+    constexpr bool NARROW = decltype(narrow_tag)::value;
     int32_t acc[F32_NC];
     if (n_chunks > 0) tmem_ld(taddr, acc);
 #pragma unroll 1
@@ -302,7 +293,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
           tp[2] = a.z + p4.z - (int32_t)kMagicBits; tp[3] = a.w + p4.w - (int32_t)kMagicBits;
         }
         if (!dst_ptr[i]) continue;
-        const float2 f0 = acc_to_float2<IN_RANGE>(a.x + p4.x, a.y + p4.y), f1 = acc_to_float2<IN_RANGE>(a.z + p4.z, a.w + p4.w);
+        const float2 f0 = acc_to_float2<NARROW>(a.x + p4.x, a.y + p4.y), f1 = acc_to_float2<NARROW>(a.z + p4.z, a.w + p4.w);
         float2 lo, hi;
         if (MODE == EPI_MERGE) {
           lo = __fmul2_rn(f0, make_float2(m4.x, m4.y)); hi = __fmul2_rn(f1, make_float2(m4.z, m4.w));
@@ -317,7 +308,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
       if (MODE != EPI_MERGE) fetch(ch + RES_SLOTS);              // the slot just read is free again
     }
   };
-  if (in_range) walk(std::true_type{}); else walk(std::false_type{});
+  if (narrow) walk(std::true_type{}); else walk(std::false_type{});
   if (MODE != EPI_MERGE) cp_async_wait<0>();                   // nothing of this tile is left in flight
   return true;
 }

@@ -8,7 +8,7 @@
 //               128-byte-swizzled K-major stages (cp.async.bulk.tensor, no multicast), completion on mbarriers;
 //   warp 1      MMA issuer: one thread feeds the tensor core; the tiles take turns on up to six TMEM accumulators, so
 //               that the epilogue of a tile overlaps the loads and MMAs of the following ones;
-//   warps 2-5   unpack producers for 4-bit / 2-bit branches: the bit-packed rows of the k-block arrive by TMA in a
+//   warps 4-7   unpack producers for 4-bit / 2-bit branches: the bit-packed rows of the k-block arrive by TMA in a
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
 //               the swizzled layout (rows whose byte pitch is no multiple of 16 cannot be described to the TMA
 //               unit and are read with plain loads instead);
@@ -37,7 +37,7 @@ constexpr int BM = 128;            // rows per tile = TMEM lanes
 constexpr int BK = 128;            // codes (bytes) per row and stage = one 128-byte swizzle row
 constexpr int UMMA_K = 32;         // codes per tcgen05.mma kind::i8
 constexpr int A_STAGE_BYTES = BM * BK;
-// warps 2..5 expand sub-byte codes (two warps left the long-K main loops of 4-bit tiles waiting for the expansion;
+// warps 4..7 expand sub-byte codes (two warps left the long-K main loops of 4-bit tiles waiting for the expansion;
 // eight cost more registers than they return)
 constexpr int UNPACK_WARPS = 4;
 // Epilogue warps.  Binary32 outputs: 8.  Code outputs: 12; fc1, whose GELU makes it the longest, 16 where every SM has two row
@@ -47,7 +47,13 @@ constexpr int UNPACK_WARPS = 4;
 // element, is faster with 12 everywhere (C = 128 at 2 x 384 x 384: 63 us against 68).
 constexpr int F32_WARPS = 8, CODE_WARPS = 12, CODE_WARPS_MANY = 16;
 constexpr int MANY_ROW_TILES = 2;              // row tiles per SM from which fc1 has CODE_WARPS_MANY
-__host__ __device__ constexpr int num_threads(int warps) { return 32 * (2 + UNPACK_WARPS + warps); }
+constexpr int FIRST_UNPACK_WARP = 4, FIRST_EPI_WARP = 8;        // warpgroups: TMA, MMA and TMEM set-up; unpack; epilogue
+__host__ __device__ constexpr int num_threads(int warps) { return 32 * (FIRST_EPI_WARP + warps); }
+// Registers.  A block is launched with what its threads divide the file into (80 a thread with 16 epilogue warps, 96 with 12); the
+// first two warpgroups give back all but SIDE_REGS and the epilogue warps of the code outputs take them.  gemm_init checks that
+// the shares fit into what the compiled kernels are launched with.
+constexpr int SIDE_REGS = 40;
+__host__ __device__ constexpr int epi_regs(int warps) { return warps == 16 ? 96 : warps == 12 ? 128 : 0; }     // 0: no exchange
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
 constexpr int MAX_RING = 6;
@@ -84,7 +90,7 @@ __host__ __device__ inline SmemLayout smem_layout(int BN, int ring, int packed_b
   L.stage_off = L.consts_off + 3 * const_cols * 4;    // binary32 epilogues: a 32 x 16 chunk per warp
   L.res_off = L.stage_off + (code_mode(mode) ? 0 : warps * EPI_STAGE_FLOATS * 4);   // and their residual rings
   L.bars_off = L.res_off + res_bytes;
-  L.total = L.bars_off + NUM_BARS * 8 + 16;                     // then TMEM base, abort flag, constants-out-of-range flag
+  L.total = L.bars_off + NUM_BARS * 8 + 16;                     // then TMEM base, abort flag, constants-out-of-range flags
   return L;
 }
 
@@ -126,14 +132,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   const uint32_t bar_tempty = bar_tfull + 8u * MAX_ACC, bar_consts = bar_tempty + 8u * MAX_ACC, bar_drain = bar_consts + 8u;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  volatile int* beyond_flag = reinterpret_cast<volatile int*>(tmem_holder + 2);
+  int* beyond_flags = reinterpret_cast<int*>(tmem_holder + 2);       // bit 0: some sum may reach 2^22; bit 1: some pattern its range
   // TMA warp: fills of ring stages so far; stages that held packed rows and the phase of the last ones (bit s of each).  Read by
   // the give-up path only.
   uint32_t fills = 0, raw_used = 0, raw_phase = 0;
 
   constexpr int NUM_EPI_WARPS = EW;
   constexpr int NUM_UNPACK_WARPS = UNPACK_WARPS, NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
-  constexpr int FIRST_EPI_WARP = 2 + NUM_UNPACK_WARPS;
   constexpr int UNPACK_ITEMS = BM * (BK / UMMA_K) / NUM_UNPACK_THREADS;   // (row, 32-code group) items per thread and stage
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -162,7 +167,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
       mbar_init(bar_tempty + 8u * a, 4u * (uint32_t)p.split);   // one arrival per epilogue warp of a group
     }
     mbar_init(bar_consts, NUM_EPI_WARPS);                       // constants of a branch: loaded / no longer in use
-    *beyond_flag = 0;
+    *beyond_flags = 0;
     mbar_init(bar_drain, 1u);                                   // tcgen05.commit of the give-up path
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -180,6 +185,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 
   if (warp == 0) {
     // ---- TMA producer ----
+    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     {
       const bool leader = elect_one();
       TileWalk w(p);
@@ -227,6 +233,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     }
   } else if (warp == 1) {
     // ---- MMA issuer ----
+    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     {
       const bool leader = elect_one();
       const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
@@ -272,9 +279,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         }
       }
     }
+  } else if (warp < FIRST_UNPACK_WARP) {
+    // (warps 2 and 3 fill up the warpgroup)
+    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
   } else if (warp < FIRST_EPI_WARP) {
     // ---- unpack producers: bit-packed rows -> one code per byte, written in the swizzled layout ----
-    const int ptid = tid - 64;                   // 0 .. NUM_UNPACK_THREADS-1
+    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
+    const int ptid = tid - 32 * FIRST_UNPACK_WARP;   // 0 .. NUM_UNPACK_THREADS-1
     TileWalk w(p);
     int slot = 0;
     uint32_t raw_next = 0;                       // bit s: parity of stage s' next packed fill
@@ -335,6 +346,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     __syncwarp();
   } else {
     // ---- epilogue warps: warp e reads TMEM lanes 32*(e%4).. of its group's tiles, every split-th chunk ----
+    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(epi_regs(EW) > 0 ? epi_regs(EW) : 24));
     const int e = warp - FIRST_EPI_WARP, q = warp & 3;         // any 4 consecutive warps cover the 4 lane quarters
     const int split = p.split, groups = p.groups, group = (e >> 2) / split, sub = (e >> 2) - group * split;
     float* stage = reinterpret_cast<float*>(smem + L.stage_off) + e * EPI_STAGE_FLOATS;
@@ -357,7 +369,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     const int last_mt = (int)(blockIdx.x + (unsigned)(p.last_step - (int)blockIdx.x) / gridDim.x * gridDim.x) / p.n_tiles;
     uint32_t consts_pass = 0;
     bool waited = false;
-    bool in_range = false;                                     // the patterns of these columns stay in range
+    bool narrow = false, in_range = false;                     // sums and patterns of these columns stay in range
     auto all_warps = [&]() -> bool {
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_consts);
@@ -371,7 +383,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
       const GemmBranch& br = p.g.br[b];
       const EpiBranch eb(br, p.g.N);
       if (b == 1 && first_mt < p.tiles_m0 && !all_warps()) { ok = false; break; }      // everybody is done with the first branch's
-      bool fits = true;
+      int beyond = 0;
       for (int i = e * 32 + lane; i < p.const_cols; i += NUM_EPI_WARPS * 32) {
         const int n = const_first + i;
         const float bias = MODE != EPI_MERGE ? __ldg(br.bias + n) : 0.0f, bound = __ldg(br.bound + n);
@@ -379,12 +391,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         c_mult[i] = __ldg(br.mult + n);
         c_bias[i] = bias;
         const float inv = !code_mode(MODE) ? 0.0f : MODE == EPI_FC1 || n < p.g.C ? br.q0.inv_scale : (n < 2 * p.g.C ? br.q1.inv_scale : br.q2.inv_scale);
-        fits &= code_mode(MODE) ? (bound + fabsf(bias)) * inv < kPatternRange : bound < INFINITY;
+        beyond |= bound < 0.0f ? 1 : 0;
+        beyond |= code_mode(MODE) && !((fabsf(bound) + fabsf(bias)) * inv < kPatternRange) ? 2 : 0;
       }
-      if (!fits) *beyond_flag = b + 1;                          // (a branch out of range takes the next one along: it is only slower)
+      if (beyond) atomicOr(beyond_flags, beyond);               // (a branch out of range takes the next one along: it is only slower)
       if (!all_warps()) { ok = false; break; }
       if (!waited) { griddep_wait(); waited = true; }           // residuals, row indices and outputs belong to earlier kernels
-      in_range = *beyond_flag == 0;
+      const int flags = *reinterpret_cast<volatile int*>(beyond_flags);
+      narrow = (flags & 1) == 0; in_range = (flags & 2) == 0;
       for (; w.mt < m_end; step(w)) {
         const int n_tile0 = w.nt * p.BN;
         const int c0 = n_tile0 - const_first;
@@ -396,7 +410,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
           return true;
         };
         if (!epilogue_warp_tile<MODE, TAPS>(br, eb, p.g.N, p.g.C, row0, lane, n_tile0, sub, split, c_total, cc,
-                                            tmem_q + (uint32_t)(acc * p.acc_stride), stage, in_range, p.g.neg_zero,
+                                            tmem_q + (uint32_t)(acc * p.acc_stride), stage, narrow, in_range, p.g.neg_zero,
                                             acc_ready, res_ring)) { ok = false; break; }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -651,6 +665,14 @@ int launch_mma_peak(int kind, int groups, unsigned long long* ns_out, int* statu
 bool gemm_init() {
   bool ok = encode_fn() != nullptr && sm_count() > 0;
   auto big_smem = [&](auto kernel) { ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess; };
+  // the register shares of the code epilogues have to add up to no more than the block is launched with
+  auto regs_fit = [&](auto kernel, int warps) {
+    cudaFuncAttributes a;
+    ok &= cudaFuncGetAttributes(&a, kernel) == cudaSuccess && FIRST_EPI_WARP * SIDE_REGS + warps * epi_regs(warps) <= (FIRST_EPI_WARP + warps) * a.numRegs;
+  };
+  regs_fit(k_gemm_tc<EPI_QKV, false, CODE_WARPS>, CODE_WARPS); regs_fit(k_gemm_tc<EPI_QKV, true, CODE_WARPS>, CODE_WARPS);
+  regs_fit(k_gemm_tc<EPI_FC1, false, CODE_WARPS>, CODE_WARPS); regs_fit(k_gemm_tc<EPI_FC1, true, CODE_WARPS>, CODE_WARPS);
+  regs_fit(k_gemm_tc<EPI_FC1, false, CODE_WARPS_MANY>, CODE_WARPS_MANY); regs_fit(k_gemm_tc<EPI_FC1, true, CODE_WARPS_MANY>, CODE_WARPS_MANY);
   big_smem(k_gemm_tc<EPI_QKV, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_QKV, true, CODE_WARPS>);
   big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS>);
   big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS_MANY>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS_MANY>);

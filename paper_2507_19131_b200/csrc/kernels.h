@@ -84,7 +84,7 @@ struct GemmBranch {
   const float* mult;         // [N]  s_a * s_w[n]
   const int32_t* pre;        // [N]  0x4B400000 - z_a * sum_k w[n][k]
   const float* bias;         // [N]  (nullable for EPI_MERGE)
-  const float* bound;        // [N]  largest |acc * mult| the channel can reach (see k_prepare_linear)
+  const float* bound;        // [N]  largest |acc * mult| the channel can reach, negative: |acc| may reach 2^22 (see k_prepare_linear)
   AQ q0, q1, q2;             // output quantizers (QKV: q,k,v; FC1: q0)
   int out_bits;
   uint8_t* out_codes;        // QKV, FC1: [M][N*out_bits/8]

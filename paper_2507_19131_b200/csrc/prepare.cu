@@ -1,31 +1,34 @@
 // One-time derived tables of a block: per-output-channel step-size products and zero-point corrections of
 // every (linear layer, branch) pair, and the relative-position bias expanded to the attention kernel's fragment order.
 #include "kernels.h"
+#include <cfloat>
 
 namespace mixaq {
 
 // one warp per output channel: mult[n] = s_a * s_w[n];
 // pre[n] = 0x4B400000 - z_a * sum_k w[n][k], what the GEMM's epilogue adds to the raw sums (see acc_to_float2);
-// bound[n]: no dequantized sum |mult * acc| exceeds it (|a - z_a| <= qmax_a, so |acc| <= qmax_a * sum_k |w[n][k]|), or
-// infinity where |acc| could reach the 2^22 that this leaves room for.
+// bound[n]: no dequantized sum |mult * acc| exceeds its magnitude; negative where |acc| could reach the 2^22 that `pre` leaves
+// room for.  The codes lie in 0 .. qmax, so acc = sum_k w (a - z) is largest with a = qmax where w > 0 and a = 0 elsewhere, and
+// smallest the other way round: half of qmax * sum |w| for a zero point in the middle of the range or weights of either sign alike.
 __global__ void __launch_bounds__(256) k_prepare_linear(const int8_t* __restrict__ w, const float* __restrict__ sw,
                                                         int N, int K, float sa, int za, int qmax, float* mult, int32_t* pre,
                                                         float* bound) {
   int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
   if (n >= N) return;
-  int s = 0, sabs = 0;
-  for (int k = lane; k < K; k += 32) { const int c = (int)w[(long)n * K + k]; s += c; sabs += c < 0 ? -c : c; }
+  int up = 0, down = 0;                                     // sum of the positive weights, of the negative ones
+  for (int k = lane; k < K; k += 32) { const int c = (int)w[(long)n * K + k]; up += c > 0 ? c : 0; down += c < 0 ? -c : 0; }
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, off);
-    sabs += __shfl_xor_sync(0xffffffffu, sabs, off);
+    up += __shfl_xor_sync(0xffffffffu, up, off);
+    down += __shfl_xor_sync(0xffffffffu, down, off);
   }
   if (lane == 0) {
-    pre[n] = (int32_t)(kMagicBits - (uint32_t)(za * s));
+    pre[n] = (int32_t)(kMagicBits - (uint32_t)(za * (up - down)));
     mult[n] = __fmul_rn(sa, sw[n]);
-    const long most = (long)qmax * sabs;
-    bound[n] = most < (1L << 22) - 16 ? fabsf(mult[n]) * (float)most * 1.0001f : INFINITY;
+    const long hi = (long)up * (qmax - za) + (long)down * za, lo = (long)up * za + (long)down * (qmax - za), most = hi > lo ? hi : lo;
+    const float limit = fabsf(mult[n]) * (float)most * 1.0001f;
+    bound[n] = most < (1L << 22) - 16 ? limit : -fmaxf(limit, FLT_MIN);
   }
 }
 
