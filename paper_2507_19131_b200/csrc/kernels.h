@@ -37,6 +37,7 @@ struct SelectArgs {
   int32_t* win_hi;           // [B*n_hi] window index of every batch slot
   int32_t* win_lo;           // [B*n_lo]
   int B, H, W, shift, nwx, nW, n_hi, n_lo, n_pr, reverse;
+  bool narrow;               // the energies are the library's own: scores are below 2^31
 };
 // selections of `count` blocks that share one energy map (all blocks of a stage): 2 launches per 24 blocks
 void launch_select(const SelectArgs* a, int count, cudaStream_t st);

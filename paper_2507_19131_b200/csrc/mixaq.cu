@@ -299,13 +299,13 @@ BlockWs carve_block(const mixaq_block_params* p, int B, int H, int W, void* base
 }
 
 SelectArgs make_select_args(const SelWs& sel, const int32_t* energy, int B, int H, int W, int shift, const Geometry& g,
-                            int reverse) {
+                            int reverse, bool own_energy) {
   SelectArgs sa;
   sa.energy = energy; sa.score = sel.score; sa.order = sel.order; sa.cls = sel.cls;
   sa.rowsrc_hi = sel.rowsrc[0]; sa.rowsrc_lo = sel.rowsrc[1]; sa.rowsrc_pr = sel.rowsrc[2];
   sa.win_hi = sel.win[0]; sa.win_lo = sel.win[1];
   sa.B = B; sa.H = H; sa.W = W; sa.shift = shift; sa.nwx = g.nwx; sa.nW = g.nW;
-  sa.n_hi = g.n_hi; sa.n_lo = g.n_lo; sa.n_pr = g.n_pr; sa.reverse = reverse;
+  sa.n_hi = g.n_hi; sa.n_lo = g.n_lo; sa.n_pr = g.n_pr; sa.reverse = reverse; sa.narrow = own_energy;
   return sa;
 }
 
@@ -570,7 +570,7 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   if (!presel) {
     const int32_t* energy = opts ? opts->energy : nullptr;
     if (!energy) { PROF(PC_ENERGY); launch_energy(x, ws.energy, (long)B * H * W, C, p->score_inv_scale, st); energy = ws.energy; }
-    SelectArgs sa = make_select_args(sel, energy, B, H, W, p->shift, g, opts ? opts->reverse : 0);
+    SelectArgs sa = make_select_args(sel, energy, B, H, W, p->shift, g, opts ? opts->reverse : 0, energy == ws.energy);
     { PROF(PC_SELECT); launch_select(&sa, 1, st); }
   }
   if (sel_out) {
@@ -930,7 +930,7 @@ mixaq_status issue_backbone(mixaq_ctx* ctx, const BackboneCall& c, bool recordin
       Geometry g = geometry(H, W, lr, pr);
       if ((size_t)g.nW * 8 > 48 * 1024) { result = fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "too many windows per image (max 6144)"); break; }
       sels[i] = carve_sel(B, H, W, ws.sel + (size_t)i * sel_stride);
-      sargs[i] = make_select_args(sels[i], ws.energy, B, H, W, p->blocks[blk + i].shift, g, ctx->reverse_selection ? 1 : 0);
+      sargs[i] = make_select_args(sels[i], ws.energy, B, H, W, p->blocks[blk + i].shift, g, ctx->reverse_selection ? 1 : 0, true);
     }
     if (result != MIXAQ_OK) break;
     g_launches = 0;

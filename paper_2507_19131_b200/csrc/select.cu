@@ -1,6 +1,7 @@
 // Window importance scoring and ratio-driven selection (MixA-Q Section 3.2; pruned class: Section 3.4).
 // Integer work throughout: int8 score codes, int32 token energies, int64 window scores, ranks by counting.
 #include "kernels.h"
+#include <climits>
 
 namespace mixaq {
 
@@ -69,16 +70,29 @@ __global__ void __launch_bounds__(256) k_window_score(const __grid_constant__ Se
   if (lane == 0) a.score[gw] = s;
 }
 
-// Rank of window w among the scores of its image, and the bookkeeping of its slot (by one warp)
-__device__ __forceinline__ void emit_window(const SelectArgs& a, int b, int w, const long long* s_score, int lane, int Hp, int Wp) {
-  const long long mine = s_score[w];
+// How many windows of an image precede window w in (score descending, index ascending), by one warp.  key: the scores in shared
+// memory (negated for the ascending order), n4 groups of four, padded with the lowest value.  Windows before w precede it with an
+// equal score too; a lane compares four per load.
+template <class Key>
+__device__ __forceinline__ int count_preceding(const Key* key, int n4, int w, int lane) {
+  struct alignas(4 * sizeof(Key)) Four { Key k[4]; };
+  const Four* four = reinterpret_cast<const Four*>(key);
+  const Key mine = key[w];
   int cnt = 0;
-  if (!a.reverse) {
-    for (int v = lane; v < a.nW; v += 32) { long long o = s_score[v]; cnt += (o > mine) || (o == mine && v < w); }
-  } else {
-    for (int v = lane; v < a.nW; v += 32) { long long o = s_score[v]; cnt += (o < mine) || (o == mine && v < w); }
+  for (int i = lane; i < n4; i += 32) {
+    const Four o = four[i];
+    // (the group that holds w: those from w on have to exceed it)
+    const Key at_least = 4 * i + 3 < w ? mine : mine + 1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cnt += o.k[j] >= at_least ? 1 : 0;
+    if (i == w >> 2)
+      for (int j = 0; j < 4; ++j) cnt += 4 * i + j < w && o.k[j] == mine ? 1 : 0;
   }
-  const int rank = __reduce_add_sync(0xffffffffu, cnt);
+  return __reduce_add_sync(0xffffffffu, cnt);
+}
+
+// The bookkeeping of the slot that window w takes with its rank (by one warp)
+__device__ __forceinline__ void emit_window(const SelectArgs& a, int b, int w, int rank, int lane, int Hp, int Wp) {
   const int c = rank < a.n_hi ? 0 : (rank < a.n_hi + a.n_lo ? 1 : 2);
   int32_t* dst; long slot;
   if (c == 0)      { slot = (long)b * a.n_hi + rank;                     dst = a.rowsrc_hi; }
@@ -93,23 +107,28 @@ __device__ __forceinline__ void emit_window(const SelectArgs& a, int b, int w, c
   for (int t = lane; t < WT; t += 32) dst[slot * WT + t] = window_src(b, a.H, a.W, Hp, Wp, a.shift, a.nwx, w, t);
 }
 
-// Rank by counting: rank(w) = #{v : v precedes w in (score desc, index asc)}; ranks are a permutation.
-// One warp per window: the lanes split the windows to compare against, the counts are summed over the warp,
-// and the lanes then write the batch bookkeeping of the window's slot (49 source-token indices) together.
+// Rank by counting: ranks are a permutation.  One warp per window: the lanes split the windows to compare against, and then
+// write the batch bookkeeping of the window's slot (49 source-token indices) together.  Bound by the comparisons (n^2 per image),
+// so scores that fit are compared as 32-bit numbers: every score made of the library's own energies does (at most
+// 49 x 1024 x 127^2); a caller's energies may not.
 constexpr int RANK_WARPS = 8;
 __global__ void __launch_bounds__(RANK_WARPS * 32) k_rank_emit(const __grid_constant__ SelectBatch batch) {
   griddep_launch();
   griddep_wait();
-  extern __shared__ long long s_score[];
+  extern __shared__ __align__(32) unsigned char s_keys[];
   const SelectArgs& a = batch.a[blockIdx.z];
-  const int b = blockIdx.y;
+  const int b = blockIdx.y, n4 = (a.nW + 3) / 4;
   const int64_t* sc = a.score + (long)b * a.nW;
-  for (int i = threadIdx.x; i < a.nW; i += blockDim.x) s_score[i] = sc[i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int w = blockIdx.x * RANK_WARPS + (threadIdx.x >> 5);
-  if (w >= a.nW) return;
-  emit_window(a, b, w, s_score, lane, (a.H + WS - 1) / WS * WS, (a.W + WS - 1) / WS * WS);
+  const int lane = threadIdx.x & 31, w = blockIdx.x * RANK_WARPS + (threadIdx.x >> 5);
+  const int Hp = (a.H + WS - 1) / WS * WS, Wp = (a.W + WS - 1) / WS * WS;
+  auto rank_with = [&](auto* key, auto lowest) {
+    for (int i = threadIdx.x; i < 4 * n4; i += blockDim.x)
+      key[i] = i < a.nW ? (decltype(lowest))(a.reverse ? -sc[i] : sc[i]) : lowest;
+    __syncthreads();
+    if (w < a.nW) emit_window(a, b, w, count_preceding(key, n4, w, lane), lane, Hp, Wp);
+  };
+  if (a.narrow) rank_with(reinterpret_cast<int*>(s_keys), (int)INT_MIN);
+  else rank_with(reinterpret_cast<long long*>(s_keys), (long long)LLONG_MIN);
 }
 
 // Score, rank and bookkeeping of one (image, block) in one CTA with a warp per window, for images of at most 32 windows:
@@ -119,7 +138,7 @@ __global__ void __launch_bounds__(RANK_WARPS * 32) k_rank_emit(const __grid_cons
 // images and the 18 blocks of a deep stage in one launch is the single kernel still 2 us faster up to 64 windows.)
 constexpr int SMALL_WINDOWS = 32;
 __global__ void __launch_bounds__(SMALL_WINDOWS * 32) k_select_small(const __grid_constant__ SelectBatch batch) {
-  __shared__ long long s_score[SMALL_WINDOWS];
+  __shared__ __align__(32) long long s_score[SMALL_WINDOWS];
   griddep_wait();
   griddep_launch();
   const SelectArgs& a = batch.a[blockIdx.y];
@@ -133,28 +152,43 @@ __global__ void __launch_bounds__(SMALL_WINDOWS * 32) k_select_small(const __gri
     }
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) { s_score[w] = s; a.score[(long)b * a.nW + w] = s; }
+    if (lane == 0) { s_score[w] = a.reverse ? -s : s; a.score[(long)b * a.nW + w] = s; }
+  } else if (lane == 0) {
+    s_score[w] = LLONG_MIN;
   }
   __syncthreads();
-  if (w < a.nW) emit_window(a, b, w, s_score, lane, Hp, Wp);
+  if (w < a.nW) emit_window(a, b, w, count_preceding(s_score, SMALL_WINDOWS / 4, w, lane), lane, Hp, Wp);
 }
 
-// One warp per (image, class): walks the windows in ascending index, 32 at a time, and appends the members of its class
-// (order-preserving compaction by ballot).
+// One CTA per image: every warp takes a run of windows, counts the members of the three classes in it, and writes them behind those
+// of the warps before it (order-preserving compaction by ballot).  One warp per class took 25 us at 3 025 windows.
+constexpr int LIST_WARPS = 32;
 struct ClassListArgs { const uint8_t* cls; int32_t* out[3]; int count[3]; int B, nW; };
-__global__ void __launch_bounds__(96) k_class_lists(ClassListArgs a) {
-  const int b = blockIdx.x, c = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int32_t* out = a.out[c];
-  if (!out) return;
-  out += (long)b * a.count[c];
+__global__ void __launch_bounds__(LIST_WARPS * 32) k_class_lists(ClassListArgs a) {
+  __shared__ int s_count[3][LIST_WARPS];
+  griddep_launch();
+  griddep_wait();
+  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint8_t* cls = a.cls + (long)b * a.nW;
-  int base = 0;
-  for (int w0 = 0; w0 < a.nW; w0 += 32) {
-    const int w = w0 + lane;
-    const bool mine = w < a.nW && cls[w] == c;
-    const unsigned m = __ballot_sync(0xffffffffu, mine);
-    if (mine) out[base + __popc(m & ((1u << lane) - 1u))] = w;
-    base += __popc(m);
+  const int per = ((a.nW + LIST_WARPS - 1) / LIST_WARPS + 31) / 32 * 32, first = warp * per, end = min(a.nW, first + per);
+  int base[3] = {0, 0, 0};
+  for (int w0 = first; w0 < end; w0 += 32) {
+    const int c = w0 + lane < end ? cls[w0 + lane] : 3;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) base[k] += __popc(__ballot_sync(0xffffffffu, c == k));
+  }
+  if (lane < 3) s_count[lane][warp] = lane == 0 ? base[0] : lane == 1 ? base[1] : base[2];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) base[k] = __reduce_add_sync(0xffffffffu, lane < warp ? s_count[k][lane] : 0);
+  for (int w0 = first; w0 < end; w0 += 32) {
+    const int c = w0 + lane < end ? cls[w0 + lane] : 3;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const unsigned m = __ballot_sync(0xffffffffu, c == k);
+      if (c == k && a.out[k]) a.out[k][(long)b * a.count[k] + base[k] + __popc(m & ((1u << lane) - 1u))] = w0 + lane;
+      base[k] += __popc(m);
+    }
   }
 }
 
@@ -162,7 +196,7 @@ void launch_class_lists(const uint8_t* cls, int B, int nW, int32_t* const out[3]
   ClassListArgs a;
   a.cls = cls; a.B = B; a.nW = nW;
   for (int c = 0; c < 3; ++c) { a.out[c] = out[c]; a.count[c] = count[c]; }
-  k_class_lists<<<B, 96, 0, st>>>(a);
+  launch_pdl(k_class_lists, dim3(B), LIST_WARPS * 32, 0, st, a);
   ++g_launches;
 }
 
@@ -188,7 +222,7 @@ void launch_select(const SelectArgs* args, int count, cudaStream_t st) {
     launch_pdl(k_window_score, dim3((nwin + 7) / 8, n), 256, 0, st, batch);
     ++g_launches;
     dim3 grid((a.nW + RANK_WARPS - 1) / RANK_WARPS, a.B, n);
-    launch_pdl(k_rank_emit, grid, RANK_WARPS * 32, (size_t)a.nW * sizeof(long long), st, batch);
+    launch_pdl(k_rank_emit, grid, RANK_WARPS * 32, (size_t)(a.nW + 3) / 4 * 4 * sizeof(long long), st, batch);
     ++g_launches;
   }
 }
