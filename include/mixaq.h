@@ -76,14 +76,13 @@ typedef struct {
   float score_inv_scale;                  /* score code = clamp(rne(x * score_inv_scale), -127, 127)       */
   void* prepared;                         /* device buffer of mixaq_block_prepared_bytes(), filled once by */
                                           /* mixaq_block_prepare(); read by every forward call             */
-  int byte_codes;                         /* storage of the block's intermediate activation codes in the workspace.
-                                             0: bit-packed at the branch's bit width (the default; a 4-bit branch
-                                             moves half the bytes of an 8-bit one).  1: one code per byte whatever
-                                             the bit width -- the same code values in [0, 2^bits), no expansion in
-                                             shared memory before the integer MMAs; for maps with many channels,
-                                             where one row tile is read by many column tiles and the codes stay in
-                                             L2, that expansion costs more than the bytes save.  Taps then hold one
-                                             code per byte too.  Workspace sizes depend on this field. */
+  int byte_codes;                         /* storage of the block's intermediate activation codes in the workspace, and
+                                             in the taps.  0 (the default): sized for codes bit-packed at the branch's
+                                             bit width.  1: one code per byte whatever the bit width -- the same code
+                                             values in [0, 2^bits), no expansion in shared memory before the integer
+                                             MMAs.  A call without taps keeps one code per byte in either case where
+                                             the workspace has room for the rows of the call; taps hold what this field
+                                             says.  Workspace sizes depend on it. */
 } mixaq_block_params;
 
 /* Patch merging between stages: 2x2 neighbours concatenated (zero padding for odd sizes) -> LN(4C) ->

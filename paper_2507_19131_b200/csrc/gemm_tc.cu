@@ -52,8 +52,8 @@ __host__ __device__ constexpr int num_threads(int warps) { return 32 * (FIRST_EP
 // Registers.  A block is launched with what its threads divide the file into (80 a thread with 16 epilogue warps, 96 with 12); the
 // first two warpgroups give back all but SIDE_REGS and the epilogue warps of the code outputs take them.  gemm_init checks that
 // the shares fit into what the compiled kernels are launched with.
-constexpr int SIDE_REGS = 40;
-__host__ __device__ constexpr int epi_regs(int warps) { return warps == 16 ? 96 : warps == 12 ? 128 : 0; }     // 0: no exchange
+constexpr int SIDE_REGS = 56;
+__host__ __device__ constexpr int epi_regs(int warps) { return warps == 16 ? 88 : warps == 12 ? 120 : 0; }     // 0: no exchange
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
 constexpr int MAX_RING = 6;

@@ -298,6 +298,28 @@ BlockWs carve_block(const mixaq_block_params* p, int B, int H, int W, void* base
   return w;
 }
 
+// The code buffers of a bit-packed block laid out anew with one byte per code, for the M[i] rows that the branches have in this call.
+// Expanding packed codes in front of every MMA costs more than their bytes save (Swin-T 800 x 1333, bit-packed against bytes: 916
+// and 841 us; Swin-S 4 x 1024 x 1024 at A4 / A2: 3 918 and 3 487), and nobody sees the storage but the taps.  The packed carving
+// sizes each branch for all rows and keeps apart what is never alive at once, so bytes fit into the same memory: x1; the q, k, v
+// codes and after them fc1's; the codes of LN1 and after them LN2's; those of the attention.  false: not enough room (hidden layers
+// beyond 10 C at two bits); ws is left as it is.
+bool carve_bytes(const mixaq_block_params* p, const int (&M)[2], void* workspace, BlockWs& ws) {
+  const size_t rows = (size_t)M[0] + M[1], C = p->dim, Hd = p->hidden, wide = std::max(3 * C, Hd);
+  Carver c(ws.a[0], false);
+  float* x1 = c.take<float>(rows * C);
+  uint8_t *big = c.take<uint8_t>(rows * wide), *ln = c.take<uint8_t>(rows * C), *o = c.take<uint8_t>(rows * C);
+  if (c.off > (size_t)((char*)workspace + ws.bytes - (char*)ws.a[0])) return false;
+  const size_t m0 = M[0];
+  for (int i = 0; i < 2; ++i) {
+    const size_t r = i == 0 ? 0 : m0;                        // the high branch's rows come first
+    ws.x1[i] = x1 + r * C;
+    ws.qkv[i] = big + r * 3 * C; ws.f2[i] = big + r * Hd;
+    ws.a[i] = ws.f1[i] = ln + r * C; ws.o[i] = o + r * C;
+  }
+  return true;
+}
+
 SelectArgs make_select_args(const SelWs& sel, const int32_t* energy, int B, int H, int W, int shift, const Geometry& g,
                             int reverse, bool own_energy) {
   SelectArgs sa;
@@ -588,8 +610,10 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   const int M[2] = {B * g.n_hi * WT, B * g.n_lo * WT};
   const int slots[2] = {B * g.n_hi, B * g.n_lo};
   const mixaq_branch_taps* tp[2] = {taps ? &taps->hi : nullptr, taps ? &taps->lo : nullptr};
-  // bits a stored code occupies: the branch's bit width (bit-packed) or a whole byte
-  const int cb[2] = {p->byte_codes ? 8 : p->hi.bits, p->byte_codes ? 8 : p->lo.bits};
+  // bits a stored code occupies: a whole byte, or the branch's bit width (bit-packed: what the taps hand out and the guard zones
+  // are laid out for)
+  const bool bytes = p->byte_codes || (!taps && guard_zones.empty() && carve_bytes(p, M, workspace, ws));
+  const int cb[2] = {bytes ? 8 : p->hi.bits, bytes ? 8 : p->lo.bits};
 
   // 2. gather + LN1 + quantize + pack
   LnBranch lb[2];

@@ -39,6 +39,22 @@ def test_gemm_tilings_around_their_limits(orc, mq, ctx, dim, windows):
     run_block_case(orc, mq, ctx, blk, x, 0.55, taps=False)
 
 
+@pytest.mark.parametrize("bits,mult,low,prune", [((8, 4), 4, 0.9, 0.0), ((4, 2), 4, 0.0, 0.0), ((2, 2), 4, 0.5, 0.3), ((2, 2), 10, 0.5, 0.0),
+                                                 ((2, 2), 12, 0.5, 0.0), ((4, 2), 4, 0.5, 1.0)])
+def test_one_code_per_byte_inside_a_packed_workspace(orc, mq, ctx, bits, mult, low, prune):
+    """Every row in one branch, hidden layers up to and beyond what the room of two-bit codes allows, all windows pruned; the
+    taps of the same call stay bit-packed."""
+    rng = np.random.default_rng(mult)
+    blk = synth.make_block(rng, 64, 2, 3, 4, *bits, share_bias=False)
+    blk.hidden = 64 * mult
+    blk.fc1, blk.fc2 = synth.make_linear(rng, blk.hidden, 64, 4), synth.make_linear(rng, 64, blk.hidden, 4)
+    for br in (blk.hi, blk.lo):
+        br.b_fc1 = (0.02 * rng.standard_normal(blk.hidden)).astype(F32)
+    x = synth.input_student_t(mult, 2, 20, 30, 64)
+    for taps in (False, True):
+        run_block_case(orc, mq, ctx, blk, x, low, prune, taps=taps)
+
+
 @pytest.mark.parametrize("dim,sign", [(128, 1), (128, -1), (192, 1), (384, -1), (384, 0)])
 def test_gemm_accumulators_beyond_the_bias_trick(orc, mq, ctx, dim, sign):
     """Weights of full magnitude: sums of 128 products of 255 x 127 stay below 2^22, from 192 on they may not, and the
