@@ -47,13 +47,18 @@ constexpr int UNPACK_WARPS = 4;
 // element, is faster with 12 everywhere (C = 128 at 2 x 384 x 384: 63 us against 68).
 constexpr int F32_WARPS = 8, CODE_WARPS = 12, CODE_WARPS_MANY = 16;
 constexpr int MANY_ROW_TILES = 2;              // row tiles per SM from which fc1 has CODE_WARPS_MANY
-constexpr int FIRST_UNPACK_WARP = 4, FIRST_EPI_WARP = 8;        // warpgroups: TMA, MMA and TMEM set-up; unpack; epilogue
-__host__ __device__ constexpr int num_threads(int warps) { return 32 * (FIRST_EPI_WARP + warps); }
-// Registers.  A block is launched with what its threads divide the file into (80 a thread with 16 epilogue warps, 96 with 12); the
-// first two warpgroups give back all but SIDE_REGS and the epilogue warps of the code outputs take them.  gemm_init checks that
-// the shares fit into what the compiled kernels are launched with.
+// Warpgroups: TMA, MMA and TMEM set-up; unpack, only in launches with bit-packed rows; epilogue
+constexpr int FIRST_UNPACK_WARP = 4;
+__host__ __device__ constexpr int first_epi_warp(bool packed) { return FIRST_UNPACK_WARP + (packed ? UNPACK_WARPS : 0); }
+__host__ __device__ constexpr int num_threads(int warps, bool packed) { return 32 * (first_epi_warp(packed) + warps); }
+// Registers.  A block is launched with what its threads divide the file into (a scheduler's 16 384 among its warps: 80 a thread with
+// 16 epilogue warps and the unpack warps, 96 without those, 96 and 128 with 12); the side warpgroups give back all but SIDE_REGS
+// and the epilogue warps of the code outputs take them.  gemm_init checks that the shares fit into what the compiled kernels are
+// launched with.
 constexpr int SIDE_REGS = 56;
-__host__ __device__ constexpr int epi_regs(int warps) { return warps == 16 ? 88 : warps == 12 ? 120 : 0; }     // 0: no exchange
+__host__ __device__ constexpr int epi_regs(int warps, bool packed) {      // 0: no exchange
+  return warps == 16 ? (packed ? 88 : 104) : warps == 12 ? (packed ? 120 : 152) : 0;
+}
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
 constexpr int MAX_RING = 6;
@@ -116,8 +121,8 @@ struct RingPos {
 // The loops of the TMA and the MMA warp bound a tile as much as the epilogue does, so they hold no division, and the whole warp
 // walks through them with one elected lane issuing: in code that a single lane runs, an MMA of up to 64 columns takes 63 cycles to
 // issue (its operands go through the uniform registers one by one), elected in a converged warp 46 to 50.
-template <int MODE, bool TAPS, int EW>
-__global__ void __launch_bounds__(num_threads(EW), 1)
+template <int MODE, bool TAPS, int EW, bool PACKED>
+__global__ void __launch_bounds__(num_threads(EW, PACKED), 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
           const __grid_constant__ CUtensorMap tmB, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -137,7 +142,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   // the give-up path only.
   uint32_t fills = 0, raw_used = 0, raw_phase = 0;
 
-  constexpr int NUM_EPI_WARPS = EW;
+  constexpr int NUM_EPI_WARPS = EW, FIRST_EPI_WARP = first_epi_warp(PACKED);
   constexpr int NUM_UNPACK_WARPS = UNPACK_WARPS, NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
   constexpr int UNPACK_ITEMS = BM * (BK / UMMA_K) / NUM_UNPACK_THREADS;   // (row, 32-code group) items per thread and stage
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -185,7 +190,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 
   if (warp == 0) {
     // ---- TMA producer ----
-    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
+    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     {
       const bool leader = elect_one();
       TileWalk w(p);
@@ -198,7 +203,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         const int m_first = b == 0 ? 0 : p.tiles_m0, m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
         if (w.mt >= m_end) continue;
         const int abits = p.g.br[b].a_bits;
-        const bool packed = abits != 8, stage_packed = packed && p.tma_packed[b];
+        const bool packed = PACKED && abits != 8, stage_packed = packed && p.tma_packed[b];
         const CUtensorMap* tmA = b == 0 ? &tmA0 : &tmA1;
         const uint32_t tx = b_bytes + (packed ? 0u : (uint32_t)A_STAGE_BYTES);
         const int pk_row = BK * abits / 8;                      // packed bytes per row and k-block
@@ -233,7 +238,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     }
   } else if (warp == 1) {
     // ---- MMA issuer ----
-    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
+    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     {
       const bool leader = elect_one();
       const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
@@ -248,7 +253,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
       for (int b = 0; b < 2 && ok; ++b) {
         const int m_end = b == 0 ? p.tiles_m0 : p.tiles_m;
         if (w.mt >= m_end) continue;
-        const bool packed = p.g.br[b].a_bits != 8;
+        const bool packed = PACKED && p.g.br[b].a_bits != 8;
         for (; w.mt < m_end && ok; w.next(p), ap.next(n_acc)) {
           // wait until the epilogue has drained this accumulator's previous use (at once in the first pass)
           if (!mbar_wait(bar_tempty + 8u * ap.slot, ap.pass ^ 1u, abort_flag)) { ok = false; break; }
@@ -281,10 +286,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     }
   } else if (warp < FIRST_UNPACK_WARP) {
     // (warps 2 and 3 fill up the warpgroup)
-    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
-  } else if (warp < FIRST_EPI_WARP) {
+    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
+  } else if (PACKED && warp < FIRST_EPI_WARP) {
     // ---- unpack producers: bit-packed rows -> one code per byte, written in the swizzled layout ----
-    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
+    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     const int ptid = tid - 32 * FIRST_UNPACK_WARP;   // 0 .. NUM_UNPACK_THREADS-1
     TileWalk w(p);
     int slot = 0;
@@ -346,7 +351,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     __syncwarp();
   } else {
     // ---- epilogue warps: warp e reads TMEM lanes 32*(e%4).. of its group's tiles, every split-th chunk ----
-    if (epi_regs(EW) > 0) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(epi_regs(EW) > 0 ? epi_regs(EW) : 24));
+    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(epi_regs(EW, PACKED) > 0 ? epi_regs(EW, PACKED) : 24));
     const int e = warp - FIRST_EPI_WARP, q = warp & 3;         // any 4 consecutive warps cover the 4 lane quarters
     const int split = p.split, groups = p.groups, group = (e >> 2) / split, sub = (e >> 2) - group * split;
     float* stage = reinterpret_cast<float*>(smem + L.stage_off) + e * EPI_STAGE_FLOATS;
@@ -485,8 +490,8 @@ Tiling pick_tiling(int unit, int N, int m_tiles, int k_blocks, int sms, int warp
   return best;
 }
 
-template <int MODE, int EW>
-bool launch_mode(const GemmArgs& g, int* status, cudaStream_t st) {
+template <int MODE, int EW, bool PACKED>
+bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
   TcParams p;
   p.g = g; p.status = status;
   p.g.neg_zero = -0.0f;
@@ -540,11 +545,16 @@ bool launch_mode(const GemmArgs& g, int* status, cudaStream_t st) {
   const size_t smem = (size_t)smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW).total + 1024 /*alignment slack*/;
   if (smem > 227 * 1024) return false;
   if (g.br[0].tap_acc || g.br[1].tap_acc)
-    launch_pdl(k_gemm_tc<MODE, true, EW>, dim3(grid), num_threads(EW), smem, st, mA[0], mA[1], mB, p);
+    launch_pdl(k_gemm_tc<MODE, true, EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);
   else
-    launch_pdl(k_gemm_tc<MODE, false, EW>, dim3(grid), num_threads(EW), smem, st, mA[0], mA[1], mB, p);
+    launch_pdl(k_gemm_tc<MODE, false, EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);
   ++g_launches;
   return true;
+}
+template <int MODE, int EW>
+bool launch_mode(const GemmArgs& g, int* status, cudaStream_t st) {
+  const bool packed = (g.br[0].M > 0 && g.br[0].a_bits != 8) || (g.br[1].M > 0 && g.br[1].a_bits != 8);
+  return packed ? launch_mode_as<MODE, EW, true>(g, status, st) : launch_mode_as<MODE, EW, false>(g, status, st);
 }
 
 }  // namespace
@@ -664,21 +674,24 @@ int launch_mma_peak(int kind, int groups, unsigned long long* ns_out, int* statu
 // opt-in to large dynamic shared memory for every epilogue mode, resolve the tensor-map encoder, read the SM count.
 bool gemm_init() {
   bool ok = encode_fn() != nullptr && sm_count() > 0;
-  auto big_smem = [&](auto kernel) { ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess; };
   // the register shares of the code epilogues have to add up to no more than the block is launched with
-  auto regs_fit = [&](auto kernel, int warps) {
+  auto set_up = [&](auto kernel, int warps, bool packed) {
     cudaFuncAttributes a;
-    ok &= cudaFuncGetAttributes(&a, kernel) == cudaSuccess && FIRST_EPI_WARP * SIDE_REGS + warps * epi_regs(warps) <= (FIRST_EPI_WARP + warps) * a.numRegs;
+    const int side = first_epi_warp(packed), regs = epi_regs(warps, packed);
+    ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess &&
+          cudaFuncGetAttributes(&a, kernel) == cudaSuccess && (regs == 0 || side * SIDE_REGS + warps * regs <= (side + warps) * a.numRegs);
   };
-  regs_fit(k_gemm_tc<EPI_QKV, false, CODE_WARPS>, CODE_WARPS); regs_fit(k_gemm_tc<EPI_QKV, true, CODE_WARPS>, CODE_WARPS);
-  regs_fit(k_gemm_tc<EPI_FC1, false, CODE_WARPS>, CODE_WARPS); regs_fit(k_gemm_tc<EPI_FC1, true, CODE_WARPS>, CODE_WARPS);
-  regs_fit(k_gemm_tc<EPI_FC1, false, CODE_WARPS_MANY>, CODE_WARPS_MANY); regs_fit(k_gemm_tc<EPI_FC1, true, CODE_WARPS_MANY>, CODE_WARPS_MANY);
-  big_smem(k_gemm_tc<EPI_QKV, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_QKV, true, CODE_WARPS>);
-  big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS>);
-  big_smem(k_gemm_tc<EPI_FC1, false, CODE_WARPS_MANY>); big_smem(k_gemm_tc<EPI_FC1, true, CODE_WARPS_MANY>);
-  big_smem(k_gemm_tc<EPI_PROJ, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_PROJ, true, F32_WARPS>);
-  big_smem(k_gemm_tc<EPI_FC2, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_FC2, true, F32_WARPS>);
-  big_smem(k_gemm_tc<EPI_MERGE, false, F32_WARPS>); big_smem(k_gemm_tc<EPI_MERGE, true, F32_WARPS>);
+  auto set_up_all = [&](auto mode_tag, auto warps_tag) {
+    constexpr int MODE = decltype(mode_tag)::value, EW = decltype(warps_tag)::value;
+    set_up(k_gemm_tc<MODE, false, EW, false>, EW, false); set_up(k_gemm_tc<MODE, true, EW, false>, EW, false);
+    set_up(k_gemm_tc<MODE, false, EW, true>, EW, true); set_up(k_gemm_tc<MODE, true, EW, true>, EW, true);
+  };
+  set_up_all(std::integral_constant<int, EPI_QKV>{}, std::integral_constant<int, CODE_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_FC1>{}, std::integral_constant<int, CODE_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_FC1>{}, std::integral_constant<int, CODE_WARPS_MANY>{});
+  set_up_all(std::integral_constant<int, EPI_PROJ>{}, std::integral_constant<int, F32_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_FC2>{}, std::integral_constant<int, F32_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_MERGE>{}, std::integral_constant<int, F32_WARPS>{});
   return ok;
 }
 
