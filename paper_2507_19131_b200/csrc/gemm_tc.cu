@@ -12,7 +12,7 @@
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
 //               the swizzled layout (rows whose byte pitch is no multiple of 16 cannot be described to the TMA
 //               unit and are read with plain loads instead);
-//   then        epilogue (12 or 16 warps for the code outputs, 8 for the binary32 outputs): tcgen05.ld (one row per thread,
+//   then        epilogue (12 warps for the code outputs, 8 or 12 for the binary32 outputs): tcgen05.ld (one row per thread,
 //               16 or 32 columns per load) + the fused epilogue of the mode.
 // Every wait on an mbarrier is bounded; on expiry the CTA raises the status word, then waits (bounded again) for the
 // copies it has issued to land and for the MMAs it has issued to retire, frees its tensor memory and returns.
@@ -40,25 +40,21 @@ constexpr int A_STAGE_BYTES = BM * BK;
 // warps 4..7 expand sub-byte codes (two warps left the long-K main loops of 4-bit tiles waiting for the expansion;
 // eight cost more registers than they return)
 constexpr int UNPACK_WARPS = 4;
-// Epilogue warps.  Binary32 outputs: 8.  Code outputs: 12; fc1, whose GELU makes it the longest, 16 where every SM has two row
-// tiles or more: whole tiles are then dealt to groups of warps (see pick_tiling) and the launch is bound by throughput (C = 256
-// at 2 x 192 x 192 tokens: 93 us with 16, 97 with 12; C = 96 at 16 x 56 x 56: 30.4 and 32.5); below that the shorter tile
-// latency of 12 warps with more registers wins (C = 384 at 16 x 14 x 14: 14.4 us against 16.1).  QKV, with less work per
-// element, is faster with 12 everywhere (C = 128 at 2 x 384 x 384: 63 us against 68).
-constexpr int F32_WARPS = 8, CODE_WARPS = 12, CODE_WARPS_MANY = 16;
-constexpr int MANY_ROW_TILES = 2;              // row tiles per SM from which fc1 has CODE_WARPS_MANY
+// Epilogue warps.  Code outputs: 12 (16 with fewer registers are no faster at any size).  Binary32 outputs: 8; 12 up to a row tile
+// per twelve SMs, where a launch is the latency of a tile or two and three warps share the columns of a lane quarter (fc2 of
+// 768 channels at 7 x 7: 6.7 against 7.7 us, at 25 x 42 8.3 against 9.2; from 26 row tiles on 8 warps are up to 10 % faster).
+constexpr int F32_WARPS = 8, F32_WARPS_FEW = 12, CODE_WARPS = 12;
+constexpr int FEW_SMS_PER_ROW_TILE = 12;
 // Warpgroups: TMA, MMA and TMEM set-up; unpack, only in launches with bit-packed rows; epilogue
 constexpr int FIRST_UNPACK_WARP = 4;
 __host__ __device__ constexpr int first_epi_warp(bool packed) { return FIRST_UNPACK_WARP + (packed ? UNPACK_WARPS : 0); }
 __host__ __device__ constexpr int num_threads(int warps, bool packed) { return 32 * (first_epi_warp(packed) + warps); }
-// Registers.  A block is launched with what its threads divide the file into (a scheduler's 16 384 among its warps: 80 a thread with
-// 16 epilogue warps and the unpack warps, 96 without those, 96 and 128 with 12); the side warpgroups give back all but SIDE_REGS
+// Registers.  A block is launched with what its threads divide the file into (a scheduler's 16 384 among its warps: 128 a thread with
+// 12 epilogue warps, 96 with the unpack warps too); the side warpgroups give back all but SIDE_REGS
 // and the epilogue warps of the code outputs take them.  gemm_init checks that the shares fit into what the compiled kernels are
 // launched with.
 constexpr int SIDE_REGS = 56;
-__host__ __device__ constexpr int epi_regs(int warps, bool packed) {      // 0: no exchange
-  return warps == 16 ? (packed ? 88 : 104) : warps == 12 ? (packed ? 120 : 152) : 0;
-}
+__host__ __device__ constexpr int epi_regs(int warps, bool packed) { return warps != 12 ? 0 : packed ? 112 : 136; }    // 0: no exchange
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
 constexpr int MAX_RING = 6;
@@ -455,32 +451,30 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 
 // ---- host side -------------------------------------------------------------------------------------
 // Tile width and the epilogue's division of labour.  The width is a multiple of 32 that divides `unit` (N; for QKV the
-// width C of a section, so that a tile has one quantizer), at most 256.  Cost in units of an epilogue warp's 32 columns
-// (about 0.6 us): a tile takes `mma` to multiply and each of its warps `epi` to convert, `groups` tiles are converted at
-// once while the next ones are multiplied, and the first tiles have nothing to hide behind.  A wide tile reads its rows
-// fewer times and pays the fixed part of the epilogue once for more columns; narrow ones spread a small problem over the
-// SMs.  The constants are a fit to the times of all (width, groups) at 13 shapes from 768 x 7 x 7 to 128 x 2 x 384 x 384.  Of
-// 80 shapes (four GEMMs of 20 maps from 7 x 7 to 2 x 384 x 384 tokens), all widths and groups of each timed, the choice is
-// within 5 % of the fastest at 73; the worst are proj with C = 192 at 16 x 28 x 28 (9.0 us at width 64, 7.5 at 192), QKV with
-// C = 768 at 4 x 32 x 32 (15.3 at 128, 13.4 at 256) and proj with C = 512 at 2 x 96 x 96 (23.9 at 256, 21.4 at 128).  A cost
-// without the overlap was up to 30 % off (fc2 with C = 1024 at 2 x 48 x 48: 50 us at the width of 256 it chose, 40 at 128).
+// width C of a section, so that a tile has one quantizer), at most 256.  A tile takes `mma` to multiply and each of its warps `epi`
+// to convert, `groups` tiles are converted at once while the next ones are multiplied, and the first tiles have nothing to hide
+// behind.  A wide tile reads its rows fewer times and pays the fixed part of the epilogue once for more columns; narrow ones spread a
+// small problem over the SMs.  The constants (microseconds, roughly) are a fit to the times of all widths and groups of the four GEMMs
+// at 25 maps from 768 x 7 x 7 to 128 x 384 x 384, each taken together with the kernel behind it: on average 2 % above the fastest
+// choice, 4 % with the constants that were fitted to the kernels before (worst: QKV with C = 512 at 14 x 14, 8.4 us against 6.6).
 struct Tiling { int bn, n_acc, groups, split; };
-Tiling pick_tiling(int unit, int N, int m_tiles, int k_blocks, int sms, int warps, int chunk) {
+Tiling pick_tiling(int mode, int unit, int N, int m_tiles, int k_blocks, int sms, int warps) {
   Tiling best = {0, 0, 0, 0};
   double best_cost = 0.0;
   const int per_quarter = warps / 4;
-  const double fixed = chunk == CODE_NC ? 0.5 : 2.5;
+  const int chunk = code_mode(mode) ? CODE_NC : F32_NC;
+  const double fixed = code_mode(mode) ? 1.14 : 4.77, per_32 = mode == EPI_QKV ? 0.183 : mode == EPI_FC1 ? 0.0775 : 0.147;
   for (int bn = 32; bn <= MAX_BN; bn += 32) {
     if (unit % bn) continue;
     const int fit = TMEM_COLS / bn < MAX_ACC ? TMEM_COLS / bn : MAX_ACC;
     const long tiles = (long)m_tiles * (N / bn), per_cta = (tiles + sms - 1) / sms;
     // a launch that leaves SMs idle has more of the L2 for each tile: width then costs less
-    const double mma = k_blocks * (0.26 + 0.16 * (bn / 32) * (tiles < sms ? (double)tiles / sms : 1.0));
+    const double mma = k_blocks * (0.256 + 0.246 * (bn / 32) * (tiles < sms ? (double)tiles / sms : 1.0));
     for (int groups = 1; groups <= per_quarter && groups <= fit; ++groups) {
       if (per_quarter % groups) continue;
       const int n_acc = fit / groups * groups;                // a group keeps to its own accumulators
       const int split = per_quarter / groups;
-      const double epi = (bn / chunk + split - 1) / split * (chunk / 32.0) + fixed;
+      const double epi = (bn / chunk + split - 1) / split * (chunk / 32.0) * per_32 + fixed;
       const long rounds = (per_cta + groups - 1) / groups;
       const double first = per_cta < groups ? per_cta * mma : groups * mma;
       const double cost = fmax(first + rounds * epi, per_cta * mma + epi);
@@ -501,7 +495,7 @@ bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
   const int sms = sm_count();
   p.tiles_m0 = t0; p.tiles_m = t0 + t1;
   p.k_blocks = (g.K + BK - 1) / BK;
-  const Tiling tl = pick_tiling(MODE == EPI_QKV ? g.C : g.N, g.N, t0 + t1, p.k_blocks, sms, EW, code_mode(MODE) ? CODE_NC : F32_NC);
+  const Tiling tl = pick_tiling(MODE, MODE == EPI_QKV ? g.C : g.N, g.N, t0 + t1, p.k_blocks, sms, EW);
   if (tl.bn == 0) return false;
   p.BN = tl.bn; p.n_acc = tl.n_acc; p.groups = tl.groups; p.split = tl.split;
   p.n_tiles = g.N / p.BN;
@@ -688,22 +682,24 @@ bool gemm_init() {
   };
   set_up_all(std::integral_constant<int, EPI_QKV>{}, std::integral_constant<int, CODE_WARPS>{});
   set_up_all(std::integral_constant<int, EPI_FC1>{}, std::integral_constant<int, CODE_WARPS>{});
-  set_up_all(std::integral_constant<int, EPI_FC1>{}, std::integral_constant<int, CODE_WARPS_MANY>{});
   set_up_all(std::integral_constant<int, EPI_PROJ>{}, std::integral_constant<int, F32_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_PROJ>{}, std::integral_constant<int, F32_WARPS_FEW>{});
   set_up_all(std::integral_constant<int, EPI_FC2>{}, std::integral_constant<int, F32_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_FC2>{}, std::integral_constant<int, F32_WARPS_FEW>{});
   set_up_all(std::integral_constant<int, EPI_MERGE>{}, std::integral_constant<int, F32_WARPS>{});
+  set_up_all(std::integral_constant<int, EPI_MERGE>{}, std::integral_constant<int, F32_WARPS_FEW>{});
   return ok;
 }
 
 bool launch_gemm(const GemmArgs& g, cudaStream_t st) {
   const long row_tiles = (long)(g.br[0].M + BM - 1) / BM + (g.br[1].M + BM - 1) / BM;
-  const bool many = row_tiles >= (long)MANY_ROW_TILES * sm_count();
+  const bool few = row_tiles * FEW_SMS_PER_ROW_TILE <= sm_count();
   switch (g.mode) {
     case EPI_QKV:   return launch_mode<EPI_QKV, CODE_WARPS>(g, g.status, st);
-    case EPI_FC1:   return many ? launch_mode<EPI_FC1, CODE_WARPS_MANY>(g, g.status, st) : launch_mode<EPI_FC1, CODE_WARPS>(g, g.status, st);
-    case EPI_PROJ:  return launch_mode<EPI_PROJ, F32_WARPS>(g, g.status, st);
-    case EPI_FC2:   return launch_mode<EPI_FC2, F32_WARPS>(g, g.status, st);
-    case EPI_MERGE: return launch_mode<EPI_MERGE, F32_WARPS>(g, g.status, st);
+    case EPI_FC1:   return launch_mode<EPI_FC1, CODE_WARPS>(g, g.status, st);
+    case EPI_PROJ:  return few ? launch_mode<EPI_PROJ, F32_WARPS_FEW>(g, g.status, st) : launch_mode<EPI_PROJ, F32_WARPS>(g, g.status, st);
+    case EPI_FC2:   return few ? launch_mode<EPI_FC2, F32_WARPS_FEW>(g, g.status, st) : launch_mode<EPI_FC2, F32_WARPS>(g, g.status, st);
+    case EPI_MERGE: return few ? launch_mode<EPI_MERGE, F32_WARPS_FEW>(g, g.status, st) : launch_mode<EPI_MERGE, F32_WARPS>(g, g.status, st);
   }
   return false;
 }

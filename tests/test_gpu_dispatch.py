@@ -39,6 +39,13 @@ def test_gemm_tilings_around_their_limits(orc, mq, ctx, dim, windows):
     run_block_case(orc, mq, ctx, blk, x, 0.55, taps=False)
 
 
+@pytest.mark.parametrize("dim,H,W", [(96, 35, 42), (96, 21, 74), (384, 35, 41), (384, 28, 56)])
+def test_gemm_epilogue_warps_around_their_limit(orc, mq, ctx, dim, H, W):
+    """12 row tiles (12 epilogue warps for the binary32 outputs) and 14 (8 warps), with remainders in the last tile."""
+    blk = synth.make_block(np.random.default_rng(dim + W), dim, dim // 32, 3, 8, 8, 4, share_bias=False)
+    run_block_case(orc, mq, ctx, blk, synth.input_student_t(dim, 1, H, W, dim), 0.5, taps=False)
+
+
 @pytest.mark.parametrize("bits,mult,low,prune", [((8, 4), 4, 0.9, 0.0), ((4, 2), 4, 0.0, 0.0), ((2, 2), 4, 0.5, 0.3), ((2, 2), 10, 0.5, 0.0),
                                                  ((2, 2), 12, 0.5, 0.0), ((4, 2), 4, 0.5, 1.0)])
 def test_one_code_per_byte_inside_a_packed_workspace(orc, mq, ctx, bits, mult, low, prune):
