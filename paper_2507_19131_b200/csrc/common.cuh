@@ -77,6 +77,17 @@ __device__ __forceinline__ float2 gelu_log2_tail2(float2 a) {      // log2 Phi(-
   q = __ffma2_rn(q, a, f2(__uint_as_float(0xbf935b8fu)));
   return __ffma2_rn(q, a, f2(__uint_as_float(0xbf7fffbeu)));
 }
+// the same, to the bit, of -a: the coefficients of odd powers change their signs
+__device__ __forceinline__ float2 gelu_log2_tail_neg2(float2 a) {
+  float2 q = f2(__uint_as_float(0x35d6f9e3u));
+  q = __ffma2_rn(q, a, f2(__uint_as_float(0x38729e20u)));
+  q = __ffma2_rn(q, a, f2(__uint_as_float(0x3a6dcc74u)));
+  q = __ffma2_rn(q, a, f2(__uint_as_float(0x3c0a3aedu)));
+  q = __ffma2_rn(q, a, f2(__uint_as_float(0x3d5c93e3u)));
+  q = __ffma2_rn(q, a, f2(__uint_as_float(0xbeeac5d4u)));
+  q = __ffma2_rn(q, a, f2(__uint_as_float(0x3f935b8fu)));
+  return __ffma2_rn(q, a, f2(__uint_as_float(0xbf7fffbeu)));
+}
 __device__ __forceinline__ float2 gelu_f2(float2 v) {
   const float2 a = make_float2(fminf(fabsf(v.x), 5.0f), fminf(fabsf(v.y), 5.0f));
   const float2 q = gelu_log2_tail2(a);
@@ -119,50 +130,25 @@ __device__ __forceinline__ uint32_t pack_const(int zp, int bits) {
   const uint32_t k = (uint32_t)zp - kMagicBits;
   return k * (bits == 8 ? 0x01010101u : (bits == 4 ? 0x11111111u : 0x55555555u));
 }
-// Four unclamped codes to one word, one per byte, clamped to [0, 2^bits - 1]: m holds the rounding patterns
-// 0x4B400000 + n, and (m << SH) + bias is (n + zp) << SH for bias = (zp - 0x4B400000) << SH, SH = 8 - bits.  The
-// saturating byte conversion then clamps both ends at once: codes above the range become 255, whose top `bits` bits are
-// all ones.  1.5 instructions per code against 3 for two binary32 clamps and a shifted add.  For bits < 8 the codes come
-// out in the top bits of their bytes.
-template <int SH>
-__device__ __forceinline__ uint32_t sat_pack4(uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3, uint32_t bias) {
-  uint32_t d;
-  asm("{\n\t.reg .b32 t;\n\t"
-      "cvt.pack.sat.u8.s32.b32 t, %4, %3, 0;\n\t"
-      "cvt.pack.sat.u8.s32.b32 %0, %2, %1, t;\n\t}"
-      : "=r"(d) : "r"((m0 << SH) + bias), "r"((m1 << SH) + bias), "r"((m2 << SH) + bias), "r"((m3 << SH) + bias));
-  return d;
+// Four unclamped codes to one word, one per byte, clamped to [0, qmax]: m holds rounding patterns 0x4B400000 + n, whose low halves
+// are n as 16-bit numbers (|n| + zp < 2^15).  zp2, qmax2: zero point and largest code in both halves of a word; the additions and
+// both ends of the clamp are one instruction for two codes.
+template <bool ADD_ZP>
+__device__ __forceinline__ uint32_t clamp_pack4(uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3, uint32_t zp2, uint32_t qmax2) {
+  const uint32_t lo = __byte_perm(m0, m1, 0x5410), hi = __byte_perm(m2, m3, 0x5410);
+  return ADD_ZP ? __byte_perm(__viaddmin_s16x2_relu(lo, zp2, qmax2), __viaddmin_s16x2_relu(hi, zp2, qmax2), 0x6420)
+                : __byte_perm(__vimin_s16x2_relu(lo, qmax2), __vimin_s16x2_relu(hi, qmax2), 0x6420);
 }
-// Stores 32 codes of one row (eight words of sat_pack4): one code per byte (cbits = 8, codes of `bits` bits) or packed at
-// cbits = bits = 4 or 2.  dst is 4 * cbits bytes aligned.
-__device__ __forceinline__ void store_sat32(uint8_t* dst, uint32_t (&w)[8], int bits, int cbits) {
+// Stores 8 codes of one row (two words of clamp_pack4): one code per byte (cbits = 8) or packed at cbits = 4 or 2.  dst is cbits
+// bytes aligned.
+__device__ __forceinline__ void store_codes8(uint8_t* dst, uint32_t w0, uint32_t w1, int cbits) {
   if (cbits == 8) {
-    if (bits < 8) {
-      const int sh = 8 - bits;
-      const uint32_t mask = bits == 4 ? 0x0F0F0F0Fu : 0x03030303u;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) w[i] = (w[i] >> sh) & mask;
-    }
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+    *reinterpret_cast<uint2*>(dst) = make_uint2(w0, w1);
   } else if (cbits == 4) {
-    // bytes 0 and 1 of a word hold codes 0 and 1 in their high nibbles: the pair is (byte 0 >> 4) | (byte 1 & 0xF0)
-    uint32_t n[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) n[i] = ((w[i] >> 4) & 0x000F000Fu) | ((w[i] >> 8) & 0x00F000F0u);
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(__byte_perm(n[0], n[1], 0x6420), __byte_perm(n[2], n[3], 0x6420),
-                                                  __byte_perm(n[4], n[5], 0x6420), __byte_perm(n[6], n[7], 0x6420));
+    *reinterpret_cast<uint32_t*>(dst) = __byte_perm(w0 | (w0 >> 4), w1 | (w1 >> 4), 0x6420);      // codes 2 i and 2 i + 1 in byte 2 i
   } else {
-    // four codes in the top two bits of four bytes to one byte
-    uint32_t n[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t t = ((w[i] >> 6) & 0x00030003u) | ((w[i] >> 12) & 0x000C000Cu);     // codes 0, 1 and codes 2, 3
-      n[i] = t | (t >> 12);
-    }
-    reinterpret_cast<uint2*>(dst)[0] =
-        make_uint2(__byte_perm(__byte_perm(n[0], n[1], 0x0040), __byte_perm(n[2], n[3], 0x0040), 0x5410),
-                   __byte_perm(__byte_perm(n[4], n[5], 0x0040), __byte_perm(n[6], n[7], 0x0040), 0x5410));
+    const uint32_t t0 = w0 | (w0 >> 6), t1 = w1 | (w1 >> 6);                                      // and then two pairs in byte 0
+    *reinterpret_cast<uint16_t*>(dst) = (uint16_t)__byte_perm(t0 | (t0 >> 12), t1 | (t1 >> 12), 0x0040);
   }
 }
 

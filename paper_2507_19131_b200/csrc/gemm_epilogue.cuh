@@ -1,12 +1,17 @@
 // Fused epilogues of the integer GEMMs (MixA-Q Section 3.2: shared integer weights, per-branch step sizes,
-// zero points and biases).  One epilogue warp owns 32 rows (one TMEM lane quarter, one row per thread) and every
-// c_step-th chunk of the tile, 32 columns wide for the code outputs and 16 for the binary32 outputs (the warps of a group
-// that share a lane quarter deal the chunks round-robin):
+// zero points and biases).  One epilogue warp owns 32 rows (one TMEM lane quarter) and every c_step-th chunk of the tile, 32
+// columns wide for the code outputs and 16 for the binary32 outputs (the warps of a group that share a lane quarter deal the
+// chunks round-robin).  A quad of lanes holds a row of a chunk, lane t of it 8 (4) consecutive channels, of rows l / 4 + 0, 8, 16,
+// 24: the accumulator is read in the layout of tmem_ld_quads and the weights arrive with their rows in the matching order
+// (make_quad_map).
 //   raw[n] = sum_k a[m][k] * w[n][k]                   with UNSIGNED activation codes a;
 //   acc[n] = raw[n] - z_a * sum_k w[n][k]              (zero-point correction, exact in int32)
 //   v[n]       = fma((float)acc[n], s_a*s_w[n], bias[n])
-// The per-column constants (pre, mult, bias) sit in shared memory; every lane reads the same
-// column, so the reads are broadcasts.
+// The per-column constants (pre, mult, bias) sit in shared memory.  With a row per lane every warp read all of a chunk's constants in
+// every lane, 12 bytes a value through a 128-byte path: a quarter of the fc1 epilogue's time and half of the QKV epilogue's.  Now a
+// value read serves four rows, and the binary32 outputs need no transposition through shared memory.  B200, 294 912 rows of 128
+// channels, before and after: QKV 58.4 -> 49.0 us, proj 60.1 -> 55.1, fc1 137.5 -> 137.2, fc2 76.1 -> 76.1; 18 432 rows of 512: QKV
+// 23.4 -> 20.4, proj 23.0 -> 20.9, fc1 46.4 -> 45.0, fc2 33.1 -> 33.8.
 #pragma once
 #include "kernels.h"
 #include "tc_ptx.cuh"
@@ -15,7 +20,7 @@
 namespace mixaq {
 
 constexpr int CODE_NC = 32, F32_NC = 16;               // columns per chunk of the code and of the binary32 epilogues
-constexpr int EPI_STAGE_FLOATS = 32 * F32_NC;          // per-warp transposition tile of the binary32 epilogues
+constexpr int EPI_CHUNK_FLOATS = 32 * F32_NC;          // a residual chunk of the binary32 epilogues
 
 struct ColConsts {                                     // shared-memory arrays indexed by the column within the tile
   const int32_t* pre; const float* mult; const float* bias;
@@ -37,39 +42,34 @@ __device__ __forceinline__ float2 acc_to_float2(int32_t a, int32_t b) {
   if (NARROW) return __fadd2_rn(make_float2(__int_as_float(a), __int_as_float(b)), f2(-12582912.0f));
   return make_float2(__int2float_rn(a - (int32_t)kMagicBits), __int2float_rn(b - (int32_t)kMagicBits));
 }
-// dequantization of NC columns; lc0 = first column in the warp's constants, n0 = its global index
-template <int MODE, bool TAPS, bool NARROW, int NC>
-__device__ __forceinline__ void dequant(const GemmBranch& br, int N, long m, bool row_ok, int n0, int lc0, const ColConsts& cc,
-                                        const int32_t* acc, float (&v)[NC]) {
-  if (TAPS && br.tap_acc && row_ok) {
-#pragma unroll
-    for (int i = 0; i < NC; ++i) br.tap_acc[m * N + n0 + i] = acc[i] + cc.pre[lc0 + i] - (int32_t)kMagicBits;
+// the constants of four columns
+struct Consts4 {
+  int4 pre; float4 mult, bias;
+  template <bool BIAS> __device__ __forceinline__ void load(const ColConsts& cc, int lc) {
+    pre = *reinterpret_cast<const int4*>(cc.pre + lc);
+    mult = *reinterpret_cast<const float4*>(cc.mult + lc);
+    bias = BIAS ? *reinterpret_cast<const float4*>(cc.bias + lc) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-#pragma unroll
-  for (int i4 = 0; i4 < NC / 4; ++i4) {
-    const int4 p4 = *reinterpret_cast<const int4*>(cc.pre + lc0 + 4 * i4);
-    const int pp[4] = {p4.x, p4.y, p4.z, p4.w};
-    const float4 m4 = *reinterpret_cast<const float4*>(cc.mult + lc0 + 4 * i4);
-    const float mm[4] = {m4.x, m4.y, m4.z, m4.w};
-    float bb[4] = {0.f, 0.f, 0.f, 0.f};
-    if (MODE != EPI_MERGE) {
-      const float4 b4 = *reinterpret_cast<const float4*>(cc.bias + lc0 + 4 * i4);
-      bb[0] = b4.x; bb[1] = b4.y; bb[2] = b4.z; bb[3] = b4.w;
-    }
-    // two columns per packed instruction (each lane rounds like the scalar fma / mul)
-#pragma unroll
-    for (int j = 0; j < 4; j += 2) {
-      const int i = 4 * i4 + j;
-      const float2 f = acc_to_float2<NARROW>(acc[i] + pp[j], acc[i + 1] + pp[j + 1]);
-      const float2 r = MODE == EPI_MERGE ? __fmul2_rn(f, make_float2(mm[j], mm[j + 1]))
-                                         : __ffma2_rn(f, make_float2(mm[j], mm[j + 1]), make_float2(bb[j], bb[j + 1]));
-      v[i] = r.x; v[i + 1] = r.y;
-    }
+};
+// Dequantization of four columns of a row, two per packed instruction (each lane rounds like the scalar fma / mul).
+// tap: where the accumulators of these columns go, or nullptr
+template <int MODE, bool TAPS, bool NARROW>
+__device__ __forceinline__ void dequant4(const Consts4& k, int32_t a0, int32_t a1, int32_t a2, int32_t a3, int32_t* tap, float2& lo, float2& hi) {
+  if (TAPS && tap) {
+    tap[0] = a0 + k.pre.x - (int32_t)kMagicBits; tap[1] = a1 + k.pre.y - (int32_t)kMagicBits;
+    tap[2] = a2 + k.pre.z - (int32_t)kMagicBits; tap[3] = a3 + k.pre.w - (int32_t)kMagicBits;
+  }
+  const float2 f0 = acc_to_float2<NARROW>(a0 + k.pre.x, a1 + k.pre.y), f1 = acc_to_float2<NARROW>(a2 + k.pre.z, a3 + k.pre.w);
+  if (MODE == EPI_MERGE) {
+    lo = __fmul2_rn(f0, make_float2(k.mult.x, k.mult.y)); hi = __fmul2_rn(f1, make_float2(k.mult.z, k.mult.w));
+  } else {
+    lo = __ffma2_rn(f0, make_float2(k.mult.x, k.mult.y), make_float2(k.bias.x, k.bias.y));
+    hi = __ffma2_rn(f1, make_float2(k.mult.z, k.mult.w), make_float2(k.bias.z, k.bias.w));
   }
 }
 
 // ---- quantizers of the code outputs ------------------------------------------------------------------------------------
-// Both leave rne(x * inv_scale) (FC1: + zp) in the low 16 bits of every pattern, unclamped; sat_pack4 adds, clamps and
+// Both leave rne(x * inv_scale) (FC1: + zp) in the low 16 bits of every pattern, unclamped; clamp_pack4 adds, clamps and
 // packs.  They need |x * inv_scale| < 2^15, which `in_range` of the caller guarantees (the channel's bound + |bias|, times
 // inv_scale); launches for which that cannot be shown take the exact functions with their binary32 clamps.
 constexpr float kPatternRange = 30000.0f;
@@ -85,32 +85,55 @@ __device__ __forceinline__ void quant_pattern2(float2 x, float inv_scale, float 
 // to the nearest integer; where it comes within the error bound of one half (see gelu_threshold) the caller recomputes.
 // The zero point is part of the rounding constant; at exact ties that changes the parity rule, and ties are recomputed.
 __device__ __forceinline__ void gelu_pattern2(float2 v, float inv_scale, float magic_zp, float& dist, uint32_t& m0, uint32_t& m1) {
-  const float2 a = make_float2(fminf(fabsf(v.x), 5.0f), fminf(fabsf(v.y), 5.0f));
-  const float2 q = gelu_log2_tail2(a);
-  const float2 h = __fmul2_rn(a, make_float2(ex2_approx(q.x), ex2_approx(q.y)));
-  const float2 g = sub2(make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f)), h);
+  const float2 a = make_float2(fmaxf(-fabsf(v.x), -5.0f), fmaxf(-fabsf(v.y), -5.0f));        // minus the contract's a
+  const float2 q = gelu_log2_tail_neg2(a);
+  const float2 g = __ffma2_rn(a, make_float2(ex2_approx(q.x), ex2_approx(q.y)), make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f)));
   const float2 r = __ffma2_rn(g, f2(inv_scale), f2(magic_zp));
   const float2 n = __fadd2_rn(f2(magic_zp), make_float2(-r.x, -r.y));          // minus the rounded value, exactly
   const float2 d = __ffma2_rn(g, f2(inv_scale), n);
-  dist = fmaxf(fmaxf(dist, fabsf(d.x)), fabsf(d.y));
+  asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(dist) : "f"(d.x), "f"(d.y));
   m0 = __float_as_uint(r.x); m1 = __float_as_uint(r.y);
 }
 // Distance of g * inv_scale from the contract's t: both exponentials are within 2^-22 of 2^q, h = a 2^q <= 0.17, so h differs
 // by at most 0.17 * 2^-21 + one rounding < 1.0e-7; g is rounded in both evaluations and t in the contract's, which adds
-// |t| * 3 * 2^-24, and |t| <= qmax + 1 for every t that is not clamped anyway; the distance itself is rounded by 2^-26.
-__device__ __forceinline__ float gelu_threshold(float inv_scale, float qmaxf) {
-  return 0.5f - __fmaf_rn(inv_scale, 1.1e-7f, (qmaxf + 2.0f) * 1.8e-7f);
+// |t| * 3 * 2^-24, and |t| <= max(code, zp) + 1 for every t that is not clamped anyway; the distance itself is rounded by 2^-26.
+// maxf: at least the codes in question and the zero point
+__device__ __forceinline__ float gelu_threshold(float inv_scale, float maxf) {
+  return 0.5f - __fmaf_rn(inv_scale, 1.1e-7f, (maxf + 2.0f) * 1.8e-7f);
+}
+
+// Four columns of two of the lane's rows by the contract's own operations, read again from tensor memory.  A function of its own: its
+// twenty constants and its temporaries would otherwise take registers of the loop that hardly ever comes here.
+template <int MODE>
+__device__ __noinline__ uint2 codes_exact8(uint32_t taddr, ColConsts cc, int lc, float inv_scale, float zpf, float qmaxf) {
+  int32_t a[8];
+  tmem_ld_quads(taddr, a);
+  Consts4 k;
+  k.load<true>(cc, lc);
+  tmem_ld_wait(a);
+  const uint32_t zp2 = (uint32_t)zpf * 0x10001u, qmax2 = (uint32_t)qmaxf * 0x10001u;
+  uint32_t w[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    float2 v0, v1;
+    uint32_t c[4];
+    dequant4<MODE, false, false>(k, a[2 * j], a[2 * j + 1], a[2 * j + 4], a[2 * j + 5], nullptr, v0, v1);
+    quant_magic2(MODE == EPI_FC1 ? gelu_f2(v0) : v0, inv_scale, -zpf, qmaxf - zpf, c[0], c[1]);
+    quant_magic2(MODE == EPI_FC1 ? gelu_f2(v1) : v1, inv_scale, -zpf, qmaxf - zpf, c[2], c[3]);
+    w[j] = clamp_pack4<true>(c[0], c[1], c[2], c[3], zp2, qmax2);
+  }
+  return make_uint2(w[0], w[1]);
 }
 
 // What a warp's epilogue needs of its branch, read once per branch (the parameters sit in constant memory, and a tile used
 // to read them again field by field).
 struct EpiBranch {
-  int M, bits, cbits;                                      // code outputs: width of the codes, bits a stored code takes
+  int M, cbits;                                            // code outputs: bits a stored code takes
   uint8_t* out_codes; float* out_f; const float* res; const int32_t* rowsrc;
   long row_bytes;                                          // code outputs: bytes of an output row
   float qmaxf;                                             // largest code
   __device__ __forceinline__ EpiBranch(const GemmBranch& b, int N)
-      : M(b.M), bits(b.q0.bits), cbits(b.out_bits), out_codes(b.out_codes), out_f(b.out_f), res(b.res), rowsrc(b.rowsrc),
+      : M(b.M), cbits(b.out_bits), out_codes(b.out_codes), out_f(b.out_f), res(b.res), rowsrc(b.rowsrc),
         row_bytes((long)N * b.out_bits / 8), qmaxf(b.q0.qmaxf) {}
 };
 
@@ -123,105 +146,109 @@ struct EpiBranch {
 template <int MODE, bool TAPS, class WaitFn>
 __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const EpiBranch& eb, int N, int C, long row0, int lane, int n_tile0,
                                                    int c_first, int c_step, int c_total, const ColConsts& cc,
-                                                   uint32_t taddr_tile, float* stage, bool narrow, bool in_range, float neg_zero, WaitFn acc_ready,
+                                                   uint32_t taddr_tile, bool narrow, bool in_range, float neg_zero, WaitFn acc_ready,
                                                    float* res_ring = nullptr /* per warp: RES_SLOTS x 32 x 16 floats */) {
-  const long m = row0 + lane;
-  const bool row_ok = m < eb.M;
+  // this lane's rows: row0 + 8 i + rsub, i = 0 ... 3; rows_left: how many of the warp's rows exist
+  const int cj = lane & 3, rsub = lane >> 2;
+  const int rows_left = row0 + 32 <= eb.M ? 32 : (int)(eb.M - row0);
   constexpr int NC = MODE == EPI_QKV || MODE == EPI_FC1 ? CODE_NC : F32_NC;
+  constexpr int LANE_COLS = NC / 4;                        // consecutive columns of a lane
   const int n_chunks = c_first < c_total ? (c_total - c_first + c_step - 1) / c_step : 0;
-  const int n_first = n_tile0 + c_first * NC;              // global column of the warp's first chunk
+  const int n_first = n_tile0 + c_first * NC + LANE_COLS * cj;   // global column of this lane's first one
+  const int lc_first = c_first * NC + LANE_COLS * cj;            // and within the tile
   const int col_step = c_step * NC;                        // distance between consecutive chunks of the warp
   const uint32_t taddr = taddr_tile + (uint32_t)(c_first * NC);
+  auto tap_at = [&](int i, int col) -> int32_t* {          // the accumulator tap of this lane's i-th row, tile column col
+    return TAPS && br.tap_acc && 8 * i + rsub < rows_left ? br.tap_acc + (row0 + 8 * i + rsub) * N + n_tile0 + col : nullptr;
+  };
 
   if (MODE == EPI_QKV || MODE == EPI_FC1) {
-    // ---- code outputs: every thread quantizes and packs the 32 codes of its own row ----
+    // ---- code outputs: a thread quantizes and packs 8 codes of each of its four rows; a quad stores 32 codes side by side ----
     // a tile lies within one of the q, k, v sections (its width divides a section's), so its quantizer is the tile's
     const AQ& q = MODE == EPI_FC1 || n_tile0 < C ? br.q0 : (n_tile0 < 2 * C ? br.q1 : br.q2);
     const float inv_scale = q.inv_scale, zpf = q.zpf;
-    const int cbits = eb.cbits, bits = eb.bits;
-    const uint32_t zbias = (MODE == EPI_FC1 ? 0u : (uint32_t)q.zp) - kMagicBits;
+    const int cbits = eb.cbits;
+    const uint32_t zp2 = (uint32_t)q.zp * 0x10001u, qmax2 = (uint32_t)eb.qmaxf * 0x10001u;
     const float magic_zp = 12582912.0f + zpf;                              // FC1
     const float thr = gelu_threshold(inv_scale, eb.qmaxf);                 // FC1
-    // this thread's output position of the warp's first chunk
-    uint8_t* out_ptr = eb.out_codes + m * eb.row_bytes + n_first * cbits / 8;
+    // this thread's output position in its first row of the warp's first chunk, and the distance of its rows
+    uint8_t* out_ptr = eb.out_codes + (row0 + rsub) * eb.row_bytes + n_first * cbits / 8;
+    const int row_step = 8 * (int)eb.row_bytes;
     const int out_step = col_step * cbits / 8;
     if (!acc_ready()) return false;
-    // the quantizer's width as a constant (a shift in the packing)
-    auto walk = [&](auto bits_tag) {
-      constexpr int SH = 8 - decltype(bits_tag)::value;
-      // 32 columns at a time, without a branch between them: the dependent chain of a value is about twenty operations
-      // long, and with four warps per scheduler only independent values hide its latency.  The accumulator comes in halves of 16
-      // columns, each requested a half ahead, the first one of the next chunk behind the second one of this.
-      int32_t first[CODE_NC / 2], second[CODE_NC / 2];
-      if (n_chunks > 0) tmem_ld(taddr, first);
+    // 32 columns at a time, without a branch between them: the dependent chain of a value is about twenty operations
+    // long, and with three warps per scheduler only independent values hide its latency.  The accumulator comes in halves of 16
+    // columns (four of this lane's in each of its rows), each requested a half ahead, the first one of the next chunk behind the
+    // second one of this.
+    int32_t first[16], second[16];
+    if (n_chunks > 0) tmem_ld_quads32(taddr, first);
 #pragma unroll 1
-      for (int ch = 0; ch < n_chunks; ++ch) {
-        const uint32_t ta = taddr + (uint32_t)(ch * col_step);
-        const int col = c_first * CODE_NC + ch * col_step;
-        uint32_t w[8];
-        float dist[4];
+    for (int ch = 0; ch < n_chunks; ++ch) {
+      const uint32_t ta = taddr + (uint32_t)(ch * col_step);
+      const int lc = lc_first + ch * col_step;
+      uint32_t w[4][2];                                                    // [row][half of the columns]
+      float dist[4];                                                       // [2 * half of the columns + half of the rows]
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (h == 0) { tmem_ld_wait(first); tmem_ld_quads32(ta + 16u, second); }
+        else        { tmem_ld_wait(second); if (ch + 1 < n_chunks) tmem_ld_quads32(ta + (uint32_t)col_step, first); }
+        const int32_t (&a)[16] = h == 0 ? first : second;
+        Consts4 k;
+        k.load<true>(cc, lc + 4 * h);
+        dist[2 * h] = 0.0f; dist[2 * h + 1] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int o = 8 * (i >> 1) + 2 * (i & 1);
+          float2 v0, v1;
+          uint32_t c[4];
+          dequant4<MODE, TAPS, false>(k, a[o], a[o + 1], a[o + 4], a[o + 5], tap_at(i, lc + 4 * h), v0, v1);
+          if (MODE == EPI_FC1) {
+            float& d = dist[2 * h + (i >> 1)];
+            gelu_pattern2(v0, inv_scale, magic_zp, d, c[0], c[1]); gelu_pattern2(v1, inv_scale, magic_zp, d, c[2], c[3]);
+          } else {
+            quant_pattern2(v0, inv_scale, neg_zero, c[0], c[1]); quant_pattern2(v1, inv_scale, neg_zero, c[2], c[3]);
+          }
+          w[i][h] = clamp_pack4<MODE != EPI_FC1>(c[0], c[1], c[2], c[3], zp2, qmax2);
+        }
+      }
+      // Half of the columns of half of the rows again by the contract's own operations: where some value of the warp is too close
+      // to a rounding boundary, and all of them where the patterns above do not hold.  A sixth of the chunks at A8 has a value
+      // within the bound for the largest code; with the bound for the lane's own codes, which are mostly small, few of them are left.
+      const bool near = MODE == EPI_FC1 && fmaxf(fmaxf(dist[0], dist[1]), fmaxf(dist[2], dist[3])) >= thr;
+      if (!in_range || (MODE == EPI_FC1 && __any_sync(0xffffffffu, near))) {
+        tmem_ld_wait(first);                                 // nothing may be on its way into registers across a call
+        uint32_t todo = 0;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-          if (g == 0) { tmem_ld_wait(first); tmem_ld(ta + CODE_NC / 2, second); }
-          if (g == 2) { tmem_ld_wait(second); if (ch + 1 < n_chunks) tmem_ld(ta + (uint32_t)col_step, first); }
-          float v[8];
-          uint32_t c[8];
-          dequant<MODE, TAPS, false, 8>(br, N, m, row_ok, n_tile0 + col + 8 * g, col + 8 * g, cc, (g < 2 ? first : second) + 8 * (g & 1), v);
-          dist[g] = 0.0f;
-#pragma unroll
-          for (int i = 0; i < 8; i += 2) {
-            if (MODE == EPI_FC1) gelu_pattern2(make_float2(v[i], v[i + 1]), inv_scale, magic_zp, dist[g], c[i], c[i + 1]);
-            else quant_pattern2(make_float2(v[i], v[i + 1]), inv_scale, neg_zero, c[i], c[i + 1]);
-          }
-          w[2 * g] = sat_pack4<SH>(c[0], c[1], c[2], c[3], zbias << SH);
-          w[2 * g + 1] = sat_pack4<SH>(c[4], c[5], c[6], c[7], zbias << SH);
+          uint32_t any = w[2 * (g & 1)][g >> 1] | w[2 * (g & 1) + 1][g >> 1];      // no code is above the bits of all of them
+          any |= any >> 16; any |= any >> 8;
+          const float t = gelu_threshold(inv_scale, fmaxf((float)(any & 0xFFu), zpf));
+          if (!in_range || __any_sync(0xffffffffu, dist[g] >= t)) todo |= 1u << g;
         }
-        // Eight columns again by the contract's own operations: where some value of the warp is too close to a rounding boundary
-        // (FC1, a sixth of the chunks at A8), and all of them where the patterns above do not hold
-        const bool near = MODE == EPI_FC1 && fmaxf(fmaxf(dist[0], dist[1]), fmaxf(dist[2], dist[3])) >= thr;
-        if (!in_range || (MODE == EPI_FC1 && __any_sync(0xffffffffu, near))) {
 #pragma unroll 1
-          for (int g = 0; g < 4; ++g) {
-            const float d = g == 0 ? dist[0] : g == 1 ? dist[1] : g == 2 ? dist[2] : dist[3];
-            if (in_range && !__any_sync(0xffffffffu, d >= thr)) continue;
-            int32_t again[8];
-            tmem_ld(ta + (uint32_t)(8 * g), again);
-            tmem_ld_wait(again);
-            float v[8];
-            uint32_t c[8];
-            dequant<MODE, TAPS, false, 8>(br, N, m, row_ok, n_tile0 + col + 8 * g, col + 8 * g, cc, again, v);
+        for (int g = 0; g < 4; ++g) {
+          if (!(todo >> g & 1u)) continue;
+          const int h = g >> 1, i0 = 2 * (g & 1);
+          const uint2 pk = codes_exact8<MODE>(ta + ((uint32_t)(8 * i0) << 16) + (uint32_t)(16 * h), cc, lc + 4 * h, inv_scale, zpf, eb.qmaxf);
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {
-              const float2 x = make_float2(v[i], v[i + 1]);
-              quant_magic2(MODE == EPI_FC1 ? gelu_f2(x) : x, inv_scale, -zpf, eb.qmaxf - zpf, c[i], c[i + 1]);
-            }
-            const uint32_t zb = (uint32_t)q.zp - kMagicBits;
-            const uint32_t w0 = sat_pack4<SH>(c[0], c[1], c[2], c[3], zb << SH), w1 = sat_pack4<SH>(c[4], c[5], c[6], c[7], zb << SH);
-            w[0] = g == 0 ? w0 : w[0]; w[1] = g == 0 ? w1 : w[1];
-            w[2] = g == 1 ? w0 : w[2]; w[3] = g == 1 ? w1 : w[3];
-            w[4] = g == 2 ? w0 : w[4]; w[5] = g == 2 ? w1 : w[5];
-            w[6] = g == 3 ? w0 : w[6]; w[7] = g == 3 ? w1 : w[7];
-          }
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) w[i][hh] = g == 2 * hh + (i >> 1) ? ((i & 1) ? pk.y : pk.x) : w[i][hh];
         }
-        if (row_ok) store_sat32(out_ptr + ch * out_step, w, bits, cbits);
       }
-    };
-    if (bits == 8) walk(std::integral_constant<int, 8>{});
-    else if (bits == 4) walk(std::integral_constant<int, 4>{});
-    else walk(std::integral_constant<int, 2>{});
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (8 * i + rsub < rows_left) store_codes8(out_ptr + i * (long)row_step + ch * out_step, w[i][0], w[i][1], cbits);
+    }
     return true;
   }
 
   // ---- binary32 outputs (proj: x1 = x_window + out; fc2: y = x1 + out scattered to the token's own position;
-  //      merge: out).  The raw sums of a 16-column chunk are transposed through shared memory so that global accesses are
-  //      64-byte runs (4 lanes per row, 8 rows per instruction), and a lane then needs the constants of 4 columns only:
-  //      these launches are bound by the load/store pipe, and constants read per row and column were a third of its work.
-  //      (32-column chunks with 128-byte runs: 86 against 68 us for a proj of 296 450 rows of 128 channels -- half the
-  //      chunks in flight per warp, and the addresses of eight rows spill.) ----
-  const int cj = lane & 3, rsub = lane >> 2;
-  long src_mine = -1;
-  if (MODE != EPI_MERGE && row_ok) src_mine = eb.rowsrc[m];
-  // this lane's four (row, 16-byte piece) positions of the warp's first chunk: residual source and output, NULL: none
+  //      merge: out).  A lane holds 16 bytes of a row, so global accesses are 64-byte runs (4 lanes per row, 8 rows per instruction)
+  //      and the constants are those of 4 columns. ----
+  int src_mine = -1;
+  if (MODE != EPI_MERGE && lane < rows_left) src_mine = eb.rowsrc[row0 + lane];
+  // this lane's four pieces of the warp's first chunk: residual source and output, NULL: none
   const float* res_ptr[4];
   float* dst_ptr[4];
 #pragma unroll
@@ -229,28 +256,26 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
     const int r = 8 * i + rsub;
     const long mr = row0 + r;
     const long s = __shfl_sync(0xffffffffu, src_mine, r);
-    const bool ok = mr < eb.M;
+    const bool ok = r < rows_left;
     long res_row, dst_row;               // row offsets (in elements), -1: none
     if (MODE == EPI_PROJ)     { res_row = (ok && s >= 0) ? s * N : -1;  dst_row = ok ? mr * N : -1; }
     else if (MODE == EPI_FC2) { res_row = (ok && s >= 0) ? mr * N : -1; dst_row = (ok && s >= 0) ? s * N : -1; }
     else                      { res_row = -1;                            dst_row = ok ? mr * N : -1; }
-    res_ptr[i] = (MODE != EPI_MERGE && res_row >= 0) ? eb.res + res_row + n_first + 4 * cj : nullptr;
-    dst_ptr[i] = dst_row >= 0 ? eb.out_f + dst_row + n_first + 4 * cj : nullptr;
+    res_ptr[i] = (MODE != EPI_MERGE && res_row >= 0) ? eb.res + res_row + n_first : nullptr;
+    dst_ptr[i] = dst_row >= 0 ? eb.out_f + dst_row + n_first : nullptr;
   }
-  // The residual rows come into shared memory by asynchronous copies, RES_SLOTS chunks ahead of their use: the copies
+  // The residual pieces come into shared memory by asynchronous copies, RES_SLOTS chunks ahead of their use: the copies
   // of a whole tile are in flight while the accumulator is still being computed, and they cost no registers.
-  // Slot ch % RES_SLOTS holds chunk ch in the layout of the transposition tile (row r, 16-byte piece j at piece
-  // j ^ ((r >> 1) & 3)).  One commit group per chunk, also when there is nothing left to fetch, so that "all but the
-  // newest RES_SLOTS - 1 groups are complete" always covers the chunk about to be used.
+  // Slot ch % RES_SLOTS holds chunk ch; a lane reads what it has copied itself, so nothing but its own copies is waited for.  One
+  // commit group per chunk, also when there is nothing left to fetch, so that "all but the newest RES_SLOTS - 1 groups are
+  // complete" always covers the chunk about to be used.
   auto fetch = [&](int ch) {
     if (MODE != EPI_MERGE && ch < n_chunks) {
-      float* slot = res_ring + (ch % RES_SLOTS) * EPI_STAGE_FLOATS;
+      float* slot = res_ring + (ch % RES_SLOTS) * EPI_CHUNK_FLOATS + 4 * lane;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = 8 * i + rsub;
-        float* dst = slot + r * F32_NC + 4 * (cj ^ ((r >> 1) & 3));
-        if (res_ptr[i]) cp_async16(dst, res_ptr[i] + ch * col_step);
-        else *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);   // a pad token's residual input is zero
+        if (res_ptr[i]) cp_async16(slot + 128 * i, res_ptr[i] + ch * col_step);
+        else *reinterpret_cast<float4*>(slot + 128 * i) = make_float4(0.f, 0.f, 0.f, 0.f);   // a pad token's residual input is zero
       }
     }
     cp_async_commit();
@@ -262,50 +287,38 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
   if (!acc_ready()) { cp_async_wait<0>(); return false; }
   auto walk = [&](auto narrow_tag) {
     constexpr bool NARROW = decltype(narrow_tag)::value;
-    int32_t acc[F32_NC];
-    if (n_chunks > 0) tmem_ld(taddr, acc);
-#pragma unroll 1
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const int lc = c_first * F32_NC + ch * col_step + 4 * cj;       // this lane's first column within the tile
-      tmem_ld_wait(acc);
-      // row `lane`, logical 16-byte piece j is stored at piece j ^ ((lane >> 1) & 3): conflict-free both ways
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        *reinterpret_cast<int4*>(stage + lane * F32_NC + 4 * (j ^ ((lane >> 1) & 3))) =
-            make_int4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-      // the TMEM load of the next chunk is in flight while this chunk is finished
-      if (ch + 1 < n_chunks) tmem_ld(taddr + (uint32_t)((ch + 1) * col_step), acc);
-      const int4 p4 = *reinterpret_cast<const int4*>(cc.pre + lc);
-      const float4 m4 = *reinterpret_cast<const float4*>(cc.mult + lc);
-      float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (MODE != EPI_MERGE) b4 = *reinterpret_cast<const float4*>(cc.bias + lc);
+    auto finish = [&](int ch, const int32_t (&a)[16]) {
+      const int lc = lc_first + ch * col_step;
+      Consts4 k;
+      k.load<MODE != EPI_MERGE>(cc, lc);
       if (MODE != EPI_MERGE) cp_async_wait<RES_SLOTS - 1>();     // this lane's copies of chunk ch have landed
-      __syncwarp();
-      const float* slot = res_ring + (ch % RES_SLOTS) * EPI_STAGE_FLOATS;
+      const float* slot = res_ring + (ch % RES_SLOTS) * EPI_CHUNK_FLOATS + 4 * lane;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = 8 * i + rsub;
-        const int off = r * F32_NC + 4 * (cj ^ ((r >> 1) & 3));
-        const int4 a = *reinterpret_cast<const int4*>(stage + off);
-        if (TAPS && br.tap_acc && row0 + r < eb.M) {
-          int32_t* tp = br.tap_acc + (row0 + r) * N + n_tile0 + lc;
-          tp[0] = a.x + p4.x - (int32_t)kMagicBits; tp[1] = a.y + p4.y - (int32_t)kMagicBits;
-          tp[2] = a.z + p4.z - (int32_t)kMagicBits; tp[3] = a.w + p4.w - (int32_t)kMagicBits;
-        }
-        if (!dst_ptr[i]) continue;
-        const float2 f0 = acc_to_float2<NARROW>(a.x + p4.x, a.y + p4.y), f1 = acc_to_float2<NARROW>(a.z + p4.z, a.w + p4.w);
+        const int o = 8 * (i >> 1) + 2 * (i & 1);
         float2 lo, hi;
-        if (MODE == EPI_MERGE) {
-          lo = __fmul2_rn(f0, make_float2(m4.x, m4.y)); hi = __fmul2_rn(f1, make_float2(m4.z, m4.w));
-        } else {
-          const float4 rr = *reinterpret_cast<const float4*>(slot + off);
-          lo = __fadd2_rn(make_float2(rr.x, rr.y), __ffma2_rn(f0, make_float2(m4.x, m4.y), make_float2(b4.x, b4.y)));
-          hi = __fadd2_rn(make_float2(rr.z, rr.w), __ffma2_rn(f1, make_float2(m4.z, m4.w), make_float2(b4.z, b4.w)));
+        dequant4<MODE, TAPS, NARROW>(k, a[o], a[o + 1], a[o + 4], a[o + 5], tap_at(i, lc), lo, hi);
+        if (!dst_ptr[i]) continue;
+        if (MODE != EPI_MERGE) {
+          const float4 rr = *reinterpret_cast<const float4*>(slot + 128 * i);
+          lo = __fadd2_rn(make_float2(rr.x, rr.y), lo); hi = __fadd2_rn(make_float2(rr.z, rr.w), hi);
         }
         *reinterpret_cast<float4*>(dst_ptr[i] + ch * col_step) = make_float4(lo.x, lo.y, hi.x, hi.y);
       }
-      __syncwarp();
       if (MODE != EPI_MERGE) fetch(ch + RES_SLOTS);              // the slot just read is free again
+    };
+    // two chunks in turn, each requested one ahead
+    int32_t even[16], odd[16];
+    if (n_chunks > 0) tmem_ld_quads32(taddr, even);
+#pragma unroll 1
+    for (int ch = 0; ch < n_chunks; ch += 2) {
+      tmem_ld_wait(even);
+      if (ch + 1 < n_chunks) tmem_ld_quads32(taddr + (uint32_t)((ch + 1) * col_step), odd);
+      finish(ch, even);
+      if (ch + 1 >= n_chunks) break;
+      tmem_ld_wait(odd);
+      if (ch + 2 < n_chunks) tmem_ld_quads32(taddr + (uint32_t)((ch + 2) * col_step), even);
+      finish(ch + 1, odd);
     }
   };
   if (narrow) walk(std::true_type{}); else walk(std::false_type{});

@@ -12,8 +12,8 @@
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
 //               the swizzled layout (rows whose byte pitch is no multiple of 16 cannot be described to the TMA
 //               unit and are read with plain loads instead);
-//   then        epilogue (12 warps for the code outputs, 8 or 12 for the binary32 outputs): tcgen05.ld (one row per thread,
-//               16 or 32 columns per load) + the fused epilogue of the mode.
+//   then        epilogue (12 warps for the code outputs, 8 or 12 for the binary32 outputs): tcgen05.ld (a quad of lanes
+//               per row, 16 columns per load) + the fused epilogue of the mode.
 // Every wait on an mbarrier is bounded; on expiry the CTA raises the status word, then waits (bounded again) for the
 // copies it has issued to land and for the MMAs it has issued to retire, frees its tensor memory and returns.
 #include "tc_ptx.cuh"
@@ -57,6 +57,7 @@ constexpr int SIDE_REGS = 56;
 __host__ __device__ constexpr int epi_regs(int warps, bool packed) { return warps != 12 ? 0 : packed ? 112 : 136; }    // 0: no exchange
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
+__host__ __device__ constexpr int lane_cols(int mode) { return (code_mode(mode) ? CODE_NC : F32_NC) / 4; }   // columns of a lane in a chunk
 constexpr int MAX_RING = 6;
 constexpr int TMEM_COLS = 512;                 // one CTA per SM: it takes all of the tensor memory
 constexpr int MAX_ACC = 6;                     // accumulators in it, as far as the tile width allows
@@ -80,16 +81,15 @@ struct TcParams {
 
 // shared-memory carve-up (offsets from the 1024-byte aligned base)
 struct SmemLayout {
-  int stage_bytes, ring_bytes, consts_off, stage_off, res_off, bars_off, total;
+  int stage_bytes, ring_bytes, consts_off, res_off, bars_off, total;
 };
 constexpr int NUM_BARS = 4 * MAX_RING + 2 * MAX_ACC + 2;        // full, empty, raw, unpacked; accumulator full, empty; constants, drain
-__host__ __device__ inline SmemLayout smem_layout(int BN, int ring, int packed_bytes, int res_bytes, int const_cols, int mode, int warps) {
+__host__ __device__ inline SmemLayout smem_layout(int BN, int ring, int packed_bytes, int res_bytes, int const_cols) {
   SmemLayout L;
   L.stage_bytes = A_STAGE_BYTES + BN * BK + packed_bytes;
   L.ring_bytes = ring * L.stage_bytes;
   L.consts_off = L.ring_bytes;                                  // (pre, mult, bias) of const_cols columns
-  L.stage_off = L.consts_off + 3 * const_cols * 4;    // binary32 epilogues: a 32 x 16 chunk per warp
-  L.res_off = L.stage_off + (code_mode(mode) ? 0 : warps * EPI_STAGE_FLOATS * 4);   // and their residual rings
+  L.res_off = L.consts_off + 3 * const_cols * 4;                // residual rings of proj and fc2
   L.bars_off = L.res_off + res_bytes;
   L.total = L.bars_off + NUM_BARS * 8 + 16;                     // then TMEM base, abort flag, constants-out-of-range flags
   return L;
@@ -125,7 +125,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;                 // swizzled tiles need 1024-byte alignment
   uint8_t* smem = smem_raw + (base - raw);
-  const SmemLayout L = smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW);
+  const SmemLayout L = smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols);
   const int stage_bytes = L.stage_bytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars_off);
   const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8u * MAX_RING, bar_raw = bar_empty + 8u * MAX_RING;
@@ -138,6 +138,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   // the give-up path only.
   uint32_t fills = 0, raw_used = 0, raw_phase = 0;
 
+  constexpr int LANE_COLS = lane_cols(MODE);
   constexpr int NUM_EPI_WARPS = EW, FIRST_EPI_WARP = first_epi_warp(PACKED);
   constexpr int NUM_UNPACK_WARPS = UNPACK_WARPS, NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
   constexpr int UNPACK_ITEMS = BM * (BK / UMMA_K) / NUM_UNPACK_THREADS;   // (row, 32-code group) items per thread and stage
@@ -212,7 +213,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
             ++fills;
             if (leader) {
               mbar_arrive_expect_tx(bar_full + o, tx);
-              tma_load_2d(sb, &tmB, kb * BK, n_row, bar_full + o);
+              tma_load_5d(sb, &tmB, kb * BK, n_row / (4 * LANE_COLS), bar_full + o);
             }
             if (!waited) { griddep_wait(); waited = true; }
             if (leader && !packed) tma_load_2d(sa, tmA, kb * BK, m_row, bar_full + o);
@@ -350,8 +351,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(epi_regs(EW, PACKED) > 0 ? epi_regs(EW, PACKED) : 24));
     const int e = warp - FIRST_EPI_WARP, q = warp & 3;         // any 4 consecutive warps cover the 4 lane quarters
     const int split = p.split, groups = p.groups, group = (e >> 2) / split, sub = (e >> 2) - group * split;
-    float* stage = reinterpret_cast<float*>(smem + L.stage_off) + e * EPI_STAGE_FLOATS;
-    float* res_ring = reinterpret_cast<float*>(smem + L.res_off) + e * RES_SLOTS * EPI_STAGE_FLOATS;
+    float* res_ring = reinterpret_cast<float*>(smem + L.res_off) + e * RES_SLOTS * EPI_CHUNK_FLOATS;
     int32_t* c_pre = reinterpret_cast<int32_t*>(smem + L.consts_off);
     float* c_mult = reinterpret_cast<float*>(c_pre + p.const_cols);
     float* c_bias = c_mult + p.const_cols;
@@ -411,7 +411,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
           return true;
         };
         if (!epilogue_warp_tile<MODE, TAPS>(br, eb, p.g.N, p.g.C, row0, lane, n_tile0, sub, split, c_total, cc,
-                                            tmem_q + (uint32_t)(acc * p.acc_stride), stage, narrow, in_range, p.g.neg_zero,
+                                            tmem_q + (uint32_t)(acc * p.acc_stride), narrow, in_range, p.g.neg_zero,
                                             acc_ready, res_ring)) { ok = false; break; }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -507,7 +507,7 @@ bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
     p.tma_packed[i] = g.br[i].M > 0 && bits != 8 && ((long)g.K * bits / 8) % 16 == 0;
     if (p.tma_packed[i]) p.packed_bytes = BM * (BK / 2);        // room for the widest packed format (4 bit)
   }
-  p.res_bytes = (g.mode == EPI_PROJ || g.mode == EPI_FC2) ? EW * RES_SLOTS * EPI_STAGE_FLOATS * 4 : 0;
+  p.res_bytes = (g.mode == EPI_PROJ || g.mode == EPI_FC2) ? EW * RES_SLOTS * EPI_CHUNK_FLOATS * 4 : 0;
   p.acc_stride = p.BN;
   CUtensorMap mA[2], mB;
   memset(mA, 0, sizeof(mA));
@@ -522,7 +522,7 @@ bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
       ok = make_map(&mA[i], g.w, (uint64_t)g.N, (uint64_t)g.K, (uint32_t)p.BN);
     if (!ok) return false;
   }
-  if (!make_map(&mB, g.w, (uint64_t)g.N, (uint64_t)g.K, (uint32_t)p.BN)) return false;
+  if (!make_quad_map(&mB, g.w, (uint64_t)g.N, (uint64_t)g.K, (uint32_t)p.BN, 4 * lane_cols(MODE))) return false;
   // a grid that is a multiple of the number of column tiles keeps every CTA on one column tile (t mod n_tiles);
   // taken only where it does not cost a wave of tiles
   int grid = total_tiles < sms ? total_tiles : sms;
@@ -535,8 +535,8 @@ bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
   p.const_cols = p.step_n == 0 || total_tiles == grid ? p.BN : g.N;
   p.last_step = total_tiles - 1;
   p.ring = MAX_RING;
-  while (p.ring > 2 && smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW).total + 1024 > 220 * 1024) --p.ring;
-  const size_t smem = (size_t)smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols, MODE, EW).total + 1024 /*alignment slack*/;
+  while (p.ring > 2 && smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols).total + 1024 > 220 * 1024) --p.ring;
+  const size_t smem = (size_t)smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols).total + 1024 /*alignment slack*/;
   if (smem > 227 * 1024) return false;
   if (g.br[0].tap_acc || g.br[1].tap_acc)
     launch_pdl(k_gemm_tc<MODE, true, EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);

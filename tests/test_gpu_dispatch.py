@@ -74,6 +74,18 @@ def test_gemm_accumulators_beyond_the_bias_trick(orc, mq, ctx, dim, sign):
     run_block_case(orc, mq, ctx, blk, synth.input_blobs(dim, 1, 17, 23, dim, bg_std=0.5, gain=4.0), 0.4)
 
 
+@pytest.mark.parametrize("dim,bits,factor", [(96, (8, 4), 20.0), (32, (4, 2), 20.0), (128, (8, 2), 20.0), (128, (8, 4), 3000.0),
+                                             (64, (4, 2), 3000.0)])
+def test_gemm_code_outputs_far_beyond_their_range(orc, mq, ctx, dim, bits, factor):
+    """Sums of which most lie beyond both ends of the codes: within the 16-bit patterns of the fast quantizers, and beyond
+    them, where all codes come from the contract's own operations; rows that are no multiple of a warp's."""
+    blk = synth.make_block(np.random.default_rng(dim), dim, dim // 32, 3, 4, *bits, share_bias=False)
+    for lin in (blk.qkv, blk.fc1):
+        lin.scale[:] = (lin.scale * F32(factor)).astype(F32)
+    for taps in (False, True):
+        run_block_case(orc, mq, ctx, blk, synth.input_student_t(dim, 1, 17, 23, dim), 0.4, taps=taps)
+
+
 @pytest.mark.parametrize("pairs", [5, 10])
 @pytest.mark.parametrize("own_stream", [False, True])
 def test_block_graphs_follow_data_buffers_and_switch(orc, mq, pairs, own_stream):
