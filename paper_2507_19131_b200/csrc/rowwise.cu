@@ -83,6 +83,8 @@ __device__ __forceinline__ void ln_g_finish(const LnBranch& br, const float (&x)
       for (int k = 0; k < o; ++k) p[k] = __fadd_rn(p[k], p[k + o]);
     return p[0];
   };
+  // the division by the number of channels: by a power of two it is a multiplication with the same rounding
+  auto over_c = [](float v) { return (C & (C - 1)) == 0 ? __fmul_rn(v, 1.0f / C) : __fdiv_rn(v, (float)C); };
   // neighbouring partials are summed as pairs (packed binary32 arithmetic: each lane adds in the same order)
   float p[P];
 #pragma unroll
@@ -92,7 +94,7 @@ __device__ __forceinline__ void ln_g_finish(const LnBranch& br, const float (&x)
     for (int i = 0; i < NG; ++i) s = __fadd2_rn(s, make_float2(x[i][k], x[i][k + 1]));
     p[k] = s.x; p[k + 1] = s.y;
   }
-  const float mean = __fdiv_rn(reduce32(p), (float)C);
+  const float mean = over_c(reduce32(p));
 #pragma unroll
   for (int k = 0; k < P; k += 2) {
     float2 v = f2(0.0f);
@@ -100,7 +102,7 @@ __device__ __forceinline__ void ln_g_finish(const LnBranch& br, const float (&x)
     for (int i = 0; i < NG; ++i) { const float2 d = sub2(make_float2(x[i][k], x[i][k + 1]), f2(mean)); v = __ffma2_rn(d, d, v); }
     p[k] = v.x; p[k + 1] = v.y;
   }
-  const float var = __fdiv_rn(reduce32(p), (float)C);
+  const float var = over_c(reduce32(p));
   const float rstd = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(var, 1e-5f)));
   if (m >= M) return;
   // the normalisation, the quantizer and the packing with the bit width as a compile-time constant (a CTA works for
@@ -219,13 +221,15 @@ __global__ void __launch_bounds__(256, (NG * (32 / G) > 24 ? 2 : 4)) k_ln_quant_
 
 // The same for batches that keep every SM busy for a while: persistent warps walk over row groups and fetch STAGES groups
 // ahead by asynchronous copies into shared memory, every thread into slots that it alone reads back (no barrier).  The plain
-// kernel alternates between waiting for its loads and computing: 45 to 50 us at 296 450 rows of 128 channels (180 MB, 3.6 to 4
-// TB/s), this one 40 (4.5 TB/s); 148 225 rows of 256 channels 26 and 21.5.  Eight lanes per row: with 16 the shuffles cost more
-// (50 us), with 4 the chain of a lane (59).
+// kernel alternates between waiting for its loads and computing.  What bounds this one is the chain of reductions and divisions of
+// a row group, so warps count for more than copies ahead: three CTAs per SM with two stages against two with three, 294 912 rows of
+// 128 channels (189 MB) 50.5 -> 35.5 us (3.7 -> 5.3 TB/s), 65 536 rows of 192 channels 13.5 -> 12.3, 73 728 rows of 256 channels
+// 18.6 -> 17.8; four CTAs 36.8 (spills at 256).  Eight lanes per row: with 16 the shuffles cost more, with 4 the chain of a lane;
+// at 384 and 512 channels, with 16 lanes, it is slower than the plain kernel (16 384 rows of 384: 8.4 -> 9.6 us).
 __device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(src) : "memory");
 }
-constexpr int LN_STAGES = 3, LN_STREAM_CTAS = 2;
+constexpr int LN_STAGES = 2, LN_STREAM_CTAS = 3;
 template <int NG, int G> constexpr int ln_stream_smem() { return LN_STAGES * NG * (32 / G) * 256 * 4; }
 template <int NG, int G>
 __global__ void __launch_bounds__(256, LN_STREAM_CTAS) k_ln_stream(LnBranch hi, LnBranch lo, int groups_hi, int groups) {
@@ -352,8 +356,9 @@ void launch_ln_g(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
   launch_pdl(k_ln_quant_g<NG, G, MERGE>, dim3(bh + bl), 256, 0, st, hi, lo, bh);
 }
 
-// elements per SM from which the streaming LayerNorm is used: below, its 16 warps have fewer than eight groups of 4 rows x 128
-// channels each, and the set-up of the persistent grid costs what the overlap gives
+// Elements per SM from which the streaming LayerNorm is used: below, its 24 warps have fewer than six groups of 4 rows x 128
+// channels each, and the set-up of the persistent grid costs more than the overlap gives (43 300 elements per SM: 66 800 rows of 96
+// channels 7.5 us by the plain kernel, 10.1 by this one; 85 000: 65 536 rows of 192 channels 13.5 by this one with two CTAs, 12.3)
 constexpr long LN_STREAM_MIN = 65536;
 template <int NG, int G>
 void launch_ln_stream(const LnBranch& hi, const LnBranch& lo, cudaStream_t st) {
@@ -378,7 +383,6 @@ void launch_ln_quant(const LnBranch& hi, const LnBranch& lo, int C, cudaStream_t
   const int rows = hi.M + lo.M;
   const int min_bits = hi.M > 0 && lo.M > 0 ? (hi.q.bits < lo.q.bits ? hi.q.bits : lo.q.bits) : (hi.M > 0 ? hi.q.bits : lo.q.bits);
   bool done = false;
-  // streaming kernel: from eight row groups per warp of the persistent grid on
   const long elems = (long)rows * C;
   if (elems >= LN_STREAM_MIN * sm_count()) {
     done = true;
