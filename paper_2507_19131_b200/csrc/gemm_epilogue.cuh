@@ -80,8 +80,8 @@ __device__ __forceinline__ void quant_pattern2(float2 x, float inv_scale, float 
   const float2 t = __fadd2_rn(__ffma2_rn(x, f2(inv_scale), f2(neg_zero)), f2(12582912.0f));
   m0 = __float_as_uint(t.x); m1 = __float_as_uint(t.y);
 }
-// FC1: code of GELU(v) from the special-function exponential instead of the contract's polynomial (a third of the
-// packed operations).  The value can differ from the contract's in the last bits, so `dist` collects the largest distance
+// FC1: code of GELU(v) from a polynomial of degree 6 and the special-function exponential instead of the contract's two polynomials
+// (a third of the packed operations).  The value can differ from the contract's in the last bits, so `dist` collects the largest distance
 // to the nearest integer; where it comes within the error bound of one half (see gelu_threshold) the caller recomputes.
 // The zero point is part of the rounding constant; at exact ties that changes the parity rule, and ties are recomputed.
 __device__ __forceinline__ void gelu_pattern2(float2 v, float inv_scale, float magic_zp, float& dist, uint32_t& m0, uint32_t& m1) {
@@ -94,12 +94,12 @@ __device__ __forceinline__ void gelu_pattern2(float2 v, float inv_scale, float m
   asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(dist) : "f"(d.x), "f"(d.y));
   m0 = __float_as_uint(r.x); m1 = __float_as_uint(r.y);
 }
-// Distance of g * inv_scale from the contract's t: both exponentials are within 2^-22 of 2^q, h = a 2^q <= 0.17, so h differs
-// by at most 0.17 * 2^-21 + one rounding < 1.0e-7; g is rounded in both evaluations and t in the contract's, which adds
+// Distance of g * inv_scale from the contract's t: the polynomials change h = a 2^q <= 0.17 by at most 6.4e-8, both exponentials are
+// within 2^-22 of theirs, so h differs by at most 6.4e-8 + 0.17 * 2^-21 + one rounding < 1.7e-7; g is rounded in both evaluations and t in the contract's, which adds
 // |t| * 3 * 2^-24, and |t| <= max(code, zp) + 1 for every t that is not clamped anyway; the distance itself is rounded by 2^-26.
 // maxf: at least the codes in question and the zero point
 __device__ __forceinline__ float gelu_threshold(float inv_scale, float maxf) {
-  return 0.5f - __fmaf_rn(inv_scale, 1.1e-7f, (maxf + 2.0f) * 1.8e-7f);
+  return 0.5f - __fmaf_rn(inv_scale, 1.9e-7f, (maxf + 2.0f) * 1.8e-7f);
 }
 
 // Four columns of two of the lane's rows by the contract's own operations, read again from tensor memory.  A function of its own: its
