@@ -228,7 +228,8 @@ mixaq_status mixaq_norm_forward(mixaq_ctx* ctx, const float* gamma, const float*
  *      weights = code x step size) with every window through the LayerNorm parameters and biases of one branch
  *      (branch 0: high, 1: low), writes its output map to y and the minimum / maximum each quantizer site saw to
  *      `ranges` (a HOST struct).  The quantizer fields of `p` are not read and `p->prepared` is not needed.
- *      mixaq_calibrate_merge does the same for a patch merging (one site: the LayerNorm output).
+ *      mixaq_calibrate_merge does the same for a patch merging (one site: the LayerNorm output).  The error of a matrix
+ *      product is a few roundings of binary64 relative to sum |a w| of the output itself, whatever the range of a row.
  *      Both synchronise the stream.  mixaq_aq_from_range is the one definition of the quantizer that covers a range:
  *      scale = (hi - lo) / (2^bits - 1), inv_scale = 1 / scale, zero_point = clamp(rne(-lo / scale), 0, 2^bits - 1). ---- */
 typedef struct { float lo, hi; } mixaq_range;

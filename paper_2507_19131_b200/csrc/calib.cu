@@ -118,70 +118,136 @@ __global__ void __launch_bounds__(256) k_cal_merge_ln(const float* __restrict__ 
 }
 
 // ---- matrix products ----------------------------------------------------------------------------------------------------
-// out[m][n] = (float)( sum_k a[m][k] * w[n][k] * sw[n]  + bias[n] ) with the sum exact or rounded in binary64, then per mode:
+// out[m][n] = (float)( sum_k a[m][k] * w[n][k] * sw[n]  + bias[n] ) with the sum to binary64 accuracy, then per mode:
 enum CalMode { CAL_QKV = 0, CAL_PROJ = 1, CAL_FC1 = 2, CAL_FC2 = 3, CAL_PLAIN = 4 };
 struct CalLinearArgs {
   const float* a; const int8_t* w; const float* sw; const float* bias;   // bias nullable
   float* out;                 // QKV, FC1, PLAIN: [M][N];  PROJ: x1 [M][N];  FC2: the output feature map
   const float* res;           // PROJ: input feature map (gathered through rowsrc);  FC2: x1 [M][N]
   const int32_t* rowsrc;      // PROJ, FC2
-  uint8_t* slices; int32_t* expo;   // workspace: [CAL_SLICES][M][K] bytes of the fixed-point rows, [M] their exponents
+  uint8_t* slices; int32_t* expo;   // workspace: [CAL_SLICES][M][K] bytes of the fixed-point rows, [M] their exponents or CAL_PLAIN_ROW
   long M; int N, K, C;        // C: width of one q/k/v section (QKV)
   uint32_t* obs;
   int* status;
 };
-// The weights are whole numbers times a step per output channel, so the product runs on the integer tensor cores: every row of
-// `a` becomes 56-bit fixed point with the row's largest exponent (values down to 2^-31 of the largest keep all their bits, the
-// others are rounded at 2^-55 of it), cut into seven bytes, the top one signed.  Each byte plane times the weight codes is an
-// exact int32 sum; the seven sums are put together in integers and three binary64 values, so an output sees at most one rounding
-// of 2^-55 per input and a handful of binary64 roundings where the plain binary64 sum has two per product.
+// The weights are whole numbers times a step per output channel, so the product runs on the integer tensor cores, by exact integer
+// slices of the operands (the Ozaki scheme): every row of `a` becomes 56-bit fixed point with the row's largest exponent, cut into
+// seven bytes, the top one signed.  Each byte plane times the weight codes is an exact int32 sum; the seven sums are put together in
+// integers and three binary64 values, a handful of binary64 roundings where the plain binary64 sum has one or two per product.
+// The 56 bits hold every bit of a value whose exponent is at most 31 below the row's largest.  A row with a smaller value (it would
+// lose bits, which are all that counts where the large ones meet weights of zero), or with an infinity or a NaN, is summed in
+// binary64 instead: k_cal_split knows it, and puts its sums where the product's epilogue then reads them.
 // A Swin-T calibration on a 200 x 334 map: 23.4 ms of products on the binary64 pipe (8.5 T products/s, about half of its rate),
-// 5.8 ms here and 1.3 ms for the byte planes.
-constexpr int CAL_NOT_FINITE = 255;      // exponent field of a row that holds an infinity or a NaN
+// 5.8 ms here and 1.35 ms for the byte planes.  One block of C = 96 on that map: 0.76 ms with usual rows, 1.8 with the rows of both
+// LayerNorms summed in binary64, 2.0 with all rows (20.7 with a serial loop per output in the product's epilogue).
+constexpr int CAL_PLAIN_ROW = 0;         // in place of the exponent (at least 1) of a row that is summed in binary64
 
-// One warp per row: the largest exponent, then the byte planes (a row of one plane is K bytes).
-__global__ void __launch_bounds__(256) k_cal_split(const float* __restrict__ a, uint8_t* __restrict__ slices,
-                                                   int32_t* __restrict__ expo, long M, int K) {
-  const long m = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (m >= M) return;
-  const uint4* row = reinterpret_cast<const uint4*>(a + m * K);
-  uint32_t top = 0;
-  for (int i = lane; i < K / 4; i += 32) {
-    const uint4 v = __ldg(row + i);
-    top = max(max(top, max(v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu)), max(v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu));
-  }
-  const int E = max(1, (int)(__reduce_max_sync(0xffffffffu, top) >> 23));
-  if (lane == 0) expo[m] = E;
-  for (int i = lane; i < K / 4; i += 32) {
-    const uint4 v = __ldg(row + i);
-    const uint32_t in[4] = {v.x, v.y, v.z, v.w};
-    uint32_t lo[4], hi[4];                                  // 56-bit two's complement: bytes 0-3 and 4-6
+// The sums of a CTA's plain rows (bit r of `todo`: row first + r), before residual and GELU, into their places of the output.
+// A thread has a column and four rows at a time, so that a weight is fetched and converted once for four products; a product of 24
+// and 8 bits is exact in binary64, and the sums run over k in ascending order.  All threads of the CTA come here together.
+constexpr int CAL_PLAIN_ROWS = 4, CAL_PLAIN_K = 128;
+__device__ __noinline__ void cal_plain_rows(const CalLinearArgs& p, bool scatter, long first, uint32_t todo, double (*sa)[CAL_PLAIN_K]) {
+  const int tid = threadIdx.x;
+  while (todo) {
+    long row[CAL_PLAIN_ROWS];
+    int rows = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = (in[j] >> 23) & 255;
-      const long long f = (in[j] & 0x7FFFFFu) | (e ? 0x800000u : 0u);
-      const int sh = (e ? e : 1) - E + 31;                  // at most 31
-      long long q = sh >= 0 ? f << sh : (sh < -25 ? 0 : (f + (1LL << (-sh - 1))) >> -sh);
-      if (in[j] >> 31) q = -q;
-      lo[j] = (uint32_t)q; hi[j] = (uint32_t)(q >> 32);
+    for (int r = 0; r < CAL_PLAIN_ROWS; ++r) {
+      row[r] = todo ? first + __ffs(todo) - 1 : row[0];
+      rows += todo ? 1 : 0;
+      todo &= todo - 1u;                                                      // (stays 0)
     }
+    for (int n0 = 0; n0 < p.N; n0 += (int)blockDim.x) {
+      const int n = n0 + tid;
+      const int8_t* w = p.w + (long)(n < p.N ? n : 0) * p.K;
+      double s[CAL_PLAIN_ROWS] = {};
+      for (int k0 = 0; k0 < p.K; k0 += CAL_PLAIN_K) {                         // K is a multiple of 32
+        const int kn = min(CAL_PLAIN_K, p.K - k0);
+        __syncthreads();
+        if (tid < kn) {
 #pragma unroll
-    for (int s = 0; s < CAL_SLICES; ++s) {
-      const uint32_t* x = s < 4 ? lo : hi;
-      const uint32_t sel = (uint32_t)(s & 3) | (uint32_t)((s & 3) + 4) << 4;
-      reinterpret_cast<uint32_t*>(slices + ((long)s * M + m) * K)[i] =
-          __byte_perm(__byte_perm(x[0], x[1], sel), __byte_perm(x[2], x[3], sel), 0x5410);
+          for (int r = 0; r < CAL_PLAIN_ROWS; ++r) sa[r][tid] = (double)__ldg(p.a + row[r] * p.K + k0 + tid);
+        }
+        __syncthreads();
+        for (int k = 0; k < kn; k += 16) {
+          const int4 w16 = __ldg(reinterpret_cast<const int4*>(w + k0 + k));
+          const int w4[4] = {w16.x, w16.y, w16.z, w16.w};
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const double c = (double)(int)(int8_t)(w4[j >> 2] >> (8 * (j & 3)));
+#pragma unroll
+            for (int r = 0; r < CAL_PLAIN_ROWS; ++r) s[r] = __fma_rn(sa[r][k + j], c, s[r]);
+          }
+        }
+      }
+      if (n >= p.N) continue;
+      const double step = (double)__ldg(p.sw + n), bias = p.bias ? (double)__ldg(p.bias + n) : 0.0;
+#pragma unroll
+      for (int r = 0; r < CAL_PLAIN_ROWS; ++r) {
+        const long dst = scatter ? (long)__ldg(p.rowsrc + row[r]) : row[r];
+        if (r < rows && dst >= 0) p.out[dst * p.N + n] = (float)__dadd_rn(__dmul_rn(s[r], step), bias);
+      }
     }
   }
+}
+
+// One warp per row: the largest exponent, then the byte planes (a row of one plane is K bytes).  scatter: row m of the output is
+// row rowsrc[m] (fc2).
+constexpr int CAL_SPLIT_WARPS = 8;
+__global__ void __launch_bounds__(32 * CAL_SPLIT_WARPS, 6) k_cal_split(const __grid_constant__ CalLinearArgs p, int scatter) {
+  __shared__ double sa[CAL_PLAIN_ROWS][CAL_PLAIN_K];
+  __shared__ uint32_t plain_rows;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, K = p.K;
+  const long first = (long)blockIdx.x * CAL_SPLIT_WARPS, m = first + warp;
+  if (threadIdx.x == 0) plain_rows = 0;
+  __syncthreads();
+  bool plain = false;
+  if (m < p.M) {
+    const uint4* row = reinterpret_cast<const uint4*>(p.a + m * K);
+    uint32_t top = 0, low = 0xFFFFFFFFu;                      // largest magnitude; smallest but zero, minus 1
+    for (int i = lane; i < K / 4; i += 32) {
+      const uint4 v = __ldg(row + i);
+      const uint32_t x = v.x & 0x7FFFFFFFu, y = v.y & 0x7FFFFFFFu, z = v.z & 0x7FFFFFFFu, w = v.w & 0x7FFFFFFFu;
+      top = max(max(top, max(x, y)), max(z, w));
+      low = min(min(low, min(x - 1u, y - 1u)), min(z - 1u, w - 1u));
+    }
+    const int E = max(1, (int)(__reduce_max_sync(0xffffffffu, top) >> 23));
+    const uint32_t least = __reduce_min_sync(0xffffffffu, low);
+    plain = E == 255 || (least != 0xFFFFFFFFu && max(1, (int)((least + 1u) >> 23)) < E - 31);
+    if (lane == 0) {
+      p.expo[m] = plain ? CAL_PLAIN_ROW : E;
+      if (plain) atomicOr(&plain_rows, 1u << warp);
+    }
+    for (int i = plain ? K : lane; i < K / 4; i += 32) {      // (what the planes of a plain row hold does not matter)
+      const uint4 v = __ldg(row + i);
+      const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+      uint32_t lo[4], hi[4];                                  // 56-bit two's complement: bytes 0-3 and 4-6
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int e = (in[j] >> 23) & 255;
+        const long long f = (in[j] & 0x7FFFFFu) | (e ? 0x800000u : 0u);
+        long long q = f << max((e ? e : 1) - E + 31, 0);      // 0 ... 31; below 0 for zeros only
+        if (in[j] >> 31) q = -q;
+        lo[j] = (uint32_t)q; hi[j] = (uint32_t)(q >> 32);
+      }
+#pragma unroll
+      for (int s = 0; s < CAL_SLICES; ++s) {
+        const uint32_t* x = s < 4 ? lo : hi;
+        const uint32_t sel = (uint32_t)(s & 3) | (uint32_t)((s & 3) + 4) << 4;
+        reinterpret_cast<uint32_t*>(p.slices + ((long)s * p.M + m) * K)[i] =
+            __byte_perm(__byte_perm(x[0], x[1], sel), __byte_perm(x[2], x[3], sel), 0x5410);
+      }
+    }
+  }
+  if (__syncthreads_or(plain)) cal_plain_rows(p, scatter != 0, first, plain_rows, sa);
 }
 
 // Persistent, one CTA per SM: warp 0 TMA, warp 1 MMA, sixteen epilogue warps (a lane quarter and 16 columns each).
 // A 128 x 64 tile has seven accumulators of 64 TMEM columns, one per byte plane.  Per 128 codes of k the weight tile is loaded
 // once and met by the seven activation tiles, which are what the loads are made of (16 KB each against 140 cycles of MMA): the
 // width of 64 is the largest with which seven accumulators fit.  What bounds it up to K = 384 is the epilogue (seven TMEM loads,
-// eight binary64 operations and two conversions an output: 16 warps 5.8 ms, 8 warps with the loop unrolled 7.9), then the loads.  Sums of more than CAL_KCHUNK products, which int32 might not
-// hold, are drained in parts.
+// eight binary64 operations and two conversions an output: 16 warps 5.8 ms, 8 warps with the loop unrolled 7.9), then the loads.
+// Sums of more than CAL_KCHUNK products, which int32 might not hold, are drained in parts.
 constexpr int CG_BM = 128, CG_BN = 64, CG_BK = 128, CG_A_RING = 8, CG_B_RING = 4, CAL_KCHUNK = 32768;
 constexpr int CG_A_BYTES = CG_BM * CG_BK, CG_B_BYTES = CG_BN * CG_BK, CG_EPI_WARPS = 16, CG_THREADS = 32 * (2 + CG_EPI_WARPS);
 constexpr int CG_EPI_COLS = CG_BN / (CG_EPI_WARPS / 4);
@@ -189,14 +255,6 @@ constexpr int CG_BARS = 2 * CG_A_RING + 2 * CG_B_RING + 3;
 constexpr int CG_COLS_OFF = CG_A_RING * CG_A_BYTES + CG_B_RING * CG_B_BYTES;             // constants of the epilogue warps' columns
 constexpr int CG_BARS_OFF = CG_COLS_OFF + CG_EPI_WARPS * CG_EPI_COLS * 16;
 constexpr int CG_SMEM = CG_BARS_OFF + CG_BARS * 8 + 16 + 1024;
-
-// The sum as it is written, for rows with infinities or NaNs: what follows from them is what the plain sum gives.
-__device__ __noinline__ float cal_plain_sum(const CalLinearArgs& p, long m, int n, double2 col) {
-  double s = 0.0;
-  for (int k = 0; k < p.K; ++k)
-    s = __dadd_rn(s, __dmul_rn((double)p.a[m * p.K + k], __dmul_rn((double)(int)p.w[(long)n * p.K + k], col.x)));
-  return (float)__dadd_rn(s, col.y);
-}
 
 template <int MODE>
 __global__ void __launch_bounds__(CG_THREADS, 1) k_cal_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -349,13 +407,9 @@ __global__ void __launch_bounds__(CG_THREADS, 1) k_cal_gemm(const __grid_constan
           }
           if (c + 1 < n_chunks) continue;
           const int n = n0 + g;
-          if (__any_sync(0xffffffffu, E == CAL_NOT_FINITE)) {
-#pragma unroll 1
-            for (int j = 0; j < 8; ++j) {
-              const float f = E == CAL_NOT_FINITE && n + j < p.N ? cal_plain_sum(p, m, n + j, cols[g + j]) : 0.0f;
+          if (E == CAL_PLAIN_ROW && store) {                      // k_cal_split has put this row's sums where the results go
 #pragma unroll
-              for (int i = 0; i < 8; ++i) if (i == j && E == CAL_NOT_FINITE) v[i] = f;
-            }
+            for (int j = 0; j < 8; ++j) if (n + j < p.N) v[j] = p.out[dst * p.N + n + j];
           }
           if (MODE == CAL_FC1) {
 #pragma unroll
@@ -547,7 +601,7 @@ bool launch_cal_linear(const CalLinearArgs& p, cudaStream_t st) {
   if (cudaFuncSetAttribute(k_cal_gemm<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, CG_SMEM) != cudaSuccess) return false;
   CUtensorMap mA, mB;
   if (!make_map(&mA, p.slices, (uint64_t)CAL_SLICES * p.M, (uint64_t)p.K, CG_BM) || !make_map(&mB, p.w, (uint64_t)p.N, (uint64_t)p.K, CG_BN)) return false;
-  k_cal_split<<<(unsigned)((p.M + 7) / 8), 256, 0, st>>>(p.a, p.slices, p.expo, p.M, p.K);
+  k_cal_split<<<(unsigned)((p.M + CAL_SPLIT_WARPS - 1) / CAL_SPLIT_WARPS), 32 * CAL_SPLIT_WARPS, 0, st>>>(p, MODE == CAL_FC2);
   const int n_tiles = (p.N + CG_BN - 1) / CG_BN;
   const int tiles = (int)((p.M + CG_BM - 1) / CG_BM) * n_tiles, sms = sm_count();
   k_cal_gemm<MODE><<<tiles < sms ? tiles : sms, CG_THREADS, CG_SMEM, st>>>(mA, mB, p, n_tiles, tiles);

@@ -230,29 +230,73 @@ def test_selection_outputs_at_odd_addresses(orc, mq, ctx, H, W):
         assert torch.equal(y, want.y)
 
 
-@pytest.mark.parametrize("N,dim", [(52, 32), (31, 32), (200, 64)])
-def test_calibration_products_of_rows_with_a_wide_range(orc, mq, ctx, N, dim):
-    """Rows whose values span 2^-45 to 1 of their largest (bits below 2^-55 of it are rounded away), ragged widths."""
+def observe_merge(mq, ctx, m, x, N):
+    """mixaq_calibrate_merge with any number of output channels (the binding allocates 2 * dim)."""
+    B, H, W, _ = x.shape
+    params, xd = mq._Dev(ctx.device), dev(x)
+    ms, r = mq.fill_merge_struct(params, m), mq.RangeS()
+    y = torch.empty((B, (H + 1) // 2, (W + 1) // 2, N), device="cuda")
+    ws = torch.empty(mq.lib().mixaq_calibrate_merge_workspace_bytes(ctypes.byref(ms), B, H, W), dtype=torch.uint8, device="cuda")
+    ctx.check(mq.lib().mixaq_calibrate_merge(ctx.h, ctypes.byref(ms), mq._ptr(xd), mq._ptr(y), B, H, W, ctypes.byref(r), mq._ptr(ws),
+                                             ctypes.c_size_t(ws.numel()), mq._stream_ptr()))
+    return y.cpu().numpy(), (r.lo, r.hi)
+
+
+@pytest.mark.parametrize("N,dim,low,large", [(52, 32, 45, False), (31, 32, 36, True), (300, 64, 45, True), (64, 32, 31, True), (96, 32, 130, True)])
+def test_calibration_products_of_rows_with_a_wide_range(orc, mq, ctx, N, dim, low, large):
+    """Rows whose values span 2^-low to 1 of their largest, ragged widths.  `large`: the channel of the largest value meets
+    weights of zero, so that the sums are those of the small values alone."""
     rng = np.random.default_rng(N)
     m = synth.make_merge(rng, dim, 8, 8)
     m.red = synth.make_linear(rng, N, 4 * dim, 8)
-    m.ln_g = np.exp2(-rng.uniform(0, 45, 4 * dim)).astype(F32)
+    m.ln_g = np.exp2(-rng.uniform(low - 1 if large else 0, low, 4 * dim)).astype(F32)
     m.ln_b = np.zeros(4 * dim, F32)
+    if large:
+        m.ln_g[5] = 1.0
+        m.red.codes[:, 5] = 0
     x = synth.input_student_t(N, 1, 23, 27, dim)
-    params, xd = mq._Dev(ctx.device), dev(x)
-    ms, r = mq.fill_merge_struct(params, m), mq.RangeS()
-    y = torch.empty((1, 12, 14, N), device="cuda")                # (the binding allocates 2 * dim channels)
-    ws = torch.empty(mq.lib().mixaq_calibrate_merge_workspace_bytes(ctypes.byref(ms), 1, 23, 27), dtype=torch.uint8, device="cuda")
-    ctx.check(mq.lib().mixaq_calibrate_merge(ctx.h, ctypes.byref(ms), mq._ptr(xd), mq._ptr(y), 1, 23, 27, ctypes.byref(r), mq._ptr(ws),
-                                             ctypes.c_size_t(ws.numel()), mq._stream_ptr()))
+    x[0, 4:9] = 0.0                                                # rows of zeros among them
+    y, got_span = observe_merge(mq, ctx, m, x, N)
     want, span = orc.merge_observe_fp(m, x)
-    assert (r.lo, r.hi) == span
-    # per input at most 2^-55 of the row's largest value, the oracle's running sum 2^-53 of sum |a w| per term, one rounding
-    # to binary32 on either side
-    w = np.abs(m.red.codes.astype(np.float64) * m.red.scale[:, None]).sum(1)
-    top = max(abs(span[0]), abs(span[1]))
-    bound = 2.0 ** -23 * np.abs(want) + (2.0 ** -55 + 4 * dim * 2.0 ** -53) * top * w
-    assert (np.abs(y.cpu().numpy().astype(np.float64) - want) <= bound).all()
+    assert got_span == span
+    # each output against sum |a w| of its own: 2^-53 per term for the running sum of either side, one rounding to binary32 each
+    pad = np.zeros((24, 28, dim), F32)
+    pad[:23, :27] = x[0]
+    ln = orc.layernorm(np.concatenate([pad[dy::2, dx::2] for dx in (0, 1) for dy in (0, 1)], axis=-1), m.ln_g, m.ln_b)
+    terms = np.abs(ln.astype(np.float64)) @ np.abs(m.red.codes.astype(np.float64) * m.red.scale[:, None].astype(np.float64)).T
+    bound = 2.0 ** -23 * np.abs(want) + 2.0 ** -149 + 2 * (4 * dim + 2) * 2.0 ** -53 * terms
+    assert (np.abs(y.astype(np.float64) - want) <= bound).all()
+    assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("shift,branch", [(0, 0), (3, 1)])
+def test_calibration_products_of_a_block_with_a_wide_range_at_every_layer(orc, mq, ctx, shift, branch):
+    """At the input of all four products one channel is near 1 and meets weights of zero, the others are near 2^-45; steps bring
+    what they leave back to the size of the residuals.  Ragged map: pad rows take no part in the last scatter."""
+    dim, small = 64, F32(2.0 ** -45)
+    blk = synth.make_block(np.random.default_rng(7 + shift), dim, dim // 32, shift, 8, 8, 4, share_bias=False)
+    for br in (blk.hi, blk.lo):
+        for g, b in ((br.ln1_g, br.ln1_b), (br.ln2_g, br.ln2_b)):
+            b[:] = 0.0
+            g[:] = g * small
+            g[3] = 1.0
+        for b in (br.b_qkv, br.b_proj, br.b_fc1, br.b_fc2):
+            b[:] = 0.0
+        br.b_fc1[7] = 4.0
+    for lin, channel in ((blk.qkv, 3), (blk.proj, 5), (blk.fc1, 3), (blk.fc2, 7)):
+        lin.codes[:, channel] = 0
+        lin.scale[:] = (lin.scale / small).astype(F32)
+    for lin, big in ((blk.qkv, 2 * dim + 5), (blk.fc1, 7)):       # and small again: the v channels but one, the hidden ones but one
+        rows = np.arange(lin.scale.size)
+        lin.scale[(rows != big) & (rows >= (2 * dim if lin is blk.qkv else 0))] *= small
+    x = synth.input_blobs(5, 2, 12, 17, dim, bg_std=0.5, gain=3.0)
+    params = mq._Dev(ctx.device)
+    y, got = mq.calibrate_block(ctx, mq.fill_block_struct(params, blk), branch, dev(x))
+    want_y, want = orc.block_observe_fp(blk, ("hi", "lo")[branch], x)
+    # a binary32 rounding (6e-8) may fall the other way in each of the products; the layers behind it amplify it by less than 100
+    assert np.abs(y.cpu().numpy() - want_y).max() <= 6e-6 * np.abs(want_y - x).max() + 2.0 ** -22 * np.abs(want_y).max()
+    for site, (lo, hi) in want.items():
+        assert max(abs(got[site][0] - lo), abs(got[site][1] - hi)) <= 6e-6 * (hi - lo), site
     assert ctx.device_status() == 0
 
 
