@@ -426,10 +426,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   __syncthreads();
   if (*abort_flag) {
     // A wait ran out.  Before the CTA may exit, the copies already issued must have landed in its shared memory and
-    // the MMAs already issued must have retired.  (1) The MMA thread commits what it has issued to a barrier of its
-    // own.  (2) The TMA thread waits, bounded, for the phase of the last fill of every stage, on the full barrier and on
+    // the MMAs already issued must have retired.  (1) The lane that issued the MMAs commits them to a barrier of their
+    // own (a commit covers what its own thread has issued; elect.sync names the same lane of a full warp every time).
+    // (2) The TMA thread waits, bounded, for the phase of the last fill of every stage, on the full barrier and on
     // the packed-rows barrier (both complete by the copies alone), and for that commit.
-    if (tid == 32) mma_commit(bar_drain);
+    if (warp == 1 && elect_one()) mma_commit(bar_drain);
     __syncthreads();
     if (tid == 0) {
       atomicExch(p.status, 1);

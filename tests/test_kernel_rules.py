@@ -1,0 +1,23 @@
+"""Rules of the machine that the GEMM kernel has to keep where no result shows it: checked on its source."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_19131_b200", "csrc")
+
+
+def kernel_source():
+    """csrc/gemm_tc.cu's k_gemm_tc without comments."""
+    text = open(os.path.join(CSRC, "gemm_tc.cu")).read()
+    body = text[text.index("k_gemm_tc(const"):text.index("// ---- host side")]
+    return re.sub(r"//[^\n]*", "", body)
+
+
+def test_the_lane_that_issued_the_mmas_commits_them_when_the_cta_gives_up():
+    """tcgen05.commit covers what the executing thread has issued.  The MMAs are issued by the lane that elect.sync names (the
+    same one for a full warp every time), so the commit in front of freeing tensor memory has to be that lane's too."""
+    body = kernel_source()
+    give_up = body[body.index("if (*abort_flag) {"):]
+    assert re.search(r"if \(warp == 1 && elect_one\(\)\) mma_commit\(bar_drain\);", give_up)
+    assert len(re.findall(r"mma_commit\(bar_drain\)", body)) == 1
+    issuer = body[body.index("} else if (warp == 1) {"):body.index("} else if (warp < FIRST_UNPACK_WARP)")]
+    assert "const bool leader = elect_one();" in issuer and re.search(r"if \(leader\) \{[^}]*mma_i8\(", issuer)
