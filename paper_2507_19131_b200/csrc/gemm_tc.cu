@@ -51,9 +51,9 @@ __host__ __device__ constexpr int first_epi_warp(bool packed) { return FIRST_UNP
 __host__ __device__ constexpr int num_threads(int warps, bool packed) { return 32 * (first_epi_warp(packed) + warps); }
 // Registers.  A block is launched with what its threads divide the file into (a scheduler's 16 384 among its warps: 128 a thread with
 // 12 epilogue warps, 96 with the unpack warps too); the side warpgroups give back all but SIDE_REGS
-// and the epilogue warps of the code outputs take them.  gemm_init checks that the shares fit into what the compiled kernels are
-// launched with.
-constexpr int SIDE_REGS = 56;
+// and the epilogue warps take them: 4 x 72 + 12 x 136 of 16 x 128, 8 x 72 + 12 x 112 of 20 x 96.  gemm_init checks that the shares fit
+// into what the compiled kernels are launched with.  (No instance spills; with 56 for the side warps six did.)
+constexpr int SIDE_REGS = 72;
 __host__ __device__ constexpr int epi_regs(int warps, bool packed) { return warps != 12 ? 0 : packed ? 112 : 136; }    // 0: no exchange
 constexpr int MAX_BN = 256;
 __host__ __device__ constexpr bool code_mode(int mode) { return mode == EPI_QKV || mode == EPI_FC1; }
@@ -142,7 +142,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   constexpr int NUM_EPI_WARPS = EW, FIRST_EPI_WARP = first_epi_warp(PACKED);
   constexpr int NUM_UNPACK_WARPS = UNPACK_WARPS, NUM_UNPACK_THREADS = NUM_UNPACK_WARPS * 32;
   constexpr int UNPACK_ITEMS = BM * (BK / UMMA_K) / NUM_UNPACK_THREADS;   // (row, 32-code group) items per thread and stage
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // The warp number through a shuffle: the compiler then knows that it is the same in all lanes and that the roles' loops run
+  // converged, and keeps addresses and descriptors in uniform registers (Swin-T 224 image / 800 x 1333: 393 / 788 us with
+  // threadIdx.x >> 5, 371 / 758 so).
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
 
   // Every launch starts with a cold constant cache, and the roles below would miss on one parameter after the other
   // (1 800 cycles until the first copy was issued): the warps touch the lines of the parameter block side by side.
@@ -184,10 +187,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_holder;
   griddep_launch();
+  // Registers change hands by whole warpgroups, whose warps all execute the same instruction: it stands in front of the roles.
+  if (epi_regs(EW, PACKED) > 0 && warp < FIRST_EPI_WARP) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
 
   if (warp == 0) {
     // ---- TMA producer ----
-    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     {
       const bool leader = elect_one();
       TileWalk w(p);
@@ -235,7 +239,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     }
   } else if (warp == 1) {
     // ---- MMA issuer ----
-    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     {
       const bool leader = elect_one();
       const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
@@ -283,10 +286,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     }
   } else if (warp < FIRST_UNPACK_WARP) {
     // (warps 2 and 3 fill up the warpgroup)
-    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
   } else if (PACKED && warp < FIRST_EPI_WARP) {
     // ---- unpack producers: bit-packed rows -> one code per byte, written in the swizzled layout ----
-    if (epi_regs(EW, PACKED) > 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SIDE_REGS));
     const int ptid = tid - 32 * FIRST_UNPACK_WARP;   // 0 .. NUM_UNPACK_THREADS-1
     TileWalk w(p);
     int slot = 0;

@@ -21,3 +21,15 @@ def test_the_lane_that_issued_the_mmas_commits_them_when_the_cta_gives_up():
     assert len(re.findall(r"mma_commit\(bar_drain\)", body)) == 1
     issuer = body[body.index("} else if (warp == 1) {"):body.index("} else if (warp < FIRST_UNPACK_WARP)")]
     assert "const bool leader = elect_one();" in issuer and re.search(r"if \(leader\) \{[^}]*mma_i8\(", issuer)
+
+
+def test_registers_are_exchanged_by_whole_warpgroups():
+    """setmaxnreg is executed by all warps of a warpgroup, the same instruction: one for the side warps in front of the split into
+    roles, one for the epilogue warps, under conditions that are the same for every four warps."""
+    text, body = open(os.path.join(CSRC, "gemm_tc.cu")).read(), kernel_source()
+    assert len(re.findall("setmaxnreg", body)) == 2
+    assert re.search(r'\n  if \(epi_regs\(EW, PACKED\) > 0 && warp < FIRST_EPI_WARP\) asm volatile\("setmaxnreg\.dec\.[^\n]*\n\s*'
+                     r'if \(warp == 0\) \{', body)
+    assert re.search(r'\n  \} else \{\s*if \(epi_regs\(EW, PACKED\) > 0\) asm volatile\("setmaxnreg\.inc\.', body)
+    number = {n: int(v) for n, v in re.findall(r"\b(FIRST_UNPACK_WARP|UNPACK_WARPS|CODE_WARPS|F32_WARPS_FEW|F32_WARPS) = (\d+)", text)}
+    assert len(number) == 5 and all(v % 4 == 0 for v in number.values())      # every boundary between roles lies between warpgroups
