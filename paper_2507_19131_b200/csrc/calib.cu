@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) k_cal_gemm(const __grid_constan
       __syncwarp();
       float lo = INFINITY, hi = -INFINITY;
       for (int c = 0; c < n_chunks; ++c) {
-        if (!mbar_wait(acc_full, fp, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(acc_full, fp, abort_flag)) { ok = false; break; }
         fp ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1

@@ -212,7 +212,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
           const int m_row = (w.mt - m_first) * BM, n_row = w.nt * BN;
           for (int kb = 0; kb < k_blocks; ++kb, rp.next(ring)) {
             const uint32_t o = 8u * (uint32_t)rp.slot;
-            if (!mbar_wait(bar_empty + o, rp.pass ^ 1u, abort_flag)) { ok = false; break; }    // (at once in the first pass)
+            if (!mbar_wait_warp(bar_empty + o, rp.pass ^ 1u, abort_flag)) { ok = false; break; }    // (at once in the first pass)
             const uint32_t sa = base + (uint32_t)(rp.slot * stage_bytes), sb = sa + A_STAGE_BYTES;
             ++fills;
             if (leader) {
@@ -256,14 +256,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         const bool packed = PACKED && p.g.br[b].a_bits != 8;
         for (; w.mt < m_end && ok; w.next(p), ap.next(n_acc)) {
           // wait until the epilogue has drained this accumulator's previous use (at once in the first pass)
-          if (!mbar_wait(bar_tempty + 8u * ap.slot, ap.pass ^ 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(bar_tempty + 8u * ap.slot, ap.pass ^ 1u, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t d_tmem = tmem_base + (uint32_t)(ap.slot * p.acc_stride);
           for (int kb = 0; kb < k_blocks; ++kb, rp.next(ring)) {
             const uint32_t o = 8u * (uint32_t)rp.slot;
-            if (!mbar_wait(bar_full + o, rp.pass, abort_flag)) { ok = false; break; }
+            if (!mbar_wait_warp(bar_full + o, rp.pass, abort_flag)) { ok = false; break; }
             if (packed) {
-              if (!mbar_wait(bar_unp + o, (unp_next >> rp.slot) & 1u, abort_flag)) { ok = false; break; }
+              if (!mbar_wait_warp(bar_unp + o, (unp_next >> rp.slot) & 1u, abort_flag)) { ok = false; break; }
               unp_next ^= 1u << rp.slot;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -313,7 +313,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         const long m0 = (long)(w.mt - m_first) * BM;
         for (int kb = 0; kb < p.k_blocks; ++kb) {
           // the TMA thread arrives on raw[s] once it owns the stage (and, when staged, the packed bytes have landed)
-          if (!mbar_wait(bar_raw + 8u * slot, (raw_next >> slot) & 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(bar_raw + 8u * slot, (raw_next >> slot) & 1u, abort_flag)) { ok = false; break; }
           raw_next ^= 1u << slot;
           uint8_t* sa = smem + (size_t)slot * stage_bytes;
           const uint8_t* sp = sa + A_STAGE_BYTES + p.BN * BK;
@@ -375,7 +375,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     auto all_warps = [&]() -> bool {
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_consts);
-      const bool done = mbar_wait(bar_consts, consts_pass, abort_flag);
+      const bool done = mbar_wait_warp(bar_consts, consts_pass, abort_flag);
       consts_pass ^= 1u;
       return done;
     };
@@ -407,7 +407,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         const ColConsts cc = {c_pre + c0, c_mult + c0, c_bias + c0};
         const long row0 = (long)(w.mt - m_first) * BM + q * 32;
         auto acc_ready = [&]() -> bool {
-          if (!mbar_wait<true>(bar_tfull + 8u * acc, acc_pass, abort_flag)) return false;
+          if (!mbar_wait_warp<true>(bar_tfull + 8u * acc, acc_pass, abort_flag)) return false;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           return true;
         };

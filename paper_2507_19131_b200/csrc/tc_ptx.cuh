@@ -47,7 +47,7 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
   return ok != 0;
 }
-// Bounded wait.  Returns false when the limit ran out or another thread of the CTA already gave up (looked at now and
+// Bounded wait of one thread.  Returns false when the limit ran out or another thread of the CTA already gave up (looked at now and
 // then only).  The waits that are not on a tile's critical path give the hardware a suspend time: the polls of the TMA and
 // MMA threads took up to a tenth of the issue slots of their schedulers.
 template <bool LATENCY = false>
@@ -56,6 +56,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   for (uint32_t it = 1; it < (LATENCY ? MAX_POLLS : MAX_SUSPENDED_POLLS); ++it) {
     if (LATENCY ? mbar_try_wait(bar, parity) : mbar_try_wait_hint(bar, parity)) return true;
     if ((it & 15u) == 0u && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+// The same by a converged warp, with one answer for all lanes: a lane that gave up while another one went on to the next aligned
+// instruction would leave that one waiting without a limit.
+template <bool LATENCY = false>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  for (uint32_t it = 1; it < (LATENCY ? MAX_POLLS : MAX_SUSPENDED_POLLS); ++it) {
+    if (__all_sync(0xffffffffu, LATENCY ? mbar_try_wait(bar, parity) : mbar_try_wait_hint(bar, parity))) return true;
+    if ((it & 15u) == 0u && __any_sync(0xffffffffu, *abort_flag != 0)) return false;
   }
   *abort_flag = 1;
   return false;

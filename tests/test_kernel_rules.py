@@ -33,3 +33,15 @@ def test_registers_are_exchanged_by_whole_warpgroups():
     assert re.search(r'\n  \} else \{\s*if \(epi_regs\(EW, PACKED\) > 0\) asm volatile\("setmaxnreg\.inc\.', body)
     number = {n: int(v) for n, v in re.findall(r"\b(FIRST_UNPACK_WARP|UNPACK_WARPS|CODE_WARPS|F32_WARPS_FEW|F32_WARPS) = (\d+)", text)}
     assert len(number) == 5 and all(v % 4 == 0 for v in number.values())      # every boundary between roles lies between warpgroups
+
+
+def test_the_lanes_of_a_warp_give_up_together():
+    """A bounded wait that runs out in one lane only would leave the others at the next aligned instruction for good: warps that
+    walk converged wait with one answer for all lanes."""
+    assert not re.findall(r"\bmbar_wait(?:<\w+>)?\(", kernel_source())
+    calib = open(os.path.join(CSRC, "calib.cu")).read()
+    epilogue = calib[calib.index("double part[CG_EPI_COLS]"):calib.index("// a wait ran out")]
+    assert not re.findall(r"\bmbar_wait(?:<\w+>)?\(", epilogue) and "mbar_wait_warp(acc_full" in epilogue
+    wait = open(os.path.join(CSRC, "tc_ptx.cuh")).read()
+    wait = wait[wait.index("bool mbar_wait_warp("):wait.index("void tma_load_2d")]
+    assert len(re.findall(r"if \(.*return", wait)) == len(re.findall(r"__(?:all|any)_sync\(0xffffffffu", wait)) == 3
