@@ -28,7 +28,8 @@ __global__ void __launch_bounds__(256) k_prepare_linear(const int8_t* __restrict
     mult[n] = __fmul_rn(sa, sw[n]);
     const long hi = (long)up * (qmax - za) + (long)down * za, lo = (long)up * za + (long)down * (qmax - za), most = hi > lo ? hi : lo;
     const float limit = fabsf(mult[n]) * (float)most * 1.0001f;
-    bound[n] = most < (1L << 22) - 16 ? limit : -fmaxf(limit, FLT_MIN);
+    // (a step that is no number leaves no bound: its column takes the contract's own operations either way)
+    bound[n] = most < (1L << 22) - 16 ? limit : limit > 0.0f ? -limit : limit == limit ? -FLT_MIN : -INFINITY;
   }
 }
 

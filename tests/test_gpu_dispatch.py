@@ -74,6 +74,19 @@ def test_gemm_accumulators_beyond_the_bias_trick(orc, mq, ctx, dim, sign):
     run_block_case(orc, mq, ctx, blk, synth.input_blobs(dim, 1, 17, 23, dim, bg_std=0.5, gain=4.0), 0.4)
 
 
+@pytest.mark.parametrize("dim", [96, 384])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_gemm_code_outputs_of_a_column_without_a_finite_step(orc, mq, ctx, dim, value):
+    """One step of a q, a k, a v and an fc1 channel is no number or infinite, in columns whose sums stay below 2^22 (dim 96) and in
+    columns whose sums may not: the codes are those of the contract (0 for what is no number)."""
+    rng = np.random.default_rng(dim)
+    blk = synth.make_block(rng, dim, dim // 32, 3, 8, 8, 4)
+    for lin, channels in ((blk.qkv, (5, dim + 9, 2 * dim + 30)), (blk.fc1, (7, 3 * dim + 1))):
+        lin.codes[list(channels)] = 127 * rng.choice([-1, 1], size=(len(channels), dim), p=[0.02, 0.98]).astype(np.int8)
+        lin.scale[list(channels)] = value
+    run_block_case(orc, mq, ctx, blk, synth.input_student_t(dim, 1, 17, 23, dim), 0.4)
+
+
 @pytest.mark.parametrize("dim,bits,factor", [(96, (8, 4), 20.0), (32, (4, 2), 20.0), (128, (8, 2), 20.0), (128, (8, 4), 3000.0),
                                              (64, (4, 2), 3000.0)])
 def test_gemm_code_outputs_far_beyond_their_range(orc, mq, ctx, dim, bits, factor):
