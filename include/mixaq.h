@@ -230,7 +230,8 @@ mixaq_status mixaq_norm_forward(mixaq_ctx* ctx, const float* gamma, const float*
  *      `ranges` (a HOST struct).  The quantizer fields of `p` are not read and `p->prepared` is not needed.
  *      mixaq_calibrate_merge does the same for a patch merging (one site: the LayerNorm output).  The error of a matrix
  *      product is a few roundings of binary64 relative to sum |a w| of the output itself, whatever the range of a row.
- *      Both synchronise the stream.  mixaq_aq_from_range is the one definition of the quantizer that covers a range:
+ *      Both synchronise the stream, and return MIXAQ_DEVICE_TIMEOUT when a bounded wait of theirs ran out (the ranges are
+ *      then left as they are; the status word is raised too).  mixaq_aq_from_range is the one definition of the quantizer that covers a range:
  *      scale = (hi - lo) / (2^bits - 1), inv_scale = 1 / scale, zero_point = clamp(rne(-lo / scale), 0, 2^bits - 1). ---- */
 typedef struct { float lo, hi; } mixaq_range;
 typedef struct { mixaq_range qkv_in, q, k, v, proj_in, fc1_in, fc2_in;

@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) k_cal_gemm(const __grid_constan
     if (tid == 32) mma_commit(drained);
     if (tid == 0) {
       atomicExch(p.status, 1);
+      p.obs[CAL_STATUS] = 1;
       auto drain = [](uint32_t bar, uint32_t parity) {
         for (uint32_t it = 0; it < (1u << 20); ++it) if (mbar_try_wait(bar, parity)) return;
       };
@@ -593,6 +594,7 @@ __global__ void __launch_bounds__(64) k_cal_attention(CalAttnArgs a) {
 __global__ void k_cal_obs_init(uint32_t* obs, int sites) {
   const int i = threadIdx.x;
   if (i < 2 * sites) obs[i] = (i & 1) ? 0u : 0xFFFFFFFFu;
+  if (i == CAL_STATUS) obs[i] = 0u;
 }
 
 template <int MODE>
@@ -633,7 +635,7 @@ static bool launch_cal_ln(const float* src, int32_t* rowsrc_out, const float* ga
 }
 
 // The floating-point block through one branch.  Workspace (floats unless noted): rowsrc int32[M], ln [M][C],
-// qkv [M][3C], o [M][C], x1 [M][C], h [M][hidden], slices, expo; obs: 16 keys (seven sites and the block's input map).
+// qkv [M][3C], o [M][C], x1 [M][C], h [M][hidden], slices, expo; obs: keys of the seven sites and the block's input map, status.
 bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
   const int C = c.C, Hd = c.hidden;
   const int Hp = (c.H + WS - 1) / WS * WS, Wp = (c.W + WS - 1) / WS * WS, nwx = Wp / WS, nW = (Hp / WS) * nwx;

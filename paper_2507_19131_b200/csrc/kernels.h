@@ -140,7 +140,7 @@ struct CalBlockArgs {
   const float *s_qkv, *s_proj, *s_fc1, *s_fc2, *relpos;
   int32_t* rowsrc; float *ln, *qkv, *o, *x1, *h;  // workspace: [M], [M][C], [M][3C], [M][C], [M][C], [M][hidden]
   uint8_t* slices; int32_t* expo;                 // workspace of the products: [7][M][max(C, hidden)] bytes, [M]
-  uint32_t* obs;                                  // 16 order-preserving keys: min, max of the seven sites and of x
+  uint32_t* obs;                                  // CAL_OBS words: order-preserving keys (min, max of the seven sites and of x), status
   int* status;
 };
 bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st);
@@ -148,11 +148,12 @@ struct CalMergeArgs {
   const float* x; float* y; int B, H, W, C, N;
   const float *ln_g, *ln_b; const int8_t* w; const float* sw;
   float* ln; uint8_t* slices; int32_t* expo;      // workspace [M][4C], [7][M][4C], [M]
-  uint32_t* obs;                                  // 2 keys
+  uint32_t* obs;                                  // the same with 2 keys
   int* status;
 };
 bool launch_calibrate_merge(const CalMergeArgs& c, cudaStream_t st);
 constexpr int CAL_SLICES = 7;                     // byte planes a calibration product cuts its input into
+constexpr int CAL_STATUS = 16, CAL_OBS = 17;      // word of the call's own status behind the 16 keys (the context's may be older)
 float cal_key_to_float(uint32_t key);
 
 // ---- preparation -----------------------------------------------------------------------------------

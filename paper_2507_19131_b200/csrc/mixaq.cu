@@ -1246,7 +1246,7 @@ CalWs carve_cal(const mixaq_block_params* p, int B, int H, int W, void* base) {
   CalWs w; Carver c(base);
   Geometry g = geometry(H, W, 0.f, 0.f);
   const size_t M = (size_t)B * g.nW * WT;
-  w.obs = c.take<uint32_t>(16);
+  w.obs = c.take<uint32_t>(CAL_OBS);
   w.rowsrc = c.take<int32_t>(M);
   w.ln = c.take<float>(M * p->dim); w.qkv = c.take<float>(M * 3 * p->dim); w.o = c.take<float>(M * p->dim);
   w.x1 = c.take<float>(M * p->dim); w.h = c.take<float>(M * p->hidden);
@@ -1254,11 +1254,12 @@ CalWs carve_cal(const mixaq_block_params* p, int B, int H, int W, void* base) {
   w.bytes = c.off;
   return w;
 }
-// reads the observers' keys back (synchronises) and decodes them
+// reads the observers' keys and the call's status back (synchronises) and decodes them
 mixaq_status read_ranges(mixaq_ctx* ctx, const uint32_t* d_obs, int sites, mixaq_range* out, cudaStream_t st) {
-  uint32_t keys[16];
-  if (cudaMemcpyAsync(keys, d_obs, sizeof(uint32_t) * 2 * sites, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  uint32_t keys[CAL_OBS];
+  if (cudaMemcpyAsync(keys, d_obs, sizeof(keys), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess) return check_cuda(ctx, "calibrate (read ranges)") == MIXAQ_OK ? MIXAQ_CUDA_ERROR : MIXAQ_CUDA_ERROR;
+  if (keys[CAL_STATUS]) return fail(ctx, MIXAQ_DEVICE_TIMEOUT, "calibrate: a bounded wait inside a product ran out");
   for (int i = 0; i < sites; ++i) { out[i].lo = cal_key_to_float(keys[2 * i]); out[i].hi = cal_key_to_float(keys[2 * i + 1]); }
   return MIXAQ_OK;
 }
@@ -1303,7 +1304,7 @@ mixaq_status mixaq_calibrate_block(mixaq_ctx* ctx, const mixaq_block_params* p, 
 size_t mixaq_calibrate_merge_workspace_bytes(const mixaq_merge_params* p, int B, int H, int W) {
   if (!p || B <= 0 || H <= 0 || W <= 0 || p->reduction.in_features <= 0) return 0;
   const size_t toks = (size_t)B * ((H + 1) / 2) * ((W + 1) / 2);
-  return carved_bytes(16 * sizeof(uint32_t)) + carved_bytes(toks * p->reduction.in_features * sizeof(float)) +
+  return carved_bytes(CAL_OBS * sizeof(uint32_t)) + carved_bytes(toks * p->reduction.in_features * sizeof(float)) +
          carved_bytes(toks * sizeof(int32_t)) + carved_bytes(CAL_SLICES * toks * p->reduction.in_features);
 }
 
@@ -1323,7 +1324,7 @@ mixaq_status mixaq_calibrate_merge(mixaq_ctx* ctx, const mixaq_merge_params* p, 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   Carver cv(workspace);
   CalMergeArgs c;
-  c.obs = cv.take<uint32_t>(16);
+  c.obs = cv.take<uint32_t>(CAL_OBS);
   const size_t toks = (size_t)B * ((H + 1) / 2) * ((W + 1) / 2);
   c.ln = cv.take<float>(toks * K);
   c.expo = cv.take<int32_t>(toks); c.slices = cv.take<uint8_t>(CAL_SLICES * toks * K);

@@ -24,6 +24,7 @@ cudaError_t fail(cudaError_t e) { last_error = e; return e; }
 extern "C" {
 FakeCounts counts;
 int fail_capture, fail_instantiate, fail_graph_launch;      // the call fails while this is set
+unsigned fake_device_word;                                   // what copies to the host find in every 32-bit word of the device
 FakeCopy last_copies[16];
 cudaStream_t capture_origins[16];                            // of the newest captures
 void fake_reset() { std::lock_guard<std::mutex> g(lock); const long live = counts.live_graphs; counts = FakeCounts(); counts.live_graphs = live; }
@@ -51,8 +52,9 @@ cudaError_t cudaMalloc(void** p, size_t) { std::lock_guard<std::mutex> g(lock); 
 cudaError_t cudaFree(void*) { return cudaSuccess; }
 cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t st) { enqueue(st); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind, cudaStream_t st) {
+cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind kind, cudaStream_t st) {
   enqueue(st);
+  if (kind == cudaMemcpyDeviceToHost) for (size_t i = 0; i < n / 4; ++i) static_cast<unsigned*>(dst)[i] = fake_device_word;
   std::lock_guard<std::mutex> g(lock);
   last_copies[counts.copies++ % 16] = {dst, src, n};
   return cudaSuccess;

@@ -40,7 +40,8 @@ def L(tmp_path_factory):
                                             os.path.join(fake, "fake_launch.cu"), os.path.join(fake, "fake_runtime.cpp"), "-ldl"])
     lib = C.CDLL(out)
     lib.mixaq_last_error.restype = C.c_char_p
-    for n in ("mixaq_block_workspace_bytes", "mixaq_backbone_workspace_bytes"):
+    for n in ("mixaq_block_workspace_bytes", "mixaq_backbone_workspace_bytes", "mixaq_calibrate_block_workspace_bytes",
+              "mixaq_calibrate_merge_workspace_bytes"):
         getattr(lib, n).restype = C.c_size_t
     return lib
 
@@ -52,7 +53,7 @@ class Host:
 
     def __init__(self, L):
         self.L, self.h, self.next = L, C.c_void_p(), 0x7000_0000_0000
-        for flag in ("fail_capture", "fail_instantiate", "fail_graph_launch"):
+        for flag in ("fail_capture", "fail_instantiate", "fail_graph_launch", "fake_device_word"):
             self.set(flag, 0)
         L.fake_reset()
         assert L.mixaq_create(C.byref(self.h), 0) == 0
@@ -302,3 +303,18 @@ def test_output_norms_run_beside_the_chain_also_after_eviction(host, stream):
     replayed = host.counts.graph_launches
     assert host.run_backbone(b, xs[0], stream) == 0 and host.counts.graph_launches == replayed + 1
     assert host.run_backbone(b, xs[1], stream) == 0 and host.counts.graph_launches == replayed + 1
+
+
+def test_a_calibration_whose_waits_ran_out_says_so(host):
+    """The status word that the product's kernels raise comes back with the ranges; the host's own copy of it is not stale."""
+    s, r = host.block(), mq.BlockRangesS()
+    m, rm = mq.MergeS(host.addr(), host.addr(), mq.AQ(8, 0.1, 10.0, 3), host.linear(64, 128), host.addr()), mq.RangeS()
+    x, y, ws = (C.c_void_p(host.addr()) for _ in range(3))
+    n = C.c_size_t(host.L.mixaq_calibrate_block_workspace_bytes(C.byref(s), 1, 14, 14))
+    nm = C.c_size_t(host.L.mixaq_calibrate_merge_workspace_bytes(C.byref(m), 1, 8, 8))
+    calls = (lambda: host.L.mixaq_calibrate_block(host.h, C.byref(s), 0, x, y, 1, 14, 14, C.byref(r), ws, n, None),
+             lambda: host.L.mixaq_calibrate_merge(host.h, C.byref(m), x, y, 1, 8, 8, C.byref(rm), ws, nm, None))
+    for call in calls:
+        for word in (0, 1, 0):
+            host.set("fake_device_word", word)
+            assert call() == (-5 if word else 0)                 # MIXAQ_DEVICE_TIMEOUT
