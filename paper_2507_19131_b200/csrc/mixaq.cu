@@ -5,6 +5,7 @@
 #include "../../include/mixaq.h"
 #include "graph_cache.h"
 #include "kernels.h"
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -302,14 +303,20 @@ BlockWs carve_block(const mixaq_block_params* p, int B, int H, int W, void* base
 // Expanding packed codes in front of every MMA costs more than their bytes save (Swin-T 800 x 1333, bit-packed against bytes: 916
 // and 841 us; Swin-S 4 x 1024 x 1024 at A4 / A2: 3 918 and 3 487), and nobody sees the storage but the taps.  The packed carving
 // sizes each branch for all rows and keeps apart what is never alive at once, so bytes fit into the same memory: x1; the q, k, v
-// codes and after them fc1's; the codes of LN1 and after them LN2's; those of the attention.  false: not enough room (hidden layers
-// beyond 10 C at two bits); ws is left as it is.
+// codes and after them fc1's; the codes of LN1 and after them LN2's; those of the attention.  Guard zones follow these buffers as they
+// do the packed ones (four in the room of twelve).  false: not enough room (hidden layers beyond 10 C at two bits); ws is left as it is.
 bool carve_bytes(const mixaq_block_params* p, const int (&M)[2], void* workspace, BlockWs& ws) {
   const size_t rows = (size_t)M[0] + M[1], C = p->dim, Hd = p->hidden, wide = std::max(3 * C, Hd);
-  Carver c(ws.a[0], false);
+  const size_t need = carved_bytes(rows * C * sizeof(float)) + carved_bytes(rows * wide) + 2 * carved_bytes(rows * C);
+  if (need > (size_t)((char*)workspace + ws.bytes - (char*)ws.a[0])) return false;
+  // the zones of the packed buffers lie inside the new ones
+  if (t_guard_log) {
+    auto inside = [&](void* zone) { return (char*)zone >= (char*)ws.a[0]; };
+    t_guard_log->erase(std::remove_if(t_guard_log->begin(), t_guard_log->end(), inside), t_guard_log->end());
+  }
+  Carver c(ws.a[0]);
   float* x1 = c.take<float>(rows * C);
   uint8_t *big = c.take<uint8_t>(rows * wide), *ln = c.take<uint8_t>(rows * C), *o = c.take<uint8_t>(rows * C);
-  if (c.off > (size_t)((char*)workspace + ws.bytes - (char*)ws.a[0])) return false;
   const size_t m0 = M[0];
   for (int i = 0; i < 2; ++i) {
     const size_t r = i == 0 ? 0 : m0;                        // the high branch's rows come first
@@ -571,9 +578,13 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   if (!workspace) return fail(ctx, MIXAQ_INVALID_ARG, "workspace is NULL");
   if (!aligned_to(workspace, 256)) return fail(ctx, MIXAQ_INVALID_ARG, "workspace must be 256-byte aligned");
   std::vector<void*> guard_zones;
-  BlockWs ws;
-  { GuardScope gs(ctx, &guard_zones); ws = carve_block(p, B, H, W, workspace); }
+  GuardScope guard_scope(ctx, &guard_zones);
+  BlockWs ws = carve_block(p, B, H, W, workspace);
   if (ws.bytes > workspace_bytes) return fail(ctx, MIXAQ_WORKSPACE_TOO_SMALL, "workspace too small");
+  const int M[2] = {B * g.n_hi * WT, B * g.n_lo * WT};
+  // bits a stored code occupies: a whole byte, or the branch's bit width (bit-packed: what the taps hand out)
+  const bool bytes = p->byte_codes || (!taps && carve_bytes(p, M, workspace, ws));
+  const int cb[2] = {bytes ? 8 : p->hi.bits, bytes ? 8 : p->lo.bits};
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const int C = p->dim, Hd = p->hidden;
   Prepared pr = carve_prepared(p, p->prepared);
@@ -607,13 +618,8 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   }
 
   const mixaq_branch* brp[2] = {&p->hi, &p->lo};
-  const int M[2] = {B * g.n_hi * WT, B * g.n_lo * WT};
   const int slots[2] = {B * g.n_hi, B * g.n_lo};
   const mixaq_branch_taps* tp[2] = {taps ? &taps->hi : nullptr, taps ? &taps->lo : nullptr};
-  // bits a stored code occupies: a whole byte, or the branch's bit width (bit-packed: what the taps hand out and the guard zones
-  // are laid out for)
-  const bool bytes = p->byte_codes || (!taps && guard_zones.empty() && carve_bytes(p, M, workspace, ws));
-  const int cb[2] = {bytes ? 8 : p->hi.bits, bytes ? 8 : p->lo.bits};
 
   // 2. gather + LN1 + quantize + pack
   LnBranch lb[2];

@@ -400,15 +400,17 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(orc, mq):
 
 
 def test_workspace_guard_zones(orc, mq):
-    """The guard zones behind every workspace buffer: untouched by a forward (block with all taps, and a small
-    backbone), and the check itself reports a byte written just past a buffer."""
+    """The guard zones behind every workspace buffer: untouched by a forward (blocks with all taps and bit-packed codes, blocks and a
+    small backbone with one code per byte), and the check itself reports a byte written just past a buffer."""
     c = mq.Context(0)
     try:
         c.set_workspace_guards(True)
-        blk = synth.make_block(np.random.default_rng(52), 64, 2, 3, 4, 8, 4)
-        x = synth.input_blobs(53, 2, 17, 23, 64, bg_std=0.5, gain=4.0)
-        run_block_case(orc, mq, c, blk, x, 0.4, 0.1)
-        assert c.device_status() == 0
+        for bits in ((8, 4), (4, 2)):
+            blk = synth.make_block(np.random.default_rng(52), 64, 2, 3, 4, *bits)
+            x = synth.input_blobs(53, 2, 17, 23, 64, bg_std=0.5, gain=4.0)
+            for taps in (True, False):
+                run_block_case(orc, mq, c, blk, x, 0.4, 0.1, taps=taps)
+                assert c.device_status() == 0
         wl = synth.tiny_backbone()
         want = orc.backbone_forward(wl.backbone, wl.x, wl.low_ratios, wl.prune_ratios)
         side = torch.cuda.Stream()

@@ -25,6 +25,10 @@ class SelectArgs(C.Structure):
                [(n, C.c_int) for n in ("B", "H", "W", "shift", "nwx", "nW", "n_hi", "n_lo", "n_pr", "reverse")]
 
 
+class Range(C.Structure):
+    _fields_ = [("at", C.c_void_p), ("bytes", C.c_size_t), ("code_bits", C.c_int)]
+
+
 class Copy(C.Structure):
     _fields_ = [("dst", C.c_void_p), ("src", C.c_void_p), ("bytes", C.c_size_t)]
 
@@ -53,7 +57,7 @@ class Host:
 
     def __init__(self, L):
         self.L, self.h, self.next = L, C.c_void_p(), 0x7000_0000_0000
-        for flag in ("fail_capture", "fail_instantiate", "fail_graph_launch", "fake_device_word"):
+        for flag in ("fail_capture", "fail_instantiate", "fail_graph_launch", "fake_device_word", "written_count"):
             self.set(flag, 0)
         L.fake_reset()
         assert L.mixaq_create(C.byref(self.h), 0) == 0
@@ -100,11 +104,11 @@ class Host:
         return self.L.mixaq_backbone_forward(self.h, C.byref(b["s"]), C.c_void_p(x), b["out"], 1, 14, 14, (C.c_float * 1)(low), None,
                                              b["ws"], b["ws_bytes"], stream if stream is not None else self.DEFAULT)
 
-    def run_block(self, s, x, y, ws, stream=None, sel=None, energy=None):
+    def run_block(self, s, x, y, ws, stream=None, sel=None, energy=None, taps=None):
         n = C.c_size_t(self.L.mixaq_block_workspace_bytes(C.byref(s), 1, 14, 14))
         return self.L.mixaq_block_forward(self.h, C.byref(s), C.c_void_p(x), C.c_void_p(y), 1, 14, 14, C.c_float(0.5), C.c_float(0.25),
                                           C.byref(mq.SelectOpts(energy, 0)), C.byref(sel) if sel is not None else None,
-                                          C.c_void_p(ws), n, None, stream if stream is not None else self.DEFAULT)
+                                          C.c_void_p(ws), n, C.byref(taps) if taps is not None else None, stream if stream is not None else self.DEFAULT)
 
     def close(self):
         assert self.L.mixaq_destroy(self.h) == 0
@@ -318,3 +322,41 @@ def test_a_calibration_whose_waits_ran_out_says_so(host):
         for word in (0, 1, 0):
             host.set("fake_device_word", word)
             assert call() == (-5 if word else 0)                 # MIXAQ_DEVICE_TIMEOUT
+
+
+@pytest.mark.parametrize("taps", [False, True])
+@pytest.mark.parametrize("bits,mult", [((8, 4), 4), ((4, 2), 4), ((2, 2), 4), ((2, 2), 64)])
+def test_guard_zones_lie_around_the_buffers_that_calls_use(host, bits, mult, taps):
+    """One code per byte inside the packed workspace, unless taps ask for packed codes or the hidden layer is too wide: with the
+    zones on as without, each buffer followed by its own zone."""
+    s, x, y, ws = host.block(dim=64, shift=3), host.addr(), host.addr(), host.addr()
+    s.hidden = s.fc1.out_features = s.fc2.in_features = 64 * mult
+    for br, b in ((s.hi, bits[0]), (s.lo, bits[1])):
+        br.bits = b
+        for n in ("qkv_in", "q", "k", "v", "proj_in", "fc1_in", "fc2_in"):
+            setattr(br, n, mq.AQ(b, 0.1, 10.0, 1))
+    found = []
+    for guards in (1, 0):
+        host.L.mixaq_set_workspace_guards(host.h, guards)
+        host.set("written_count", 0)
+        assert host.run_block(s, x, y, ws, taps=mq.Taps() if taps else None) == 0
+        n = C.c_int.in_dll(host.L, "written_count").value
+        found.append([(r.at, r.bytes, r.code_bits) for r in (Range * 256).in_dll(host.L, "written")[:n]])
+    assert found[0] == found[1] and len(found[0]) == 2 * 6
+    packed = taps or mult == 64
+    assert [r[2] for r in found[0] if r[2]] == 5 * (list(bits) if packed else [8, 8])
+    zones = (C.c_void_p * 64).in_dll(host.L, "guard_zones")[:C.c_int.in_dll(host.L, "guard_count").value]
+    end = ws + host.L.mixaq_block_workspace_bytes(C.byref(s), 1, 14, 14)
+    for z in zones:
+        assert ws < z <= end - 256
+        assert all(z + 256 <= at or at + size <= z for at, size, _ in found[0])
+    # what lies side by side or overlaps (both branches' rows, buffers that take turns) has one zone behind it
+    groups = []
+    for at, size, _ in sorted(found[0]):
+        if groups and at <= groups[-1][1]:
+            groups[-1][1] = max(groups[-1][1], at + size)
+        else:
+            groups.append([at, at + size])
+    assert len(groups) == (12 if packed else 4)
+    for (_, last), following in zip(groups, [g[0] for g in groups[1:]] + [end]):
+        assert sum(last <= z < following for z in zones) == 1
