@@ -486,6 +486,10 @@ Tiling pick_tiling(int mode, int unit, int N, int m_tiles, int k_blocks, int sms
   return best;
 }
 
+// Bit-packed launches of a block are those of calls with taps, and of blocks whose hidden layer is too wide for byte codes in their
+// workspace (see carve_bytes): they share the instance with the tap.  Patch merging packs its codes and has no tap.
+__host__ __device__ constexpr bool always_taps(int mode, bool packed) { return packed && mode != EPI_MERGE; }
+
 template <int MODE, int EW, bool PACKED>
 bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
   TcParams p;
@@ -540,10 +544,11 @@ bool launch_mode_as(const GemmArgs& g, int* status, cudaStream_t st) {
   while (p.ring > 2 && smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols).total + 1024 > 220 * 1024) --p.ring;
   const size_t smem = (size_t)smem_layout(p.BN, p.ring, p.packed_bytes, p.res_bytes, p.const_cols).total + 1024 /*alignment slack*/;
   if (smem > 227 * 1024) return false;
-  if (g.br[0].tap_acc || g.br[1].tap_acc)
-    launch_pdl(k_gemm_tc<MODE, true, EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);
+  constexpr bool TAPS = MODE != EPI_MERGE;
+  if (TAPS && (g.br[0].tap_acc || g.br[1].tap_acc))
+    launch_pdl(k_gemm_tc<MODE, TAPS, EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);
   else
-    launch_pdl(k_gemm_tc<MODE, false, EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);
+    launch_pdl(k_gemm_tc<MODE, always_taps(MODE, PACKED), EW, PACKED>, dim3(grid), num_threads(EW, PACKED), smem, st, mA[0], mA[1], mB, p);
   ++g_launches;
   return true;
 }
@@ -679,8 +684,9 @@ bool gemm_init() {
   };
   auto set_up_all = [&](auto mode_tag, auto warps_tag) {
     constexpr int MODE = decltype(mode_tag)::value, EW = decltype(warps_tag)::value;
-    set_up(k_gemm_tc<MODE, false, EW, false>, EW, false); set_up(k_gemm_tc<MODE, true, EW, false>, EW, false);
-    set_up(k_gemm_tc<MODE, false, EW, true>, EW, true); set_up(k_gemm_tc<MODE, true, EW, true>, EW, true);
+    constexpr bool TAPS = MODE != EPI_MERGE;                  // (a merge has none)
+    set_up(k_gemm_tc<MODE, false, EW, false>, EW, false); set_up(k_gemm_tc<MODE, TAPS, EW, false>, EW, false);
+    set_up(k_gemm_tc<MODE, always_taps(MODE, true), EW, true>, EW, true);
   };
   set_up_all(std::integral_constant<int, EPI_QKV>{}, std::integral_constant<int, CODE_WARPS>{});
   set_up_all(std::integral_constant<int, EPI_FC1>{}, std::integral_constant<int, CODE_WARPS>{});

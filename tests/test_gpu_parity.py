@@ -281,7 +281,8 @@ def _full_backbone_case(orc, mq, ctx, wl):
     side.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(side):
         xd = dev(wl.x)
-        # every block bit-packed, then the storage the benchmark uses (one code per byte from 384 channels on)
+        # workspaces sized for bit-packed codes (which calls without taps lay out anew, one code per byte), then those that the
+        # benchmark uses (sized for one code per byte from 384 channels on)
         for byte_min in (None, 384):
             dbb = mq.DeviceBackbone(ctx, wl.backbone, wl.B, wl.H, wl.W, byte_codes_min_dim=byte_min)
             for call in range(2):
@@ -291,7 +292,7 @@ def _full_backbone_case(orc, mq, ctx, wl):
                 for st, (g, w) in enumerate(zip(got, want)):
                     g = g.cpu().numpy()
                     assert_close_rel(g, w)
-                    assert np.array_equal(g, w), f"stage {st} (call {call}, byte codes from {byte_min}) not bit-identical"
+                    assert np.array_equal(g, w), f"stage {st} (call {call}, workspaces for byte codes from {byte_min}) not bit-identical"
             del dbb
     torch.cuda.current_stream().wait_stream(side)
 
@@ -310,6 +311,14 @@ def test_config4_swin_s_1024_full_size_three_classes(orc, mq, ctx):
 def test_config5_swin_b_1536_full_size(orc, mq, ctx):
     """Swin-B, B=2, 384x384 tokens, W8, A8/A4, clustered high-norm regions, ratio 0.5."""
     _full_backbone_case(orc, mq, ctx, synth.config5(ratio=0.5))
+
+
+@pytest.mark.parametrize("dim,H,W,w_bits,bits", [(96, 200, 334, 4, (8, 4)), (96, 256, 256, 4, (4, 2)), (128, 384, 384, 8, (8, 4)),
+                                                 (384, 64, 64, 4, (4, 2)), (768, 25, 42, 4, (8, 4))])
+def test_blocks_at_full_size_with_bit_packed_codes(orc, mq, ctx, dim, H, W, w_bits, bits):
+    """First and late blocks of the three configurations with all taps: the GEMMs that expand packed rows, at their sizes."""
+    blk = synth.make_block(np.random.default_rng(dim + H), dim, dim // 32, 3, w_bits, *bits)
+    run_block_case(orc, mq, ctx, blk, synth.input_blobs(H, 1, H, W, dim, bg_std=0.3, gain=3.0), 0.5)
 
 
 @pytest.mark.parametrize("B,Hi,Wi,C0", [(2, 16, 20, 32), (1, 13, 18, 96), (1, 7, 5, 32), (1, 800, 1333, 96)])
