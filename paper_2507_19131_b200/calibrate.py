@@ -38,15 +38,6 @@ def _upload_stream(device) -> torch.cuda.Stream:
     return _upload_streams[device]
 
 
-def _deep_copy(bb, pool):
-    """copy.deepcopy(bb) with the weight codes, nearly all of its bytes, copied by `pool` (numpy copies without holding the
-    interpreter; fresh pages are what the time goes into): 14 ms for a Swin-T on one thread."""
-    lins = [lin for b in bb.blocks for lin in (b.qkv, b.proj, b.fc1, b.fc2)] + [m.red for m in bb.merges]
-    arrays = {id(lin.codes): lin.codes for lin in lins if type(lin.codes) is np.ndarray and not lin.codes.dtype.hasobject}
-    copies = list(pool.map(lambda a: a.copy(order="K"), arrays.values()))
-    return copy.deepcopy(bb, dict(zip(arrays, copies)))
-
-
 def calibrate_backbone(ctx: "mq.Context", bb, x0: np.ndarray):
     """Returns a deep copy of `bb` whose activation quantizers (both branches of every block, every merge) and score
     steps come from the calibration sample x0 [B,H,W,C0].  Every block is calibrated on the full feature map, once
