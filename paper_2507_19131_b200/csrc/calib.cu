@@ -658,7 +658,7 @@ bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
   if (!launch_cal_ln(c.x1, nullptr, c.ln2_g, c.ln2_b, c.ln, M, C, 0, c.H, c.W, c.shift, nwx, nW, c.obs, 5, -1, st)) return false;
   l.a = c.ln; l.w = c.w_fc1; l.sw = c.s_fc1; l.bias = c.b_fc1; l.out = c.h; l.res = nullptr; l.N = Hd; l.K = C;
   if (!launch_cal_linear<CAL_FC1>(l, st)) return false;
-  l.a = c.h; l.w = c.w_fc2; l.sw = c.s_fc2; l.bias = c.b_fc2; l.out = c.y; l.res = c.x1; l.N = C; l.K = Hd;
+  l.a = c.h; l.w = c.w_fc2; l.sw = c.s_fc2; l.bias = c.b_fc2; l.out = c.y; l.res = c.x1; l.N = C; l.K = Hd; l.slices = c.slices_fc2;
   if (!launch_cal_linear<CAL_FC2>(l, st)) return false;
   return true;
 }

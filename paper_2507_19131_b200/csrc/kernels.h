@@ -139,7 +139,8 @@ struct CalBlockArgs {
   const int8_t *w_qkv, *w_proj, *w_fc1, *w_fc2;
   const float *s_qkv, *s_proj, *s_fc1, *s_fc2, *relpos;
   int32_t* rowsrc; float *ln, *qkv, *o, *x1, *h;  // workspace: [M], [M][C], [M][3C], [M][C], [M][C], [M][hidden]
-  uint8_t* slices; int32_t* expo;                 // workspace of the products: [7][M][max(C, hidden)] bytes, [M]
+  uint8_t *slices, *slices_fc2; int32_t* expo;    // workspace of the products: [7][M][C] bytes, fc2's [7][M][hidden], which may lie
+                                                  // over ln, qkv, o and slices, [M]
   uint32_t* obs;                                  // CAL_OBS words: order-preserving keys (min, max of the seven sites and of x), status
   int* status;
 };

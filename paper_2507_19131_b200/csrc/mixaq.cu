@@ -1247,16 +1247,22 @@ mixaq_status mixaq_set_graph_cache(mixaq_ctx* ctx, int enabled) {
 // -------------------------------------------------------------------------------------------------
 // calibration (Section 4.3)
 namespace {
-struct CalWs { int32_t *rowsrc, *expo; float *ln, *qkv, *o, *x1, *h; uint8_t* slices; uint32_t* obs; size_t bytes; };
+struct CalWs { int32_t *rowsrc, *expo; float *ln, *qkv, *o, *x1, *h; uint8_t *slices, *slices_fc2; uint32_t* obs; size_t bytes; };
 CalWs carve_cal(const mixaq_block_params* p, int B, int H, int W, void* base) {
   CalWs w; Carver c(base);
   Geometry g = geometry(H, W, 0.f, 0.f);
   const size_t M = (size_t)B * g.nW * WT;
   w.obs = c.take<uint32_t>(CAL_OBS);
   w.rowsrc = c.take<int32_t>(M);
-  w.ln = c.take<float>(M * p->dim); w.qkv = c.take<float>(M * 3 * p->dim); w.o = c.take<float>(M * p->dim);
+  w.expo = c.take<int32_t>(M);
   w.x1 = c.take<float>(M * p->dim); w.h = c.take<float>(M * p->hidden);
-  w.expo = c.take<int32_t>(M); w.slices = c.take<uint8_t>(CAL_SLICES * M * std::max(p->dim, p->hidden));
+  // fc2's byte planes, which are the largest, start where the inputs of the products before it lay: 48 C bytes a row at hidden = 4 C
+  // (68 C with a place of their own, 40 C for the arrays that are not planes)
+  const size_t shared = c.off;
+  w.ln = c.take<float>(M * p->dim); w.qkv = c.take<float>(M * 3 * p->dim); w.o = c.take<float>(M * p->dim);
+  const size_t planes = CAL_SLICES * M * p->dim, planes_fc2 = CAL_SLICES * M * p->hidden, dead = c.off - shared;
+  w.slices_fc2 = reinterpret_cast<uint8_t*>(w.ln);
+  w.slices = c.take<uint8_t>(std::max(planes, planes_fc2 > dead ? planes_fc2 - dead : 0));
   w.bytes = c.off;
   return w;
 }
@@ -1298,7 +1304,7 @@ mixaq_status mixaq_calibrate_block(mixaq_ctx* ctx, const mixaq_block_params* p, 
   c.w_qkv = p->qkv.codes; c.w_proj = p->proj.codes; c.w_fc1 = p->fc1.codes; c.w_fc2 = p->fc2.codes;
   c.s_qkv = p->qkv.scale; c.s_proj = p->proj.scale; c.s_fc1 = p->fc1.scale; c.s_fc2 = p->fc2.scale; c.relpos = p->relpos_table;
   c.rowsrc = ws.rowsrc; c.ln = ws.ln; c.qkv = ws.qkv; c.o = ws.o; c.x1 = ws.x1; c.h = ws.h; c.obs = ws.obs;
-  c.slices = ws.slices; c.expo = ws.expo; c.status = ctx->d_status;
+  c.slices = ws.slices; c.slices_fc2 = ws.slices_fc2; c.expo = ws.expo; c.status = ctx->d_status;
   g_launches = 0;
   if (!launch_calibrate_block(c, st)) return fail(ctx, MIXAQ_UNSUPPORTED_SHAPE, "calibrate_block: unsupported dim");
   ctx->launches = g_launches;

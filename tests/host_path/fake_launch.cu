@@ -7,6 +7,7 @@ extern "C" {
 mixaq::SelectArgs last_select;
 struct Range { const void* at; size_t bytes; int code_bits; };      // code_bits: 0 for binary32
 Range written[256]; int written_count;                              // what the kernels since fake_reset write, guard zones apart
+const void* last_calibration[10];
 const void* guard_zones[64]; int guard_count;                       // the zones of the last check
 }
 static void note(const void* at, size_t elements, int bits) {
@@ -51,7 +52,11 @@ void launch_prepare_linear(const int8_t*, const float*, int, int, float, int, in
 void launch_prepare_relbias(const float*, int, float*, cudaStream_t st) { LAUNCH(st); }
 void launch_wait_probe(int*, cudaStream_t st) { LAUNCH(st); }
 int launch_mma_peak(int, int, unsigned long long*, int*, cudaStream_t) { return 0; }
-bool launch_calibrate_block(const CalBlockArgs&, cudaStream_t st) { LAUNCH(st); return true; }
+bool launch_calibrate_block(const CalBlockArgs& c, cudaStream_t st) {
+  const void* at[10] = {c.obs, c.rowsrc, c.expo, c.x1, c.h, c.ln, c.qkv, c.o, c.slices, c.slices_fc2};
+  for (int i = 0; i < 10; ++i) last_calibration[i] = at[i];
+  LAUNCH(st); return true;
+}
 bool launch_calibrate_merge(const CalMergeArgs&, cudaStream_t st) { LAUNCH(st); return true; }
 float cal_key_to_float(uint32_t) { return 0.f; }
 }  // namespace mixaq

@@ -360,3 +360,26 @@ def test_guard_zones_lie_around_the_buffers_that_calls_use(host, bits, mult, tap
     assert len(groups) == (12 if packed else 4)
     for (_, last), following in zip(groups, [g[0] for g in groups[1:]] + [end]):
         assert sum(last <= z < following for z in zones) == 1
+
+
+@pytest.mark.parametrize("mult", [1, 4, 16])
+def test_calibration_workspace_shares_memory_of_what_is_dead(host, mult):
+    """fc2's byte planes lie over what no product behind fc1 reads; nothing else overlaps."""
+    dim, s = 96, host.block(dim=96)
+    s.hidden = s.fc1.out_features = s.fc2.in_features = dim * mult
+    ws, x, y, r = host.addr(), C.c_void_p(host.addr()), C.c_void_p(host.addr()), mq.BlockRangesS()
+    M = 2 * 9 * 49                                                        # 2 maps of 17 x 20: 9 windows each
+    bytes_ = host.L.mixaq_calibrate_block_workspace_bytes(C.byref(s), 2, 17, 20)
+    assert host.L.mixaq_calibrate_block(host.h, C.byref(s), 0, x, y, 2, 17, 20, C.byref(r), C.c_void_p(ws), C.c_size_t(bytes_), None) == 0
+    names = ("obs", "rowsrc", "expo", "x1", "h", "ln", "qkv", "o", "slices", "slices_fc2")
+    size = dict(obs=4 * 17, rowsrc=4 * M, expo=4 * M, x1=4 * M * dim, h=4 * M * s.hidden, ln=4 * M * dim, qkv=12 * M * dim, o=4 * M * dim,
+                slices=7 * M * dim, slices_fc2=7 * M * s.hidden)
+    at = dict(zip(names, (C.c_void_p * 10).in_dll(host.L, "last_calibration")))
+    over = {"ln", "qkv", "o", "slices"}                                   # what slices_fc2 may overlap
+    for a in names:
+        assert ws <= at[a] and at[a] + size[a] <= ws + bytes_ and at[a] % 256 == 0
+        for b in names:
+            if a < b and not ({a, b} - over == {"slices_fc2"}):
+                assert at[a] + size[a] <= at[b] or at[b] + size[b] <= at[a], (a, b)
+    if mult == 4:
+        assert bytes_ <= M * (48 * dim + 8) + 10 * 512
