@@ -10,6 +10,12 @@ run agrees with them to about 1e-4 relative in the smallest coefficients and exa
 maximum error is within a fraction of a percent of the optimum; `check()` measures both.  Re-deriving them does not
 change the contract: the frozen words do.
 
+A third polynomial is no part of the contract: the one that the fc1 epilogue evaluates first, degree 6 in -a.  It approximates the
+contract's degree-7 polynomial Q with a small largest error of a * 2^q (weight a * 2^Q(a) * ln 2), from a linear program on a grid; in
+binary32 the rounding of the evaluation is the larger part of the error, so a finer fit gains little (6.0e-8 against 6.3e-8).  The
+epilogue compares each value's distance from a rounding boundary with a bound that rests on that error and takes the contract's
+own operations where it is too close; `check_fast_gelu()` fits again.
+
   python oracle/fit_contract_polynomials.py        # prints frozen and re-derived coefficients and their errors
 """
 from __future__ import annotations
@@ -30,6 +36,10 @@ TARGETS = {
     "exp2": (lambda t: np.exp2(t), 5, -0.5, 0.5),
     "log2_phi_neg": (lambda a: log_ndtr(-np.asarray(a, dtype=np.float64)) / math.log(2.0), 7, 0.0, 5.0),
 }
+
+
+# of (-a)^0, (-a)^1, ...: the words in csrc/common.cuh (gelu_log2_tail_neg2)
+FAST_GELU = [0xbf7fffe5, 0x3f935ab1, 0xbeead2f4, 0x3d5bddca, 0x3c07b015, 0x3a5a8f53, 0x3829e7cb]
 
 
 def word_to_float(w: int) -> float:
@@ -95,7 +105,34 @@ def check():
     return out
 
 
+def check_fast_gelu(grid_points: int = 4001):
+    """Largest weighted error of the frozen words and of a fresh fit (binary64, dense grid), largest difference of the two
+    polynomials' values of a * 2^q."""
+    from scipy.optimize import linprog
+    contract = np.array([word_to_float(w) for w in FROZEN["log2_phi_neg"]])
+
+    def target(a):
+        q = np.polyval(contract[::-1], a)
+        return q, a * np.exp2(q) * math.log(2.0)
+    a = 2.5 * (1.0 - np.cos(np.linspace(0.0, math.pi, grid_points)))          # denser at the ends
+    q, weight = target(a)
+    cheb = np.polynomial.chebyshev.chebvander(a / 2.5 - 1.0, 6)
+    scale = 1e8                                                               # the solver's tolerances are absolute
+    rows = weight[:, None] * cheb * scale
+    ones = np.ones((a.size, 1))
+    res = linprog(np.r_[np.zeros(7), 1.0], A_ub=np.block([[rows, -ones], [-rows, -ones]]),
+                  b_ub=np.r_[weight * q, -weight * q] * scale, bounds=[(None, None)] * 8, method="highs")
+    fitted = np.polynomial.Chebyshev(res.x[:7], domain=[0.0, 5.0])
+    frozen = np.array([word_to_float(w) for w in FAST_GELU])
+    dense = np.linspace(0.0, 5.0, 200001)
+    q, weight = target(dense)
+    p = np.polyval(frozen[::-1], -dense)
+    return {"max_err_frozen": float(np.abs(weight * (p - q)).max()), "max_err_fitted": float(np.abs(weight * (fitted(dense) - q)).max()),
+            "max_diff_to_fit": float(np.abs(weight * (p - fitted(dense))).max())}
+
+
 if __name__ == "__main__":
+    print("fast GELU", check_fast_gelu())
     for name, r in check().items():
         print(name)
         print("  frozen  ", " ".join("0x%08x" % w for w in r["frozen_words"]))

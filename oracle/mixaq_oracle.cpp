@@ -403,6 +403,30 @@ void orc_layernorm(const float* x, long rows, int C, const float* g, const float
 }
 void orc_exp2(const float* t, long n, float* y) { for (long i = 0; i < n; ++i) y[i] = exp2_clamped(t[i]); }
 void orc_gelu(const float* x, long n, float* y) { for (long i = 0; i < n; ++i) y[i] = gelu1(x[i]); }
+double orc_gelu_tail_gap(const float* p, int degree, float lo, float hi, long step, float* at, double* top) {
+  const long first = f2i(lo), last = f2i(hi);          // positive numbers: their bit patterns ascend with them
+  double worst = -1.0, largest = 0.0;
+  float where = lo;
+#pragma omp parallel
+  {
+    double mine = -1.0, my_largest = 0.0;
+    float my_where = lo;
+#pragma omp for schedule(static)
+    for (long i = 0; i < (last - first) / step + 1; ++i) {
+      const float a = i2f((int)(first + i * step));
+      float u = p[degree], q = kGeluQ[7];
+      for (int k = degree - 1; k >= 0; --k) u = std::fmaf(u, -a, p[k]);
+      for (int k = 6; k >= 0; --k) q = std::fmaf(q, a, kGeluQ[k]);
+      const double h = (double)a * std::exp2((double)q), d = std::fabs((double)a * std::exp2((double)u) - h);
+      if (d > mine) { mine = d; my_where = a; }
+      my_largest = std::max(my_largest, h);
+    }
+#pragma omp critical
+    { if (mine > worst) { worst = mine; where = my_where; } largest = std::max(largest, my_largest); }
+  }
+  *at = where; *top = largest;
+  return worst;
+}
 void orc_softmax_rows(const float* s, long rows, int T, float* p) {
   for (long r = 0; r < rows; ++r) softmax_row(s + r * T, T, p + r * T);
 }

@@ -84,6 +84,10 @@ void  orc_unpack(const uint8_t* packed, long rows, int cols, int bits, uint8_t* 
 void  orc_layernorm(const float* x, long rows, int C, const float* g, const float* b, float* y);
 void  orc_exp2(const float* t, long n, float* y);
 void  orc_gelu(const float* x, long n, float* y);
+/* largest |a * 2^p(-a) - a * 2^q(a)| over the binary32 numbers a of [lo, hi] (every step-th one): p a polynomial given by its
+ * coefficients (constant first), q the contract's log2 Phi(-a); both by Horner with fused multiply-adds in binary32, the rest in
+ * binary64.  at: where; top: the largest a * 2^q(a) met. */
+double orc_gelu_tail_gap(const float* p, int degree, float lo, float hi, long step, float* at, double* top);
 void  orc_softmax_rows(const float* s, long rows, int T, float* p);
 void  orc_int_gemm(const uint8_t* a, long M, int K, int za, const int8_t* w, int N, int32_t* acc);
 /* source token (y*W+x) of in-window position t of window w under a cyclic shift, or -1 for a pad token */

@@ -76,6 +76,7 @@ def lib():
         _lib.orc_low_count.restype = C.c_int
         _lib.orc_low_count.argtypes = [C.c_double, C.c_int]
         _lib.orc_window_token.restype = C.c_long
+        _lib.orc_gelu_tail_gap.restype = C.c_double
         _lib.orc_get_threads.restype = C.c_int
     return _lib
 
@@ -189,6 +190,14 @@ def gelu(x):
     y = np.empty_like(x)
     lib().orc_gelu(_p(x), C.c_long(x.size), _p(y))
     return y
+
+
+def gelu_tail_gap(coef, lo: float, hi: float, step: int = 1):
+    """(largest difference, where, largest a * Phi(-a)) over the binary32 numbers of [lo, hi]; see orc_gelu_tail_gap."""
+    coef = np.ascontiguousarray(coef, np.float32)
+    at, top = C.c_float(), C.c_double()
+    gap = lib().orc_gelu_tail_gap(_p(coef), C.c_int(coef.size - 1), C.c_float(lo), C.c_float(hi), C.c_long(step), C.byref(at), C.byref(top))
+    return gap, at.value, top.value
 
 
 def softmax_rows(s):

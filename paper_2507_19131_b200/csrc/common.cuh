@@ -77,9 +77,9 @@ __device__ __forceinline__ float2 gelu_log2_tail2(float2 a) {      // log2 Phi(-
   q = __ffma2_rn(q, a, f2(__uint_as_float(0xbf935b8fu)));
   return __ffma2_rn(q, a, f2(__uint_as_float(0xbf7fffbeu)));
 }
-// Nearly the same of -a, for values that are checked before they decide a code: degree 6, the minimax fit (linear program, weighted
-// with a 2^q ln 2) to the polynomial above.  a 2^q differs by at most 6.4e-8, evaluated as here in binary32 over all a in [2^-5, 5] and
-// every eighth one in [2^-12, 2^-5); below it is smaller than a.
+// Nearly the same of -a, for values that are checked before they decide a code: degree 6, fitted (linear program, weighted
+// with a 2^q ln 2) to the polynomial above (oracle/fit_contract_polynomials.py).  a 2^q differs by at most 6.4e-8, evaluated as here in
+// binary32 over every a in [2^-12, 5]; below it differs by less than 1e-9.
 __device__ __forceinline__ float2 gelu_log2_tail_neg2(float2 a) {
   float2 q = f2(__uint_as_float(0x3829e7cbu));
   q = __ffma2_rn(q, a, f2(__uint_as_float(0x3a5a8f53u)));

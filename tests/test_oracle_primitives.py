@@ -141,6 +141,29 @@ def test_contract_polynomials_are_the_minimax_fits_the_fit_script_derives(orc):
     assert np.array_equal(orc.exp2(f), p)
 
 
+def test_fast_gelu_polynomial_and_its_error_bound(orc):
+    """The degree-6 polynomial that the fc1 epilogue evaluates first: its words are those of the kernel, they are near the minimax fit
+    to the contract's polynomial (2.1e-8 in binary64; rounded coefficients 2.5e-8), and the bound that the epilogue's check rests on
+    holds over every binary32 argument."""
+    import os
+    import re
+    from oracle import fit_contract_polynomials as fit
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_19131_b200", "csrc")
+    text = open(os.path.join(csrc, "common.cuh")).read()
+    body = text[text.index("float2 gelu_log2_tail_neg2("):]
+    body = body[:body.index("}")]
+    assert [int(w, 16) for w in re.findall(r"0x([0-9a-f]{8})u", body)] == fit.FAST_GELU[::-1]
+    r = fit.check_fast_gelu()
+    assert r["max_err_frozen"] < 3.6e-8 and 2.0e-8 < r["max_err_fitted"] < 2.2e-8 and r["max_diff_to_fit"] < 1.6e-8, r
+    coef = [F32(fit.word_to_float(w)) for w in fit.FAST_GELU]
+    gap, at, top = orc.gelu_tail_gap(coef, 2.0 ** -12, 5.0)
+    assert gap <= 6.4e-8 and top <= 0.17, (gap, at, top)
+    assert orc.gelu_tail_gap(coef, 2.0 ** -126, 2.0 ** -12, 97)[0] <= 1e-9
+    # the epilogue's constant: that gap, 2^-22 relative of either exponential, one rounding of h
+    bound = float(re.search(r"__fmaf_rn\(inv_scale, ([0-9.e-]+)f,", open(os.path.join(csrc, "gemm_epilogue.cuh")).read()).group(1))
+    assert 6.4e-8 + 0.17 * (2 * 2.0 ** -22 + 2.0 ** -24) < 1.7e-7 < bound
+
+
 def test_softmax_rows(orc):
     rng = np.random.default_rng(11)
     s = (rng.standard_normal((200, 49)) * 4).astype(F32)
