@@ -192,7 +192,8 @@ def run_ours(args):
     torch.cuda.set_stream(torch.cuda.Stream())
     ctx = mq.Context(local)
     K, Wm = args.steps, max(args.warmup, 3)
-    # storage of the blocks' intermediate codes: bit-packed below this many channels, one code per byte from there on
+    # workspaces of blocks with at least this many channels are sized for one code per byte, the others for bit-packed codes (calls
+    # without taps keep one code per byte in either)
     BYTE_MIN = args.byte_codes_min_dim if args.byte_codes_min_dim > 0 else None
 
     def barrier():
@@ -389,7 +390,7 @@ def run_ours(args):
     e2e = time_e2e(args.ratio, K, Wm)
     e2e_value = replicas.job_throughput(wl_images(e2e["wl"]), K, world, e2e["ms"])
 
-    # the same forward with every block's codes bit-packed (what the expansion in shared memory costs in stages 3-4)
+    # the same forward with every block's workspace sized for bit-packed codes (its calls lay it out anew for bytes)
     packed_value = None
     if BYTE_MIN is not None and world == 1:
         n_p = max(3, K // 2)
@@ -465,8 +466,8 @@ def run_ours(args):
                    "weights": "W%d (int8 container)" % bbm.blocks[0].qkv.bits,
                    "act_bits_high_low": [bbm.blocks[0].hi.bits, bbm.blocks[0].lo.bits], "low_ratio": args.ratio,
                    "prune_ratio": (main["wl"].prune_ratios or [0.0])[0],
-                   "code_storage": ("bit-packed in every block" if BYTE_MIN is None else
-                                    f"bit-packed in blocks of fewer than {BYTE_MIN} channels, one code per byte from {BYTE_MIN} on"),
+                   "code_storage": ("one code per byte; workspaces sized for bit-packed codes in " +
+                                    ("every block" if BYTE_MIN is None else f"blocks of fewer than {BYTE_MIN} channels")),
                    "l2": f"flushed between timed iterations ({L2_FLUSH_BYTES >> 20} MiB write)",
                    "parallelism": "replicas only (one image per GPU, no collective)"},
         "clocks": main["clocks"],
@@ -480,7 +481,7 @@ def run_ours(args):
         "gpu_launches": main["launches"] * K,
         "roofline": roof,
         "kernels": kernels,
-        "value_all_bit_packed": packed_value,
+        "value_all_packed_workspaces": packed_value,
         "low_ratio_sweep_images_per_sec": sweep,
         "paper_cost_model": cost,
         "value_with_stem": stem,
@@ -614,8 +615,8 @@ def main():
                     help="also sweep the low-bit ratio for --config 4 (0 ... 0.75) or 5 (0 ... 0.8); config 3 sweeps by default")
     ap.add_argument("--no-cpu-baseline", dest="cpu_baseline", action="store_false")
     ap.add_argument("--byte-codes-min-dim", type=int, default=384,
-                    help="blocks with at least this many channels store their intermediate codes one per byte "
-                         "(mixaq_block_params.byte_codes); 0: every block bit-packs")
+                    help="blocks with at least this many channels have workspaces sized for one code per byte "
+                         "(mixaq_block_params.byte_codes); 0: none, every workspace is sized for bit-packed codes")
     args = ap.parse_args()
     global CONFIG
     CONFIG = args.config

@@ -498,8 +498,8 @@ class DeviceBackbone:
     """All parameters of a backbone on the device, prepared; owns the workspace and the stage outputs.
     embed: stem parameters (object with ln_g, ln_b, bias, aq, proj) -- the forward then takes the IMAGE [B,H0,W0,3];
     norms: one (gamma, beta) pair of numpy vectors per stage -- the stage outputs are then LayerNormed.
-    byte_codes_min_dim: blocks with at least this many channels keep their intermediate codes one per byte
-    (mixaq_block_params.byte_codes); None: every block bit-packs."""
+    byte_codes_min_dim: blocks with at least this many channels have workspaces sized for one code per byte
+    (mixaq_block_params.byte_codes); None: every workspace is sized for bit-packed codes."""
 
     def __init__(self, ctx: Context, bb, B: int, H0: int, W0: int, embed=None, norms=None, byte_codes_min_dim=None):
         self.ctx, self.bb, self.B, self.H0, self.W0 = ctx, bb, B, H0, W0

@@ -95,8 +95,9 @@ __device__ __forceinline__ void gelu_pattern2(float2 v, float inv_scale, float m
   m0 = __float_as_uint(r.x); m1 = __float_as_uint(r.y);
 }
 // Distance of g * inv_scale from the contract's t: the polynomials change h = a 2^q <= 0.17 by at most 6.4e-8, both exponentials are
-// within 2^-22 of theirs, so h differs by at most 6.4e-8 + 0.17 * 2^-21 + one rounding < 1.7e-7; g is rounded in both evaluations and t in the contract's, which adds
-// |t| * 3 * 2^-24, and |t| <= max(code, zp) + 1 for every t that is not clamped anyway; the distance itself is rounded by 2^-26.
+// within 2^-22 of theirs, so h differs by at most 6.4e-8 + 0.17 * 2^-21 + one rounding < 1.7e-7; g is rounded in both evaluations
+// and t in the contract's, which adds |t| * 3 * 2^-24, and |t| <= max(code, zp) + 1 for every t that is not clamped anyway; the
+// distance itself is rounded by 2^-26.
 // maxf: at least the codes in question and the zero point
 __device__ __forceinline__ float gelu_threshold(float inv_scale, float maxf) {
   return 0.5f - __fmaf_rn(inv_scale, 1.9e-7f, (maxf + 2.0f) * 1.8e-7f);

@@ -12,7 +12,7 @@
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
 //               the swizzled layout (rows whose byte pitch is no multiple of 16 cannot be described to the TMA
 //               unit and are read with plain loads instead);
-//   then        epilogue (12 warps for the code outputs, 8 or 12 for the binary32 outputs): tcgen05.ld (a quad of lanes
+//   then        epilogue (12 warps for the code outputs, 8 for the binary32 outputs): tcgen05.ld (a quad of lanes
 //               per row, 16 columns per load) + the fused epilogue of the mode.
 // Every wait on an mbarrier is bounded; on expiry the CTA raises the status word, then waits (bounded again) for the
 // copies it has issued to land and for the MMAs it has issued to retire, frees its tensor memory and returns.
@@ -40,18 +40,17 @@ constexpr int A_STAGE_BYTES = BM * BK;
 // warps 4..7 expand sub-byte codes (two warps left the long-K main loops of 4-bit tiles waiting for the expansion;
 // eight cost more registers than they return)
 constexpr int UNPACK_WARPS = 4;
-// Epilogue warps.  Code outputs: 12 (16 with fewer registers are no faster at any size).  Binary32 outputs: 8; 12 up to a row tile
-// per twelve SMs, where a launch is the latency of a tile or two and three warps share the columns of a lane quarter (fc2 of
-// 768 channels at 7 x 7: 6.7 against 7.7 us, at 25 x 42 8.3 against 9.2; from 26 row tiles on 8 warps are up to 10 % faster).
-constexpr int F32_WARPS = 8, F32_WARPS_FEW = 12, CODE_WARPS = 12;
-constexpr int FEW_SMS_PER_ROW_TILE = 12;
+// Epilogue warps.  Code outputs: 12 (16 with fewer registers are no faster at any size).  Binary32 outputs: 8, which are as fast as 12
+// for few row tiles and up to 16 % faster for many (best tiling of either, fc2 of 768 channels at 7 x 7: 6.7 against 6.8 us, at 25 x 42
+// 8.1 against 8.5, at 4 x 32 x 32 15.3 against 18.2).
+constexpr int F32_WARPS = 8, CODE_WARPS = 12;
 // Warpgroups: TMA, MMA and TMEM set-up; unpack, only in launches with bit-packed rows; epilogue
 constexpr int FIRST_UNPACK_WARP = 4;
 __host__ __device__ constexpr int first_epi_warp(bool packed) { return FIRST_UNPACK_WARP + (packed ? UNPACK_WARPS : 0); }
 __host__ __device__ constexpr int num_threads(int warps, bool packed) { return 32 * (first_epi_warp(packed) + warps); }
-// Registers.  A block is launched with what its threads divide the file into (a scheduler's 16 384 among its warps: 128 a thread with
-// 12 epilogue warps, 96 with the unpack warps too); the side warpgroups give back all but SIDE_REGS
-// and the epilogue warps take them: 4 x 72 + 12 x 136 of 16 x 128, 8 x 72 + 12 x 112 of 20 x 96.  gemm_init checks that the shares fit
+// Registers.  With 12 epilogue warps a block is launched with what its threads divide the file into (a scheduler's 16 384 among its
+// warps: 128 a thread, 96 with the unpack warps too); the side warpgroups give back all but SIDE_REGS and the epilogue warps take
+// them: 4 x 72 + 12 x 136 of 16 x 128, 8 x 72 + 12 x 112 of 20 x 96.  gemm_init checks that the shares fit
 // into what the compiled kernels are launched with.  (No instance spills; with 56 for the side warps six did.)
 constexpr int SIDE_REGS = 72;
 __host__ __device__ constexpr int epi_regs(int warps, bool packed) { return warps != 12 ? 0 : packed ? 112 : 136; }    // 0: no exchange
@@ -116,7 +115,7 @@ struct RingPos {
 //
 // The loops of the TMA and the MMA warp bound a tile as much as the epilogue does, so they hold no division, and the whole warp
 // walks through them with one elected lane issuing: in code that a single lane runs, an MMA of up to 64 columns takes 63 cycles to
-// issue (its operands go through the uniform registers one by one), elected in a converged warp 46 to 50.
+// issue, elected in a converged warp 45 to 51.
 template <int MODE, bool TAPS, int EW, bool PACKED>
 __global__ void __launch_bounds__(num_threads(EW, PACKED), 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
@@ -456,9 +455,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 // width C of a section, so that a tile has one quantizer), at most 256.  A tile takes `mma` to multiply and each of its warps `epi`
 // to convert, `groups` tiles are converted at once while the next ones are multiplied, and the first tiles have nothing to hide
 // behind.  A wide tile reads its rows fewer times and pays the fixed part of the epilogue once for more columns; narrow ones spread a
-// small problem over the SMs.  The constants (microseconds, roughly) are a fit to the times of all widths and groups of the four GEMMs
-// at 25 maps from 768 x 7 x 7 to 128 x 384 x 384, each taken together with the kernel behind it: on average 2 % above the fastest
-// choice, 4 % with the constants that were fitted to the kernels before (worst: QKV with C = 512 at 14 x 14, 8.4 us against 6.6).
+// small problem over the SMs.  The constants (microseconds, roughly) were fitted to the times of all widths and groups of the four GEMMs
+// at 25 maps from 768 x 7 x 7 to 128 x 384 x 384, each taken together with the kernel behind it.  With the present kernels the choice
+// is 2.2 % above the fastest on average, within 10 % at 96 of 100.
 struct Tiling { int bn, n_acc, groups, split; };
 Tiling pick_tiling(int mode, int unit, int N, int m_tiles, int k_blocks, int sms, int warps) {
   Tiling best = {0, 0, 0, 0};
@@ -691,23 +690,18 @@ bool gemm_init() {
   set_up_all(std::integral_constant<int, EPI_QKV>{}, std::integral_constant<int, CODE_WARPS>{});
   set_up_all(std::integral_constant<int, EPI_FC1>{}, std::integral_constant<int, CODE_WARPS>{});
   set_up_all(std::integral_constant<int, EPI_PROJ>{}, std::integral_constant<int, F32_WARPS>{});
-  set_up_all(std::integral_constant<int, EPI_PROJ>{}, std::integral_constant<int, F32_WARPS_FEW>{});
   set_up_all(std::integral_constant<int, EPI_FC2>{}, std::integral_constant<int, F32_WARPS>{});
-  set_up_all(std::integral_constant<int, EPI_FC2>{}, std::integral_constant<int, F32_WARPS_FEW>{});
   set_up_all(std::integral_constant<int, EPI_MERGE>{}, std::integral_constant<int, F32_WARPS>{});
-  set_up_all(std::integral_constant<int, EPI_MERGE>{}, std::integral_constant<int, F32_WARPS_FEW>{});
   return ok;
 }
 
 bool launch_gemm(const GemmArgs& g, cudaStream_t st) {
-  const long row_tiles = (long)(g.br[0].M + BM - 1) / BM + (g.br[1].M + BM - 1) / BM;
-  const bool few = row_tiles * FEW_SMS_PER_ROW_TILE <= sm_count();
   switch (g.mode) {
     case EPI_QKV:   return launch_mode<EPI_QKV, CODE_WARPS>(g, g.status, st);
     case EPI_FC1:   return launch_mode<EPI_FC1, CODE_WARPS>(g, g.status, st);
-    case EPI_PROJ:  return few ? launch_mode<EPI_PROJ, F32_WARPS_FEW>(g, g.status, st) : launch_mode<EPI_PROJ, F32_WARPS>(g, g.status, st);
-    case EPI_FC2:   return few ? launch_mode<EPI_FC2, F32_WARPS_FEW>(g, g.status, st) : launch_mode<EPI_FC2, F32_WARPS>(g, g.status, st);
-    case EPI_MERGE: return few ? launch_mode<EPI_MERGE, F32_WARPS_FEW>(g, g.status, st) : launch_mode<EPI_MERGE, F32_WARPS>(g, g.status, st);
+    case EPI_PROJ:  return launch_mode<EPI_PROJ, F32_WARPS>(g, g.status, st);
+    case EPI_FC2:   return launch_mode<EPI_FC2, F32_WARPS>(g, g.status, st);
+    case EPI_MERGE: return launch_mode<EPI_MERGE, F32_WARPS>(g, g.status, st);
   }
   return false;
 }

@@ -57,7 +57,7 @@ DEFAULT_METRICS = [
 
 
 # the sources that hold the device code of the GEMM kernel whose DRAM traffic is recorded
-GEMM_KERNEL_SOURCES = ("common.cuh", "gemm_epilogue.cuh", "gemm_tc.cu", "kernels.h")
+GEMM_KERNEL_SOURCES = ("common.cuh", "gemm_epilogue.cuh", "gemm_tc.cu", "kernels.h", "tc_ptx.cuh")
 
 
 def kernel_source_digest() -> str:

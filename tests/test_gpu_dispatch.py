@@ -41,7 +41,7 @@ def test_gemm_tilings_around_their_limits(orc, mq, ctx, dim, windows):
 
 @pytest.mark.parametrize("dim,H,W", [(96, 35, 42), (96, 21, 74), (384, 35, 41), (384, 28, 56)])
 def test_gemm_epilogue_warps_around_their_limit(orc, mq, ctx, dim, H, W):
-    """12 row tiles (12 epilogue warps for the binary32 outputs) and 14 (8 warps), with remainders in the last tile."""
+    """12 and 14 row tiles, with remainders in the last tile."""
     blk = synth.make_block(np.random.default_rng(dim + W), dim, dim // 32, 3, 8, 8, 4, share_bias=False)
     run_block_case(orc, mq, ctx, blk, synth.input_student_t(dim, 1, H, W, dim), 0.5, taps=False)
 

@@ -31,8 +31,8 @@ def test_registers_are_exchanged_by_whole_warpgroups():
     assert re.search(r'\n  if \(epi_regs\(EW, PACKED\) > 0 && warp < FIRST_EPI_WARP\) asm volatile\("setmaxnreg\.dec\.[^\n]*\n\s*'
                      r'if \(warp == 0\) \{', body)
     assert re.search(r'\n  \} else \{\s*if \(epi_regs\(EW, PACKED\) > 0\) asm volatile\("setmaxnreg\.inc\.', body)
-    number = {n: int(v) for n, v in re.findall(r"\b(FIRST_UNPACK_WARP|UNPACK_WARPS|CODE_WARPS|F32_WARPS_FEW|F32_WARPS) = (\d+)", text)}
-    assert len(number) == 5 and all(v % 4 == 0 for v in number.values())      # every boundary between roles lies between warpgroups
+    number = {n: int(v) for n, v in re.findall(r"\b(FIRST_UNPACK_WARP|UNPACK_WARPS|CODE_WARPS|F32_WARPS) = (\d+)", text)}
+    assert len(number) == 4 and all(v % 4 == 0 for v in number.values())      # every boundary between roles lies between warpgroups
 
 
 def test_the_lanes_of_a_warp_give_up_together():
