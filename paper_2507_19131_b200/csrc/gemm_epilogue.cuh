@@ -11,7 +11,8 @@
 // every lane, 12 bytes a value through a 128-byte path: a quarter of the fc1 epilogue's time and half of the QKV epilogue's.  Now a
 // value read serves four rows, and the binary32 outputs need no transposition through shared memory.  B200, 294 912 rows of 128
 // channels, before and after: QKV 58.4 -> 49.0 us, proj 60.1 -> 55.1, fc1 137.5 -> 137.2, fc2 76.1 -> 76.1; 18 432 rows of 512: QKV
-// 23.4 -> 20.4, proj 23.0 -> 20.9, fc1 46.4 -> 45.0, fc2 33.1 -> 33.8.
+// 23.4 -> 20.4, proj 23.0 -> 20.9, fc1 46.4 -> 45.0, fc2 33.1 -> 33.8.  Since the warp number comes through a shuffle (gemm_tc.cu):
+// 47.7, 54.0, 120.1, 74.8 and 20.4, 20.1, 40.1, 34.0.
 #pragma once
 #include "kernels.h"
 #include "tc_ptx.cuh"

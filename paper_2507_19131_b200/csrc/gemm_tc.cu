@@ -6,7 +6,7 @@
 // Persistent, warp-specialised: one CTA per SM walks over the output tiles t = blockIdx.x, + gridDim.x, ...
 //   warp 0      TMA producer: weight tile and (8-bit branches) activation tile of every k-block into a ring of
 //               128-byte-swizzled K-major stages (cp.async.bulk.tensor, no multicast), completion on mbarriers;
-//   warp 1      MMA issuer: one thread feeds the tensor core; the tiles take turns on up to six TMEM accumulators, so
+//   warp 1      MMA issuer: one elected lane feeds the tensor core; the tiles take turns on up to six TMEM accumulators, so
 //               that the epilogue of a tile overlaps the loads and MMAs of the following ones;
 //   warps 4-7   unpack producers for 4-bit / 2-bit branches: the bit-packed rows of the k-block arrive by TMA in a
 //               staging slot of the stage; these warps expand them to one code per byte, shared to shared, into
@@ -111,7 +111,7 @@ struct RingPos {
   __device__ __forceinline__ void next(int n) { if (++slot == n) { slot = 0; pass ^= 1u; } }
 };
 
-// TAPS: the accumulator tap is compiled in only for calls that ask for it
+// TAPS: the accumulator tap is compiled in only for calls that ask for it (and where always_taps says so)
 //
 // The loops of the TMA and the MMA warp bound a tile as much as the epilogue does, so they hold no division, and the whole warp
 // walks through them with one elected lane issuing: in code that a single lane runs, an MMA of up to 64 columns takes 63 cycles to
@@ -428,7 +428,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
     // A wait ran out.  Before the CTA may exit, the copies already issued must have landed in its shared memory and
     // the MMAs already issued must have retired.  (1) The lane that issued the MMAs commits them to a barrier of their
     // own (a commit covers what its own thread has issued; elect.sync names the same lane of a full warp every time).
-    // (2) The TMA thread waits, bounded, for the phase of the last fill of every stage, on the full barrier and on
+    // (2) A thread of the TMA warp waits, bounded, for the phase of the last fill of every stage, on the full barrier and on
     // the packed-rows barrier (both complete by the copies alone), and for that commit.
     if (warp == 1 && elect_one()) mma_commit(bar_drain);
     __syncthreads();

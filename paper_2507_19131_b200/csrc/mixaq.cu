@@ -723,7 +723,7 @@ static bool caller_is_capturing(cudaStream_t st) {
 // The call `forward(stream, recording)` with this key: replayed when it was recorded before, recorded (and launched) when
 // that is worth it and works, else issued on the caller's stream: recording takes device memory, which a call does not
 // otherwise need, so that it fails is no reason for the call to fail.  What a call costs (us, Swin-T forwards on the default stream,
-// waited for one by one; 224 x 224 image / 800 x 1333 map): 473 / 902 replayed, 514 / 939 issued, 1 026 / 1 341 recorded.
+// waited for one by one; 224 x 224 image / 800 x 1333 map): 393 / 802 replayed, 433 / 801 issued, 798 / 1 119 recorded.
 // Calls are recorded on a stream of the context's own: the legacy default stream cannot be captured, and while another one
 // is, it refuses what other threads put on it (a blocking one makes work on the default stream fail too).
 // The caller holds graph_lock.
@@ -777,8 +777,8 @@ mixaq_status mixaq_block_forward(mixaq_ctx* ctx, const mixaq_block_params* p, co
                               taps, nullptr, st);
   };
   // A call repeated with the same arguments replays a graph: issuing its eleven launches and their tensor maps takes the
-  // host longer than a small block takes the GPU (C = 96 at 56 x 56: 58 us a call without a replay, 40 with; C = 384 at
-  // 50 x 84 with pruning, bound by the GPU but for the gaps between stream launches: 72 and 66).
+  // host longer than a small block takes the GPU (C = 96 at 56 x 56: 41 to 51 us a call without a replay, 31 with; C = 384 at
+  // 50 x 84 with pruning, bound by the GPU but for the gaps between stream launches: 54.5 and 51.5).
   if (!ctx || !p || taps || !ctx->graph_cache || ctx->profiling || ctx->guards || ctx->nvtx) return forward(user_stream);
   if (caller_is_capturing(user_stream)) return forward(user_stream);
   std::string key;
