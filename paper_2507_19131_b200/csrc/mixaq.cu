@@ -602,8 +602,9 @@ static mixaq_status block_forward_impl(mixaq_ctx* ctx, const mixaq_block_params*
   }
   if (!presel) {
     const int32_t* energy = opts ? opts->energy : nullptr;
-    if (!energy) { PROF(PC_ENERGY); launch_energy(x, ws.energy, (long)B * H * W, C, p->score_inv_scale, st); energy = ws.energy; }
-    SelectArgs sa = make_select_args(sel, energy, B, H, W, p->shift, g, opts ? opts->reverse : 0, energy == ws.energy);
+    const bool own_energy = !energy;
+    if (own_energy) { PROF(PC_ENERGY); launch_energy(x, ws.energy, (long)B * H * W, C, p->score_inv_scale, st); energy = ws.energy; }
+    SelectArgs sa = make_select_args(sel, energy, B, H, W, p->shift, g, opts ? opts->reverse : 0, own_energy);
     { PROF(PC_SELECT); launch_select(&sa, 1, st); }
   }
   if (sel_out) {

@@ -30,6 +30,20 @@ def test_window_selection_by_window_count(orc, mq, ctx, H, W):
         run_block_case(orc, mq, ctx, blk, x, low, prune, reverse=rev, taps=False)
 
 
+@pytest.mark.parametrize("reverse", [False, True])
+@pytest.mark.parametrize("H,W", [(21, 28), (56, 56)])
+def test_window_selection_by_a_callers_large_energies(orc, mq, ctx, H, W, reverse):
+    """A caller's energies up to 2^31: window scores beyond 2^32 whose lower halves are in another order."""
+    rng = np.random.default_rng(H)
+    blk, x = synth.make_block(rng, 32, 1, 3, 8, 8, 4), synth.input_student_t(W, 2, H, W, 32)
+    energy = rng.integers(0, 2 ** 31, size=(2, H, W)).astype(np.int32)
+    ref = orc.block_forward(blk, x, 0.5, 0.25, energy_map=energy, reverse=reverse)
+    assert (ref.scores > 2 ** 32).all() and (np.argsort(ref.scores) != np.argsort(ref.scores.astype(np.int32))).any()
+    got = mq.block_forward(ctx, mq.DeviceBlock(ctx, blk), dev(x), 0.5, 0.25, energy=dev(energy), reverse=reverse, selection=True)
+    for name, want in (("scores", ref.scores), ("order", ref.order), ("cls", ref.cls), ("y", ref.y)):
+        assert np.array_equal(getattr(got, name).cpu().numpy(), want), name
+
+
 @pytest.mark.parametrize("dim,windows", [(32, (27, 28)), (32, (28, 28)), (64, (28, 28)), (96, (28, 28)), (1024, (1, 2))])
 def test_gemm_tilings_around_their_limits(orc, mq, ctx, dim, windows):
     """Row tiles just below and above the limit of the 16 epilogue warps, tile widths 32 to 256, more accumulators than

@@ -22,7 +22,7 @@ class Counts(C.Structure):
 
 class SelectArgs(C.Structure):
     _fields_ = [(n, C.c_void_p) for n in ("energy", "score", "order", "cls", "rowsrc_hi", "rowsrc_lo", "rowsrc_pr", "win_hi", "win_lo")] + \
-               [(n, C.c_int) for n in ("B", "H", "W", "shift", "nwx", "nW", "n_hi", "n_lo", "n_pr", "reverse")]
+               [(n, C.c_int) for n in ("B", "H", "W", "shift", "nwx", "nW", "n_hi", "n_lo", "n_pr", "reverse")] + [("narrow", C.c_bool)]
 
 
 class Range(C.Structure):
@@ -184,6 +184,16 @@ def test_selection_outputs_at_any_address(host, off_cls, off_order, off_score):
         assert got % size == 0
         assert got == want if want % size == 0 else late.pop(want) == (got, 4 * size)      # 4 windows of a 14 x 14 map
     assert not late
+
+
+def test_only_scores_of_the_librarys_own_energies_are_ranked_in_32_bits(host):
+    """A caller's energies may be of any size, wherever their map lies (the library's own is the first buffer of the workspace)."""
+    x, y, ws = host.addr(), host.addr(), host.addr()
+    narrow = []
+    for energy in (None, host.addr(), ws):
+        assert host.run_block(host.block(), x, y, ws, energy=energy) == 0
+        narrow.append(SelectArgs.in_dll(host.L, "last_select").narrow)
+    assert narrow == [True, False, False]
 
 
 def test_misaligned_arrays_are_refused_before_a_launch(host):
