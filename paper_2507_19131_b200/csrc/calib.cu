@@ -380,6 +380,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) k_cal_gemm(const __grid_constan
 #pragma unroll 1
         for (int g = 0; g < CG_EPI_COLS; g += 8) {
           int32_t S[CAL_SLICES][8];
+          __syncwarp();                                           // rows that are not stored left the pass before early
 #pragma unroll
           for (int s = 0; s < CAL_SLICES; ++s) tmem_ld(taddr + (uint32_t)(s * CG_BN + g), S[s]);
 #pragma unroll

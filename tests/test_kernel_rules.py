@@ -45,3 +45,14 @@ def test_the_lanes_of_a_warp_give_up_together():
     wait = open(os.path.join(CSRC, "tc_ptx.cuh")).read()
     wait = wait[wait.index("bool mbar_wait_warp("):wait.index("void tma_load_2d")]
     assert len(re.findall(r"if \(.*return", wait)) == len(re.findall(r"__(?:all|any)_sync\(0xffffffffu", wait)) == 3
+
+
+def test_tensor_memory_is_read_by_converged_warps():
+    """tcgen05.ld is for all lanes of a warp at once.  The calibration products' epilogue loops over it, and lanes whose row is not
+    stored leave a pass early, so every pass begins with a __syncwarp."""
+    calib = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "calib.cu")).read())
+    reads = [m.start() for m in re.finditer(r"\btmem_ld\(", calib)]
+    assert len(reads) == 1
+    loop = calib[calib.index("for (int g = 0; g < CG_EPI_COLS; g += 8) {"):]
+    assert "continue;" in loop[:loop.index("observe_warp(")]
+    assert re.match(r"[^{]*\{\s*int32_t S\[CAL_SLICES\]\[8\];\s*__syncwarp\(\);\s*#pragma unroll\s*for [^;]*;[^;]*;[^;]*tmem_ld\(", loop)
