@@ -212,6 +212,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
           }
           w[i][h] = clamp_pack4<MODE != EPI_FC1>(c[0], c[1], c[2], c[3], zp2, qmax2);
         }
+        if (TAPS) __syncwarp();                              // (rows that exist were tapped)
       }
       // Half of the columns of half of the rows again by the contract's own operations: where some value of the warp is too close
       // to a rounding boundary, and all of them where the patterns above do not hold.  A sixth of the chunks at A8 has a value
@@ -241,6 +242,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (8 * i + rsub < rows_left) store_codes8(out_ptr + i * (long)row_step + ch * out_step, w[i][0], w[i][1], cbits);
+      __syncwarp();                                          // tensor memory is read by all lanes at once
     }
     return true;
   }
@@ -308,6 +310,7 @@ __device__ __forceinline__ bool epilogue_warp_tile(const GemmBranch& br, const E
         *reinterpret_cast<float4*>(dst_ptr[i] + ch * col_step) = make_float4(lo.x, lo.y, hi.x, hi.y);
       }
       if (MODE != EPI_MERGE) fetch(ch + RES_SLOTS);              // the slot just read is free again
+      __syncwarp();                                              // (lanes without a place to store to went another way)
     };
     // two chunks in turn, each requested one ahead
     int32_t even[16], odd[16];

@@ -48,11 +48,16 @@ def test_the_lanes_of_a_warp_give_up_together():
 
 
 def test_tensor_memory_is_read_by_converged_warps():
-    """tcgen05.ld is for all lanes of a warp at once.  The calibration products' epilogue loops over it, and lanes whose row is not
-    stored leave a pass early, so every pass begins with a __syncwarp."""
-    calib = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "calib.cu")).read())
-    reads = [m.start() for m in re.finditer(r"\btmem_ld\(", calib)]
-    assert len(reads) == 1
+    """tcgen05.ld and its wait are for all lanes of a warp at once.  Lanes whose row is not stored leave a pass of an epilogue's loop
+    early, so there is a __syncwarp between that and the next read."""
+    def source(name):
+        return re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    calib = source("calib.cu")
+    assert len(re.findall(r"\btmem_ld\(", calib)) == 1
     loop = calib[calib.index("for (int g = 0; g < CG_EPI_COLS; g += 8) {"):]
     assert "continue;" in loop[:loop.index("observe_warp(")]
     assert re.match(r"[^{]*\{\s*int32_t S\[CAL_SLICES\]\[8\];\s*__syncwarp\(\);\s*#pragma unroll\s*for [^;]*;[^;]*;[^;]*tmem_ld\(", loop)
+    gemm = source("gemm_epilogue.cuh")
+    assert re.search(r"clamp_pack4<MODE != EPI_FC1>\([^;]*;\s*\}\s*if \(TAPS\) __syncwarp\(\);\s*\}", gemm)          # taps of a half
+    assert re.search(r"rows_left\) store_codes8\([^;]*;\s*__syncwarp\(\);\s*\}\s*return true;", gemm)                 # code outputs
+    assert re.search(r"if \(!dst_ptr\[i\]\) continue;", gemm) and re.search(r"fetch\(ch \+ RES_SLOTS\);\s*__syncwarp\(\);\s*\};", gemm)
