@@ -46,7 +46,7 @@ def test_window_selection_by_a_callers_large_energies(orc, mq, ctx, H, W, revers
 
 @pytest.mark.parametrize("dim,windows", [(32, (27, 28)), (32, (28, 28)), (64, (28, 28)), (96, (28, 28)), (1024, (1, 2))])
 def test_gemm_tilings_around_their_limits(orc, mq, ctx, dim, windows):
-    """Row tiles just below and above the limit of the 16 epilogue warps, tile widths 32 to 256, more accumulators than
+    """Just fewer and just more than two row tiles per SM, tile widths 32 to 256, more accumulators than
     tiles, remainders in the last row tile of both branches."""
     blk = synth.make_block(np.random.default_rng(dim), dim, dim // 32, 0, 4, 8, 4, share_bias=False)
     x = synth.input_student_t(dim, 1, 7 * windows[0], 7 * windows[1] - 2, dim)
